@@ -1,5 +1,6 @@
 // Context, workspace, error reporting and the exclusive scan used by the
 // binning stages.
+#include <math.h>
 #include <stdarg.h>
 #include <stdio.h>
 #include <string.h>
@@ -301,6 +302,52 @@ __global__ void k_selftest_wait(long long cycles, DevStatus *st) {
     }
 }
 
+// Computed once per process in the host's long double (one eighth of the
+// circle, the rest by symmetry), rounded to each type.
+static const FftTables &host_fft_tables() {
+    static const FftTables *t = [] {
+        FftTables *h = new FftTables;
+        constexpr int n = 2048;
+        const long double tau = 6.283185307179586476925286766559005768L, q62 = 4611686018427387904.0L;
+        for (int k = 0; k < n; ++k) {
+            const int oct = k / (n / 8), r = oct & 1 ? n / 8 - k % (n / 8) : k % (n / 8);
+            const long double c0 = cosl(tau * r / n), s0 = sinl(tau * r / n);
+            // octants 1, 2, 5, 6 swap sine and cosine; 2 to 5 have a negative cosine, 4 to 7 a negative sine
+            const bool swap = ((oct + 1) & 2) != 0;
+            const long double c = (oct >= 2 && oct <= 5 ? -1.0L : 1.0L) * (swap ? s0 : c0);
+            const long double s = (oct >= 4 ? -1.0L : 1.0L) * (swap ? c0 : s0);
+            h->roots32[k] = make_float2((float)c, (float)-s);
+            h->trig32[k] = make_float2((float)c, (float)s);
+            h->trig64[k] = make_double2((double)c, (double)s);
+            const long long v[2] = {llrintl(c * q62), llrintl(-s * q62)};
+            int b[4];
+            for (int a = 0; a < 2; ++a) {
+                b[2 * a] = (int)((v[a] + (1LL << 31)) >> 32);
+                b[2 * a + 1] = (int)(v[a] - (long long)b[2 * a] * (1LL << 32));
+            }
+            h->roots_fx[k] = make_int4(b[0], b[1], b[2], b[3]);
+        }
+        return h;
+    }();
+    return *t;
+}
+
+cudaError_t make_fft_tables(FftTables **out, cudaStream_t s) {
+    *out = nullptr;
+    const FftTables &h = host_fft_tables();
+    void *d = nullptr;
+    cudaError_t e = cudaMalloc(&d, sizeof(FftTables));
+    if (e != cudaSuccess) return e;
+    e = cudaMemcpyAsync(d, &h, sizeof(FftTables), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) {
+        cudaFree(d);
+        return e;
+    }
+    *out = (FftTables *)d;
+    return cudaSuccess;
+}
+
 static cudaEvent_t take_event(ib_ctx *c) {
     if (!c->pool.empty()) {
         cudaEvent_t e = c->pool.back();
@@ -386,6 +433,16 @@ int ib_ctx_create(ib_ctx **ctx, size_t workspace_bytes) {
         cudaFree(c->ws);
         delete c;
         return set_error(IB_ERR_CUDA, "context stream/event creation failed");
+    }
+    if (make_fft_tables(&c->fft_tab, c->fork_stream) != cudaSuccess) {
+        cudaGetLastError();
+        for (cudaEvent_t ev : c->fork_ev) cudaEventDestroy(ev);
+        cudaStreamDestroy(c->fork_stream);
+        cudaFreeHost(c->h_nlev);
+        cudaFree(c->status);
+        cudaFree(c->ws);
+        delete c;
+        return set_error(IB_ERR_CUDA, "transform tables");
     }
     c->pass_kernels = IB_PASSES_AUTO;
     c->vol_split = 0;  // automatic
@@ -511,6 +568,7 @@ int ib_ctx_destroy(ib_ctx *c) {
         if (c->stage_ev[k]) cudaEventDestroy(c->stage_ev[k]);
     }
     cudaFree(c->ws);
+    cudaFree(c->fft_tab);
     cudaFree(c->status);
     delete c;
     return IB_OK;

@@ -1,0 +1,302 @@
+// Line FFTs of the fluid step in registers, for FP32 and for FP64 fields.
+//
+// Form: Stockham passes of radix up to E with E complex points per thread
+// (Govindaraju et al. 2008, "High performance discrete Fourier transforms on
+// graphics processors"): the thread t of a line holds the points t + TPL m
+// (TPL = N / E threads per line) before and after the transform, and the
+// passes exchange through shared memory.  Two arithmetics:
+//
+//  * Fp32: float pairs.
+//  * Fx64: 64-bit block fixed point, the transform of FP64 fields.  GB300
+//    issues 2 FP64 operations per clock and SM (a warp instruction holds the
+//    pipe for 16 clocks) but 64 or more integer ones.  A line's components
+//    are scaled by one power of two, so that the largest has B = 62 - log2 N
+//    bits and no sum of the transform can overflow, and rounded to integers;
+//    butterflies are then exact 64-bit additions, and only the products with
+//    twiddle factors (Q62) round, to one unit of 2^-B of the line's largest
+//    component, where an FP64 transform rounds every addition to 2^-53 of its
+//    own, up to sqrt(N) times larger, result.  The result goes back to FP64
+//    with one rounding.  A line with a NaN or an infinity gives NaN.
+#pragma once
+
+#include "gbib_internal.cuh"
+
+namespace gbib {
+
+constexpr int kRootBits = 11;            // the tables hold the 2048th roots of unity
+constexpr int kRoots = 1 << kRootBits;
+
+// ---------------------------------------------------------------------------
+// arithmetic
+// ---------------------------------------------------------------------------
+struct Fx64On32;
+struct Fp32 {
+    using Pressure = Fx64On32;           // the pressure solve's x passes
+    using Real = float;                  // the field's element
+    using C = float2;                    // a point in registers
+    using Mem = float2;                  // a point in memory
+    using W = float2;                    // a twiddle factor
+    static constexpr bool kFixed = false;
+    static __host__ __device__ constexpr int points(int logN) {
+        return logN == 7 || logN == 8 || logN == 10 ? 16 : 8;
+    }
+    // adjacent lines of one CTA in the strided passes: 128-byte rows (64 for
+    // long lines, which fill the CTA's threads and shared memory)
+    static __host__ __device__ constexpr int lanes(int logN) { return logN >= 9 ? 8 : 16; }
+};
+struct Fx64 {
+    using Pressure = Fx64;
+    using Real = double;
+    using C = longlong2;
+    using Mem = double2;
+    using W = int4;                      // (re hi, re lo, im hi, im lo) in Q62, signed halves
+    static constexpr bool kFixed = true;
+    static __host__ __device__ constexpr int points(int) { return 8; }
+    static __host__ __device__ constexpr int lanes(int logN) { return logN >= 10 ? 4 : 8; }
+};
+
+// Fx64's arithmetic on FP32 values: the x passes of the FP32 pressure solve.
+// They bring the error of the pressure's nearly checkerboard modes down to
+// what the right-hand side's own rounding leaves (the first pass spreads its
+// rounding over all modes, and these are amplified most), and the last pass
+// adds none to the gradient.
+struct Fx64On32 : Fx64 {
+    using Real = float;
+    using Mem = float2;
+};
+
+__device__ __forceinline__ float2 operator+(float2 a, float2 b) { return {a.x + b.x, a.y + b.y}; }
+__device__ __forceinline__ float2 operator-(float2 a, float2 b) { return {a.x - b.x, a.y - b.y}; }
+__device__ __forceinline__ longlong2 operator+(longlong2 a, longlong2 b) { return {a.x + b.x, a.y + b.y}; }
+__device__ __forceinline__ longlong2 operator-(longlong2 a, longlong2 b) { return {a.x - b.x, a.y - b.y}; }
+
+// a times -i (forward) or +i (inverse)
+template <bool INV, typename C> __device__ __forceinline__ C rot90(C a) {
+    return INV ? C{-a.y, a.x} : C{a.y, -a.x};
+}
+
+// Balanced halves: a = hi 2^32 + lo with lo signed.
+struct Halves {
+    int hi, lo;
+};
+__device__ __forceinline__ Halves halves(long long a) {
+    const int lo = (int)(unsigned)a;
+    return {(int)(a >> 32) + (int)((unsigned)lo >> 31), lo};
+}
+// S 2^64 + T 2^32 (T with its rounding half) as a Q62 product's integer
+__device__ __forceinline__ long long q62(long long S, long long T) { return (S << 2) + (T >> 30); }
+constexpr long long kQ62Half = 1LL << 29;
+
+__device__ __forceinline__ long long fx_mul(long long a, int bh, int bl) {
+    const Halves h = halves(a);
+    return q62((long long)h.hi * bh, (long long)h.hi * bl + ((long long)h.lo * bh + kQ62Half));
+}
+
+template <bool INV> __device__ __forceinline__ float2 cmulw(float2 a, float2 w) {
+    const float s = INV ? -w.y : w.y;
+    return {fmaf(a.x, w.x, -(a.y * s)), fmaf(a.x, s, a.y * w.x)};
+}
+template <bool INV> __device__ __forceinline__ longlong2 cmulw(longlong2 a, int4 w) {
+    const Halves x = halves(a.x), y = halves(a.y);
+    const int ih = INV ? -w.z : w.z, il = INV ? -w.w : w.w, nh = -ih, nl = -il;
+    const long long sr = (long long)x.hi * w.x + (long long)y.hi * nh;
+    const long long si = (long long)x.hi * ih + (long long)y.hi * w.x;
+    const long long tr = (long long)x.hi * w.y + ((long long)x.lo * w.x + ((long long)y.hi * nl +
+                         ((long long)y.lo * nh + kQ62Half)));
+    const long long ti = (long long)x.hi * il + ((long long)x.lo * ih + ((long long)y.hi * w.y +
+                         ((long long)y.lo * w.x + kQ62Half)));
+    return {q62(sr, tr), q62(si, ti)};
+}
+
+// a times the real constants cos(pi/4), cos(pi/8), sin(pi/8) in Q62 halves
+struct Q62Const {
+    int hi, lo;
+};
+constexpr Q62Const q62_const(long long v) {
+    return {(int)((v + 0x80000000LL) >> 32), (int)(v - (((v + 0x80000000LL) >> 32) << 32))};
+}
+constexpr long long kHalfRoot = 3260954456333195553LL;  // round(2^62 / sqrt 2)
+__device__ __forceinline__ float mul_half_root(float a) { return a * 0.70710678118654752f; }
+__device__ __forceinline__ long long mul_half_root(long long a) {
+    constexpr Q62Const c = q62_const(kHalfRoot);
+    return fx_mul(a, c.hi, c.lo);
+}
+
+// ---------------------------------------------------------------------------
+// butterflies, natural order in and out
+// ---------------------------------------------------------------------------
+template <bool INV, typename C> __device__ __forceinline__ void radix2(C &a, C &b) {
+    const C t = a - b;
+    a = a + b;
+    b = t;
+}
+template <bool INV, typename C> __device__ __forceinline__ void radix4(C &x0, C &x1, C &x2, C &x3) {
+    const C a = x0 + x2, b = x0 - x2, c = x1 + x3, d = rot90<INV>(x1 - x3);
+    x0 = a + c;
+    x1 = b + d;
+    x2 = a - c;
+    x3 = b - d;
+}
+// times exp(-+ i pi / 4) and exp(-+ 3 i pi / 4)
+template <bool INV, typename C> __device__ __forceinline__ C rot45(C a) {
+    return INV ? C{mul_half_root(a.x - a.y), mul_half_root(a.x + a.y)}
+               : C{mul_half_root(a.x + a.y), mul_half_root(a.y - a.x)};
+}
+template <bool INV, typename C> __device__ __forceinline__ C rot135(C a) { return rot90<INV>(rot45<INV>(a)); }
+
+template <bool INV, typename C> __device__ __forceinline__ void radix8(C *x) {
+    radix4<INV>(x[0], x[2], x[4], x[6]);
+    radix4<INV>(x[1], x[3], x[5], x[7]);
+    const C o1 = rot45<INV>(x[3]), o2 = rot90<INV>(x[5]), o3 = rot135<INV>(x[7]);
+    const C e0 = x[0], e1 = x[2], e2 = x[4], e3 = x[6], o0 = x[1];
+    x[0] = e0 + o0, x[4] = e0 - o0;
+    x[1] = e1 + o1, x[5] = e1 - o1;
+    x[2] = e2 + o2, x[6] = e2 - o2;
+    x[3] = e3 + o3, x[7] = e3 - o3;
+}
+// FP32 only: two radix-4 stages with the 16th roots between them
+template <bool INV> __device__ __forceinline__ void radix16(float2 *x) {
+    constexpr float c = 0.92387953251128674f, s = 0.38268343236508977f;
+    const float2 w1 = {c, -s}, w3 = {s, -c}, w9 = {-c, s};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) radix4<INV>(x[k], x[k + 4], x[k + 8], x[k + 12]);
+    // point n2 + 4 k1 holds the sub-transform k1 of the residue n2: times w16^(n2 k1)
+    x[5] = cmulw<INV>(x[5], w1);
+    x[6] = rot45<INV>(x[6]);
+    x[7] = cmulw<INV>(x[7], w3);
+    x[9] = rot45<INV>(x[9]);
+    x[10] = rot90<INV>(x[10]);
+    x[11] = rot135<INV>(x[11]);
+    x[13] = cmulw<INV>(x[13], w3);
+    x[14] = rot135<INV>(x[14]);
+    x[15] = cmulw<INV>(x[15], w9);
+    float2 y[16];
+#pragma unroll
+    for (int k1 = 0; k1 < 4; ++k1) {
+        radix4<INV>(x[4 * k1], x[4 * k1 + 1], x[4 * k1 + 2], x[4 * k1 + 3]);
+#pragma unroll
+        for (int k2 = 0; k2 < 4; ++k2) y[k1 + 4 * k2] = x[4 * k1 + k2];
+    }
+#pragma unroll
+    for (int k = 0; k < 16; ++k) x[k] = y[k];
+}
+template <int R, bool INV, typename C> __device__ __forceinline__ void radix(C *x) {
+    if constexpr (R == 2) radix2<INV>(x[0], x[1]);
+    else if constexpr (R == 4) radix4<INV>(x[0], x[1], x[2], x[3]);
+    else if constexpr (R == 8) radix8<INV>(x);
+    else radix16<INV>(x);
+}
+
+// ---------------------------------------------------------------------------
+// a line's transform: v[m] is the point t + TPL m on entry and on exit
+// ---------------------------------------------------------------------------
+// `at(p)`: index of the line's point p in the CTA's shared buffer (every
+// thread of the CTA calls this together).
+template <class A, int LOGN, bool INV, int NS, typename At>
+__device__ __forceinline__ void fft_passes(typename A::C *v, int t, typename A::C *sm, At at,
+                                           const typename A::W *__restrict__ roots) {
+    using C = typename A::C;
+    constexpr int N = 1 << LOGN, E = A::points(LOGN), TPL = N / E, R = N / NS < E ? N / NS : E, B = E / R;
+#pragma unroll
+    for (int b = 0; b < B; ++b) {
+        const int j = t + b * TPL, k = j & (NS - 1);
+        C x[R];
+#pragma unroll
+        for (int i = 0; i < R; ++i) x[i] = v[b + i * B];
+        if constexpr (NS > 1) {
+#pragma unroll
+            for (int i = 1; i < R; ++i) x[i] = cmulw<INV>(x[i], __ldg(roots + k * i * (kRoots / (NS * R))));
+        }
+        radix<R, INV>(x);
+#pragma unroll
+        for (int i = 0; i < R; ++i) v[b + i * B] = x[i];
+    }
+    if constexpr (NS * R < N) {
+        __syncthreads();
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+            const int j = t + b * TPL, k = j & (NS - 1), p = (j - k) * R + k;
+#pragma unroll
+            for (int i = 0; i < R; ++i) sm[at(p + i * NS)] = v[b + i * B];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int m = 0; m < E; ++m) v[m] = sm[at(t + TPL * m)];
+        fft_passes<A, LOGN, INV, NS * R>(v, t, sm, at, roots);
+    }
+}
+template <class A, int LOGN, bool INV, typename At>
+__device__ __forceinline__ void fft_line(typename A::C *v, int t, typename A::C *sm, At at,
+                                         const typename A::W *__restrict__ roots) {
+    fft_passes<A, LOGN, INV, 1>(v, t, sm, at, roots);
+}
+
+// ---------------------------------------------------------------------------
+// floating point <-> block fixed point
+// ---------------------------------------------------------------------------
+// A value's magnitude as an ordered integer (for FP64 its high word), and the
+// exponent field of the largest (at least 1).
+__device__ __forceinline__ int magnitude(double x) { return (int)((unsigned)__double2hiint(x) & 0x7fffffffu); }
+__device__ __forceinline__ int magnitude(float x) { return (int)((unsigned)__float_as_int(x) & 0x7fffffffu); }
+template <typename R> __device__ __forceinline__ int exponent_of(int mag) {
+    const int e = mag >> (sizeof(R) == 8 ? 20 : 23);
+    return e ? e : 1;
+}
+
+constexpr int fx_bits(int logN) { return 62 - logN; }
+
+// x 2^(B - (emax - bias + 1)) rounded; emax the line's largest exponent field,
+// bias 1023 or 127.
+template <int B> __device__ __forceinline__ long long fixed_of(unsigned long long m63, int e, int emax, bool neg) {
+    // the mantissa in 63 bits, then right by emax - e + 63 - B >= 1
+    int s = emax - (e ? e : 1) + 63 - B;
+    s = s > 64 ? 64 : s;
+    const unsigned long long r = ((m63 >> (s - 1)) + 1) >> 1;
+    return neg ? -(long long)r : (long long)r;
+}
+template <int B> __device__ __forceinline__ long long to_fixed(double x, int emax) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const int e = (int)(b >> 52) & 0x7ff;
+    return fixed_of<B>(((b & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull)) << 10, e, emax, (long long)b < 0);
+}
+template <int B> __device__ __forceinline__ long long to_fixed(float x, int emax) {
+    const unsigned b = (unsigned)__float_as_int(x);
+    const int e = (int)(b >> 23) & 0xff;
+    return fixed_of<B>((unsigned long long)((b & 0x7fffffu) | (e ? 1u << 23 : 0u)) << 39, e, emax, (int)b < 0);
+}
+
+// The inverse, F 2^(emax - bias + 1 - B); NaN for a line that held a NaN or an
+// infinity.
+template <int B> __device__ __forceinline__ void from_fixed(long long F, int emax, double &out) {
+    const unsigned long long u = F < 0 ? 0ull - (unsigned long long)F : (unsigned long long)F;
+    const int lz = __clzll((long long)u);
+    const unsigned long long n = u << (lz & 63);
+    const unsigned long long m = (n >> 11) + ((n >> 10) & 1ull);  // 53 bits, rounded
+    const int e = 64 - lz + emax - B;                             // biased exponent of the leading bit
+    unsigned long long r = ((unsigned long long)(unsigned)(e - 1) << 52) + m;
+    if (emax == 0x7ff) r = 0x7ff8000000000000ull;
+    else if (u == 0) r = 0;
+    else if (e < 1 || e > 2045) {
+        // at or beyond the ends of the normal range: two scalings
+        const int k = emax - 1022 - B;
+        r = (unsigned long long)__double_as_longlong(ldexp(ldexp((double)(long long)u, k / 2), k - k / 2));
+    }
+    out = __longlong_as_double((long long)(r | ((unsigned long long)F & 0x8000000000000000ull)));
+}
+template <int B> __device__ __forceinline__ void from_fixed(long long F, int emax, float &out) {
+    const unsigned long long u = F < 0 ? 0ull - (unsigned long long)F : (unsigned long long)F;
+    const int lz = __clzll((long long)u);
+    const unsigned long long n = u << (lz & 63);
+    const unsigned m = (unsigned)(n >> 40) + ((unsigned)(n >> 39) & 1u);  // 24 bits, rounded
+    const int e = 64 - lz + emax - B;
+    unsigned r = ((unsigned)(e - 1) << 23) + m;
+    if (emax == 0xff) r = 0x7fc00000u;
+    else if (u == 0) r = 0;
+    else if (e < 1 || e > 253) {
+        const int k = emax - 126 - B;
+        r = (unsigned)__float_as_int(ldexpf(ldexpf((float)(long long)u, k / 2), k - k / 2));
+    }
+    out = __int_as_float((int)(r | (F < 0 ? 0x80000000u : 0u)));
+}
+
+}  // namespace gbib

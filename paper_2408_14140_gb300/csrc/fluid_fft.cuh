@@ -1,0 +1,388 @@
+// The spectral solves of the fluid step: a real field of n0 x n1 x n2 values
+// as its half spectrum in x, n2 planes of n1 rows of n0/2 complex points, and
+// the points kx = n0/2 beside it (n2 rows of n1).  Five passes over these:
+//   x forward (from the real field), y forward,
+//   z: forward, the operator's inverse symbol, inverse -- in one kernel,
+//   y inverse, x inverse (to the real field).
+// Every pass reads and writes each point once, so a field moves 10 times its
+// bytes, half of what a complex field with a zero imaginary part would.
+//
+// x forward takes two rows (planes 2z', 2z'+1) as the real and the imaginary
+// part of one complex line Z and separates their spectra A, B by
+// A(k) = (Z(k) + conj Z(n0-k))/2, B(k) = (Z(k) - conj Z(n0-k))/2i; x inverse
+// puts Z = A + iB together again.
+//
+// Two denser packings measured worse errors in FP32 and were not kept: planes
+// packed through all passes (the symbols of kz and kz + n2/2 applied to the
+// packed spectrum) gave 1.2 to 1.5 times the projection's error of u, and
+// kx = 0 and n0/2 sharing a point up to 4 times its error of p, since the
+// rounding of the large modes then reaches the nearly checkerboard ones, which
+// the pressure solve amplifies by up to 1e5.
+#pragma once
+
+#include "fft_core.cuh"
+
+namespace gbib {
+
+// Operators diagonal in Fourier space.
+enum { kSolveHelmholtz = 0, kSolveDivGrad = 1 };
+struct SymbolArgs {
+    int kind;
+    double scale;  // 1 / (points of the transform) and, for div grad, the constant factor
+    double g;      // Helmholtz: 4 coef / h^2
+};
+
+// The half spectrum of one field: `c` the points kx < n0/2, `ny` those of
+// kx = n0/2; fields follow one another in both.
+template <class A> struct Spectrum {
+    typename A::Mem *c, *ny;
+};
+
+// The launches (one field, or ncomp fields one after another in memory).
+template <class A>
+struct FftGrid {
+    int n[3], log2n[3];
+    const typename A::W *roots;                 // [kRoots]
+    const typename A::Mem *trig;                // [kRoots] (cos, sin)(2 pi k / kRoots)
+};
+
+template <int TPL, bool FAST_T>
+struct LineMax {
+    // The largest of a line's values over its TPL threads.  FAST_T: the
+    // line's threads are neighbours in the CTA; else `lanes` lines interleave.
+    __device__ static __forceinline__ int get(int v, int *slot, int line, int lanes) {
+        if (FAST_T) {
+#pragma unroll
+            for (int o = (TPL < 32 ? TPL : 32) / 2; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+            if (TPL <= 32) return v;
+            if ((threadIdx.x & 31) == 0) atomicMax(slot + line, v);
+        } else {
+            for (int o = lanes; o < 32; o <<= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+            atomicMax(slot + line, v);
+        }
+        __syncthreads();
+        return slot[line];
+    }
+};
+// A thread's points of a line to the transform's arithmetic and back.
+// `slot`: the lines' maxima (zeroed); returns the line's exponent.
+template <class A, int E, int BITS, int TPL, bool FAST_T>
+__device__ __forceinline__ int points_in(const typename A::Mem (&z)[E], typename A::C (&v)[E], int *slot, int line,
+                                         int lanes) {
+    if constexpr (A::kFixed) {
+        int h = 0;
+#pragma unroll
+        for (int m = 0; m < E; ++m) h = max(h, max(magnitude(z[m].x), magnitude(z[m].y)));
+        const int emax = exponent_of<typename A::Real>(LineMax<TPL, FAST_T>::get(h, slot, line, lanes));
+#pragma unroll
+        for (int m = 0; m < E; ++m) v[m] = typename A::C{to_fixed<BITS>(z[m].x, emax), to_fixed<BITS>(z[m].y, emax)};
+        return emax;
+    } else {
+#pragma unroll
+        for (int m = 0; m < E; ++m) v[m] = typename A::C{z[m].x, z[m].y};
+        return 0;
+    }
+}
+template <class A, int BITS> __device__ __forceinline__ typename A::Mem point_out(typename A::C v, int emax) {
+    typename A::Mem z;
+    if constexpr (A::kFixed) {
+        from_fixed<BITS>(v.x, emax, z.x);
+        from_fixed<BITS>(v.y, emax, z.y);
+    } else {
+        z.x = v.x;
+        z.y = v.y;
+    }
+    return z;
+}
+
+// ---- x: the real field's row pairs <-> the half spectrum ----------------------
+enum { kXForward = 0, kXField = 1, kXPressure = 2 };
+
+template <class A, int LOGN> struct XShape {
+    static constexpr int N = 1 << LOGN, E = A::points(LOGN), TPL = N / E;
+    static constexpr int LPC = TPL >= 128 ? 1 : 128 / TPL;  // lines (row pairs) of one CTA
+    static constexpr int T = TPL * LPC;
+    static constexpr int PITCH = N + N / E;                 // one point of padding per E: conflict-free writes
+    static constexpr size_t smem = (size_t)LPC * PITCH * sizeof(typename A::C);
+    static constexpr int BITS = fx_bits(LOGN) - 1;          // one more bit for the sums of the separation
+};
+
+// kXField writes the field; kXPressure writes p' over the old pressure and
+// beside it, for FP64 fields, the difference p_old - p', whose gradient is all
+// the projection needs; for FP32 fields p_old itself, since the difference's
+// rounding would show in u.
+template <class A, int LOGN, int MODE>
+__global__ void __launch_bounds__(XShape<A, LOGN>::T)
+k_fft_x(const typename A::Real *__restrict__ src, Spectrum<A> sp, typename A::Real *__restrict__ dst,
+        typename A::Real *__restrict__ old, int log1, int log2, const typename A::W *__restrict__ roots) {
+    using S = XShape<A, LOGN>;
+    using C = typename A::C;
+    using R = typename A::Real;
+    using Mem = typename A::Mem;
+    constexpr int N = S::N, E = S::E, TPL = S::TPL;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int s_max[S::LPC];
+    C *sm = (C *)smem_raw;
+    const int t = threadIdx.x % TPL, l = threadIdx.x / TPL;
+    const long long line = (long long)blockIdx.x * S::LPC + l;  // z' n1 + y
+    const long long n1 = 1LL << log1, plane = n1 << LOGN;
+    const long long row = ((line >> log1) * 2 * n1 + (line & (n1 - 1))) << LOGN;  // of plane 2z'
+    const long long comp = (long long)blockIdx.y << (LOGN + log1 + log2);
+    Mem *ca = sp.c + ((comp + row) >> 1), *cb = ca + (plane >> 1);  // the two rows' half spectra
+    Mem *na = sp.ny + ((comp + row) >> LOGN), *nb = na + n1;         // and their points n0/2
+    if (A::kFixed && TPL > 32) {
+        if (threadIdx.x < S::LPC) s_max[threadIdx.x] = 0;
+        __syncthreads();
+    }
+    auto at = [l](int p) { return l * S::PITCH + p + p / E; };
+    grid_dep_wait();
+    C v[E];
+    int emax;
+    if constexpr (MODE == kXForward) {
+        Mem z[E];
+#pragma unroll
+        for (int m = 0; m < E; ++m) {
+            const R *r = src + comp + row + t + TPL * m;
+            z[m] = Mem{r[0], r[plane]};
+        }
+        emax = points_in<A, E, S::BITS, TPL, true>(z, v, s_max, l, 0);
+    } else {
+        // Z(k) = A(k) + i B(k), Z(n0 - k) = conj A(k) + i conj B(k); real points
+        // at 0 and n0/2.  The sums are formed in the transform's arithmetic.
+        Mem a[E], b[E];
+        C va[E], vb[E];
+        int h = 0;
+#pragma unroll
+        for (int m = 0; m < E; ++m) {
+            const int p = t + TPL * m, k = m >= E / 2 ? (N - p) & (N / 2 - 1) : p;
+            const bool mid = m == E / 2 && t == 0;
+            a[m] = *(mid ? na : ca + k), b[m] = *(mid ? nb : cb + k);
+            if (mid || p == 0) a[m].y = b[m].y = 0;
+            if (A::kFixed)
+                h = max(h, max(max(magnitude(a[m].x), magnitude(a[m].y)), max(magnitude(b[m].x), magnitude(b[m].y))));
+        }
+        emax = 0;
+        if constexpr (A::kFixed) emax = exponent_of<R>(LineMax<TPL, true>::get(h, s_max, l, 0));
+#pragma unroll
+        for (int m = 0; m < E; ++m) {
+            if constexpr (A::kFixed) {
+                va[m] = C{to_fixed<S::BITS>(a[m].x, emax), to_fixed<S::BITS>(a[m].y, emax)};
+                vb[m] = C{to_fixed<S::BITS>(b[m].x, emax), to_fixed<S::BITS>(b[m].y, emax)};
+            } else {
+                va[m] = C{a[m].x, a[m].y};
+                vb[m] = C{b[m].x, b[m].y};
+            }
+            v[m] = m >= E / 2 ? C{va[m].x + vb[m].y, vb[m].x - va[m].y} : C{va[m].x - vb[m].y, va[m].y + vb[m].x};
+        }
+    }
+    fft_line<A, LOGN, MODE != kXForward>(v, t, sm, at, roots);
+    grid_dep_launch();
+    if constexpr (MODE == kXForward) {
+        // separation: the thread's lower points k < n0/2 and their mirrors from
+        // shared memory; twice A or B comes in (one more bit of the integers)
+        auto put = [&](Mem *at, decltype(v[0].x) x, decltype(v[0].x) y) {
+            const Mem z = point_out<A, S::BITS + 1>(C{x, y}, emax);
+            *at = A::kFixed ? z : Mem{(R)0.5 * z.x, (R)0.5 * z.y};
+        };
+        __syncthreads();
+#pragma unroll
+        for (int m = 0; m < E; ++m)
+            if (m >= E / 2 || m == 0) sm[at(t + TPL * m)] = v[m];
+        __syncthreads();
+#pragma unroll
+        for (int m = 0; m < E / 2; ++m) {
+            const int k = t + TPL * m;
+            const C n = sm[at((N - k) & (N - 1))];
+            put(ca + k, v[m].x + n.x, v[m].y - n.y);
+            put(cb + k, v[m].y + n.y, n.x - v[m].x);
+        }
+        if (t == 0) {
+            const C n = v[E / 2];
+            put(na, n.x + n.x, n.x - n.x);
+            put(nb, n.y + n.y, n.y - n.y);
+        }
+    } else {
+#pragma unroll
+        for (int m = 0; m < E; ++m) {
+            const Mem z = point_out<A, S::BITS>(v[m], emax);
+            const long long i0 = comp + row + t + TPL * m, i1 = i0 + plane;
+            if (MODE == kXPressure) {
+                const R a = dst[i0], b = dst[i1];
+                old[i0] = sizeof(R) == 8 ? a - z.x : a;
+                old[i1] = sizeof(R) == 8 ? b - z.y : b;
+            }
+            dst[i0] = z.x;
+            dst[i1] = z.y;
+        }
+    }
+}
+
+// ---- y: lines of stride n0/2 = 2^logr points, adjacent lines in adjacent threads
+template <class A, int LOGN> struct YShape {
+    static constexpr int N = 1 << LOGN, E = A::points(LOGN), TPL = N / E;
+    static constexpr int L0 = A::lanes(LOGN), LANES = L0 * TPL >= 128 ? L0 : 128 / TPL;
+    static constexpr int T = TPL * LANES;
+    static constexpr size_t smem = (size_t)LANES * N * sizeof(typename A::C);
+};
+
+template <class A, int LOGN, bool INV>
+__global__ void __launch_bounds__(YShape<A, LOGN>::T)
+k_fft_y(Spectrum<A> sp, int logr, int log2, const typename A::W *__restrict__ roots) {
+    using S = YShape<A, LOGN>;
+    using C = typename A::C;
+    constexpr int E = S::E, TPL = S::TPL, LANES = S::LANES;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int s_max[LANES];
+    C *sm = (C *)smem_raw;
+    const int t = threadIdx.x / LANES, l = threadIdx.x % LANES;
+    // LANES lines in (z, kx) order, after them the n2 lines of kx = n0/2
+    const int regular = (1 << (logr + log2)) / LANES;
+    const bool last = (int)blockIdx.x >= regular;
+    const int q = (last ? (int)blockIdx.x - regular : (int)blockIdx.x) * LANES + l;
+    const bool active = !last || q < 1 << log2;
+    const int step = last ? 0 : logr;  // log2 of the points' stride
+    typename A::Mem *cl = last ? sp.ny + ((long long)blockIdx.y << (LOGN + log2)) + ((long long)q << LOGN)
+                               : sp.c + ((long long)blockIdx.y << (LOGN + logr + log2)) +
+                                     ((long long)(q >> logr) << (LOGN + logr)) + (q & ((1 << logr) - 1));
+    if (A::kFixed) {
+        for (int i = threadIdx.x; i < LANES; i += S::T) s_max[i] = 0;
+        __syncthreads();
+    }
+    grid_dep_wait();
+    typename A::Mem z[E];
+#pragma unroll
+    for (int m = 0; m < E; ++m) z[m] = active ? cl[(long long)(t + TPL * m) << step] : typename A::Mem{0, 0};
+    C v[E];
+    const int emax = points_in<A, E, fx_bits(LOGN), TPL, false>(z, v, s_max, l, LANES);
+    auto at = [l](int p) { return p * LANES + l; };
+    fft_line<A, LOGN, INV>(v, t, sm, at, roots);
+    grid_dep_launch();
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+        z[m] = point_out<A, fx_bits(LOGN)>(v[m], emax);
+        if (active) cl[(long long)(t + TPL * m) << step] = z[m];
+    }
+}
+
+// ---- z: forward, symbol, inverse --------------------------------------------
+template <class A, int LOGN> struct ZShape {
+    static constexpr int N = 1 << LOGN, E = A::points(LOGN), TPL = N / E;
+    static constexpr int L0 = A::lanes(LOGN), LANES = L0 * TPL >= 128 ? L0 : 128 / TPL;
+    static constexpr int T = TPL * LANES;
+    static constexpr size_t points = (size_t)LANES * N * sizeof(typename A::C);
+    static constexpr size_t smem = points + (size_t)(N / 2 + 1) * LANES * sizeof(typename A::Real);
+};
+
+// The inverse symbol times the scale at squared sines and cosines of the half angles.
+template <typename R>
+__device__ __forceinline__ R inverse_symbol(const SymbolArgs &sy, R sx, R cx, R sy2, R cy, R sz, R cz) {
+    if (sy.kind == kSolveHelmholtz) return (R)sy.scale / fma((R)sy.g, sx + sy2 + sz, (R)1);
+    // D G's symbol over -4/h^2, zero on its null modes
+    const R d = sx * cy * cz + sy2 * cx * cz + sz * cx * cy;
+    return d <= (R)3e-13 ? (R)0 : (R)sy.scale / d;
+}
+
+template <class A, int LOGN>
+__global__ void __launch_bounds__(ZShape<A, LOGN>::T)
+k_fft_z(Spectrum<A> sp, int logr, int log1, SymbolArgs sy, const typename A::W *__restrict__ roots,
+        const typename A::Mem *__restrict__ trig) {
+    using S = ZShape<A, LOGN>;
+    using C = typename A::C;
+    using R = typename A::Real;
+    using Mem = typename A::Mem;
+    constexpr int N = S::N, E = S::E, TPL = S::TPL, LANES = S::LANES;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int s_max[2][LANES];
+    C *sm = (C *)smem_raw;
+    R *fs = (R *)(smem_raw + S::points);  // [N/2 + 1][LANES] inverse symbols (even in kz)
+    const int l = threadIdx.x % LANES, t = threadIdx.x / LANES;
+    // LANES lines in (ky, kx) order, after them the n1 lines of kx = n0/2
+    const int regular = (1 << (logr + log1)) / LANES;
+    const bool last = (int)blockIdx.x >= regular;
+    const int q = (last ? (int)blockIdx.x - regular : (int)blockIdx.x) * LANES + l;
+    const bool active = !last || q < 1 << log1;
+    const int kx = last ? 1 << logr : q & ((1 << logr) - 1), ky = last ? q & ((1 << log1) - 1) : q >> logr;
+    const int shift = last ? log1 : logr + log1;  // log2 of the points' stride
+    Mem *cl = (last ? sp.ny : sp.c) + ((long long)blockIdx.y << (LOGN + shift)) + q;
+    if (A::kFixed)
+        for (int i = threadIdx.x; i < 2 * LANES; i += S::T) (&s_max[0][0])[i] = 0;
+    {
+        // the thread's lane's symbol at kz = t, t + TPL, ... <= n2/2
+        const Mem hx = __ldg(trig + kx * (kRoots / 4 >> logr)), hy = __ldg(trig + ky * (kRoots / 2 >> log1));
+        const R sx = hx.y * hx.y, cx = hx.x * hx.x, s1 = hy.y * hy.y, c1 = hy.x * hy.x;
+        for (int kz = t; kz <= N / 2; kz += TPL) {
+            const Mem hz = __ldg(trig + kz * (kRoots / 2 / N));
+            fs[kz * LANES + l] = inverse_symbol<R>(sy, sx, cx, s1, c1, hz.y * hz.y, hz.x * hz.x);
+        }
+    }
+    if (A::kFixed) __syncthreads();
+    grid_dep_wait();
+    Mem z[E];
+#pragma unroll
+    for (int m = 0; m < E; ++m) z[m] = active ? cl[(long long)(t + TPL * m) << shift] : Mem{0, 0};
+    C v[E];
+    int emax = points_in<A, E, fx_bits(LOGN), TPL, false>(z, v, s_max[0], l, LANES);
+    auto at = [l](int p) { return p * LANES + l; };
+    fft_line<A, LOGN, false>(v, t, sm, at, roots);
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+        z[m] = point_out<A, fx_bits(LOGN)>(v[m], emax);
+    }
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+        const int k = t + TPL * m;
+        const R f = fs[(k <= N / 2 ? k : N - k) * LANES + l];
+        z[m] = Mem{f * z[m].x, f * z[m].y};
+    }
+    emax = points_in<A, E, fx_bits(LOGN), TPL, false>(z, v, s_max[1], l, LANES);
+    fft_line<A, LOGN, true>(v, t, sm, at, roots);
+    grid_dep_launch();
+    if (active) {
+#pragma unroll
+        for (int m = 0; m < E; ++m) {
+            z[m] = point_out<A, fx_bits(LOGN)>(v[m], emax);
+            cl[(long long)(t + TPL * m) << shift] = z[m];
+        }
+    }
+}
+
+// ---- launches (defined per arithmetic in their own translation units) --------
+template <class A> cudaError_t fft_x(int mode, const FftGrid<A> &g, int ncomp, const typename A::Real *src,
+                                     Spectrum<A> sp, typename A::Real *dst, typename A::Real *old, cudaStream_t s);
+template <class A> cudaError_t fft_y(bool inverse, const FftGrid<A> &g, int ncomp, Spectrum<A> sp, cudaStream_t s);
+template <class A> cudaError_t fft_z(const FftGrid<A> &g, int ncomp, Spectrum<A> sp, const SymbolArgs &sy,
+                                     cudaStream_t s);
+
+template <typename Kern, typename... Args>
+inline cudaError_t launch_fft(Kern kern, dim3 grid, int threads, size_t smem, cudaStream_t s, Args... args) {
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    return launch_pdl(kern, grid, dim3(threads), smem, s, args...);
+}
+
+template <class A, int LOGN>
+cudaError_t launch_x(int mode, const FftGrid<A> &g, int ncomp, const typename A::Real *src, Spectrum<A> sp,
+                     typename A::Real *dst, typename A::Real *old, cudaStream_t s) {
+    using S = XShape<A, LOGN>;
+    const dim3 grid(g.n[1] * (g.n[2] / 2) / S::LPC, ncomp);
+    auto k = mode == kXForward ? k_fft_x<A, LOGN, kXForward>
+                               : (mode == kXField ? k_fft_x<A, LOGN, kXField> : k_fft_x<A, LOGN, kXPressure>);
+    return launch_fft(k, grid, S::T, S::smem, s, src, sp, dst, old, g.log2n[1], g.log2n[2], g.roots);
+}
+template <class A, int LOGN>
+cudaError_t launch_y(bool inverse, const FftGrid<A> &g, int ncomp, Spectrum<A> sp, cudaStream_t s) {
+    using S = YShape<A, LOGN>;
+    const dim3 grid(g.n[0] / 2 * g.n[2] / S::LANES + (g.n[2] + S::LANES - 1) / S::LANES, ncomp);
+    auto k = inverse ? k_fft_y<A, LOGN, true> : k_fft_y<A, LOGN, false>;
+    return launch_fft(k, grid, S::T, S::smem, s, sp, g.log2n[0] - 1, g.log2n[2], g.roots);
+}
+template <class A, int LOGN>
+cudaError_t launch_z(const FftGrid<A> &g, int ncomp, Spectrum<A> sp, const SymbolArgs &sy, cudaStream_t s) {
+    using S = ZShape<A, LOGN>;
+    const dim3 grid(g.n[0] / 2 * g.n[1] / S::LANES + (g.n[1] + S::LANES - 1) / S::LANES, ncomp);
+    return launch_fft(k_fft_z<A, LOGN>, grid, S::T, S::smem, s, sp, g.log2n[0] - 1, g.log2n[1], sy, g.roots, g.trig);
+}
+
+}  // namespace gbib

@@ -10,337 +10,342 @@
 //   L_c u (cells) = 7-point Laplacian per component
 // The implicit solves -- (I - nu dt/2 L_c) for Crank-Nicolson viscosity and
 // D G for the pressure -- are diagonal in Fourier space on a periodic grid
-// and are done exactly with a radix-2 FFT along each axis (Stockham
-// autosort in shared memory, one CTA per group of lines), so every grid axis
-// must be a power of two.  Convection div(u u)^{n+1/2} is a second-order
+// and are done exactly with FFTs (fluid_fft.cuh), so every grid axis must be
+// a power of two.  Convection div(u u)^{n+1/2} is a second-order
 // Godunov edge extrapolation: per face, states from both neighbours by a
 // Taylor step along monotonized-central limited slopes, the normal velocity
 // from the Burgers Riemann solution of the two normal states, the state
 // upwinded by it, and the flux difference over the cell.
-#include "gbib_internal.cuh"
+//
+// The stencil kernels march along z: a thread owns a column (i, j) of a chunk
+// of planes, keeps what the next plane needs again in registers and reads the
+// in-plane neighbours through L1.  All sizes are powers of two, so periodic
+// indices are masks.
+#include "fluid_fft.cuh"
 
 namespace gbib {
 
-template <typename T> struct Cx;
-template <> struct Cx<float> { using type = float2; };
-template <> struct Cx<double> { using type = double2; };
+struct LevelDims {
+    int n0, n1, n2, zc;  // zc: planes of one CTA's chunk
+};
 
-template <typename C> __device__ __forceinline__ C cadd(C a, C b) { return {a.x + b.x, a.y + b.y}; }
-template <typename C> __device__ __forceinline__ C csub(C a, C b) { return {a.x - b.x, a.y - b.y}; }
-template <typename C> __device__ __forceinline__ C cmul(C a, C b) {
-    return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};
+// The thread's column and its chunk of planes.
+struct Column {
+    int i, j, k0, k1;
+    __device__ __forceinline__ Column(const LevelDims &d)
+        : i(blockIdx.x * blockDim.x + threadIdx.x), j(blockIdx.y * blockDim.y + threadIdx.y), k0(blockIdx.z * d.zc),
+          k1(blockIdx.z * d.zc + d.zc) {}
+};
+
+// Half the monotonized-central slope from the differences a (below) and b
+// (above) and their sum s: min(|a|, |b|, |s|/4) with their sign, 0 at extrema.
+__device__ __forceinline__ float half_slope(float a, float b, float s) {
+    const float m = fminf(fminf(fabsf(a), fabsf(b)), 0.25f * fabsf(s));
+    return a * b > 0.0f ? copysignf(m, s) : 0.0f;
 }
-
-__device__ __forceinline__ void sincos_pi(float x, float *s, float *c) { sincospif(x, s, c); }
-__device__ __forceinline__ void sincos_pi(double x, double *s, double *c) { sincospi(x, s, c); }
-
-constexpr int kFftThreads = 256;
-constexpr int kFftPoints = 2048;  // points of one CTA (lines x length)
-
-// Lines of one CTA along `axis`.
-__host__ __device__ inline int fft_lines(int N, int axis, int n0) {
-    int L = kFftPoints / N;
-    L = L < 1 ? 1 : (L > 8 ? 8 : L);
-    if (axis > 0 && L > n0) L = n0;
-    return L;
+// For FP64 the comparisons run on the integer pipe: the order of non-negative
+// doubles is that of their bits.
+__device__ __forceinline__ double half_slope(double a, double b, double s) {
+    const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b), is = __double_as_longlong(0.25 * s);
+    constexpr long long mag = 0x7fffffffffffffffLL;
+    const long long m = min(min(ia & mag, ib & mag), is & mag);
+    return (ia ^ ib) < 0 ? 0.0 : __longlong_as_double(m | (ia & ~mag));
 }
+__device__ __forceinline__ bool positive(float x) { return x > 0.0f; }
+__device__ __forceinline__ bool positive(double x) { return __double_as_longlong(x) > 0; }
+__device__ __forceinline__ bool negative(float x) { return x < 0.0f; }
+__device__ __forceinline__ bool negative(double x) { return 2 * __double_as_longlong(x) != 0 && __double_as_longlong(x) < 0; }
 
-// One radix-2 Stockham FFT of length N = 2^logN along `axis` for L lines per
-// CTA: stage t combines x[q + s p] and x[q + s (p + m)] (s = 2^t,
-// m = N / 2^(t+1)) into y[q + 2 s p] = a + b and y[q + s (2p + 1)] = (a - b) w^p
-// with w = exp(-+ 2 pi i s / N).  inverse: conjugate twiddles, no scaling.
+// Fluxes of all three components through a face with states l and r, the
+// normal component being a (Burgers Riemann solution, upwinded).
 template <typename T>
-__global__ void __launch_bounds__(kFftThreads) k_fft_axis(typename Cx<T>::type *data, int n0, int n1, int n2,
-                                                          int axis, int logN, int inverse) {
-    using C = typename Cx<T>::type;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int N = 1 << logN;
-    const int L = fft_lines(N, axis, n0);
-    C *buf0 = (C *)smem_raw;
-    C *buf1 = buf0 + (size_t)L * N;
-    C *tw = buf1 + (size_t)L * N;
-    const long long stride = axis == 0 ? 1 : (axis == 1 ? (long long)n0 : (long long)n0 * n1);
-    const long long nlines = (long long)n0 * n1 * n2 / N;
-    for (int k = threadIdx.x; k < N / 2; k += blockDim.x) {
-        T s, c;
-        sincos_pi((T)(2 * k) / (T)N, &s, &c);
-        tw[k] = C{c, inverse ? s : -s};
-    }
-    for (long long l0 = (long long)blockIdx.x * L; l0 < nlines; l0 += (long long)gridDim.x * L) {
-        // base offset of line l0 + l
-        auto base = [&](long long l) -> long long {
-            if (axis == 0) return l * n0;
-            if (axis == 1) return (l / n0) * (long long)n0 * n1 + l % n0;
-            return l;  // axis 2: l = y n0 + x
-        };
-        __syncthreads();
-        for (int t = threadIdx.x; t < L * N; t += blockDim.x) {
-            // axis 0: consecutive threads walk one line; else consecutive lines (adjacent x)
-            const int l = axis == 0 ? t / N : t % L, j = axis == 0 ? t % N : t / L;
-            buf0[l * N + j] = data[base(l0 + l) + j * stride];
-        }
-        __syncthreads();
-        C *x = buf0, *y = buf1;
-        for (int st = 0; st < logN; ++st) {
-            const int s = 1 << st, m = N >> (st + 1);
-            for (int t = threadIdx.x; t < L * (N / 2); t += blockDim.x) {
-                const int l = t / (N / 2), bfl = t % (N / 2);
-                const int p = bfl / s, q = bfl % s;
-                const C a = x[l * N + q + s * p], b = x[l * N + q + s * (p + m)];
-                y[l * N + q + 2 * s * p] = cadd(a, b);
-                y[l * N + q + s * (2 * p + 1)] = cmul(csub(a, b), tw[p * s]);
-            }
-            __syncthreads();
-            C *tmp = x;
-            x = y;
-            y = tmp;
-        }
-        for (int t = threadIdx.x; t < L * N; t += blockDim.x) {
-            const int l = axis == 0 ? t / N : t % L, j = axis == 0 ? t % N : t / L;
-            data[base(l0 + l) + j * stride] = x[l * N + j];
-        }
-    }
+__device__ __forceinline__ void upwind_flux(const T l[3], const T r[3], int a, T flux[3]) {
+    const T s = l[a] + r[a];
+    const bool up = positive(s) && positive(l[a]), down = negative(s) && negative(r[a]);
+    const T un = up ? l[a] : (down ? r[a] : (T)0);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) flux[c] = un * (up ? l[c] : r[c]);
 }
 
-// theta_a = 2 pi k_a / n_a of FFT index i (frequencies above n/2 are negative)
+// Flux difference and second difference of the three components along axis a
+// at the middle of five cells v.  k = dt / h.
 template <typename T>
-__device__ __forceinline__ T half_theta_pi(int i, int n) {
-    // theta / 2 / pi = k / n, with k in (-n/2, n/2]
-    const int k = i <= n / 2 ? i : i - n;
-    return (T)k / (T)n;
-}
-
-// Multiplies the spectrum by the inverse of the operator's symbol and by
-// 1 / (n0 n1 n2) (the inverse FFT is unscaled).
-//   kind 0: (I - coef L_c)^-1, L_c symbol -(4/h^2) sum sin^2(theta/2)
-//   kind 1: coef (D G)^-1, D G symbol -(4/h^2) sum_a sin^2 prod_b cos^2, 0 on its null modes
-template <typename T>
-__global__ void k_symbol(typename Cx<T>::type *data, int n0, int n1, int n2, int kind, double coef, double h) {
-    const long long N = (long long)n0 * n1 * n2;
-    const T inv_n = (T)(1.0 / (double)N);
-    const T c4 = (T)(4.0 / (h * h));
-    for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < N;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(idx % n0), j = (int)((idx / n0) % n1), k = (int)(idx / ((long long)n0 * n1));
-        T sx, cx, sy, cy, sz, cz;
-        sincos_pi(half_theta_pi<T>(i, n0), &sx, &cx);
-        sincos_pi(half_theta_pi<T>(j, n1), &sy, &cy);
-        sincos_pi(half_theta_pi<T>(k, n2), &sz, &cz);
-        sx *= sx, cx *= cx, sy *= sy, cy *= cy, sz *= sz, cz *= cz;
-        T f;
-        if (kind == 0) {
-            f = inv_n / ((T)1 + (T)coef * c4 * (sx + sy + sz));
-        } else {
-            const T lam = -c4 * (sx * cy * cz + sy * cx * cz + sz * cx * cy);
-            f = fabs(lam) <= (T)1e-13 * (T)3 * c4 ? (T)0 : (T)coef * inv_n / lam;
-        }
-        data[idx].x *= f;
-        data[idx].y *= f;
-    }
-}
-
-template <typename T>
-__device__ __forceinline__ T mc_slope(T um, T u0, T up) {
-    const T a = u0 - um, b = up - u0;
-    const T mag = fmin(fmin((T)2 * fabs(a), (T)2 * fabs(b)), (T)0.5 * fabs(a + b));
-    return a * b > (T)0 ? copysign(mag, a + b) : (T)0;
-}
-
-// Flux of all three components through the face between cells i and i+1
-// along axis a, from the cells i-1 .. i+2 (v[0..3][c]).
-template <typename T>
-__device__ __forceinline__ void face_flux(const T v[4][3], int a, T dt, T h, T flux[3]) {
-    T left[3], right[3];
+__device__ __forceinline__ void axis_terms(const T v[5][3], int a, T k, T conv[3], T lap[3]) {
+    T lm[3], rm[3], lp[3], rp[3];  // states at the faces -1/2 and +1/2
+    const T cl0 = fma(-k, v[1][a], (T)1), cr1 = fma(k, v[2][a], (T)1), cl1 = fma(-k, v[2][a], (T)1),
+            cr2 = fma(k, v[3][a], (T)1);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const T sl = mc_slope(v[0][c], v[1][c], v[2][c]);
-        const T sr = mc_slope(v[1][c], v[2][c], v[3][c]);
-        left[c] = v[1][c] + ((T)0.5 - dt * v[1][a] / ((T)2 * h)) * sl;
-        right[c] = v[2][c] - ((T)0.5 + dt * v[2][a] / ((T)2 * h)) * sr;
+        const T d0 = v[1][c] - v[0][c], d1 = v[2][c] - v[1][c], d2 = v[3][c] - v[2][c], d3 = v[4][c] - v[3][c];
+        const T s0 = half_slope(d0, d1, d0 + d1), s1 = half_slope(d1, d2, d1 + d2), s2 = half_slope(d2, d3, d2 + d3);
+        lm[c] = fma(cl0, s0, v[1][c]);
+        rm[c] = fma(-cr1, s1, v[2][c]);
+        lp[c] = fma(cl1, s1, v[2][c]);
+        rp[c] = fma(-cr2, s2, v[3][c]);
+        lap[c] += d2 - d1;
     }
-    const T lv = left[a], rv = right[a];
-    const T un = (lv > (T)0 && lv + rv > (T)0) ? lv : ((rv < (T)0 && lv + rv < (T)0) ? rv : (T)0);
+    T fm[3], fp[3];
+    upwind_flux(lm, rm, a, fm);
+    upwind_flux(lp, rp, a, fp);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const T s = un > (T)0 ? left[c] : (un < (T)0 ? right[c] : (T)0.5 * (left[c] + right[c]));
-        flux[c] = un * s;
-    }
+    for (int c = 0; c < 3; ++c) conv[c] += fp[c] - fm[c];
 }
 
-__device__ __forceinline__ int wrapi(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
+// A cell's gradient sums from its corners on one node plane: x and y
+// differences, and the corners themselves for the z differences.  Differences
+// are taken before anything is added: a sum of pressures would leave its
+// rounding in the gradient.
+template <typename T>
+__device__ __forceinline__ void plane_corners(T p00, T p10, T p01, T p11, T &gx, T &gy, T s[4]) {
+    gx = (p10 - p00) + (p11 - p01);
+    gy = (p01 - p00) + (p11 - p10);
+    s[0] = p00, s[1] = p10, s[2] = p01, s[3] = p11;
+}
+// The z sum between two node planes; s0 becomes s1.
+template <typename T> __device__ __forceinline__ T z_corners(T s0[4], const T s1[4]) {
+    const T r = ((s1[0] - s0[0]) + (s1[1] - s0[1])) + ((s1[2] - s0[2]) + (s1[3] - s0[3]));
+#pragma unroll
+    for (int o = 0; o < 4; ++o) s0[o] = s1[o];
+    return r;
+}
 
 // Right-hand side of the predictor at every cell,
-//   u^n + dt (-div(u u) - G p / rho + (nu / 2) L_c u^n + g),
-// packed for the spectral solve: (x, y) components as one complex field, z
-// as the real part of another (the symbol is real and even, so the two
-// real fields of one complex field stay separate).
+//   u^n + dt (-div(u u) - G p / rho + (nu / 2) L_c u^n + g).
+// Along z the five cells, the lower face's flux and the middle cell's states
+// stay in registers from plane to plane.
+struct RhsArgs {
+    double k;            // dt / h
+    double cc, cg, cl;   // -dt / h, -dt / (4 h rho), nu dt / (2 h^2)
+    double dg[3];        // dt g
+};
+constexpr int kStencilThreads = 256;
 template <typename T>
-__global__ void k_predictor_rhs(DevGrid g, const T *__restrict__ u, const T *__restrict__ p, double rho_f, double nu,
-                                double gx, double gy, double gz, double dt, typename Cx<T>::type *c0,
-                                typename Cx<T>::type *c1) {
-    const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
-    const long long N = (long long)n0 * n1 * n2;
-    const T h = (T)g.h, tdt = (T)dt;
-    for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < N;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(idx % n0), j = (int)((idx / n0) % n1), k = (int)(idx / ((long long)n0 * n1));
-        auto cell = [&](int di, int dj, int dk) {
-            return ((long long)wrapi(k + dk, n2) * n1 + wrapi(j + dj, n1)) * n0 + wrapi(i + di, n0);
-        };
+__global__ void __launch_bounds__(kStencilThreads) k_predictor_rhs(LevelDims d, const T *__restrict__ u,
+                                                                   const T *__restrict__ p, RhsArgs a,
+                                                                   T *__restrict__ out) {
+    const Column q(d);
+    const int m0 = d.n0 - 1, m1 = d.n1 - 1, m2 = d.n2 - 1;
+    const size_t plane = (size_t)d.n0 * d.n1, N = plane * d.n2;
+    const T k = (T)a.k, cc = (T)a.cc, cg = (T)a.cg, cl = (T)a.cl;
+    const int row = q.j * d.n0, i0 = row + q.i;
+    int ix[4], iy[4];  // in-plane neighbours -2, -1, +1, +2
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+        const int s = o < 2 ? o - 2 : o - 1;
+        ix[o] = row + ((q.i + s) & m0);
+        iy[o] = ((q.j + s) & m1) * d.n0 + q.i;
+    }
+    const int px = row + ((q.i + 1) & m0), py = ((q.j + 1) & m1) * d.n0 + q.i, pxy = ((q.j + 1) & m1) * d.n0 + ((q.i + 1) & m0);
+    auto corners = [&](int kk, T &gx, T &gy, T s[4]) {
+        const T *pk = p + (size_t)kk * plane;
+        plane_corners(pk[i0], pk[px], pk[py], pk[pxy], gx, gy, s);
+    };
+    grid_dep_wait();
+    T z[5][3];
+#pragma unroll
+    for (int o = 0; o < 4; ++o)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) z[o][c] = u[c * N + (size_t)((q.k0 + o - 2) & m2) * plane + i0];
+    // the lower face's flux and the middle cell's left states, as the loop carries them
+    T fm[3], left[3], gx0, gy0, s0[4];
+    {
+        const T cl0 = fma(-k, z[1][2], (T)1), cr1 = fma(k, z[2][2], (T)1), cl1 = fma(-k, z[2][2], (T)1);
+        T l[3], r[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const T d0 = z[1][c] - z[0][c], d1 = z[2][c] - z[1][c], d2 = z[3][c] - z[2][c];
+            const T s1 = half_slope(d1, d2, d1 + d2);
+            l[c] = fma(cl0, half_slope(d0, d1, d0 + d1), z[1][c]);
+            r[c] = fma(-cr1, s1, z[2][c]);
+            left[c] = fma(cl1, s1, z[2][c]);
+        }
+        upwind_flux(l, r, 2, fm);
+    }
+    corners(q.k0, gx0, gy0, s0);
+    for (int kk = q.k0; kk < q.k1; ++kk) {
+        const size_t base = (size_t)kk * plane;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) z[4][c] = u[c * N + (size_t)((kk + 2) & m2) * plane + i0];
         T conv[3] = {0, 0, 0}, lap[3] = {0, 0, 0};
-        T u0[3];
+        T v[5][3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) u0[c] = u[c * N + idx];
+        for (int c = 0; c < 3; ++c) {
+            v[2][c] = z[2][c];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            T v[5][3];  // cells -2 .. +2 along a
-#pragma unroll
-            for (int o = 0; o < 5; ++o) {
-                const long long cc = cell(a == 0 ? o - 2 : 0, a == 1 ? o - 2 : 0, a == 2 ? o - 2 : 0);
-#pragma unroll
-                for (int c = 0; c < 3; ++c) v[o][c] = o == 2 ? u0[c] : u[c * N + cc];
-            }
-            T fm[3], fp[3];
-            face_flux<T>(*(const T(*)[4][3])&v[0], a, tdt, h, fm);  // face i - 1/2 (cells i-2 .. i+1)
-            face_flux<T>(*(const T(*)[4][3])&v[1], a, tdt, h, fp);  // face i + 1/2 (cells i-1 .. i+2)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                conv[c] += (fp[c] - fm[c]) / h;
-                lap[c] += (v[3][c] - (T)2 * v[2][c] + v[1][c]) / (h * h);
-            }
+            for (int o = 0; o < 4; ++o) v[o < 2 ? o : o + 1][c] = u[c * N + base + ix[o]];
         }
-        // G p at the cell: node (i, j, k) is the cell's lower corner
-        T pc[2][2][2];
-#pragma unroll
-        for (int dk = 0; dk < 2; ++dk)
-#pragma unroll
-            for (int dj = 0; dj < 2; ++dj)
-#pragma unroll
-                for (int di = 0; di < 2; ++di) pc[dk][dj][di] = p[cell(di, dj, dk)];
-        const T q = (T)0.25 / h;
-        T gp[3];
-        {
-            T d00 = pc[0][0][1] - pc[0][0][0], d10 = pc[0][1][1] - pc[0][1][0];
-            T d01 = pc[1][0][1] - pc[1][0][0], d11 = pc[1][1][1] - pc[1][1][0];
-            gp[0] = q * (d00 + d10 + d01 + d11);
-            d00 = pc[0][1][0] - pc[0][0][0], d10 = pc[0][1][1] - pc[0][0][1];
-            d01 = pc[1][1][0] - pc[1][0][0], d11 = pc[1][1][1] - pc[1][0][1];
-            gp[1] = q * (d00 + d10 + d01 + d11);
-            d00 = pc[1][0][0] - pc[0][0][0], d10 = pc[1][0][1] - pc[0][0][1];
-            d01 = pc[1][1][0] - pc[0][1][0], d11 = pc[1][1][1] - pc[0][1][1];
-            gp[2] = q * (d00 + d10 + d01 + d11);
-        }
-        const T gv[3] = {(T)gx, (T)gy, (T)gz};
-        T r[3];
+        axis_terms(v, 0, k, conv, lap);
 #pragma unroll
         for (int c = 0; c < 3; ++c)
-            r[c] = u0[c] + tdt * (-conv[c] - gp[c] / (T)rho_f + (T)(0.5 * nu) * lap[c] + gv[c]);
-        c0[idx] = typename Cx<T>::type{r[0], r[1]};
-        c1[idx] = typename Cx<T>::type{r[2], (T)0};
+#pragma unroll
+            for (int o = 0; o < 4; ++o) v[o < 2 ? o : o + 1][c] = u[c * N + base + iy[o]];
+        axis_terms(v, 1, k, conv, lap);
+        {
+            const T cr = fma(k, z[3][2], (T)1), cn = fma(-k, z[3][2], (T)1);
+            T r[3], next[3], fp[3];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const T d1 = z[2][c] - z[1][c], d2 = z[3][c] - z[2][c], d3 = z[4][c] - z[3][c];
+                const T s = half_slope(d2, d3, d2 + d3);
+                r[c] = fma(-cr, s, z[3][c]);
+                next[c] = fma(cn, s, z[3][c]);
+                lap[c] += d2 - d1;
+            }
+            upwind_flux(left, r, 2, fp);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                conv[c] += fp[c] - fm[c];
+                fm[c] = fp[c];
+                left[c] = next[c];
+            }
+        }
+        T gx1, gy1, s1[4];
+        corners((kk + 1) & m2, gx1, gy1, s1);
+        const T gp[3] = {gx0 + gx1, gy0 + gy1, z_corners(s0, s1)};
+        gx0 = gx1, gy0 = gy1;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            out[c * N + base + i0] = fma(cl, lap[c], fma(cc, conv[c], fma(cg, gp[c], z[2][c] + (T)a.dg[c])));
+#pragma unroll
+            for (int o = 0; o < 4; ++o) z[o][c] = z[o + 1][c];
+        }
     }
 }
 
-template <typename T>
-__global__ void k_unpack_velocity(long long N, const typename Cx<T>::type *c0, const typename Cx<T>::type *c1,
-                                  T *u) {
-    for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < N;
-         idx += (long long)gridDim.x * blockDim.x) {
-        u[idx] = c0[idx].x;
-        u[N + idx] = c0[idx].y;
-        u[2 * N + idx] = c1[idx].x;
+// A sum of differences.  FP32: compensated (Knuth's TwoSum of every
+// difference and every addition), since the solve amplifies the rounding of
+// the nearly checkerboard modes most, up to 1e5 times at 256^3, and a plain
+// sum leaves there what a difference of single-precision velocities does not.
+template <typename T> struct DiffSum {
+    T s;
+    __device__ __forceinline__ void clear() { s = 0; }
+    __device__ __forceinline__ void add(T a, T b) { s += a - b; }
+    __device__ __forceinline__ void add(const DiffSum &o) { s += o.s; }
+    __device__ __forceinline__ T value() const { return s; }
+};
+template <> struct DiffSum<float> {
+    float s, e;
+    __device__ __forceinline__ void clear() { s = e = 0.0f; }
+    __device__ __forceinline__ float two_sum(float a, float b, float &err) const {
+        const float t = __fadd_rn(a, b), bb = __fsub_rn(t, a);
+        err = __fadd_rn(__fsub_rn(a, __fsub_rn(t, bb)), __fsub_rn(b, bb));
+        return t;
     }
-}
+    __device__ __forceinline__ void add(float a, float b) {
+        float e0, e1;
+        const float d = two_sum(a, -b, e0);
+        s = two_sum(s, d, e1);
+        e = __fadd_rn(e, __fadd_rn(e0, e1));
+    }
+    __device__ __forceinline__ void add(const DiffSum &o) {
+        float e1;
+        s = two_sum(s, o.s, e1);
+        e = __fadd_rn(e, __fadd_rn(o.e, e1));
+    }
+    __device__ __forceinline__ float value() const { return __fadd_rn(s, e); }
+};
 
-// G of a nodal field at cell (i, j, k), component a.
-template <typename T, typename F>
-__device__ __forceinline__ void grad_at_cell(F nodal, T h, T out[3]) {
-    T pc[2][2][2];
-#pragma unroll
-    for (int dk = 0; dk < 2; ++dk)
-#pragma unroll
-        for (int dj = 0; dj < 2; ++dj)
-#pragma unroll
-            for (int di = 0; di < 2; ++di) pc[dk][dj][di] = nodal(di, dj, dk);
-    const T q = (T)0.25 / h;
-    out[0] = q * ((pc[0][0][1] - pc[0][0][0]) + (pc[0][1][1] - pc[0][1][0]) + (pc[1][0][1] - pc[1][0][0]) +
-                  (pc[1][1][1] - pc[1][1][0]));
-    out[1] = q * ((pc[0][1][0] - pc[0][0][0]) + (pc[0][1][1] - pc[0][0][1]) + (pc[1][1][0] - pc[1][0][0]) +
-                  (pc[1][1][1] - pc[1][0][1]));
-    out[2] = q * ((pc[1][0][0] - pc[0][0][0]) + (pc[1][0][1] - pc[0][0][1]) + (pc[1][1][0] - pc[0][1][0]) +
-                  (pc[1][1][1] - pc[0][1][1]));
-}
-
-// D V at every node, V = u*/dt + G p_old / rho_f (Eq. ns_lp1) formed at the
-// eight cells around the node; the result is the real part of the spectrum
-// buffer.
+// D V at every node, V = u*/dt + G p_old / rho_f (Eq. ns_lp1).  D u is the sum
+// over the planes k - 1 and k of the in-plane differences; D G p is the
+// 27-point operator formed from in-plane second differences (so a constant
+// pressure cancels exactly): with r the second x difference of a row, y that
+// of the column along y and z along z,
+//   16 h^2 D G p = (3 r- + 2 r0 + 3 r+ + 8 y)(k-1) + the same (k+1)
+//                  + 2 (r- - 2 r0 + r+)(k) + 16 z.
 template <typename T>
-__global__ void k_projection_div(DevGrid g, const T *__restrict__ u, const T *__restrict__ p, double rho_f, double dt,
-                                 typename Cx<T>::type *c) {
-    const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
-    const long long N = (long long)n0 * n1 * n2;
-    const T h = (T)g.h, idt = (T)(1.0 / dt), irho = (T)(1.0 / rho_f);
-    for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < N;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(idx % n0), j = (int)((idx / n0) % n1), k = (int)(idx / ((long long)n0 * n1));
-        // the cells around node (i, j, k): (i-1|i, j-1|j, k-1|k)
-        T V[2][2][2][3];
+__global__ void __launch_bounds__(kStencilThreads) k_projection_div(LevelDims d, const T *__restrict__ u,
+                                                                    const T *__restrict__ p, double cu, double cp,
+                                                                    T *__restrict__ out) {
+    const Column q(d);
+    const int m0 = d.n0 - 1, m1 = d.n1 - 1, m2 = d.n2 - 1;
+    const size_t plane = (size_t)d.n0 * d.n1, N = plane * d.n2;
+    const int xm = (q.i - 1) & m0, xp = (q.i + 1) & m0, x0 = q.i;
+    const int ym = ((q.j - 1) & m1) * d.n0, yp = ((q.j + 1) & m1) * d.n0, y0 = q.j * d.n0;
+    auto pressure = [&](int kk, T &a, T &b, T &c) {
+        const T *pk = p + (size_t)kk * plane;
+        c = pk[y0 + x0];
+        const T cm = pk[ym + x0], cp1 = pk[yp + x0];
+        const T r0 = (pk[y0 + xp] - c) - (c - pk[y0 + xm]);
+        const T rm = (pk[ym + xp] - cm) - (cm - pk[ym + xm]);
+        const T rp = (pk[yp + xp] - cp1) - (cp1 - pk[yp + xm]);
+        const T yy = (cp1 - c) - (c - cm), s = rm + rp;
+        a = fma((T)3, s, fma((T)2, r0, (T)8 * yy));
+        b = fma((T)-2, r0, s);
+    };
+    // differences of u around the node: x and y parts in the plane, and the z
+    // component's four values, whose differences between planes are taken
+    // before they are added
+    auto velocity = [&](int kk, DiffSum<T> &xy, T w[4]) {
+        const T *uk = u + (size_t)kk * plane;
+        const T *vk = uk + N, *wk = vk + N;
+        xy.clear();
+        xy.add(uk[y0 + x0], uk[y0 + xm]);
+        xy.add(uk[ym + x0], uk[ym + xm]);
+        xy.add(vk[y0 + x0], vk[ym + x0]);
+        xy.add(vk[y0 + xm], vk[ym + xm]);
+        w[0] = wk[y0 + x0], w[1] = wk[y0 + xm], w[2] = wk[ym + x0], w[3] = wk[ym + xm];
+    };
+    grid_dep_wait();
+    T am, bm, cm, a0, b0, c0, wm[4];
+    DiffSum<T> xym;
+    pressure((q.k0 - 1) & m2, am, bm, cm);
+    pressure(q.k0, a0, b0, c0);
+    T dzm = c0 - cm;
+    velocity((q.k0 - 1) & m2, xym, wm);
+    for (int kk = q.k0; kk < q.k1; ++kk) {
+        T a1, b1, c1, w[4];
+        DiffSum<T> xy;
+        pressure((kk + 1) & m2, a1, b1, c1);
+        velocity(kk, xy, w);
+        const T dz = c1 - c0;
+        const T dgp = fma((T)16, dz - dzm, fma((T)2, b0, am + a1));
+        xym.add(xy);
 #pragma unroll
-        for (int ck = 0; ck < 2; ++ck)
+        for (int o = 0; o < 4; ++o) xym.add(w[o], wm[o]);
+        out[(size_t)kk * plane + y0 + x0] = fma((T)cp, dgp, (T)cu * xym.value());
+        am = a0, a0 = a1, b0 = b1, c0 = c1, dzm = dz, xym = xy;
 #pragma unroll
-            for (int cj = 0; cj < 2; ++cj)
-#pragma unroll
-                for (int ci = 0; ci < 2; ++ci) {
-                    const int ii = wrapi(i - 1 + ci, n0), jj = wrapi(j - 1 + cj, n1), kk = wrapi(k - 1 + ck, n2);
-                    const long long cidx = ((long long)kk * n1 + jj) * n0 + ii;
-                    T gp[3];
-                    grad_at_cell<T>([&](int di, int dj, int dk) {
-                        return p[((long long)wrapi(kk + dk, n2) * n1 + wrapi(jj + dj, n1)) * n0 + wrapi(ii + di, n0)];
-                    }, h, gp);
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) V[ck][cj][ci][a] = u[a * N + cidx] * idt + gp[a] * irho;
-                }
-        const T q = (T)0.25 / h;
-        T d = q * ((V[1][1][1][0] - V[1][1][0][0]) + (V[0][1][1][0] - V[0][1][0][0]) +
-                   (V[1][0][1][0] - V[1][0][0][0]) + (V[0][0][1][0] - V[0][0][0][0]));
-        d += q * ((V[1][1][1][1] - V[1][0][1][1]) + (V[0][1][1][1] - V[0][0][1][1]) +
-                  (V[1][1][0][1] - V[1][0][0][1]) + (V[0][1][0][1] - V[0][0][0][1]));
-        d += q * ((V[1][1][1][2] - V[0][1][1][2]) + (V[1][0][1][2] - V[0][0][1][2]) +
-                  (V[1][1][0][2] - V[0][1][0][2]) + (V[1][0][0][2] - V[0][0][0][2]));
-        c[idx] = typename Cx<T>::type{d, (T)0};
+        for (int o = 0; o < 4; ++o) wm[o] = w[o];
     }
 }
 
 // u^{n+1} = dt (V - G p_new / rho_f) = u* + (dt / rho_f) G (p_old - p_new)
-// (Eq. ns_lp3), p_new the real part of the solved buffer.
+// (Eq. ns_lp3).  FP64: q holds p_old - p_new; FP32: q holds p_old and p p_new
+// (fluid_fft.cuh, kXPressure).
 template <typename T>
-__global__ void k_projection_update(DevGrid g, T *__restrict__ u, const T *__restrict__ p,
-                                    const typename Cx<T>::type *__restrict__ c, double rho_f, double dt) {
-    const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
-    const long long N = (long long)n0 * n1 * n2;
-    const T h = (T)g.h, s = (T)(dt / rho_f);
-    for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < N;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(idx % n0), j = (int)((idx / n0) % n1), k = (int)(idx / ((long long)n0 * n1));
-        auto node = [&](int di, int dj, int dk) {
-            return ((long long)wrapi(k + dk, n2) * n1 + wrapi(j + dj, n1)) * n0 + wrapi(i + di, n0);
-        };
-        T go[3], gn[3];
-        grad_at_cell<T>([&](int di, int dj, int dk) { return p[node(di, dj, dk)]; }, h, go);
-        grad_at_cell<T>([&](int di, int dj, int dk) { return c[node(di, dj, dk)].x; }, h, gn);
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const T V = u[a * N + idx] / (T)dt + go[a] / (T)rho_f;
-            u[a * N + idx] = (T)dt * (V - gn[a] / (T)rho_f);
+__global__ void __launch_bounds__(kStencilThreads) k_projection_update(LevelDims d, T *__restrict__ u,
+                                                                       const T *__restrict__ q,
+                                                                       const T *__restrict__ p, double cg) {
+    constexpr bool kTwo = sizeof(T) == 4;
+    const Column o(d);
+    const int m0 = d.n0 - 1, m1 = d.n1 - 1, m2 = d.n2 - 1;
+    const size_t plane = (size_t)d.n0 * d.n1, N = plane * d.n2;
+    const int i0 = o.j * d.n0 + o.i, px = o.j * d.n0 + ((o.i + 1) & m0), py = ((o.j + 1) & m1) * d.n0 + o.i,
+              pxy = ((o.j + 1) & m1) * d.n0 + ((o.i + 1) & m0);
+    auto corners = [&](const T *f, int kk, T &gx, T &gy, T s[4]) {
+        const T *pk = f + (size_t)kk * plane;
+        plane_corners(pk[i0], pk[px], pk[py], pk[pxy], gx, gy, s);
+    };
+    grid_dep_wait();
+    T gx0, gy0, s0[4], hx0 = 0, hy0 = 0, r0[4];
+    corners(q, o.k0, gx0, gy0, s0);
+    if (kTwo) corners(p, o.k0, hx0, hy0, r0);
+    for (int kk = o.k0; kk < o.k1; ++kk) {
+        T gx1, gy1, s1[4], hx1, hy1, r1[4];
+        corners(q, (kk + 1) & m2, gx1, gy1, s1);
+        T *uk = u + (size_t)kk * plane + i0;
+        const T u0 = uk[0], u1 = uk[N], u2 = uk[2 * N];
+        T g[3] = {gx0 + gx1, gy0 + gy1, z_corners(s0, s1)};
+        if (kTwo) {
+            corners(p, (kk + 1) & m2, hx1, hy1, r1);
+            g[0] -= hx0 + hx1, g[1] -= hy0 + hy1, g[2] -= z_corners(r0, r1);
+            hx0 = hx1, hy0 = hy1;
         }
-        (void)s;
+        uk[0] = fma((T)cg, g[0], u0);
+        uk[N] = fma((T)cg, g[1], u1);
+        uk[2 * N] = fma((T)cg, g[2], u2);
+        gx0 = gx1, gy0 = gy1;
     }
-}
-
-template <typename T>
-__global__ void k_take_pressure(long long N, const typename Cx<T>::type *c, T *p) {
-    for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < N;
-         idx += (long long)gridDim.x * blockDim.x)
-        p[idx] = c[idx].x;
 }
 
 static int ilog2_exact(int n) {
@@ -361,73 +366,94 @@ static int check_fluid_grid(const ib_grid *grid) {
     return IB_OK;
 }
 
-// 3D FFT (forward or inverse, unscaled) of a complex field in place.
-template <typename T>
-static int fft3(ib_ctx *ctx, typename Cx<T>::type *c, const int n[3], int inverse, cudaStream_t s) {
-    using C = typename Cx<T>::type;
-    for (int axis = 0; axis < 3; ++axis) {
-        const int N = n[axis], logN = ilog2_exact(N);
-        const int L = fft_lines(N, axis, n[0]);
-        const size_t smem = ((size_t)2 * L * N + N / 2) * sizeof(C);
-        cudaFuncSetAttribute(k_fft_axis<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        const long long nlines = (long long)n[0] * n[1] * n[2] / N;
-        long long blocks = (nlines + L - 1) / L;
-        const long long cap = (long long)ctx->sm_count * 16;
-        if (blocks > cap) blocks = cap;
-        k_fft_axis<T><<<(int)blocks, kFftThreads, smem, s>>>(c, n[0], n[1], n[2], axis, logN, inverse);
+// Launch shape of the stencil kernels: 32 x 8 columns (16 x 16 on the smallest
+// grids) and chunks of planes, at most 32 and at least 4, that give each SM
+// several CTAs.
+struct StencilGrid {
+    LevelDims d;
+    dim3 grid, block;
+    StencilGrid(ib_ctx *ctx, const int n[3]) : d{n[0], n[1], n[2], 32} {
+        block = dim3(n[0] < 32 ? 16 : 32, n[0] < 32 ? 16 : 8, 1);
+        const long long tiles = (long long)(n[0] / block.x) * (n[1] / block.y);
+        if (d.zc > n[2]) d.zc = n[2];
+        while (d.zc > 4 && tiles * (n[2] / d.zc) < 6LL * ctx->sm_count) d.zc /= 2;
+        grid = dim3(n[0] / block.x, n[1] / block.y, n[2] / d.zc);
     }
-    return check_launch("fft");
+};
+
+template <class A> static FftGrid<A> fft_grid(ib_ctx *ctx, const int n[3]) {
+    FftGrid<A> g;
+    for (int a = 0; a < 3; ++a) g.n[a] = n[a], g.log2n[a] = ilog2_exact(n[a]);
+    if constexpr (A::kFixed) g.roots = ctx->fft_tab->roots_fx;
+    else g.roots = ctx->fft_tab->roots32;
+    if constexpr (sizeof(typename A::Real) == 8) g.trig = ctx->fft_tab->trig64;
+    else g.trig = ctx->fft_tab->trig32;
+    return g;
 }
 
-static int elem_blocks(long long n, int sm) {
-    long long b = (n + 255) / 256, cap = (long long)sm * 16;
-    return (int)(b < 1 ? 1 : (b < cap ? b : cap));
+// The spectral solve of ncomp fields from `src` to `dst`: x passes in the
+// arithmetic X, the others in A.
+template <class X, class A>
+static cudaError_t solve(ib_ctx *ctx, const int n[3], int ncomp, const typename A::Real *src, Spectrum<A> c,
+                         const SymbolArgs &sy, int out, typename A::Real *dst, typename A::Real *old, cudaStream_t s) {
+    const FftGrid<X> gx = fft_grid<X>(ctx, n);
+    const FftGrid<A> g = fft_grid<A>(ctx, n);
+    const Spectrum<X> cx = {c.c, c.ny};
+    cudaError_t e = fft_x<X>(kXForward, gx, ncomp, src, cx, nullptr, nullptr, s);
+    if (e == cudaSuccess) e = fft_y<A>(false, g, ncomp, c, s);
+    if (e == cudaSuccess) e = fft_z<A>(g, ncomp, c, sy, s);
+    if (e == cudaSuccess) e = fft_y<A>(true, g, ncomp, c, s);
+    if (e == cudaSuccess) e = fft_x<X>(out, gx, ncomp, nullptr, cx, dst, old, s);
+    return e;
 }
 
-template <typename T>
+template <class A>
 static int run_predictor(ib_ctx *ctx, const ib_grid *grid, const void *u, const void *p, double rho_f, double mu,
                          const double g[3], double dt, void *u_star, cudaStream_t s) {
-    using C = typename Cx<T>::type;
-    const DevGrid dg = make_dev_grid(grid);
-    const long long N = (long long)grid->n[0] * grid->n[1] * grid->n[2];
+    using T = typename A::Real;
+    const size_t N = (size_t)grid->n[0] * grid->n[1] * grid->n[2];
+    const double h = grid->h, nu = mu / rho_f;
     Arena ar(ctx);
-    C *c0 = ar.take<C>(N), *c1 = ar.take<C>(N);
+    const size_t ny = (size_t)grid->n[1] * grid->n[2];
+    Spectrum<A> c;
+    c.c = ar.take<typename A::Mem>(3 * (N / 2));
+    c.ny = ar.take<typename A::Mem>(3 * ny);
     if (!ar.ok()) return oom_error(ar.used, ar.cap);
-    const int nb = elem_blocks(N, ctx->sm_count);
-    const double nu = mu / rho_f;
+    const StencilGrid sg(ctx, grid->n);
+    const RhsArgs a = {dt / h, -dt / h, -dt / (4.0 * h * rho_f), 0.5 * nu * dt / (h * h), {dt * g[0], dt * g[1], dt * g[2]}};
+    const double points = (double)N;  // the transforms are unscaled
+    const SymbolArgs sy = {kSolveHelmholtz, 1.0 / points, 0.5 * nu * dt * 4.0 / (h * h)};
     PhaseTimer tm(ctx, IB_PHASE_FLUID_PREDICTOR, s);
-    k_predictor_rhs<T><<<nb, 256, 0, s>>>(dg, (const T *)u, (const T *)p, rho_f, nu, g[0], g[1], g[2], dt, c0, c1);
-    for (C *c : {c0, c1}) {
-        int rc = fft3<T>(ctx, c, grid->n, 0, s);
-        if (rc) return rc;
-        k_symbol<T><<<nb, 256, 0, s>>>(c, grid->n[0], grid->n[1], grid->n[2], 0, 0.5 * nu * dt, grid->h);
-        rc = fft3<T>(ctx, c, grid->n, 1, s);
-        if (rc) return rc;
-    }
-    k_unpack_velocity<T><<<nb, 256, 0, s>>>(N, c0, c1, (T *)u_star);
+    // the right-hand side in u_star, the point buffers in the workspace
+    cudaError_t e = launch_pdl(k_predictor_rhs<T>, sg.grid, sg.block, 0, s, sg.d, (const T *)u, (const T *)p, a, (T *)u_star);
+    if (e == cudaSuccess) e = solve<A, A>(ctx, grid->n, 3, (const T *)u_star, c, sy, kXField, (T *)u_star, nullptr, s);
+    if (e != cudaSuccess) return set_error(IB_ERR_CUDA, "fluid_predictor: %s", cudaGetErrorString(e));
     return check_launch("fluid_predictor");
 }
 
-template <typename T>
+template <class A>
 static int run_projection(ib_ctx *ctx, const ib_grid *grid, void *u, void *p, double rho_f, double dt,
                           cudaStream_t s) {
-    using C = typename Cx<T>::type;
-    const DevGrid dg = make_dev_grid(grid);
-    const long long N = (long long)grid->n[0] * grid->n[1] * grid->n[2];
+    using T = typename A::Real;
+    const size_t N = (size_t)grid->n[0] * grid->n[1] * grid->n[2];
+    const double h = grid->h;
     Arena ar(ctx);
-    C *c = ar.take<C>(N);
+    Spectrum<A> c;
+    c.c = ar.take<typename A::Mem>(N / 2);
+    c.ny = ar.take<typename A::Mem>((size_t)grid->n[1] * grid->n[2]);
+    T *q = ar.take<T>(N);
     if (!ar.ok()) return oom_error(ar.used, ar.cap);
-    const int nb = elem_blocks(N, ctx->sm_count);
-    PhaseTimer tm(ctx, IB_PHASE_FLUID_PROJECTION, s);
-    k_projection_div<T><<<nb, 256, 0, s>>>(dg, (const T *)u, (const T *)p, rho_f, dt, c);
-    int rc = fft3<T>(ctx, c, grid->n, 0, s);
-    if (rc) return rc;
+    const StencilGrid sg(ctx, grid->n);
     // p_new = rho_f (D G)^-1 D V   (Eq. ns_lp2 with L p = div((1/rho_f) grad p))
-    k_symbol<T><<<nb, 256, 0, s>>>(c, grid->n[0], grid->n[1], grid->n[2], 1, rho_f, grid->h);
-    rc = fft3<T>(ctx, c, grid->n, 1, s);
-    if (rc) return rc;
-    k_projection_update<T><<<nb, 256, 0, s>>>(dg, (T *)u, (const T *)p, c, rho_f, dt);
-    k_take_pressure<T><<<nb, 256, 0, s>>>(N, c, (T *)p);
+    const SymbolArgs sy = {kSolveDivGrad, -rho_f * h * h / 4.0 / (double)N, 0.0};
+    PhaseTimer tm(ctx, IB_PHASE_FLUID_PROJECTION, s);
+    cudaError_t e = launch_pdl(k_projection_div<T>, sg.grid, sg.block, 0, s, sg.d, (const T *)u, (const T *)p,
+                               0.25 / (h * dt), 0.0625 / (h * h * rho_f), q);
+    if (e == cudaSuccess) e = solve<typename A::Pressure, A>(ctx, grid->n, 1, q, c, sy, kXPressure, (T *)p, q, s);
+    if (e == cudaSuccess)
+        e = launch_pdl(k_projection_update<T>, sg.grid, sg.block, 0, s, sg.d, (T *)u, (const T *)q,
+                       (const T *)p, dt / (4.0 * h * rho_f));
+    if (e != cudaSuccess) return set_error(IB_ERR_CUDA, "level_projection: %s", cudaGetErrorString(e));
     return check_launch("level_projection");
 }
 
@@ -447,8 +473,8 @@ int fluid_predictor(ib_ctx *ctx, const ib_grid *grid, const void *u, const void 
         !isfinite(g[1]) || !isfinite(g[2]))
         return set_error(IB_ERR_INVALID, "rho_f > 0, mu >= 0, dt > 0 and g must be finite");
     if (grid->prec == IB_F64)
-        return run_predictor<double>(ctx, grid, u, p, rho_f, mu, g, dt, u_star, (cudaStream_t)stream);
-    return run_predictor<float>(ctx, grid, u, p, rho_f, mu, g, dt, u_star, (cudaStream_t)stream);
+        return run_predictor<Fx64>(ctx, grid, u, p, rho_f, mu, g, dt, u_star, (cudaStream_t)stream);
+    return run_predictor<Fp32>(ctx, grid, u, p, rho_f, mu, g, dt, u_star, (cudaStream_t)stream);
 }
 
 int level_projection(ib_ctx *ctx, const ib_grid *grid, void *u, void *p, double rho_f, double dt, void *stream) {
@@ -457,8 +483,8 @@ int level_projection(ib_ctx *ctx, const ib_grid *grid, void *u, void *p, double 
     if (rc) return rc;
     if (!u || !p) return set_error(IB_ERR_INVALID, "NULL array");
     if (!(rho_f > 0.0) || !(dt > 0.0) || !isfinite(dt)) return set_error(IB_ERR_INVALID, "rho_f > 0 and dt > 0");
-    if (grid->prec == IB_F64) return run_projection<double>(ctx, grid, u, p, rho_f, dt, (cudaStream_t)stream);
-    return run_projection<float>(ctx, grid, u, p, rho_f, dt, (cudaStream_t)stream);
+    if (grid->prec == IB_F64) return run_projection<Fx64>(ctx, grid, u, p, rho_f, dt, (cudaStream_t)stream);
+    return run_projection<Fp32>(ctx, grid, u, p, rho_f, dt, (cudaStream_t)stream);
 }
 
 }  // extern "C"

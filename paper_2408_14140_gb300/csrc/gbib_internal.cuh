@@ -180,6 +180,20 @@ __device__ __forceinline__ bool finite3(const double *v) {
 #include <utility>
 #include <vector>
 
+namespace gbib {
+// The 2048th roots of unity, exp(-2 pi i k / 2048): (cos, -sin) in FP32 and as
+// balanced Q62 halves (re hi, re lo, im hi, im lo), and (cos, sin) in both
+// field types for the operators' symbols.
+struct FftTables {
+    float2 roots32[2048], trig32[2048];
+    int4 roots_fx[2048];
+    double2 trig64[2048];
+};
+// Device copy of the tables (nullptr and a CUDA error on failure); `s` is a
+// stream of the context's, waited for.
+cudaError_t make_fft_tables(FftTables **out, cudaStream_t s);
+}  // namespace gbib
+
 struct ib_ctx {
     int device;
     int sm_count;
@@ -211,6 +225,7 @@ struct ib_ctx {
     size_t stage_cap[kStageSlots];
     cudaEvent_t stage_ev[kStageSlots];
     int stage_next;
+    gbib::FftTables *fft_tab;  // device: roots of unity of the fluid step's transforms
 };
 
 // A batch's case table uploaded once (ib_batch_table_create): device memory
