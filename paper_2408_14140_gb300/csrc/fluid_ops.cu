@@ -29,6 +29,7 @@ struct LevelDims {
     int n0, n1, n2, zc;  // zc: planes of one CTA's chunk
 };
 
+constexpr int kStencilThreads = 256;
 // The thread's column and its chunk of planes.
 struct Column {
     int i, j, k0, k1;
@@ -36,60 +37,6 @@ struct Column {
         : i(blockIdx.x * blockDim.x + threadIdx.x), j(blockIdx.y * blockDim.y + threadIdx.y), k0(blockIdx.z * d.zc),
           k1(blockIdx.z * d.zc + d.zc) {}
 };
-
-// Half the monotonized-central slope from the differences a (below) and b
-// (above) and their sum s: min(|a|, |b|, |s|/4) with their sign, 0 at extrema.
-__device__ __forceinline__ float half_slope(float a, float b, float s) {
-    const float m = fminf(fminf(fabsf(a), fabsf(b)), 0.25f * fabsf(s));
-    return a * b > 0.0f ? copysignf(m, s) : 0.0f;
-}
-// For FP64 the comparisons run on the integer pipe: the order of non-negative
-// doubles is that of their bits.
-__device__ __forceinline__ double half_slope(double a, double b, double s) {
-    const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b), is = __double_as_longlong(0.25 * s);
-    constexpr long long mag = 0x7fffffffffffffffLL;
-    const long long m = min(min(ia & mag, ib & mag), is & mag);
-    return (ia ^ ib) < 0 ? 0.0 : __longlong_as_double(m | (ia & ~mag));
-}
-__device__ __forceinline__ bool positive(float x) { return x > 0.0f; }
-__device__ __forceinline__ bool positive(double x) { return __double_as_longlong(x) > 0; }
-__device__ __forceinline__ bool negative(float x) { return x < 0.0f; }
-__device__ __forceinline__ bool negative(double x) { return 2 * __double_as_longlong(x) != 0 && __double_as_longlong(x) < 0; }
-
-// Fluxes of all three components through a face with states l and r, the
-// normal component being a (Burgers Riemann solution, upwinded).
-template <typename T>
-__device__ __forceinline__ void upwind_flux(const T l[3], const T r[3], int a, T flux[3]) {
-    const T s = l[a] + r[a];
-    const bool up = positive(s) && positive(l[a]), down = negative(s) && negative(r[a]);
-    const T un = up ? l[a] : (down ? r[a] : (T)0);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) flux[c] = un * (up ? l[c] : r[c]);
-}
-
-// Flux difference and second difference of the three components along axis a
-// at the middle of five cells v.  k = dt / h.
-template <typename T>
-__device__ __forceinline__ void axis_terms(const T v[5][3], int a, T k, T conv[3], T lap[3]) {
-    T lm[3], rm[3], lp[3], rp[3];  // states at the faces -1/2 and +1/2
-    const T cl0 = fma(-k, v[1][a], (T)1), cr1 = fma(k, v[2][a], (T)1), cl1 = fma(-k, v[2][a], (T)1),
-            cr2 = fma(k, v[3][a], (T)1);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const T d0 = v[1][c] - v[0][c], d1 = v[2][c] - v[1][c], d2 = v[3][c] - v[2][c], d3 = v[4][c] - v[3][c];
-        const T s0 = half_slope(d0, d1, d0 + d1), s1 = half_slope(d1, d2, d1 + d2), s2 = half_slope(d2, d3, d2 + d3);
-        lm[c] = fma(cl0, s0, v[1][c]);
-        rm[c] = fma(-cr1, s1, v[2][c]);
-        lp[c] = fma(cl1, s1, v[2][c]);
-        rp[c] = fma(-cr2, s2, v[3][c]);
-        lap[c] += d2 - d1;
-    }
-    T fm[3], fp[3];
-    upwind_flux(lm, rm, a, fm);
-    upwind_flux(lp, rp, a, fp);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) conv[c] += fp[c] - fm[c];
-}
 
 // A cell's gradient sums from its corners on one node plane: x and y
 // differences, and the corners themselves for the z differences.  Differences
@@ -109,107 +56,393 @@ template <typename T> __device__ __forceinline__ T z_corners(T s0[4], const T s1
     return r;
 }
 
-// Right-hand side of the predictor at every cell,
-//   u^n + dt (-div(u u) - G p / rho + (nu / 2) L_c u^n + g).
-// Along z the five cells, the lower face's flux and the middle cell's states
-// stay in registers from plane to plane.
+// ---- the predictor's right-hand side in three arithmetics --------------------
 struct RhsArgs {
     double k;            // dt / h
     double cc, cg, cl;   // -dt / h, -dt / (4 h rho), nu dt / (2 h^2)
     double dg[3];        // dt g
 };
-constexpr int kStencilThreads = 256;
-template <typename T>
-__global__ void __launch_bounds__(kStencilThreads) k_predictor_rhs(LevelDims d, const T *__restrict__ u,
-                                                                   const T *__restrict__ p, RhsArgs a,
-                                                                   T *__restrict__ out) {
-    const Column q(d);
-    const int m0 = d.n0 - 1, m1 = d.n1 - 1, m2 = d.n2 - 1;
-    const size_t plane = (size_t)d.n0 * d.n1, N = plane * d.n2;
-    const T k = (T)a.k, cc = (T)a.cc, cg = (T)a.cg, cl = (T)a.cl;
-    const int row = q.j * d.n0, i0 = row + q.i;
-    int ix[4], iy[4];  // in-plane neighbours -2, -1, +1, +2
-#pragma unroll
-    for (int o = 0; o < 4; ++o) {
-        const int s = o < 2 ? o - 2 : o - 1;
-        ix[o] = row + ((q.i + s) & m0);
-        iy[o] = ((q.j + s) & m1) * d.n0 + q.i;
+
+// FP32 and FP64 as they stand.  kc: a cell's dt/h u_a; up / down: its states
+// towards the faces above and below, v +- (1 -+ c) m; half_slope: half the
+// monotonized-central slope from the differences a (below) and b (above),
+// min(|a|, |b|, |a + b| / 4) with their sign, 0 at extrema.
+template <typename R> struct PlainNum {
+    using T = R;
+    using V = R;
+    R k, cc, cg, cl;
+    __device__ PlainNum(const RhsArgs &a, int, int) : k((R)a.k), cc((R)a.cc), cg((R)a.cg), cl((R)a.cl) {}
+    __device__ __forceinline__ V u(T x) const { return x; }
+    __device__ __forceinline__ V p(T x) const { return x; }
+    __device__ __forceinline__ V kc(V v) const { return k * v; }
+    __device__ __forceinline__ V up(V v, V c, V m) const { return fma((R)1 - c, m, v); }
+    __device__ __forceinline__ V down(V v, V c, V m) const { return fma((R)-1 - c, m, v); }
+    __device__ __forceinline__ V half_slope(V a, V b) const {
+        const R s = a + b, m = fmin(fmin(fabs(a), fabs(b)), (R)0.25 * fabs(s));
+        return a * b > (R)0 ? copysign(m, s) : (R)0;
     }
-    const int px = row + ((q.i + 1) & m0), py = ((q.j + 1) & m1) * d.n0 + q.i, pxy = ((q.j + 1) & m1) * d.n0 + ((q.i + 1) & m0);
-    auto corners = [&](int kk, T &gx, T &gy, T s[4]) {
-        const T *pk = p + (size_t)kk * plane;
-        plane_corners(pk[i0], pk[px], pk[py], pk[pxy], gx, gy, s);
-    };
-    grid_dep_wait();
-    T z[5][3];
+    __device__ __forceinline__ bool positive(V x) const { return x > (R)0; }
+    __device__ __forceinline__ bool negative(V x) const { return x < (R)0; }
+    __device__ __forceinline__ V product(V un, V s) const { return un * s; }
+    __device__ __forceinline__ T result(T u0, V lap, V conv, V gp, double dg) const {
+        return fma(cl, lap, fma(cc, conv, fma(cg, gp, u0 + (R)dg)));
+    }
+};
+
+// FP64 fields in 64-bit fixed point: u in units of 2^(eu), p of 2^(ep), so that
+// the field's largest |u| and |p| have 59 bits; differences and sums are then
+// exact, and what a small value loses in its conversion is 2^-60 of the
+// field's largest one.  Products round to one unit.  The FP64 pipe (a warp
+// instruction in 16 clocks of an SM) forms only the final sum.
+struct FixedNum {
+    using T = double;
+    using V = long long;
+    static constexpr int kBits = 59;
+    int eu, ep;
+    Halves kk;           // dt/h in units: c = kk v / 2^62 in Q58
+    double cc, cg, cl;   // with the units' powers of two
+    // the ranges in which no sum overflows: |u| and |p| within 2^(+-400) and a
+    // Courant number dt/h max|u| (of the power of two above the maximum) up to 2
+    __device__ static bool fits(const RhsArgs &a, int mu, int mp) {
+        const int e = exponent_of<double>(mu), f = exponent_of<double>(mp);
+        return abs(e - 1023) <= 400 && (f <= 1 || abs(f - 1023) <= 400) && a.k * pow2(e - 1022) <= 2.0;
+    }
+    __device__ static double pow2(int e) { return __hiloint2double((e + 1023) << 20, 0); }
+    __device__ FixedNum(const RhsArgs &a, int mu, int mp)
+        : eu(exponent_of<double>(mu)), ep(exponent_of<double>(mp)) {
+        const int su = eu - 1022 - kBits, sp = ep > 1 ? ep - 1022 - kBits : 0;
+        kk = halves(__double2ll_rn(a.k * pow2(su) * pow2(58 + 62)));
+        cc = a.cc * pow2(2 * su + 63);
+        cg = ep > 1 ? a.cg * pow2(sp) : 0.0;  // a pressure of 0 (or below 2^-1022)
+        cl = a.cl * pow2(su);
+    }
+    __device__ __forceinline__ V u(T x) const { return to_fixed<kBits>(x, eu); }
+    __device__ __forceinline__ V p(T x) const { return to_fixed<kBits>(x, ep); }
+    // a b / 2^SH, rounded
+    template <int SH> __device__ __forceinline__ static V mul(Halves x, Halves y) {
+        const long long s = (long long)x.hi * y.hi;
+        const long long t = (long long)x.hi * y.lo + ((long long)x.lo * y.hi + (1LL << (SH - 33)));
+        return SH == 64 ? s + (t >> 32) : (long long)((unsigned long long)s << (64 - SH)) + (t >> (SH - 32));
+    }
+    // Q61: the Q58 product shifted (its rounding counts against a slope only)
+    __device__ __forceinline__ V kc(V v) const { return mul<62>(halves(v), kk) << 3; }
+    __device__ __forceinline__ V up(V v, V c, V m) const { return v + mul<61>(halves((1LL << 61) - c), halves(m)); }
+    __device__ __forceinline__ V down(V v, V c, V m) const { return v - mul<61>(halves((1LL << 61) + c), halves(m)); }
+    __device__ __forceinline__ V half_slope(V a, V b) const {
+        const V s = a >> 63, x = (a ^ s) - s, y = (b ^ s) - s;  // |a|, |b| where the signs agree
+        V m = x < y ? x : y;
+        const V q = (x + y) >> 2;
+        m = m < q ? m : q;
+        return (a ^ b) < 0 ? 0 : (m ^ s) - s;
+    }
+    __device__ __forceinline__ bool positive(V x) const { return x > 0; }
+    __device__ __forceinline__ bool negative(V x) const { return x < 0; }
+    __device__ __forceinline__ V product(V un, V s) const { return mul<64>(halves(un << 1), halves(s)); }
+    __device__ __forceinline__ T result(T u0, V lap, V conv, V gp, double dg) const {
+        return fma(cl, (double)lap, fma(cc, (double)conv, fma(cg, (double)gp, u0 + dg)));
+    }
+};
+
+// Fluxes of all three components through a face with states l and r, the
+// normal component being a (Burgers Riemann solution, upwinded).
+template <class Q>
+__device__ __forceinline__ void upwind_flux(const Q &q, const typename Q::V l[3], const typename Q::V r[3], int a,
+                                            typename Q::V flux[3]) {
+    const typename Q::V s = l[a] + r[a];
+    const bool up = q.positive(s) && q.positive(l[a]), down = q.negative(s) && q.negative(r[a]);
+    const typename Q::V un = up ? l[a] : (down ? r[a] : 0);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) flux[c] = q.product(un, up ? l[c] : r[c]);
+}
+
+// Right-hand side of the predictor at every cell,
+//   u^n + dt (-div(u u) - G p / rho + (nu / 2) L_c u^n + g),
+// every slope, state and flux formed once.  A CTA marches a TX x TY tile of
+// columns along z: 256 threads own a column each and keep its five cells, the
+// lower z face's flux and the z states in registers; the plane's cells are in
+// shared memory with a halo of two.  A cell's two states along x and y come
+// from its slope; the face above takes the neighbour's lower state (x: the next
+// lane's by a shuffle, y: through shared memory) and passes its flux on the
+// same way.  Three more warps own the halo: they load and convert it and form
+// the tile's outer states and fluxes.
+template <int TX> struct RhsTile {
+    static constexpr int TY = 256 / TX, CELLS = 256, HALO = 96, T = CELLS + HALO;
+    static constexpr int UX = TX + 4, UY = TY + 4, ITEMS = 4 * TX + 4 * TY;  // halo cells of one component
+    static constexpr int PER = (3 * ITEMS + HALO - 1) / HALO;
+};
+template <class V, int TX> struct RhsShared {
+    using S = RhsTile<TX>;
+    V u[3][S::UY][S::UX];
+    V p[S::TY + 1][TX + 1];
+    V ry[3][S::TY + 1][TX], fy[3][S::TY + 1][TX];  // lower y states, lower y faces' fluxes
+    V rx[3][S::TY], fx[3][S::TY];                  // the states above and the fluxes below the tile in x
+};
+
+// A cell's slope terms along one axis (stride of the shared plane): the
+// state towards the upper face and the lower one.
+template <class Q>
+__device__ __forceinline__ typename Q::V states(const Q &q, typename Q::V vm, typename Q::V v0, typename Q::V vp,
+                                                typename Q::V c, typename Q::V &up, typename Q::V &down) {
+    const typename Q::V a = v0 - vm, b = vp - v0, m = q.half_slope(a, b);
+    up = q.up(v0, c, m);
+    down = q.down(v0, c, m);
+    return b - a;
+}
+
+template <class Q, int TX>
+__device__ __forceinline__ void rhs_tile(const Q q, const LevelDims &d, const typename Q::T *__restrict__ u,
+                                         const typename Q::T *__restrict__ p, const RhsArgs &a,
+                                         typename Q::T *__restrict__ out, RhsShared<typename Q::V, TX> &s) {
+    using S = RhsTile<TX>;
+    using T = typename Q::T;
+    using V = typename Q::V;
+    constexpr int TY = S::TY;
+    const int m0 = d.n0 - 1, m1 = d.n1 - 1, m2 = d.n2 - 1, tid = threadIdx.x;
+    const size_t plane = (size_t)d.n0 * d.n1, N = plane * d.n2;
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, k0 = blockIdx.z * d.zc, k1 = k0 + d.zc;
+    if (tid >= S::CELLS) {
+        // ---- the halo's warps ----
+        const int h = tid - S::CELLS;
+        int off[S::PER], at[S::PER];
+        T raw[S::PER];
+        V *const flat = &s.u[0][0][0];
+#pragma unroll
+        for (int r = 0; r < S::PER; ++r) {
+            const int e = h + r * S::HALO, c = e / S::ITEMS, i = e % S::ITEMS;
+            int x, y;
+            if (i < 4 * TY) y = i >> 2, x = (i & 3) < 2 ? (i & 3) - 2 : TX + (i & 3) - 2;
+            else x = (i - 4 * TY) % TX, y = (i - 4 * TY) / TX, y = y < 2 ? y - 2 : TY + y - 2;
+            at[r] = e < 3 * S::ITEMS ? (c * S::UY + y + 2) * S::UX + x + 2 : -1;
+            off[r] = ((y0 + y) & m1) * d.n0 + ((x0 + x) & m0);
+            if (at[r] >= 0) raw[r] = u[c * N + (size_t)k0 * plane + off[r]];
+        }
+        // pressure nodes above the tile in x and y
+        const bool edge = h < TX + TY + 1;
+        const int ex = h < TX ? h : TX, ey = h < TX ? TY : h - TX;  // (TX, TY) is the last one's
+        const int eo = ((y0 + ey) & m1) * d.n0 + ((x0 + ex) & m0);
+        T praw = 0;
+        if (edge) {
+            s.p[ey][ex] = q.p(p[(size_t)k0 * plane + eo]);
+            praw = p[(size_t)((k0 + 1) & m2) * plane + eo];
+        }
+        __syncthreads();  // the first plane's nodes there
+        __syncthreads();  // and read
+        // the tile's outer faces: lower ones (their flux), then upper ones (the state above)
+        const bool low = h < TX + TY, face = h < 2 * (TX + TY);
+        const int f = low ? h : h - (TX + TY);
+        const bool ax = f < TY;               // an x face of row f, or a y face of column f - TY
+        const int fi = ax ? f : f - TY;
+        const V *b = ax ? &s.u[0][fi + 2][low ? 1 : TX + 2] : &s.u[0][low ? 1 : TY + 2][fi + 2];  // the outer cell
+        const int st = ax ? 1 : S::UX;
+        constexpr int CS = S::UX * S::UY;
+        for (int kk = k0; kk < k1; ++kk) {
+#pragma unroll
+            for (int r = 0; r < S::PER; ++r)
+                if (at[r] >= 0) flat[at[r]] = q.u(raw[r]);
+            if (edge) s.p[ey][ex] = q.p(praw);
+            __syncthreads();  // A
+            if (kk + 1 < k1) {
+#pragma unroll
+                for (int r = 0; r < S::PER; ++r)
+                    if (at[r] >= 0)
+                        raw[r] = u[(h + r * S::HALO) / S::ITEMS * N + (size_t)(kk + 1) * plane + off[r]];
+                if (edge) praw = p[(size_t)((kk + 2) & m2) * plane + eo];
+            }
+            if (face) {
+                const V vn = b[(ax ? 0 : 1) * CS];
+                V up[3], down[3];
+                const V c = q.kc(vn);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const V *e = b + k * CS;
+                    states(q, e[-st], e[0], e[st], c, up[k], down[k]);
+                }
+                if (low) {
+                    V u1[3], d1[3], fl[3];
+                    const V c1 = q.kc(b[(ax ? 0 : 1) * CS + st]);
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        const V *e = b + k * CS + st;
+                        states(q, e[-st], e[0], e[st], c1, u1[k], d1[k]);
+                    }
+                    if (ax) upwind_flux(q, up, d1, 0, fl);
+                    else upwind_flux(q, up, d1, 1, fl);
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) (ax ? s.fx[k][fi] : s.fy[k][0][fi]) = fl[k];
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) (ax ? s.rx[k][fi] : s.ry[k][TY][fi]) = down[k];
+                }
+            }
+            __syncthreads();  // B
+            __syncthreads();  // C
+        }
+        return;
+    }
+    // ---- the cells' threads ----
+    const int tx = tid % TX, ty = tid / TX, i0 = (y0 + ty) * d.n0 + x0 + tx;
+    const unsigned mask = 0xffffffffu;
+    V z[5][3], left[3], fm[3], s0[4];
+    T mid[3], nxt[3];  // the middle cell's own values (its plane and the next)
 #pragma unroll
     for (int o = 0; o < 4; ++o)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) z[o][c] = u[c * N + (size_t)((q.k0 + o - 2) & m2) * plane + i0];
-    // the lower face's flux and the middle cell's left states, as the loop carries them
-    T fm[3], left[3], gx0, gy0, s0[4];
+        for (int c = 0; c < 3; ++c) {
+            const T v = u[c * N + (size_t)((k0 + o - 2) & m2) * plane + i0];
+            z[o][c] = q.u(v);
+            if (o == 2) mid[c] = v;
+            if (o == 3) nxt[c] = v;
+        }
+    s.p[ty][tx] = q.p(p[(size_t)k0 * plane + i0]);
     {
-        const T cl0 = fma(-k, z[1][2], (T)1), cr1 = fma(k, z[2][2], (T)1), cl1 = fma(-k, z[2][2], (T)1);
-        T l[3], r[3];
+        V l[3], r[3], x;
+        const V cl = q.kc(z[1][2]), cn = q.kc(z[2][2]);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const T d0 = z[1][c] - z[0][c], d1 = z[2][c] - z[1][c], d2 = z[3][c] - z[2][c];
-            const T s1 = half_slope(d1, d2, d1 + d2);
-            l[c] = fma(cl0, half_slope(d0, d1, d0 + d1), z[1][c]);
-            r[c] = fma(-cr1, s1, z[2][c]);
-            left[c] = fma(cl1, s1, z[2][c]);
+            states(q, z[0][c], z[1][c], z[2][c], cl, l[c], x);
+            states(q, z[1][c], z[2][c], z[3][c], cn, left[c], r[c]);
         }
-        upwind_flux(l, r, 2, fm);
+        upwind_flux(q, l, r, 2, fm);
     }
-    corners(q.k0, gx0, gy0, s0);
-    for (int kk = q.k0; kk < q.k1; ++kk) {
-        const size_t base = (size_t)kk * plane;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) z[4][c] = u[c * N + (size_t)((kk + 2) & m2) * plane + i0];
-        T conv[3] = {0, 0, 0}, lap[3] = {0, 0, 0};
-        T v[5][3];
+    __syncthreads();  // the first plane's nodes there
+    V gx0, gy0;
+    plane_corners(s.p[ty][tx], s.p[ty][tx + 1], s.p[ty + 1][tx], s.p[ty + 1][tx + 1], gx0, gy0, s0);
+    __syncthreads();  // and read
+    T praw = p[(size_t)((k0 + 1) & m2) * plane + i0];
+    for (int kk = k0; kk < k1; ++kk) {
+        T far[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            v[2][c] = z[2][c];
-#pragma unroll
-            for (int o = 0; o < 4; ++o) v[o < 2 ? o : o + 1][c] = u[c * N + base + ix[o]];
+            far[c] = u[c * N + (size_t)((kk + 2) & m2) * plane + i0];
+            s.u[c][ty + 2][tx + 2] = z[2][c];
         }
-        axis_terms(v, 0, k, conv, lap);
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-#pragma unroll
-            for (int o = 0; o < 4; ++o) v[o < 2 ? o : o + 1][c] = u[c * N + base + iy[o]];
-        axis_terms(v, 1, k, conv, lap);
+        s.p[ty][tx] = q.p(praw);
+        __syncthreads();  // A
+        if (kk + 1 < k1) praw = p[(size_t)((kk + 2) & m2) * plane + i0];
+        V lap[3], conv[3], ly[3];
         {
-            const T cr = fma(k, z[3][2], (T)1), cn = fma(-k, z[3][2], (T)1);
-            T r[3], next[3], fp[3];
+            const V c = q.kc(z[2][1]);
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const T d1 = z[2][c] - z[1][c], d2 = z[3][c] - z[2][c], d3 = z[4][c] - z[3][c];
-                const T s = half_slope(d2, d3, d2 + d3);
-                r[c] = fma(-cr, s, z[3][c]);
-                next[c] = fma(cn, s, z[3][c]);
-                lap[c] += d2 - d1;
-            }
-            upwind_flux(left, r, 2, fp);
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                conv[c] += fp[c] - fm[c];
-                fm[c] = fp[c];
-                left[c] = next[c];
+            for (int k = 0; k < 3; ++k) {
+                V r;
+                lap[k] = states(q, s.u[k][ty + 1][tx + 2], z[2][k], s.u[k][ty + 3][tx + 2], c, ly[k], r);
+                s.ry[k][ty][tx] = r;
             }
         }
-        T gx1, gy1, s1[4];
-        corners((kk + 1) & m2, gx1, gy1, s1);
-        const T gp[3] = {gx0 + gx1, gy0 + gy1, z_corners(s0, s1)};
+        V lx[3], rx[3];
+        {
+            const V c = q.kc(z[2][0]);
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                lap[k] += states(q, s.u[k][ty + 2][tx + 1], z[2][k], s.u[k][ty + 2][tx + 3], c, lx[k], rx[k]);
+        }
+        V gx1, gy1, s1[4];
+        plane_corners(s.p[ty][tx], s.p[ty][tx + 1], s.p[ty + 1][tx], s.p[ty + 1][tx + 1], gx1, gy1, s1);
+        const V gp[3] = {gx0 + gx1, gy0 + gy1, z_corners(s0, s1)};
         gx0 = gx1, gy0 = gy1;
+        __syncthreads();  // B
+        V fy[3];
+        {
+            V r[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            out[c * N + base + i0] = fma(cl, lap[c], fma(cc, conv[c], fma(cg, gp[c], z[2][c] + (T)a.dg[c])));
+            for (int k = 0; k < 3; ++k) r[k] = s.ry[k][ty + 1][tx];
+            upwind_flux(q, ly, r, 1, fy);
 #pragma unroll
-            for (int o = 0; o < 4; ++o) z[o][c] = z[o + 1][c];
+            for (int k = 0; k < 3; ++k) s.fy[k][ty + 1][tx] = fy[k];
+        }
+        {
+            V r[3], f[3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                r[k] = __shfl_down_sync(mask, rx[k], 1, TX);
+                if (tx == TX - 1) r[k] = s.rx[k][ty];
+            }
+            upwind_flux(q, lx, r, 0, f);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                V b = __shfl_up_sync(mask, f[k], 1, TX);
+                if (tx == 0) b = s.fx[k][ty];
+                conv[k] = f[k] - b;
+            }
+        }
+        {
+            V r[3], f[3], next[3];
+            const V c = q.kc(z[3][2]);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                z[4][k] = q.u(far[k]);
+                states(q, z[2][k], z[3][k], z[4][k], c, next[k], r[k]);
+                lap[k] += (z[3][k] - z[2][k]) - (z[2][k] - z[1][k]);
+            }
+            upwind_flux(q, left, r, 2, f);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                conv[k] += f[k] - fm[k];
+                fm[k] = f[k];
+                left[k] = next[k];
+            }
+        }
+        __syncthreads();  // C
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            conv[k] += fy[k] - s.fy[k][ty][tx];
+            out[k * N + (size_t)kk * plane + i0] = q.result(mid[k], lap[k], conv[k], gp[k], a.dg[k]);
+            mid[k] = nxt[k];
+            nxt[k] = far[k];
+#pragma unroll
+            for (int o = 0; o < 4; ++o) z[o][k] = z[o + 1][k];
         }
     }
+}
+
+// FP64: fixed point where the field's maxima fit it, else (a NaN, an infinity,
+// a Courant number above 2) FP64 as it stands.
+template <typename T, int TX>
+__global__ void __launch_bounds__(RhsTile<TX>::T) k_predictor_rhs(LevelDims d, const T *__restrict__ u,
+                                                                  const T *__restrict__ p, RhsArgs a,
+                                                                  const int *__restrict__ maxima, T *__restrict__ out) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    RhsShared<T, TX> &s = *(RhsShared<T, TX> *)smem_raw;
+    grid_dep_wait();
+    if constexpr (sizeof(T) == 8) {
+        const int mu = maxima[0], mp = maxima[1];
+        if (FixedNum::fits(a, mu, mp)) {
+            rhs_tile<FixedNum, TX>(FixedNum(a, mu, mp), d, u, p, a, out, *(RhsShared<long long, TX> *)smem_raw);
+            return;
+        }
+    }
+    rhs_tile<PlainNum<T>, TX>(PlainNum<T>(a, 0, 0), d, u, p, a, out, s);
+}
+
+// The largest magnitudes (high words) of an FP64 velocity field and a nodal
+// field, into words that are zero before.
+constexpr int kMaxThreads = 512;
+__global__ void __launch_bounds__(kMaxThreads) k_field_maxima(long long N, const double2 *__restrict__ u,
+                                                              const double2 *__restrict__ p, int *__restrict__ maxima) {
+    __shared__ int s_max[2];
+    if (threadIdx.x < 2) s_max[threadIdx.x] = 0;
+    __syncthreads();
+    const long long step = (long long)gridDim.x * kMaxThreads;
+    int m[2] = {0, 0};
+    const long long first = (long long)blockIdx.x * kMaxThreads + threadIdx.x;
+#pragma unroll
+    for (int f = 0; f < 2; ++f) {
+        const double2 *v = f ? p : u;
+        const long long n = f ? N / 2 : 3 * (N / 2);
+        int x = 0;
+#pragma unroll 4
+        for (long long i = first; i < n; i += step) {
+            const double2 w = v[i];
+            x = max(x, max(magnitude(w.x), magnitude(w.y)));
+        }
+        m[f] = __reduce_max_sync(0xffffffffu, x);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(&s_max[0], m[0]);
+        atomicMax(&s_max[1], m[1]);
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) atomicMax(maxima + threadIdx.x, s_max[threadIdx.x]);
 }
 
 // A sum of differences.  FP32: compensated (Knuth's TwoSum of every
@@ -407,6 +640,21 @@ static cudaError_t solve(ib_ctx *ctx, const int n[3], int ncomp, const typename 
     return e;
 }
 
+template <typename T, int TX>
+static cudaError_t launch_rhs(ib_ctx *ctx, LevelDims d, const void *u, const void *p, const RhsArgs &a,
+                              const int *maxima, void *out, cudaStream_t s) {
+    using S = RhsTile<TX>;
+    const size_t smem = sizeof(RhsShared<T, TX>);
+    auto k = k_predictor_rhs<T, TX>;
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const long long tiles = (long long)(d.n0 / TX) * (d.n1 / S::TY);
+    d.zc = d.n2 < 32 ? d.n2 : 32;
+    while (d.zc > 4 && tiles * (d.n2 / d.zc) < 4LL * ctx->sm_count) d.zc /= 2;
+    return launch_pdl(k, dim3(d.n0 / TX, d.n1 / S::TY, d.n2 / d.zc), dim3(S::T), smem, s, d, (const T *)u, (const T *)p,
+                      a, maxima, (T *)out);
+}
+
 template <class A>
 static int run_predictor(ib_ctx *ctx, const ib_grid *grid, const void *u, const void *p, double rho_f, double mu,
                          const double g[3], double dt, void *u_star, cudaStream_t s) {
@@ -418,6 +666,7 @@ static int run_predictor(ib_ctx *ctx, const ib_grid *grid, const void *u, const 
     Spectrum<A> c;
     c.c = ar.take<typename A::Mem>(3 * (N / 2));
     c.ny = ar.take<typename A::Mem>(3 * ny);
+    int *maxima = ar.take<int>(2);
     if (!ar.ok()) return oom_error(ar.used, ar.cap);
     const StencilGrid sg(ctx, grid->n);
     const RhsArgs a = {dt / h, -dt / h, -dt / (4.0 * h * rho_f), 0.5 * nu * dt / (h * h), {dt * g[0], dt * g[1], dt * g[2]}};
@@ -425,7 +674,16 @@ static int run_predictor(ib_ctx *ctx, const ib_grid *grid, const void *u, const 
     const SymbolArgs sy = {kSolveHelmholtz, 1.0 / points, 0.5 * nu * dt * 4.0 / (h * h)};
     PhaseTimer tm(ctx, IB_PHASE_FLUID_PREDICTOR, s);
     // the right-hand side in u_star, the point buffers in the workspace
-    cudaError_t e = launch_pdl(k_predictor_rhs<T>, sg.grid, sg.block, 0, s, sg.d, (const T *)u, (const T *)p, a, (T *)u_star);
+    cudaError_t e = cudaSuccess;
+    if constexpr (sizeof(T) == 8) {
+        e = cudaMemsetAsync(maxima, 0, 2 * sizeof(int), s);
+        if (e == cudaSuccess) {
+            k_field_maxima<<<2 * ctx->sm_count, kMaxThreads, 0, s>>>((long long)N, (const double2 *)u, (const double2 *)p, maxima);
+            e = cudaGetLastError();
+        }
+    }
+    if (e == cudaSuccess) e = sg.d.n0 >= 32 ? launch_rhs<T, 32>(ctx, sg.d, u, p, a, maxima, u_star, s)
+                                            : launch_rhs<T, 16>(ctx, sg.d, u, p, a, maxima, u_star, s);
     if (e == cudaSuccess) e = solve<A, A>(ctx, grid->n, 3, (const T *)u_star, c, sy, kXField, (T *)u_star, nullptr, s);
     if (e != cudaSuccess) return set_error(IB_ERR_CUDA, "fluid_predictor: %s", cudaGetErrorString(e));
     return check_launch("fluid_predictor");
