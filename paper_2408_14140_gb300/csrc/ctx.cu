@@ -309,24 +309,31 @@ static const FftTables &host_fft_tables() {
         FftTables *h = new FftTables;
         constexpr int n = 2048;
         const long double tau = 6.283185307179586476925286766559005768L, q62 = 4611686018427387904.0L;
+        std::vector<long double> cs(n), sn(n);
         for (int k = 0; k < n; ++k) {
             const int oct = k / (n / 8), r = oct & 1 ? n / 8 - k % (n / 8) : k % (n / 8);
             const long double c0 = cosl(tau * r / n), s0 = sinl(tau * r / n);
             // octants 1, 2, 5, 6 swap sine and cosine; 2 to 5 have a negative cosine, 4 to 7 a negative sine
             const bool swap = ((oct + 1) & 2) != 0;
-            const long double c = (oct >= 2 && oct <= 5 ? -1.0L : 1.0L) * (swap ? s0 : c0);
-            const long double s = (oct >= 4 ? -1.0L : 1.0L) * (swap ? c0 : s0);
-            h->roots32[k] = make_float2((float)c, (float)-s);
-            h->trig32[k] = make_float2((float)c, (float)s);
-            h->trig64[k] = make_double2((double)c, (double)s);
-            const long long v[2] = {llrintl(c * q62), llrintl(-s * q62)};
-            int b[4];
-            for (int a = 0; a < 2; ++a) {
-                b[2 * a] = (int)((v[a] + (1LL << 31)) >> 32);
-                b[2 * a + 1] = (int)(v[a] - (long long)b[2 * a] * (1LL << 32));
-            }
-            h->roots_fx[k] = make_int4(b[0], b[1], b[2], b[3]);
+            cs[k] = (oct >= 2 && oct <= 5 ? -1.0L : 1.0L) * (swap ? s0 : c0);
+            sn[k] = (oct >= 4 ? -1.0L : 1.0L) * (swap ? c0 : s0);
+            h->trig32[k] = make_float2((float)cs[k], (float)sn[k]);
+            h->trig64[k] = make_double2((double)cs[k], (double)sn[k]);
         }
+        int o = 0;
+        for (const TwiddlePass &p : kTwiddlePasses)
+            for (int j = 0; j < p.r; ++j)
+                for (int k = 0; k < p.ns; ++k, ++o) {
+                    const int q = j * k * (n / (p.ns * p.r));  // below n
+                    h->tw32[o] = make_float2((float)cs[q], (float)-sn[q]);
+                    const long long v[2] = {llrintl(cs[q] * q62), llrintl(-sn[q] * q62)};
+                    int b[4];
+                    for (int a = 0; a < 2; ++a) {
+                        b[2 * a] = (int)((v[a] + (1LL << 31)) >> 32);
+                        b[2 * a + 1] = (int)(v[a] - (long long)b[2 * a] * (1LL << 32));
+                    }
+                    h->tw_fx[o] = make_int4(b[0], b[1], b[2], b[3]);
+                }
         return h;
     }();
     return *t;

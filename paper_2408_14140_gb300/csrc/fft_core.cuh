@@ -23,8 +23,7 @@
 
 namespace gbib {
 
-constexpr int kRootBits = 11;            // the tables hold the 2048th roots of unity
-constexpr int kRoots = 1 << kRootBits;
+constexpr int kRoots = 2048;              // (cos, sin)(2 pi k / kRoots), for the symbols
 
 // ---------------------------------------------------------------------------
 // arithmetic
@@ -194,7 +193,7 @@ template <int R, bool INV, typename C> __device__ __forceinline__ void radix(C *
 // thread of the CTA calls this together).
 template <class A, int LOGN, bool INV, int NS, typename At>
 __device__ __forceinline__ void fft_passes(typename A::C *v, int t, typename A::C *sm, At at,
-                                           const typename A::W *__restrict__ roots) {
+                                           const typename A::W *__restrict__ tw) {
     using C = typename A::C;
     constexpr int N = 1 << LOGN, E = A::points(LOGN), TPL = N / E, R = N / NS < E ? N / NS : E, B = E / R;
 #pragma unroll
@@ -205,12 +204,13 @@ __device__ __forceinline__ void fft_passes(typename A::C *v, int t, typename A::
         for (int i = 0; i < R; ++i) x[i] = v[b + i * B];
         if constexpr (NS > 1) {
 #pragma unroll
-            for (int i = 1; i < R; ++i) x[i] = cmulw<INV>(x[i], __ldg(roots + k * i * (kRoots / (NS * R))));
+            for (int i = 1; i < R; ++i) x[i] = cmulw<INV>(x[i], __ldg(tw + (twiddle_offset(NS, R) + i * NS) + k));
         }
         radix<R, INV>(x);
 #pragma unroll
         for (int i = 0; i < R; ++i) v[b + i * B] = x[i];
     }
+    static_assert(NS == 1 || twiddle_offset(NS, R) >= 0, "a pass without twiddle factors");
     if constexpr (NS * R < N) {
         __syncthreads();
 #pragma unroll
@@ -222,13 +222,13 @@ __device__ __forceinline__ void fft_passes(typename A::C *v, int t, typename A::
         __syncthreads();
 #pragma unroll
         for (int m = 0; m < E; ++m) v[m] = sm[at(t + TPL * m)];
-        fft_passes<A, LOGN, INV, NS * R>(v, t, sm, at, roots);
+        fft_passes<A, LOGN, INV, NS * R>(v, t, sm, at, tw);
     }
 }
 template <class A, int LOGN, bool INV, typename At>
 __device__ __forceinline__ void fft_line(typename A::C *v, int t, typename A::C *sm, At at,
-                                         const typename A::W *__restrict__ roots) {
-    fft_passes<A, LOGN, INV, 1>(v, t, sm, at, roots);
+                                         const typename A::W *__restrict__ tw) {
+    fft_passes<A, LOGN, INV, 1>(v, t, sm, at, tw);
 }
 
 // ---------------------------------------------------------------------------

@@ -30,6 +30,10 @@ struct SymbolArgs {
     int kind;
     double scale;  // 1 / (points of the transform) and, for div grad, the constant factor
     double g;      // Helmholtz: 4 coef / h^2
+    float scale32, g32;
+    SymbolArgs(int k, double s, double c) : kind(k), scale(s), g(c), scale32((float)s), g32((float)c) {}
+    __device__ __forceinline__ void get(double &s, double &c) const { s = scale, c = g; }
+    __device__ __forceinline__ void get(float &s, float &c) const { s = scale32, c = g32; }
 };
 
 // The half spectrum of one field: `c` the points kx < n0/2, `ny` those of
@@ -42,7 +46,7 @@ template <class A> struct Spectrum {
 template <class A>
 struct FftGrid {
     int n[3], log2n[3];
-    const typename A::W *roots;                 // [kRoots]
+    const typename A::W *tw;                    // [kTwiddles]
     const typename A::Mem *trig;                // [kRoots] (cos, sin)(2 pi k / kRoots)
 };
 
@@ -114,7 +118,7 @@ template <class A, int LOGN> struct XShape {
 template <class A, int LOGN, int MODE>
 __global__ void __launch_bounds__(XShape<A, LOGN>::T)
 k_fft_x(const typename A::Real *__restrict__ src, Spectrum<A> sp, typename A::Real *__restrict__ dst,
-        typename A::Real *__restrict__ old, int log1, int log2, const typename A::W *__restrict__ roots) {
+        typename A::Real *__restrict__ old, int log1, int log2, const typename A::W *__restrict__ tw) {
     using S = XShape<A, LOGN>;
     using C = typename A::C;
     using R = typename A::Real;
@@ -175,7 +179,7 @@ k_fft_x(const typename A::Real *__restrict__ src, Spectrum<A> sp, typename A::Re
             v[m] = m >= E / 2 ? C{va[m].x + vb[m].y, vb[m].x - va[m].y} : C{va[m].x - vb[m].y, va[m].y + vb[m].x};
         }
     }
-    fft_line<A, LOGN, MODE != kXForward>(v, t, sm, at, roots);
+    fft_line<A, LOGN, MODE != kXForward>(v, t, sm, at, tw);
     grid_dep_launch();
     if constexpr (MODE == kXForward) {
         // separation: the thread's lower points k < n0/2 and their mirrors from
@@ -227,7 +231,7 @@ template <class A, int LOGN> struct YShape {
 
 template <class A, int LOGN, bool INV>
 __global__ void __launch_bounds__(YShape<A, LOGN>::T)
-k_fft_y(Spectrum<A> sp, int logr, int log2, const typename A::W *__restrict__ roots) {
+k_fft_y(Spectrum<A> sp, int logr, int log2, const typename A::W *__restrict__ tw) {
     using S = YShape<A, LOGN>;
     using C = typename A::C;
     constexpr int E = S::E, TPL = S::TPL, LANES = S::LANES;
@@ -255,7 +259,7 @@ k_fft_y(Spectrum<A> sp, int logr, int log2, const typename A::W *__restrict__ ro
     C v[E];
     const int emax = points_in<A, E, fx_bits(LOGN), TPL, false>(z, v, s_max, l, LANES);
     auto at = [l](int p) { return p * LANES + l; };
-    fft_line<A, LOGN, INV>(v, t, sm, at, roots);
+    fft_line<A, LOGN, INV>(v, t, sm, at, tw);
     grid_dep_launch();
 #pragma unroll
     for (int m = 0; m < E; ++m) {
@@ -276,15 +280,17 @@ template <class A, int LOGN> struct ZShape {
 // The inverse symbol times the scale at squared sines and cosines of the half angles.
 template <typename R>
 __device__ __forceinline__ R inverse_symbol(const SymbolArgs &sy, R sx, R cx, R sy2, R cy, R sz, R cz) {
-    if (sy.kind == kSolveHelmholtz) return (R)sy.scale / fma((R)sy.g, sx + sy2 + sz, (R)1);
+    R scale, g;
+    sy.get(scale, g);
+    if (sy.kind == kSolveHelmholtz) return scale / fma(g, sx + sy2 + sz, (R)1);
     // D G's symbol over -4/h^2, zero on its null modes
     const R d = sx * cy * cz + sy2 * cx * cz + sz * cx * cy;
-    return d <= (R)3e-13 ? (R)0 : (R)sy.scale / d;
+    return d <= (R)3e-13 ? (R)0 : scale / d;
 }
 
 template <class A, int LOGN>
 __global__ void __launch_bounds__(ZShape<A, LOGN>::T)
-k_fft_z(Spectrum<A> sp, int logr, int log1, SymbolArgs sy, const typename A::W *__restrict__ roots,
+k_fft_z(Spectrum<A> sp, int logr, int log1, SymbolArgs sy, const typename A::W *__restrict__ tw,
         const typename A::Mem *__restrict__ trig) {
     using S = ZShape<A, LOGN>;
     using C = typename A::C;
@@ -323,7 +329,7 @@ k_fft_z(Spectrum<A> sp, int logr, int log1, SymbolArgs sy, const typename A::W *
     C v[E];
     int emax = points_in<A, E, fx_bits(LOGN), TPL, false>(z, v, s_max[0], l, LANES);
     auto at = [l](int p) { return p * LANES + l; };
-    fft_line<A, LOGN, false>(v, t, sm, at, roots);
+    fft_line<A, LOGN, false>(v, t, sm, at, tw);
 #pragma unroll
     for (int m = 0; m < E; ++m) {
         z[m] = point_out<A, fx_bits(LOGN)>(v[m], emax);
@@ -335,7 +341,7 @@ k_fft_z(Spectrum<A> sp, int logr, int log1, SymbolArgs sy, const typename A::W *
         z[m] = Mem{f * z[m].x, f * z[m].y};
     }
     emax = points_in<A, E, fx_bits(LOGN), TPL, false>(z, v, s_max[1], l, LANES);
-    fft_line<A, LOGN, true>(v, t, sm, at, roots);
+    fft_line<A, LOGN, true>(v, t, sm, at, tw);
     grid_dep_launch();
     if (active) {
 #pragma unroll
@@ -369,20 +375,20 @@ cudaError_t launch_x(int mode, const FftGrid<A> &g, int ncomp, const typename A:
     const dim3 grid(g.n[1] * (g.n[2] / 2) / S::LPC, ncomp);
     auto k = mode == kXForward ? k_fft_x<A, LOGN, kXForward>
                                : (mode == kXField ? k_fft_x<A, LOGN, kXField> : k_fft_x<A, LOGN, kXPressure>);
-    return launch_fft(k, grid, S::T, S::smem, s, src, sp, dst, old, g.log2n[1], g.log2n[2], g.roots);
+    return launch_fft(k, grid, S::T, S::smem, s, src, sp, dst, old, g.log2n[1], g.log2n[2], g.tw);
 }
 template <class A, int LOGN>
 cudaError_t launch_y(bool inverse, const FftGrid<A> &g, int ncomp, Spectrum<A> sp, cudaStream_t s) {
     using S = YShape<A, LOGN>;
     const dim3 grid(g.n[0] / 2 * g.n[2] / S::LANES + (g.n[2] + S::LANES - 1) / S::LANES, ncomp);
     auto k = inverse ? k_fft_y<A, LOGN, true> : k_fft_y<A, LOGN, false>;
-    return launch_fft(k, grid, S::T, S::smem, s, sp, g.log2n[0] - 1, g.log2n[2], g.roots);
+    return launch_fft(k, grid, S::T, S::smem, s, sp, g.log2n[0] - 1, g.log2n[2], g.tw);
 }
 template <class A, int LOGN>
 cudaError_t launch_z(const FftGrid<A> &g, int ncomp, Spectrum<A> sp, const SymbolArgs &sy, cudaStream_t s) {
     using S = ZShape<A, LOGN>;
     const dim3 grid(g.n[0] / 2 * g.n[1] / S::LANES + (g.n[1] + S::LANES - 1) / S::LANES, ncomp);
-    return launch_fft(k_fft_z<A, LOGN>, grid, S::T, S::smem, s, sp, g.log2n[0] - 1, g.log2n[1], sy, g.roots, g.trig);
+    return launch_fft(k_fft_z<A, LOGN>, grid, S::T, S::smem, s, sp, g.log2n[0] - 1, g.log2n[1], sy, g.tw, g.trig);
 }
 
 }  // namespace gbib

@@ -70,8 +70,10 @@ struct RhsArgs {
 template <typename R> struct PlainNum {
     using T = R;
     using V = R;
-    R k, cc, cg, cl;
-    __device__ PlainNum(const RhsArgs &a, int, int) : k((R)a.k), cc((R)a.cc), cg((R)a.cg), cl((R)a.cl) {}
+    static constexpr bool kExact = true;  // u() loses nothing
+    R k, cc, cg, cl, dg[3];
+    __device__ PlainNum(const RhsArgs &a, int, int)
+        : k((R)a.k), cc((R)a.cc), cg((R)a.cg), cl((R)a.cl), dg{(R)a.dg[0], (R)a.dg[1], (R)a.dg[2]} {}
     __device__ __forceinline__ V u(T x) const { return x; }
     __device__ __forceinline__ V p(T x) const { return x; }
     __device__ __forceinline__ V kc(V v) const { return k * v; }
@@ -84,8 +86,8 @@ template <typename R> struct PlainNum {
     __device__ __forceinline__ bool positive(V x) const { return x > (R)0; }
     __device__ __forceinline__ bool negative(V x) const { return x < (R)0; }
     __device__ __forceinline__ V product(V un, V s) const { return un * s; }
-    __device__ __forceinline__ T result(T u0, V lap, V conv, V gp, double dg) const {
-        return fma(cl, lap, fma(cc, conv, fma(cg, gp, u0 + (R)dg)));
+    __device__ __forceinline__ T result(T u0, V lap, V conv, V gp, int c) const {
+        return fma(cl, lap, fma(cc, conv, fma(cg, gp, u0 + dg[c])));
     }
 };
 
@@ -97,10 +99,12 @@ template <typename R> struct PlainNum {
 struct FixedNum {
     using T = double;
     using V = long long;
+    static constexpr bool kExact = false;
     static constexpr int kBits = 59;
     int eu, ep;
     Halves kk;           // dt/h in units: c = kk v / 2^62 in Q58
     double cc, cg, cl;   // with the units' powers of two
+    const double *dg;
     // the ranges in which no sum overflows: |u| and |p| within 2^(+-400) and a
     // Courant number dt/h max|u| (of the power of two above the maximum) up to 2
     __device__ static bool fits(const RhsArgs &a, int mu, int mp) {
@@ -109,7 +113,7 @@ struct FixedNum {
     }
     __device__ static double pow2(int e) { return __hiloint2double((e + 1023) << 20, 0); }
     __device__ FixedNum(const RhsArgs &a, int mu, int mp)
-        : eu(exponent_of<double>(mu)), ep(exponent_of<double>(mp)) {
+        : eu(exponent_of<double>(mu)), ep(exponent_of<double>(mp)), dg(a.dg) {
         const int su = eu - 1022 - kBits, sp = ep > 1 ? ep - 1022 - kBits : 0;
         kk = halves(__double2ll_rn(a.k * pow2(su) * pow2(58 + 62)));
         cc = a.cc * pow2(2 * su + 63);
@@ -138,8 +142,8 @@ struct FixedNum {
     __device__ __forceinline__ bool positive(V x) const { return x > 0; }
     __device__ __forceinline__ bool negative(V x) const { return x < 0; }
     __device__ __forceinline__ V product(V un, V s) const { return mul<64>(halves(un << 1), halves(s)); }
-    __device__ __forceinline__ T result(T u0, V lap, V conv, V gp, double dg) const {
-        return fma(cl, (double)lap, fma(cc, (double)conv, fma(cg, (double)gp, u0 + dg)));
+    __device__ __forceinline__ T result(T u0, V lap, V conv, V gp, int c) const {
+        return fma(cl, (double)lap, fma(cc, (double)conv, fma(cg, (double)gp, u0 + dg[c])));
     }
 };
 
@@ -283,16 +287,10 @@ __device__ __forceinline__ void rhs_tile(const Q q, const LevelDims &d, const ty
     const int tx = tid % TX, ty = tid / TX, i0 = (y0 + ty) * d.n0 + x0 + tx;
     const unsigned mask = 0xffffffffu;
     V z[5][3], left[3], fm[3], s0[4];
-    T mid[3], nxt[3];  // the middle cell's own values (its plane and the next)
 #pragma unroll
     for (int o = 0; o < 4; ++o)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const T v = u[c * N + (size_t)((k0 + o - 2) & m2) * plane + i0];
-            z[o][c] = q.u(v);
-            if (o == 2) mid[c] = v;
-            if (o == 3) nxt[c] = v;
-        }
+        for (int c = 0; c < 3; ++c) z[o][c] = q.u(u[c * N + (size_t)((k0 + o - 2) & m2) * plane + i0]);
     s.p[ty][tx] = q.p(p[(size_t)k0 * plane + i0]);
     {
         V l[3], r[3], x;
@@ -341,6 +339,12 @@ __device__ __forceinline__ void rhs_tile(const Q q, const LevelDims &d, const ty
         const V gp[3] = {gx0 + gx1, gy0 + gy1, z_corners(s0, s1)};
         gx0 = gx1, gy0 = gy1;
         __syncthreads();  // B
+        T mid[3];  // the cell's own values (fixed point: read again, the conversion may have rounded them)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            if constexpr (!Q::kExact) mid[k] = u[k * N + (size_t)kk * plane + i0];
+            else mid[k] = z[2][k];
+        }
         V fy[3];
         {
             V r[3];
@@ -386,9 +390,7 @@ __device__ __forceinline__ void rhs_tile(const Q q, const LevelDims &d, const ty
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             conv[k] += fy[k] - s.fy[k][ty][tx];
-            out[k * N + (size_t)kk * plane + i0] = q.result(mid[k], lap[k], conv[k], gp[k], a.dg[k]);
-            mid[k] = nxt[k];
-            nxt[k] = far[k];
+            out[k * N + (size_t)kk * plane + i0] = q.result(mid[k], lap[k], conv[k], gp[k], k);
 #pragma unroll
             for (int o = 0; o < 4; ++o) z[o][k] = z[o + 1][k];
         }
@@ -398,7 +400,7 @@ __device__ __forceinline__ void rhs_tile(const Q q, const LevelDims &d, const ty
 // FP64: fixed point where the field's maxima fit it, else (a NaN, an infinity,
 // a Courant number above 2) FP64 as it stands.
 template <typename T, int TX>
-__global__ void __launch_bounds__(RhsTile<TX>::T) k_predictor_rhs(LevelDims d, const T *__restrict__ u,
+__global__ void __launch_bounds__(RhsTile<TX>::T, sizeof(T) == 8 ? 2 : 3) k_predictor_rhs(LevelDims d, const T *__restrict__ u,
                                                                   const T *__restrict__ p, RhsArgs a,
                                                                   const int *__restrict__ maxima, T *__restrict__ out) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -617,8 +619,8 @@ struct StencilGrid {
 template <class A> static FftGrid<A> fft_grid(ib_ctx *ctx, const int n[3]) {
     FftGrid<A> g;
     for (int a = 0; a < 3; ++a) g.n[a] = n[a], g.log2n[a] = ilog2_exact(n[a]);
-    if constexpr (A::kFixed) g.roots = ctx->fft_tab->roots_fx;
-    else g.roots = ctx->fft_tab->roots32;
+    if constexpr (A::kFixed) g.tw = ctx->fft_tab->tw_fx;
+    else g.tw = ctx->fft_tab->tw32;
     if constexpr (sizeof(typename A::Real) == 8) g.trig = ctx->fft_tab->trig64;
     else g.trig = ctx->fft_tab->trig32;
     return g;
@@ -671,7 +673,7 @@ static int run_predictor(ib_ctx *ctx, const ib_grid *grid, const void *u, const 
     const StencilGrid sg(ctx, grid->n);
     const RhsArgs a = {dt / h, -dt / h, -dt / (4.0 * h * rho_f), 0.5 * nu * dt / (h * h), {dt * g[0], dt * g[1], dt * g[2]}};
     const double points = (double)N;  // the transforms are unscaled
-    const SymbolArgs sy = {kSolveHelmholtz, 1.0 / points, 0.5 * nu * dt * 4.0 / (h * h)};
+    const SymbolArgs sy(kSolveHelmholtz, 1.0 / points, 0.5 * nu * dt * 4.0 / (h * h));
     PhaseTimer tm(ctx, IB_PHASE_FLUID_PREDICTOR, s);
     // the right-hand side in u_star, the point buffers in the workspace
     cudaError_t e = cudaSuccess;
@@ -703,7 +705,7 @@ static int run_projection(ib_ctx *ctx, const ib_grid *grid, void *u, void *p, do
     if (!ar.ok()) return oom_error(ar.used, ar.cap);
     const StencilGrid sg(ctx, grid->n);
     // p_new = rho_f (D G)^-1 D V   (Eq. ns_lp2 with L p = div((1/rho_f) grad p))
-    const SymbolArgs sy = {kSolveDivGrad, -rho_f * h * h / 4.0 / (double)N, 0.0};
+    const SymbolArgs sy(kSolveDivGrad, -rho_f * h * h / 4.0 / (double)N, 0.0);
     PhaseTimer tm(ctx, IB_PHASE_FLUID_PROJECTION, s);
     cudaError_t e = launch_pdl(k_projection_div<T>, sg.grid, sg.block, 0, s, sg.d, (const T *)u, (const T *)p,
                                0.25 / (h * dt), 0.0625 / (h * h * rho_f), q);

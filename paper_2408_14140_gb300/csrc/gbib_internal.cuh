@@ -181,12 +181,32 @@ __device__ __forceinline__ bool finite3(const double *v) {
 #include <vector>
 
 namespace gbib {
-// The 2048th roots of unity, exp(-2 pi i k / 2048): (cos, -sin) in FP32 and as
-// balanced Q62 halves (re hi, re lo, im hi, im lo), and (cos, sin) in both
-// field types for the operators' symbols.
+// The twiddle factors exp(-2 pi i k j / (NS R)) of a pass of radix R over
+// sub-transforms of length NS, [j][k] with k < NS, so that neighbouring lanes
+// (neighbouring k) read neighbouring factors: gathered from one table of roots
+// they took up to 32 L1 wavefronts a load, and the x passes were bound by them
+// (105 us a pass of 256^3 in FP32, 96 % of L1).
+struct TwiddlePass {
+    int ns, r;
+};
+constexpr TwiddlePass kTwiddlePasses[] = {{8, 8}, {8, 4}, {8, 2}, {64, 8}, {64, 4}, {64, 2}, {512, 2}, {16, 16},
+                                          {16, 8}, {256, 4}};
+__host__ __device__ constexpr int twiddle_offset(int ns, int r) {
+    int o = 0;
+    for (const TwiddlePass &p : kTwiddlePasses) {
+        if (p.ns == ns && p.r == r) return o;
+        o += p.ns * p.r;
+    }
+    return r == 1 ? o : -1;
+}
+constexpr int kTwiddles = twiddle_offset(0, 1);  // the table's length
+
+// Tables of the fluid step's transforms: twiddle factors (cos, -sin) in FP32
+// and as balanced Q62 halves (re hi, re lo, im hi, im lo), and (cos, sin)(2 pi
+// k / 2048) in both field types for the operators' symbols.
 struct FftTables {
-    float2 roots32[2048], trig32[2048];
-    int4 roots_fx[2048];
+    float2 tw32[kTwiddles], trig32[2048];
+    int4 tw_fx[kTwiddles];
     double2 trig64[2048];
 };
 // Device copy of the tables (nullptr and a CUDA error on failure); `s` is a
