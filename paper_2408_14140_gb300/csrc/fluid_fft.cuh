@@ -50,48 +50,70 @@ struct FftGrid {
     const typename A::Mem *trig;                // [kRoots] (cos, sin)(2 pi k / kRoots)
 };
 
-template <int TPL, bool FAST_T>
-struct LineMax {
-    // The largest of a line's values over its TPL threads.  FAST_T: the
-    // line's threads are neighbours in the CTA; else `lanes` lines interleave.
-    __device__ static __forceinline__ int get(int v, int *slot, int line, int lanes) {
-        if (FAST_T) {
+// The unit of a line from its threads' points: mag[] the larger component's
+// magnitude of each point.  FAST_T: the line's threads are neighbours in the
+// CTA; else `lanes` lines interleave.  slot[0], slot[1]: the lines' words for
+// the maximum and the sum, zero before (unused with FAST_T up to a warp).
+template <class A, int M, int TPL, bool FAST_T>
+__device__ __forceinline__ int points_unit(const int (&mag)[M], int *max_slot, int *sum_slot, int line, int lanes) {
+    using R = typename A::Real;
+    int h = 0;
 #pragma unroll
-            for (int o = (TPL < 32 ? TPL : 32) / 2; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-            if (TPL <= 32) return v;
-            if ((threadIdx.x & 31) == 0) atomicMax(slot + line, v);
-        } else {
-            for (int o = lanes; o < 32; o <<= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-            atomicMax(slot + line, v);
-        }
-        __syncthreads();
-        return slot[line];
+    for (int m = 0; m < M; ++m) h = max(h, mag[m]);
+    if (FAST_T) {
+#pragma unroll
+        for (int o = (TPL < 32 ? TPL : 32) / 2; o > 0; o >>= 1) h = max(h, __shfl_xor_sync(0xffffffffu, h, o));
+    } else {
+        for (int o = lanes; o < 32; o <<= 1) h = max(h, __shfl_xor_sync(0xffffffffu, h, o));
     }
-};
-// A thread's points of a line to the transform's arithmetic and back.
-// `slot`: the lines' maxima (zeroed); returns the line's exponent.
-template <class A, int E, int BITS, int TPL, bool FAST_T>
-__device__ __forceinline__ int points_in(const typename A::Mem (&z)[E], typename A::C (&v)[E], int *slot, int line,
-                                         int lanes) {
+    const bool shared = !FAST_T || TPL > 32, first = FAST_T ? (threadIdx.x & 31) == 0 : (int)(threadIdx.x & 31) < lanes;
+    if (shared) {
+        if (first) atomicMax(max_slot + line, h);
+        __syncthreads();
+        h = max_slot[line];
+    }
+    const int emax = exponent_of<R>(h);
+    unsigned s = 0;
+#pragma unroll
+    for (int m = 0; m < M; ++m) s += bound_of<R>(mag[m], emax);
+    if (FAST_T) {
+#pragma unroll
+        for (int o = (TPL < 32 ? TPL : 32) / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    } else {
+        for (int o = lanes; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    }
+    if (shared) {
+        if (first) atomicAdd((unsigned *)sum_slot + line, s);
+        __syncthreads();
+        s = (unsigned)sum_slot[line];
+    }
+    return line_unit<R>(emax, s);
+}
+
+// A thread's points of a line to the transform's arithmetic and back; returns
+// the line's unit.
+template <class A, int E, int TPL, bool FAST_T>
+__device__ __forceinline__ int points_in(const typename A::Mem (&z)[E], typename A::C (&v)[E], int *max_slot,
+                                         int *sum_slot, int line, int lanes) {
     if constexpr (A::kFixed) {
-        int h = 0;
+        int mag[E];
 #pragma unroll
-        for (int m = 0; m < E; ++m) h = max(h, max(magnitude(z[m].x), magnitude(z[m].y)));
-        const int emax = exponent_of<typename A::Real>(LineMax<TPL, FAST_T>::get(h, slot, line, lanes));
+        for (int m = 0; m < E; ++m) mag[m] = max(magnitude(z[m].x), magnitude(z[m].y));
+        const int unit = points_unit<A, E, TPL, FAST_T>(mag, max_slot, sum_slot, line, lanes);
 #pragma unroll
-        for (int m = 0; m < E; ++m) v[m] = typename A::C{to_fixed<BITS>(z[m].x, emax), to_fixed<BITS>(z[m].y, emax)};
-        return emax;
+        for (int m = 0; m < E; ++m) v[m] = typename A::C{to_fixed(z[m].x, unit), to_fixed(z[m].y, unit)};
+        return unit;
     } else {
 #pragma unroll
         for (int m = 0; m < E; ++m) v[m] = typename A::C{z[m].x, z[m].y};
         return 0;
     }
 }
-template <class A, int BITS> __device__ __forceinline__ typename A::Mem point_out(typename A::C v, int emax) {
+template <class A> __device__ __forceinline__ typename A::Mem point_out(typename A::C v, int unit) {
     typename A::Mem z;
     if constexpr (A::kFixed) {
-        from_fixed<BITS>(v.x, emax, z.x);
-        from_fixed<BITS>(v.y, emax, z.y);
+        from_fixed(v.x, unit, z.x);
+        from_fixed(v.y, unit, z.y);
     } else {
         z.x = v.x;
         z.y = v.y;
@@ -108,24 +130,24 @@ template <class A, int LOGN> struct XShape {
     static constexpr int T = TPL * LPC;
     static constexpr int PITCH = N + N / E;                 // one point of padding per E: conflict-free writes
     static constexpr size_t smem = (size_t)LPC * PITCH * sizeof(typename A::C);
-    static constexpr int BITS = fx_bits(LOGN) - 1;          // one more bit for the sums of the separation
 };
 
 // kXField writes the field; kXPressure writes p' over the old pressure and
 // beside it, for FP64 fields, the difference p_old - p', whose gradient is all
-// the projection needs; for FP32 fields p_old itself, since the difference's
-// rounding would show in u.
+// the projection needs, and the difference's largest magnitude (high word) in
+// *maxold; for FP32 fields p_old itself, since the difference's rounding would
+// show in u.
 template <class A, int LOGN, int MODE>
 __global__ void __launch_bounds__(XShape<A, LOGN>::T)
 k_fft_x(const typename A::Real *__restrict__ src, Spectrum<A> sp, typename A::Real *__restrict__ dst,
-        typename A::Real *__restrict__ old, int log1, int log2, const typename A::W *__restrict__ tw) {
+        typename A::Real *__restrict__ old, int *__restrict__ maxold, int log1, int log2, const typename A::W *__restrict__ tw) {
     using S = XShape<A, LOGN>;
     using C = typename A::C;
     using R = typename A::Real;
     using Mem = typename A::Mem;
     constexpr int N = S::N, E = S::E, TPL = S::TPL;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int s_max[S::LPC];
+    __shared__ int s_line[2][S::LPC];
     C *sm = (C *)smem_raw;
     const int t = threadIdx.x % TPL, l = threadIdx.x / TPL;
     const long long line = (long long)blockIdx.x * S::LPC + l;  // z' n1 + y
@@ -135,13 +157,13 @@ k_fft_x(const typename A::Real *__restrict__ src, Spectrum<A> sp, typename A::Re
     Mem *ca = sp.c + ((comp + row) >> 1), *cb = ca + (plane >> 1);  // the two rows' half spectra
     Mem *na = sp.ny + ((comp + row) >> LOGN), *nb = na + n1;         // and their points n0/2
     if (A::kFixed && TPL > 32) {
-        if (threadIdx.x < S::LPC) s_max[threadIdx.x] = 0;
+        if (threadIdx.x < 2 * S::LPC) (&s_line[0][0])[threadIdx.x] = 0;
         __syncthreads();
     }
     auto at = [l](int p) { return l * S::PITCH + p + p / E; };
     grid_dep_wait();
     C v[E];
-    int emax;
+    int unit;
     if constexpr (MODE == kXForward) {
         Mem z[E];
 #pragma unroll
@@ -149,29 +171,29 @@ k_fft_x(const typename A::Real *__restrict__ src, Spectrum<A> sp, typename A::Re
             const R *r = src + comp + row + t + TPL * m;
             z[m] = Mem{r[0], r[plane]};
         }
-        emax = points_in<A, E, S::BITS, TPL, true>(z, v, s_max, l, 0);
+        unit = points_in<A, E, TPL, true>(z, v, s_line[0], s_line[1], l, 0);
     } else {
         // Z(k) = A(k) + i B(k), Z(n0 - k) = conj A(k) + i conj B(k); real points
         // at 0 and n0/2.  The sums are formed in the transform's arithmetic.
         Mem a[E], b[E];
         C va[E], vb[E];
-        int h = 0;
+        int mag[2 * E];
 #pragma unroll
         for (int m = 0; m < E; ++m) {
             const int p = t + TPL * m, k = m >= E / 2 ? (N - p) & (N / 2 - 1) : p;
             const bool mid = m == E / 2 && t == 0;
             a[m] = *(mid ? na : ca + k), b[m] = *(mid ? nb : cb + k);
             if (mid || p == 0) a[m].y = b[m].y = 0;
-            if (A::kFixed)
-                h = max(h, max(max(magnitude(a[m].x), magnitude(a[m].y)), max(magnitude(b[m].x), magnitude(b[m].y))));
+            mag[2 * m] = max(magnitude(a[m].x), magnitude(a[m].y));
+            mag[2 * m + 1] = max(magnitude(b[m].x), magnitude(b[m].y));
         }
-        emax = 0;
-        if constexpr (A::kFixed) emax = exponent_of<R>(LineMax<TPL, true>::get(h, s_max, l, 0));
+        unit = 0;
+        if constexpr (A::kFixed) unit = points_unit<A, 2 * E, TPL, true>(mag, s_line[0], s_line[1], l, 0);
 #pragma unroll
         for (int m = 0; m < E; ++m) {
             if constexpr (A::kFixed) {
-                va[m] = C{to_fixed<S::BITS>(a[m].x, emax), to_fixed<S::BITS>(a[m].y, emax)};
-                vb[m] = C{to_fixed<S::BITS>(b[m].x, emax), to_fixed<S::BITS>(b[m].y, emax)};
+                va[m] = C{to_fixed(a[m].x, unit), to_fixed(a[m].y, unit)};
+                vb[m] = C{to_fixed(b[m].x, unit), to_fixed(b[m].y, unit)};
             } else {
                 va[m] = C{a[m].x, a[m].y};
                 vb[m] = C{b[m].x, b[m].y};
@@ -184,8 +206,9 @@ k_fft_x(const typename A::Real *__restrict__ src, Spectrum<A> sp, typename A::Re
     if constexpr (MODE == kXForward) {
         // separation: the thread's lower points k < n0/2 and their mirrors from
         // shared memory; twice A or B comes in (one more bit of the integers)
+        const int half = unit == kUnitNan ? unit : unit - 1;
         auto put = [&](Mem *at, decltype(v[0].x) x, decltype(v[0].x) y) {
-            const Mem z = point_out<A, S::BITS + 1>(C{x, y}, emax);
+            const Mem z = point_out<A>(C{x, y}, half);
             *at = A::kFixed ? z : Mem{(R)0.5 * z.x, (R)0.5 * z.y};
         };
         __syncthreads();
@@ -206,17 +229,24 @@ k_fft_x(const typename A::Real *__restrict__ src, Spectrum<A> sp, typename A::Re
             put(nb, n.y + n.y, n.y - n.y);
         }
     } else {
+        int big = 0;
 #pragma unroll
         for (int m = 0; m < E; ++m) {
-            const Mem z = point_out<A, S::BITS>(v[m], emax);
+            const Mem z = point_out<A>(v[m], unit);
             const long long i0 = comp + row + t + TPL * m, i1 = i0 + plane;
             if (MODE == kXPressure) {
                 const R a = dst[i0], b = dst[i1];
-                old[i0] = sizeof(R) == 8 ? a - z.x : a;
-                old[i1] = sizeof(R) == 8 ? b - z.y : b;
+                const R c = sizeof(R) == 8 ? a - z.x : a, e = sizeof(R) == 8 ? b - z.y : b;
+                old[i0] = c;
+                old[i1] = e;
+                if (sizeof(R) == 8) big = max(big, max(magnitude(c), magnitude(e)));
             }
             dst[i0] = z.x;
             dst[i1] = z.y;
+        }
+        if (MODE == kXPressure && sizeof(R) == 8) {
+            big = __reduce_max_sync(0xffffffffu, big);
+            if ((threadIdx.x & 31) == 0 && big > *(volatile int *)maxold) atomicMax(maxold, big);
         }
     }
 }
@@ -236,7 +266,7 @@ k_fft_y(Spectrum<A> sp, int logr, int log2, const typename A::W *__restrict__ tw
     using C = typename A::C;
     constexpr int E = S::E, TPL = S::TPL, LANES = S::LANES;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int s_max[LANES];
+    __shared__ int s_line[2][LANES];
     C *sm = (C *)smem_raw;
     const int t = threadIdx.x / LANES, l = threadIdx.x % LANES;
     // LANES lines in (z, kx) order, after them the n2 lines of kx = n0/2
@@ -249,7 +279,7 @@ k_fft_y(Spectrum<A> sp, int logr, int log2, const typename A::W *__restrict__ tw
                                : sp.c + ((long long)blockIdx.y << (LOGN + logr + log2)) +
                                      ((long long)(q >> logr) << (LOGN + logr)) + (q & ((1 << logr) - 1));
     if (A::kFixed) {
-        for (int i = threadIdx.x; i < LANES; i += S::T) s_max[i] = 0;
+        for (int i = threadIdx.x; i < 2 * LANES; i += S::T) (&s_line[0][0])[i] = 0;
         __syncthreads();
     }
     grid_dep_wait();
@@ -257,13 +287,13 @@ k_fft_y(Spectrum<A> sp, int logr, int log2, const typename A::W *__restrict__ tw
 #pragma unroll
     for (int m = 0; m < E; ++m) z[m] = active ? cl[(long long)(t + TPL * m) << step] : typename A::Mem{0, 0};
     C v[E];
-    const int emax = points_in<A, E, fx_bits(LOGN), TPL, false>(z, v, s_max, l, LANES);
+    const int unit = points_in<A, E, TPL, false>(z, v, s_line[0], s_line[1], l, LANES);
     auto at = [l](int p) { return p * LANES + l; };
     fft_line<A, LOGN, INV>(v, t, sm, at, tw);
     grid_dep_launch();
 #pragma unroll
     for (int m = 0; m < E; ++m) {
-        z[m] = point_out<A, fx_bits(LOGN)>(v[m], emax);
+        z[m] = point_out<A>(v[m], unit);
         if (active) cl[(long long)(t + TPL * m) << step] = z[m];
     }
 }
@@ -298,7 +328,7 @@ k_fft_z(Spectrum<A> sp, int logr, int log1, SymbolArgs sy, const typename A::W *
     using Mem = typename A::Mem;
     constexpr int N = S::N, E = S::E, TPL = S::TPL, LANES = S::LANES;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int s_max[2][LANES];
+    __shared__ int s_line[4][LANES];
     C *sm = (C *)smem_raw;
     R *fs = (R *)(smem_raw + S::points);  // [N/2 + 1][LANES] inverse symbols (even in kz)
     const int l = threadIdx.x % LANES, t = threadIdx.x / LANES;
@@ -311,7 +341,7 @@ k_fft_z(Spectrum<A> sp, int logr, int log1, SymbolArgs sy, const typename A::W *
     const int shift = last ? log1 : logr + log1;  // log2 of the points' stride
     Mem *cl = (last ? sp.ny : sp.c) + ((long long)blockIdx.y << (LOGN + shift)) + q;
     if (A::kFixed)
-        for (int i = threadIdx.x; i < 2 * LANES; i += S::T) (&s_max[0][0])[i] = 0;
+        for (int i = threadIdx.x; i < 4 * LANES; i += S::T) (&s_line[0][0])[i] = 0;
     {
         // the thread's lane's symbol at kz = t, t + TPL, ... <= n2/2
         const Mem hx = __ldg(trig + kx * (kRoots / 4 >> logr)), hy = __ldg(trig + ky * (kRoots / 2 >> log1));
@@ -327,12 +357,12 @@ k_fft_z(Spectrum<A> sp, int logr, int log1, SymbolArgs sy, const typename A::W *
 #pragma unroll
     for (int m = 0; m < E; ++m) z[m] = active ? cl[(long long)(t + TPL * m) << shift] : Mem{0, 0};
     C v[E];
-    int emax = points_in<A, E, fx_bits(LOGN), TPL, false>(z, v, s_max[0], l, LANES);
+    int unit = points_in<A, E, TPL, false>(z, v, s_line[0], s_line[1], l, LANES);
     auto at = [l](int p) { return p * LANES + l; };
     fft_line<A, LOGN, false>(v, t, sm, at, tw);
 #pragma unroll
     for (int m = 0; m < E; ++m) {
-        z[m] = point_out<A, fx_bits(LOGN)>(v[m], emax);
+        z[m] = point_out<A>(v[m], unit);
     }
 #pragma unroll
     for (int m = 0; m < E; ++m) {
@@ -340,13 +370,13 @@ k_fft_z(Spectrum<A> sp, int logr, int log1, SymbolArgs sy, const typename A::W *
         const R f = fs[(k <= N / 2 ? k : N - k) * LANES + l];
         z[m] = Mem{f * z[m].x, f * z[m].y};
     }
-    emax = points_in<A, E, fx_bits(LOGN), TPL, false>(z, v, s_max[1], l, LANES);
+    unit = points_in<A, E, TPL, false>(z, v, s_line[2], s_line[3], l, LANES);
     fft_line<A, LOGN, true>(v, t, sm, at, tw);
     grid_dep_launch();
     if (active) {
 #pragma unroll
         for (int m = 0; m < E; ++m) {
-            z[m] = point_out<A, fx_bits(LOGN)>(v[m], emax);
+            z[m] = point_out<A>(v[m], unit);
             cl[(long long)(t + TPL * m) << shift] = z[m];
         }
     }
@@ -354,7 +384,7 @@ k_fft_z(Spectrum<A> sp, int logr, int log1, SymbolArgs sy, const typename A::W *
 
 // ---- launches (defined per arithmetic in their own translation units) --------
 template <class A> cudaError_t fft_x(int mode, const FftGrid<A> &g, int ncomp, const typename A::Real *src,
-                                     Spectrum<A> sp, typename A::Real *dst, typename A::Real *old, cudaStream_t s);
+                                     Spectrum<A> sp, typename A::Real *dst, typename A::Real *old, int *maxold, cudaStream_t s);
 template <class A> cudaError_t fft_y(bool inverse, const FftGrid<A> &g, int ncomp, Spectrum<A> sp, cudaStream_t s);
 template <class A> cudaError_t fft_z(const FftGrid<A> &g, int ncomp, Spectrum<A> sp, const SymbolArgs &sy,
                                      cudaStream_t s);
@@ -370,12 +400,12 @@ inline cudaError_t launch_fft(Kern kern, dim3 grid, int threads, size_t smem, cu
 
 template <class A, int LOGN>
 cudaError_t launch_x(int mode, const FftGrid<A> &g, int ncomp, const typename A::Real *src, Spectrum<A> sp,
-                     typename A::Real *dst, typename A::Real *old, cudaStream_t s) {
+                     typename A::Real *dst, typename A::Real *old, int *maxold, cudaStream_t s) {
     using S = XShape<A, LOGN>;
     const dim3 grid(g.n[1] * (g.n[2] / 2) / S::LPC, ncomp);
     auto k = mode == kXForward ? k_fft_x<A, LOGN, kXForward>
                                : (mode == kXField ? k_fft_x<A, LOGN, kXField> : k_fft_x<A, LOGN, kXPressure>);
-    return launch_fft(k, grid, S::T, S::smem, s, src, sp, dst, old, g.log2n[1], g.log2n[2], g.tw);
+    return launch_fft(k, grid, S::T, S::smem, s, src, sp, dst, old, maxold, g.log2n[1], g.log2n[2], g.tw);
 }
 template <class A, int LOGN>
 cudaError_t launch_y(bool inverse, const FftGrid<A> &g, int ncomp, Spectrum<A> sp, cudaStream_t s) {

@@ -80,8 +80,17 @@ template <typename R> struct PlainNum {
     __device__ __forceinline__ V up(V v, V c, V m) const { return fma((R)1 - c, m, v); }
     __device__ __forceinline__ V down(V v, V c, V m) const { return fma((R)-1 - c, m, v); }
     __device__ __forceinline__ V half_slope(V a, V b) const {
-        const R s = a + b, m = fmin(fmin(fabs(a), fabs(b)), (R)0.25 * fabs(s));
-        return a * b > (R)0 ? copysign(m, s) : (R)0;
+        if constexpr (sizeof(R) == 8) {
+            // comparisons on the integer pipe: the order of non-negative doubles is that of their bits
+            constexpr long long mag = 0x7fffffffffffffffLL;
+            const long long x = __double_as_longlong(a), y = __double_as_longlong(b),
+                            z = __double_as_longlong(0.25 * (a + b));
+            const long long m = min(min(x & mag, y & mag), z & mag);
+            return (x ^ y) < 0 ? 0.0 : __longlong_as_double(m | (x & ~mag));
+        } else {
+            const R s = a + b, m = fmin(fmin(fabs(a), fabs(b)), (R)0.25 * fabs(s));
+            return a * b > (R)0 ? copysign(m, s) : (R)0;
+        }
     }
     __device__ __forceinline__ bool positive(V x) const { return x > (R)0; }
     __device__ __forceinline__ bool negative(V x) const { return x < (R)0; }
@@ -120,8 +129,8 @@ struct FixedNum {
         cg = ep > 1 ? a.cg * pow2(sp) : 0.0;  // a pressure of 0 (or below 2^-1022)
         cl = a.cl * pow2(su);
     }
-    __device__ __forceinline__ V u(T x) const { return to_fixed<kBits>(x, eu); }
-    __device__ __forceinline__ V p(T x) const { return to_fixed<kBits>(x, ep); }
+    __device__ __forceinline__ V u(T x) const { return to_fixed(x, eu - kBits); }
+    __device__ __forceinline__ V p(T x) const { return to_fixed(x, ep - kBits); }
     // a b / 2^SH, rounded
     template <int SH> __device__ __forceinline__ static V mul(Halves x, Halves y) {
         const long long s = (long long)x.hi * y.hi;
@@ -397,23 +406,22 @@ __device__ __forceinline__ void rhs_tile(const Q q, const LevelDims &d, const ty
     }
 }
 
-// FP64: fixed point where the field's maxima fit it, else (a NaN, an infinity,
-// a Courant number above 2) FP64 as it stands.
-template <typename T, int TX>
-__global__ void __launch_bounds__(RhsTile<TX>::T, sizeof(T) == 8 ? 2 : 3) k_predictor_rhs(LevelDims d, const T *__restrict__ u,
-                                                                  const T *__restrict__ p, RhsArgs a,
-                                                                  const int *__restrict__ maxima, T *__restrict__ out) {
+// FP64 fields: the fixed-point kernel where the field's maxima fit it, else (a
+// NaN, an infinity, a Courant number above 2) the plain one, each returning at
+// once where the other serves.  (Both paths in one kernel took its registers
+// for both: the plain one spilled, 2.0 ms at 128^3 against 0.6.)
+template <class Q, int TX, int MINB>
+__global__ void __launch_bounds__(RhsTile<TX>::T, MINB)
+k_predictor_rhs(LevelDims d, const typename Q::T *__restrict__ u, const typename Q::T *__restrict__ p, RhsArgs a,
+                const int *__restrict__ maxima, typename Q::T *__restrict__ out) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    RhsShared<T, TX> &s = *(RhsShared<T, TX> *)smem_raw;
     grid_dep_wait();
-    if constexpr (sizeof(T) == 8) {
-        const int mu = maxima[0], mp = maxima[1];
-        if (FixedNum::fits(a, mu, mp)) {
-            rhs_tile<FixedNum, TX>(FixedNum(a, mu, mp), d, u, p, a, out, *(RhsShared<long long, TX> *)smem_raw);
-            return;
-        }
+    int mu = 0, mp = 0;
+    if constexpr (sizeof(typename Q::T) == 8) {
+        mu = maxima[0], mp = maxima[1];
+        if (FixedNum::fits(a, mu, mp) == Q::kExact) return;
     }
-    rhs_tile<PlainNum<T>, TX>(PlainNum<T>(a, 0, 0), d, u, p, a, out, s);
+    rhs_tile<Q, TX>(Q(a, mu, mp), d, u, p, a, out, *(RhsShared<typename Q::V, TX> *)smem_raw);
 }
 
 // The largest magnitudes (high words) of an FP64 velocity field and a nodal
@@ -445,6 +453,17 @@ __global__ void __launch_bounds__(kMaxThreads) k_field_maxima(long long N, const
     }
     __syncthreads();
     if (threadIdx.x < 2) atomicMax(maxima + threadIdx.x, s_max[threadIdx.x]);
+}
+
+// Maxima (high words) that the linear stencils' fixed point takes: their unit
+// is a normal double, the values finite; or 0.
+__device__ __forceinline__ bool fixed_range(int a, int b) {
+    const int e = a >> 20, f = b >> 20;
+    return (a == 0 || (e >= 64 && e <= 2000)) && (b == 0 || (f >= 64 && f <= 2000));
+}
+// 2^(the unit's exponent) of a field in B bits of its largest value; 0 for a field of zeros.
+__device__ __forceinline__ double fixed_unit(int mag, int B) {
+    return mag ? __hiloint2double((exponent_of<double>(mag) + 1 - B) << 20, 0) : 0.0;
 }
 
 // A sum of differences.  FP32: compensated (Knuth's TwoSum of every
@@ -490,6 +509,7 @@ template <> struct DiffSum<float> {
 template <typename T>
 __global__ void __launch_bounds__(kStencilThreads) k_projection_div(LevelDims d, const T *__restrict__ u,
                                                                     const T *__restrict__ p, double cu, double cp,
+                                                                    const int *__restrict__ maxima,
                                                                     T *__restrict__ out) {
     const Column q(d);
     const int m0 = d.n0 - 1, m1 = d.n1 - 1, m2 = d.n2 - 1;
@@ -521,6 +541,7 @@ __global__ void __launch_bounds__(kStencilThreads) k_projection_div(LevelDims d,
         w[0] = wk[y0 + x0], w[1] = wk[y0 + xm], w[2] = wk[ym + x0], w[3] = wk[ym + xm];
     };
     grid_dep_wait();
+    if (sizeof(T) == 8 && fixed_range(maxima[0], maxima[1])) return;  // k_projection_div_fixed
     T am, bm, cm, a0, b0, c0, wm[4];
     DiffSum<T> xym;
     pressure((q.k0 - 1) & m2, am, bm, cm);
@@ -550,7 +571,8 @@ __global__ void __launch_bounds__(kStencilThreads) k_projection_div(LevelDims d,
 template <typename T>
 __global__ void __launch_bounds__(kStencilThreads) k_projection_update(LevelDims d, T *__restrict__ u,
                                                                        const T *__restrict__ q,
-                                                                       const T *__restrict__ p, double cg) {
+                                                                       const T *__restrict__ p, double cg,
+                                                                       const int *__restrict__ maxima) {
     constexpr bool kTwo = sizeof(T) == 4;
     const Column o(d);
     const int m0 = d.n0 - 1, m1 = d.n1 - 1, m2 = d.n2 - 1;
@@ -562,6 +584,7 @@ __global__ void __launch_bounds__(kStencilThreads) k_projection_update(LevelDims
         plane_corners(pk[i0], pk[px], pk[py], pk[pxy], gx, gy, s);
     };
     grid_dep_wait();
+    if (sizeof(T) == 8 && fixed_range(maxima[2], 0)) return;  // k_projection_update_fixed
     T gx0, gy0, s0[4], hx0 = 0, hy0 = 0, r0[4];
     corners(q, o.k0, gx0, gy0, s0);
     if (kTwo) corners(p, o.k0, hx0, hy0, r0);
@@ -580,6 +603,133 @@ __global__ void __launch_bounds__(kStencilThreads) k_projection_update(LevelDims
         uk[N] = fma((T)cg, g[1], u1);
         uk[2 * N] = fma((T)cg, g[2], u2);
         gx0 = gx1, gy0 = gy1;
+    }
+}
+
+// The two projection stencils of FP64 fields in 64-bit fixed point, units of
+// the field's largest value: the sums are exact in any order, so they are
+// formed from a plane's corner and edge sums in shared memory, and the FP64
+// pipe, which bound the plain kernels (705 and 306 us at 512x128x128), only
+// scales the result.  u has 58 bits (24 terms), p 56 (coefficients up to 96 in
+// all), p_old - p_new 59 (8 terms).
+template <int TX> struct PlaneTile {
+    static constexpr int TY = kStencilThreads / TX;
+};
+
+// Per step k: the cells' plane k and the nodes' plane k + 1 in shared memory,
+// double buffered; out at the nodes' plane k.
+template <int TX>
+__global__ void __launch_bounds__(kStencilThreads, 4)
+k_projection_div_fixed(LevelDims d, const double *__restrict__ u, const double *__restrict__ p, double cu, double cp,
+                       const int *__restrict__ maxima, double *__restrict__ out) {
+    constexpr int TY = PlaneTile<TX>::TY, BU = 58, BP = 56;
+    constexpr int UH = TX + TY + 1, PH = 2 * (TX + 2) + 2 * TY;  // halo values of a component, of the nodes
+    static_assert(3 * UH + PH <= kStencilThreads, "one halo value a thread");
+    __shared__ long long su[2][3][TY + 1][TX + 1], sp[2][TY + 2][TX + 2];
+    const int m0 = d.n0 - 1, m1 = d.n1 - 1, m2 = d.n2 - 1, tid = threadIdx.x;
+    const size_t plane = (size_t)d.n0 * d.n1, N = plane * d.n2;
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, k0 = blockIdx.z * d.zc, k1 = k0 + d.zc;
+    const int tx = tid % TX, ty = tid / TX, i0 = (y0 + ty) * d.n0 + x0 + tx;
+    // the thread's halo value: a cell below the tile (component hc) or a node around it (hc = 3)
+    int hc = tid < 3 * UH ? tid / UH : (tid < 3 * UH + PH ? 3 : 4), hx, hy;
+    if (hc < 3) {
+        const int i = tid % UH;  // column -1 from row -1, then row -1
+        hx = i <= TY ? -1 : i - TY - 1;
+        hy = i <= TY ? i - 1 : -1;
+    } else {
+        const int i = tid - 3 * UH;  // rows -1 and TY, then columns -1 and TX
+        if (i < 2 * (TX + 2)) hx = i % (TX + 2) - 1, hy = i < TX + 2 ? -1 : TY;
+        else hx = (i & 1) ? TX : -1, hy = (i - 2 * (TX + 2)) >> 1;
+    }
+    const int ho = ((y0 + hy) & m1) * d.n0 + ((x0 + hx) & m0);
+    const double *hsrc = (hc < 3 ? u + hc * N : p) + ho;
+    grid_dep_wait();
+    const int mu = maxima[0], mp = maxima[1];
+    if (!fixed_range(mu, mp)) return;  // k_projection_div
+    const int eu = exponent_of<double>(mu), ep = exponent_of<double>(mp);
+    cu *= fixed_unit(mu, BU);
+    cp *= fixed_unit(mp, BP);
+    double ru[3], rp, rh = 0;
+    auto load = [&](int k) {
+        const size_t uk = (size_t)(k & m2) * plane, pk = (size_t)((k + 1) & m2) * plane;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) ru[c] = u[c * N + uk + i0];
+        rp = p[pk + i0];
+        if (hc < 4) rh = hsrc[hc < 3 ? uk : pk];
+    };
+    load(k0 - 2);
+    long long xy0 = 0, w0 = 0, am = 0, a0 = 0, b0 = 0;
+    for (int k = k0 - 2; k < k1; ++k) {
+        const int b = k & 1;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) su[b][c][ty + 1][tx + 1] = to_fixed(ru[c], eu - BU);
+        sp[b][ty + 1][tx + 1] = to_fixed(rp, ep - BP);
+        if (hc < 3) su[b][hc][hy + 1][hx + 1] = to_fixed(rh, eu - BU);
+        else if (hc == 3) sp[b][hy + 1][hx + 1] = to_fixed(rh, ep - BP);
+        if (k + 1 < k1) load(k + 1);
+        __syncthreads();
+        const long long(*U)[TX + 1] = su[b][0], (*V)[TX + 1] = su[b][1], (*W)[TX + 1] = su[b][2];
+        const long long(*P)[TX + 2] = sp[b];
+        const int i = tx + 1, j = ty + 1;
+        const long long xy = (U[j][i] - U[j][i - 1]) + (U[j - 1][i] - U[j - 1][i - 1]) + (V[j][i] - V[j - 1][i]) +
+                             (V[j][i - 1] - V[j - 1][i - 1]);
+        const long long w = (W[j][i] + W[j][i - 1]) + (W[j - 1][i] + W[j - 1][i - 1]);
+        const long long c = (P[j - 1][i - 1] + P[j - 1][i + 1]) + (P[j + 1][i - 1] + P[j + 1][i + 1]);
+        const long long e = (P[j - 1][i] + P[j + 1][i]) + (P[j][i - 1] + P[j][i + 1]), m = P[j][i];
+        // 16 h^2 D G p = (3c + 2e - 4m)(k-1) + (2c - 4e - 24m)(k) + (3c + 2e - 4m)(k+1)
+        const long long a1 = 3 * c + 2 * (e - 2 * m), b1 = 2 * (c - 2 * e - 12 * m);
+        if (k >= k0) {
+            const long long du = (xy0 + xy) + (w - w0), dg = am + b0 + a1;
+            out[(size_t)k * plane + i0] = fma(cp, (double)dg, cu * (double)du);
+        }
+        xy0 = xy, w0 = w, am = a0, a0 = a1, b0 = b1;
+    }
+}
+
+template <int TX>
+__global__ void __launch_bounds__(kStencilThreads, 4)
+k_projection_update_fixed(LevelDims d, double *__restrict__ u, const double *__restrict__ q, double cg,
+                          const int *__restrict__ maxima) {
+    constexpr int TY = PlaneTile<TX>::TY, B = 59, QH = TX + TY + 1;
+    __shared__ long long sq[2][TY + 1][TX + 1];
+    const int m0 = d.n0 - 1, m1 = d.n1 - 1, m2 = d.n2 - 1, tid = threadIdx.x;
+    const size_t plane = (size_t)d.n0 * d.n1, N = plane * d.n2;
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, k0 = blockIdx.z * d.zc, k1 = k0 + d.zc;
+    const int tx = tid % TX, ty = tid / TX, i0 = (y0 + ty) * d.n0 + x0 + tx;
+    // halo nodes: column TX up to row TY, then row TY
+    const int hx = tid <= TY ? TX : tid - TY - 1, hy = tid <= TY ? tid : TY;
+    const int ho = ((y0 + hy) & m1) * d.n0 + ((x0 + hx) & m0);
+    grid_dep_wait();
+    const int mq = maxima[2];
+    if (!fixed_range(mq, 0)) return;  // k_projection_update
+    const int eq = exponent_of<double>(mq);
+    cg *= fixed_unit(mq, B);
+    double rq, rh = 0, v[3];
+    auto load = [&](int k) {  // nodes' plane k + 1, cells' plane k
+        const size_t qk = (size_t)((k + 1) & m2) * plane;
+        rq = q[qk + i0];
+        if (tid < QH) rh = q[qk + ho];
+    };
+    load(k0 - 1);
+    long long gx0 = 0, gy0 = 0, s0 = 0;
+    for (int k = k0 - 1; k < k1; ++k) {
+        const int b = k & 1;
+        sq[b][ty][tx] = to_fixed(rq, eq - B);
+        if (tid < QH) sq[b][hy][hx] = to_fixed(rh, eq - B);
+        if (k + 1 < k1) load(k + 1);
+        double *uk = u + (size_t)k * plane + i0;
+        if (k >= k0)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) v[c] = uk[c * N];
+        __syncthreads();
+        const long long q00 = sq[b][ty][tx], q10 = sq[b][ty][tx + 1], q01 = sq[b][ty + 1][tx], q11 = sq[b][ty + 1][tx + 1];
+        const long long gx = (q10 + q11) - (q00 + q01), gy = (q01 + q11) - (q00 + q10), s = (q00 + q10) + (q01 + q11);
+        if (k >= k0) {
+            uk[0] = fma(cg, (double)(gx0 + gx), v[0]);
+            uk[N] = fma(cg, (double)(gy0 + gy), v[1]);
+            uk[2 * N] = fma(cg, (double)(s - s0), v[2]);
+        }
+        gx0 = gx, gy0 = gy, s0 = s;
     }
 }
 
@@ -630,24 +780,35 @@ template <class A> static FftGrid<A> fft_grid(ib_ctx *ctx, const int n[3]) {
 // arithmetic X, the others in A.
 template <class X, class A>
 static cudaError_t solve(ib_ctx *ctx, const int n[3], int ncomp, const typename A::Real *src, Spectrum<A> c,
-                         const SymbolArgs &sy, int out, typename A::Real *dst, typename A::Real *old, cudaStream_t s) {
+                         const SymbolArgs &sy, int out, typename A::Real *dst, typename A::Real *old, int *maxima,
+                         cudaStream_t s) {
     const FftGrid<X> gx = fft_grid<X>(ctx, n);
     const FftGrid<A> g = fft_grid<A>(ctx, n);
     const Spectrum<X> cx = {c.c, c.ny};
-    cudaError_t e = fft_x<X>(kXForward, gx, ncomp, src, cx, nullptr, nullptr, s);
+    cudaError_t e = fft_x<X>(kXForward, gx, ncomp, src, cx, nullptr, nullptr, nullptr, s);
     if (e == cudaSuccess) e = fft_y<A>(false, g, ncomp, c, s);
     if (e == cudaSuccess) e = fft_z<A>(g, ncomp, c, sy, s);
     if (e == cudaSuccess) e = fft_y<A>(true, g, ncomp, c, s);
-    if (e == cudaSuccess) e = fft_x<X>(out, gx, ncomp, nullptr, cx, dst, old, s);
+    if (e == cudaSuccess) e = fft_x<X>(out, gx, ncomp, nullptr, cx, dst, old, maxima, s);
     return e;
 }
 
-template <typename T, int TX>
+// Maxima of u and p into the first of `words` zeroed words.
+static cudaError_t field_maxima(ib_ctx *ctx, size_t N, const double *u, const double *p, int *maxima, int words,
+                                cudaStream_t s) {
+    const cudaError_t e = cudaMemsetAsync(maxima, 0, words * sizeof(int), s);
+    if (e != cudaSuccess) return e;
+    k_field_maxima<<<2 * ctx->sm_count, kMaxThreads, 0, s>>>((long long)N, (const double2 *)u, (const double2 *)p, maxima);
+    return cudaGetLastError();
+}
+
+template <class Q, int TX, int MINB>
 static cudaError_t launch_rhs(ib_ctx *ctx, LevelDims d, const void *u, const void *p, const RhsArgs &a,
                               const int *maxima, void *out, cudaStream_t s) {
     using S = RhsTile<TX>;
-    const size_t smem = sizeof(RhsShared<T, TX>);
-    auto k = k_predictor_rhs<T, TX>;
+    using T = typename Q::T;
+    const size_t smem = sizeof(RhsShared<typename Q::V, TX>);
+    auto k = k_predictor_rhs<Q, TX, MINB>;
     const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const long long tiles = (long long)(d.n0 / TX) * (d.n1 / S::TY);
@@ -655,6 +816,21 @@ static cudaError_t launch_rhs(ib_ctx *ctx, LevelDims d, const void *u, const voi
     while (d.zc > 4 && tiles * (d.n2 / d.zc) < 4LL * ctx->sm_count) d.zc /= 2;
     return launch_pdl(k, dim3(d.n0 / TX, d.n1 / S::TY, d.n2 / d.zc), dim3(S::T), smem, s, d, (const T *)u, (const T *)p,
                       a, maxima, (T *)out);
+}
+// CTAs per SM: FP32 three (56 registers), fixed point two (80, some spilled: 22
+// warps hide more than 11 without), plain FP64 one.
+template <int TX>
+static cudaError_t predictor_rhs(ib_ctx *ctx, const LevelDims &d, const float *u, const float *p, const RhsArgs &a, int *,
+                                 float *out, cudaStream_t s) {
+    return launch_rhs<PlainNum<float>, TX, 3>(ctx, d, u, p, a, nullptr, out, s);
+}
+template <int TX>
+static cudaError_t predictor_rhs(ib_ctx *ctx, const LevelDims &d, const double *u, const double *p, const RhsArgs &a,
+                                 int *maxima, double *out, cudaStream_t s) {
+    cudaError_t e = field_maxima(ctx, (size_t)d.n0 * d.n1 * d.n2, u, p, maxima, 2, s);
+    if (e == cudaSuccess) e = launch_rhs<FixedNum, TX, 2>(ctx, d, u, p, a, maxima, out, s);
+    if (e == cudaSuccess) e = launch_rhs<PlainNum<double>, TX, 1>(ctx, d, u, p, a, maxima, out, s);
+    return e;
 }
 
 template <class A>
@@ -676,17 +852,9 @@ static int run_predictor(ib_ctx *ctx, const ib_grid *grid, const void *u, const 
     const SymbolArgs sy(kSolveHelmholtz, 1.0 / points, 0.5 * nu * dt * 4.0 / (h * h));
     PhaseTimer tm(ctx, IB_PHASE_FLUID_PREDICTOR, s);
     // the right-hand side in u_star, the point buffers in the workspace
-    cudaError_t e = cudaSuccess;
-    if constexpr (sizeof(T) == 8) {
-        e = cudaMemsetAsync(maxima, 0, 2 * sizeof(int), s);
-        if (e == cudaSuccess) {
-            k_field_maxima<<<2 * ctx->sm_count, kMaxThreads, 0, s>>>((long long)N, (const double2 *)u, (const double2 *)p, maxima);
-            e = cudaGetLastError();
-        }
-    }
-    if (e == cudaSuccess) e = sg.d.n0 >= 32 ? launch_rhs<T, 32>(ctx, sg.d, u, p, a, maxima, u_star, s)
-                                            : launch_rhs<T, 16>(ctx, sg.d, u, p, a, maxima, u_star, s);
-    if (e == cudaSuccess) e = solve<A, A>(ctx, grid->n, 3, (const T *)u_star, c, sy, kXField, (T *)u_star, nullptr, s);
+    cudaError_t e = sg.d.n0 >= 32 ? predictor_rhs<32>(ctx, sg.d, (const T *)u, (const T *)p, a, maxima, (T *)u_star, s)
+                                  : predictor_rhs<16>(ctx, sg.d, (const T *)u, (const T *)p, a, maxima, (T *)u_star, s);
+    if (e == cudaSuccess) e = solve<A, A>(ctx, grid->n, 3, (const T *)u_star, c, sy, kXField, (T *)u_star, nullptr, nullptr, s);
     if (e != cudaSuccess) return set_error(IB_ERR_CUDA, "fluid_predictor: %s", cudaGetErrorString(e));
     return check_launch("fluid_predictor");
 }
@@ -702,17 +870,31 @@ static int run_projection(ib_ctx *ctx, const ib_grid *grid, void *u, void *p, do
     c.c = ar.take<typename A::Mem>(N / 2);
     c.ny = ar.take<typename A::Mem>((size_t)grid->n[1] * grid->n[2]);
     T *q = ar.take<T>(N);
+    int *maxima = ar.take<int>(3);
     if (!ar.ok()) return oom_error(ar.used, ar.cap);
     const StencilGrid sg(ctx, grid->n);
     // p_new = rho_f (D G)^-1 D V   (Eq. ns_lp2 with L p = div((1/rho_f) grad p))
     const SymbolArgs sy(kSolveDivGrad, -rho_f * h * h / 4.0 / (double)N, 0.0);
     PhaseTimer tm(ctx, IB_PHASE_FLUID_PROJECTION, s);
-    cudaError_t e = launch_pdl(k_projection_div<T>, sg.grid, sg.block, 0, s, sg.d, (const T *)u, (const T *)p,
-                               0.25 / (h * dt), 0.0625 / (h * h * rho_f), q);
-    if (e == cudaSuccess) e = solve<typename A::Pressure, A>(ctx, grid->n, 1, q, c, sy, kXPressure, (T *)p, q, s);
+    cudaError_t e = cudaSuccess;
+    const double cu = 0.25 / (h * dt), cp = 0.0625 / (h * h * rho_f), cg = dt / (4.0 * h * rho_f);
+    const dim3 block1(kStencilThreads);
+    if constexpr (sizeof(T) == 8) {
+        e = field_maxima(ctx, N, (const double *)u, (const double *)p, maxima, 3, s);
+        auto k = sg.d.n0 >= 32 ? k_projection_div_fixed<32> : k_projection_div_fixed<16>;
+        if (e == cudaSuccess)
+            e = launch_pdl(k, sg.grid, block1, 0, s, sg.d, (const double *)u, (const double *)p, cu, cp, maxima, (double *)q);
+    }
     if (e == cudaSuccess)
-        e = launch_pdl(k_projection_update<T>, sg.grid, sg.block, 0, s, sg.d, (T *)u, (const T *)q,
-                       (const T *)p, dt / (4.0 * h * rho_f));
+        e = launch_pdl(k_projection_div<T>, sg.grid, sg.block, 0, s, sg.d, (const T *)u, (const T *)p, cu, cp, maxima, q);
+    if (e == cudaSuccess)
+        e = solve<typename A::Pressure, A>(ctx, grid->n, 1, q, c, sy, kXPressure, (T *)p, q, maxima + 2, s);
+    if constexpr (sizeof(T) == 8) {
+        auto k = sg.d.n0 >= 32 ? k_projection_update_fixed<32> : k_projection_update_fixed<16>;
+        if (e == cudaSuccess) e = launch_pdl(k, sg.grid, block1, 0, s, sg.d, (double *)u, (const double *)q, cg, maxima);
+    }
+    if (e == cudaSuccess)
+        e = launch_pdl(k_projection_update<T>, sg.grid, sg.block, 0, s, sg.d, (T *)u, (const T *)q, (const T *)p, cg, maxima);
     if (e != cudaSuccess) return set_error(IB_ERR_CUDA, "level_projection: %s", cudaGetErrorString(e));
     return check_launch("level_projection");
 }

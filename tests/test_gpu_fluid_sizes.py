@@ -104,3 +104,22 @@ def test_zero_and_nonfinite_fields(api, prec):
         assert not torch.isfinite(u).any()
     ctx.status()
     ctx.close()
+
+
+@pytest.mark.parametrize("n", [(16, 32, 64), (64, 16, 16)])
+@pytest.mark.parametrize("scale,cfl", [(1.0, 5.0), (2.0 ** 500, 0.1), (2.0 ** -500, 0.1), (1.0, 0.1)])
+def test_predictor_beyond_the_fixed_point_range(api, n, scale, cfl):
+    """FP64 right-hand sides outside the fixed-point kernel's range (Courant
+    number above 2, |u| beyond 2^400) and inside it, and a pressure of zero:
+    all at the FP64 gate.  Scaling u by s, p by s^2 and dt by 1/s scales the
+    step by s."""
+    h, u, p = inputs(n, 0, 13)
+    dt = cfl * h / np.abs(u).max()
+    ctx = api.Context()
+    for q in (p, 0 * p):
+        ref = fluid.predictor(u, q, 1.0, 0.01, (0.0, 0.0, 0.0), dt, h)
+        us = ctx.fluid_predictor(dev(u * scale, torch.float64), dev(q * scale * scale, torch.float64), h, 1.0,
+                                 0.01 * scale, (0.0, 0.0, 0.0), dt / scale)
+        assert nerr(us / scale, ref) <= TOL[0]
+    ctx.status()
+    ctx.close()
