@@ -267,6 +267,17 @@ __device__ __forceinline__ long long to_fixed(float x, int unit) {
     return fixed_of((unsigned long long)((b & 0x7fffffu) | (e ? 1u << 23 : 0u)) << 39, e, unit, (int)b < 0);
 }
 
+// u units at or beyond the ends of the normal range, by two scalings; calls,
+// so that the transforms' code stays small.
+static __device__ __noinline__ unsigned long long scaled_bits64(unsigned long long u, int unit) {
+    const int k = unit - 1022;
+    return (unsigned long long)__double_as_longlong(ldexp(ldexp((double)(long long)u, k / 2), k - k / 2));
+}
+static __device__ __noinline__ unsigned scaled_bits32(unsigned long long u, int unit) {
+    const int k = unit - 126;
+    return (unsigned)__float_as_int(ldexpf(ldexpf((float)(long long)u, k / 2), k - k / 2));
+}
+
 // F units, rounded; NaN for kUnitNan.
 __device__ __forceinline__ void from_fixed(long long F, int unit, double &out) {
     const unsigned long long u = F < 0 ? 0ull - (unsigned long long)F : (unsigned long long)F;
@@ -277,11 +288,7 @@ __device__ __forceinline__ void from_fixed(long long F, int unit, double &out) {
     unsigned long long r = ((unsigned long long)(unsigned)(e - 1) << 52) + m;
     if (unit == kUnitNan) r = 0x7ff8000000000000ull;
     else if (u == 0) r = 0;
-    else if (e < 1 || e > 2045) {
-        // at or beyond the ends of the normal range: two scalings
-        const int k = unit - 1022;
-        r = (unsigned long long)__double_as_longlong(ldexp(ldexp((double)(long long)u, k / 2), k - k / 2));
-    }
+    else if (e < 1 || e > 2045) r = scaled_bits64(u, unit);
     out = __longlong_as_double((long long)(r | ((unsigned long long)F & 0x8000000000000000ull)));
 }
 __device__ __forceinline__ void from_fixed(long long F, int unit, float &out) {
@@ -293,10 +300,7 @@ __device__ __forceinline__ void from_fixed(long long F, int unit, float &out) {
     unsigned r = ((unsigned)(e - 1) << 23) + m;
     if (unit == kUnitNan) r = 0x7fc00000u;
     else if (u == 0) r = 0;
-    else if (e < 1 || e > 253) {
-        const int k = unit - 126;
-        r = (unsigned)__float_as_int(ldexpf(ldexpf((float)(long long)u, k / 2), k - k / 2));
-    }
+    else if (e < 1 || e > 253) r = scaled_bits32(u, unit);
     out = __int_as_float((int)(r | (F < 0 ? 0x80000000u : 0u)));
 }
 

@@ -307,16 +307,42 @@ template <class A, int LOGN> struct ZShape {
     static constexpr size_t smem = points + (size_t)(N / 2 + 1) * LANES * sizeof(typename A::Real);
 };
 
-// The inverse symbol times the scale at squared sines and cosines of the half angles.
-template <typename R>
-__device__ __forceinline__ R inverse_symbol(const SymbolArgs &sy, R sx, R cx, R sy2, R cy, R sz, R cz) {
-    R scale, g;
-    sy.get(scale, g);
-    if (sy.kind == kSolveHelmholtz) return scale / fma(g, sx + sy2 + sz, (R)1);
-    // D G's symbol over -4/h^2, zero on its null modes
-    const R d = sx * cy * cz + sy2 * cx * cz + sz * cx * cy;
-    return d <= (R)3e-13 ? (R)0 : scale / d;
-}
+// The operator along a line (kx, ky), in the squared sine and cosine sz, cz of
+// kz's half angle: Helmholtz 1 + g (sx + sy + sz); D G over -4/h^2,
+// (sx cy + sy cx) cz + (cx cy) sz, as p cz + q sz.  inverse(): the scale over
+// it, 0 on D G's null modes.
+template <typename R> struct LineSymbol {
+    R p, q, scale;
+    bool helmholtz;
+    __device__ __forceinline__ LineSymbol(const SymbolArgs &sy, R sx, R cx, R sy2, R cy) {
+        R g;
+        sy.get(scale, g);
+        helmholtz = sy.kind == kSolveHelmholtz;
+        p = helmholtz ? fma(g, sx + sy2, (R)1) : sx * cy + sy2 * cx;
+        q = helmholtz ? g : cx * cy;
+    }
+    __device__ __forceinline__ R inverse(R sz, R cz) const {
+        const R d = helmholtz ? fma(q, sz, p) : fma(p, cz, q * sz);
+        if (!helmholtz && d <= (R)3e-13) return (R)0;
+        return quotient(scale, d);
+    }
+    __device__ static __forceinline__ float quotient(float a, float d) {
+        if (!(d < 1e37f)) return a / d;
+        const float y = __fdividef(1.0f, d), x = a * y;
+        return fmaf(fmaf(-d, x, a), y, x);
+    }
+    // The FP64 pipe bounds the z pass (16 clocks an operation), so the
+    // reciprocal comes from the 20-bit approximation by one step of third
+    // order, y (1 + e + e^2) with e = 1 - d y, and the quotient's remainder
+    // corrects it: six operations, within an ulp of the division's.
+    __device__ static __forceinline__ double quotient(double a, double d) {
+        if (!(d < 1e300)) return a / d;
+        double y;
+        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+        const double e = fma(-d, y, 1.0), r = fma(y, fma(e, e, e), y), x = a * r;
+        return fma(fma(-d, x, a), r, x);
+    }
+};
 
 template <class A, int LOGN>
 __global__ void __launch_bounds__(ZShape<A, LOGN>::T)
@@ -345,10 +371,10 @@ k_fft_z(Spectrum<A> sp, int logr, int log1, SymbolArgs sy, const typename A::W *
     {
         // the thread's lane's symbol at kz = t, t + TPL, ... <= n2/2
         const Mem hx = __ldg(trig + kx * (kRoots / 4 >> logr)), hy = __ldg(trig + ky * (kRoots / 2 >> log1));
-        const R sx = hx.y * hx.y, cx = hx.x * hx.x, s1 = hy.y * hy.y, c1 = hy.x * hy.x;
+        const LineSymbol<R> sym(sy, hx.y * hx.y, hx.x * hx.x, hy.y * hy.y, hy.x * hy.x);
         for (int kz = t; kz <= N / 2; kz += TPL) {
             const Mem hz = __ldg(trig + kz * (kRoots / 2 / N));
-            fs[kz * LANES + l] = inverse_symbol<R>(sy, sx, cx, s1, c1, hz.y * hz.y, hz.x * hz.x);
+            fs[kz * LANES + l] = sym.inverse(hz.y * hz.y, hz.x * hz.x);
         }
     }
     if (A::kFixed) __syncthreads();
