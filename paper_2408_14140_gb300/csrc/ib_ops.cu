@@ -844,14 +844,6 @@ __global__ void k_marker_order(int P, const int *__restrict__ moff, const int *_
     }
 }
 
-// ---------------------------------------------------------------------------
-// per-slot sort by (row, marker) and row starts.  Tiles with at most
-// kWarpSort candidates are sorted by one warp each (bitonic network in
-// registers, the sorted keys then kept in a warp-private shared-memory
-// region); larger tiles by a whole CTA (bitonic network in shared memory).
-// ---------------------------------------------------------------------------
-constexpr int kWarpSort = 256;
-
 // Case of dense global-tile slot d: the last case whose tile_off <= d.
 __device__ __forceinline__ int case_of_tile(const CaseTab &ct, uint32_t d) {
     if (!ct.arr) return 0;
@@ -914,346 +906,420 @@ __device__ __forceinline__ unsigned long long slot_key(const DevGrid &g, const u
     return ((unsigned long long)bin << 32) | m;
 }
 
-// Writes the sorted candidates, their x offsets and the row starts of slot cs
-// from keys[0..nc) (sorted); `lane`/`nl` split the work over nl threads.
-__device__ __forceinline__ void slot_emit(const DevGrid &g, const uint64_t *anchor, const unsigned long long *keys,
-                                          int nc, uint32_t b, int cs, const int lo[3], const Slots &sl, int lane,
-                                          int nl) {
-    for (int i = lane; i < nc; i += nl) sl.cand[b + i] = (uint32_t)(keys[i] & 0xffffffffu);
-    if (!sl.bins) return;
+// The bins' starts of slot cs (only the particle-resident form reads them):
+// bin_of(i) the bin of sorted candidate i; `lane`/`nl` split the work.
+template <class Bin>
+__device__ __forceinline__ void slot_bins(int nc, int cs, const Slots &sl, int lane, int nl, Bin bin_of) {
     uint16_t *bs = sl.bins + (size_t)cs * kBins;
     for (int r = lane; r < kBins; r += nl) {
         // first index whose bin >= r
         int a = 0, e = nc;
         while (a < e) {
             const int mid = (a + e) >> 1;
-            if ((int)(keys[mid] >> 32) < r) a = mid + 1;
+            if (bin_of(mid) < r) a = mid + 1;
             else e = mid;
         }
         bs[r] = (uint16_t)(r == kBins - 1 ? nc : a);
     }
 }
 
-// Sorts 32 R keys held by one warp, element e = 32 r + lane in x[r], with a
-// bitonic network in registers: partners in other lanes come by shuffle,
-// partners in the same lane are compared directly.
-template <int R>
-__device__ __forceinline__ void warp_bitonic(unsigned long long (&x)[R], int lane) {
+// ---------------------------------------------------------------------------
+// sorted candidates and per-cell gather lists.  A cell's contributions are the
+// candidates whose stencil covers it.  The bin walk of gather_cell visits a
+// tile's bins in ascending (anchor z, y, x) order and a bin's candidates in
+// index order -- in ascending candidate index, the order the tile's candidates
+// are sorted in -- so listing every cell's candidates in ascending index
+// reproduces its summation order.
+//
+// A stencil is a product of three ranges, so cell (x, y, z)'s candidates are
+// the intersection of three bit sets over the candidates: those covering
+// column x, row y and plane z of the tile.  The 24 bit sets come from warp
+// ballots, 32 candidates at a time; a cell's pair count is the population of
+// its intersection, and its list the set bits in ascending order -- no
+// ranking, no atomics and no walk over the candidates.  Only the cells with a
+// list (about a third of the tile's) get a thread for the emission, and the
+// list goes through shared memory, so that pair words and weights leave in
+// coalesced rows.
+//
+// A tile has about 70 candidates and 950 pairs: a CTA of four warps takes one,
+// ten CTAs an SM (eight warps a tile idled in barriers; one warp a tile was
+// bound by its own latency).  It sorts by rank: every thread counts the keys
+// below its own, 32 bits wide, the bin and the marker's distance from the
+// tile's first one (64 where that does not fit).  Tiles of more than kListCand
+// candidates go to a second kernel, whose CTAs sort them by a bitonic network.
+// ---------------------------------------------------------------------------
+constexpr int kListThreads = 128;
+constexpr int kListCtas = 10;               // CTAs of an SM
+constexpr int kListCand = 512;
+constexpr int kListStash = 1792;           // pairs a CTA stages in shared memory (more: memory)
+constexpr int kPairThreads = 256;          // the large tiles' CTAs
+constexpr int kPairWarps = kPairThreads / 32;
+constexpr int kPairWords = kMaxCand / 32;  // words of a bit set
+constexpr int kPairStash = 4096;
+constexpr int kMarkBits = 21;
+static_assert(kTileCells == 4 * kListThreads && kTileCells == 2 * kPairThreads && kBins <= 1 << (32 - kMarkBits),
+              "tile lists");
+
+struct CtaLists {
+    unsigned long long keys[kMaxCand];
+    unsigned set[3 * kTile][kPairWords + 1];
+    int2 band[kTileCells];
+    short first[kMaxCand];
+    int wp[kPairWarps], wb[kPairWarps];
+};
+// (the pairs replace the keys)
+static_assert(sizeof(uint32_t) * kPairStash <= sizeof(unsigned long long) * kMaxCand, "stash");
+
+// Tile coordinates + 3 of a bin's anchor (past the tile for the last bin).
+__device__ __forceinline__ int3 bin_anchor(int bin) {
+    const int row = bin / kBinsPerRow;
+    return make_int3(bin - row * kBinsPerRow, row % kRow, row / kRow);
+}
+
+// Pair words [0, np) from `src` (the staged list, or memory) and the weights.
+template <typename T, class Mark>
+__device__ __forceinline__ void pair_weights(const uint32_t *src, uint32_t *pairs, PS<T> *pw, int np, bool stash,
+                                             const PS<T> *__restrict__ wts, int t0, int nt, Mark mark) {
+    // kPwU pairs per thread at a time: the axis weights of a batch are loaded
+    // together
+    constexpr int kPwU = 4;
+    for (int k0 = t0; k0 < np; k0 += kPwU * nt) {
+        unsigned pk[kPwU];
+        PS<T> wx[kPwU], wy[kPwU], wz[kPwU];
 #pragma unroll
-    for (int k = 2; k <= 32 * R; k <<= 1)
-#pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            if (j >= 32) {
-                const int jr = j >> 5;
-#pragma unroll
-                for (int r = 0; r < R; ++r)
-                    if ((r & jr) == 0) {
-                        const bool asc = ((32 * r + lane) & k) == 0;
-                        const unsigned long long a = x[r], b = x[r | jr];
-                        const bool sw = (a > b) == asc;
-                        x[r] = sw ? b : a;
-                        x[r | jr] = sw ? a : b;
-                    }
-            } else {
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const unsigned long long y = __shfl_xor_sync(0xffffffffu, x[r], j);
-                    // the lower index of a pair keeps the minimum in an
-                    // ascending block, the maximum in a descending one
-                    const bool take_min = ((lane & j) == 0) == (((32 * r + lane) & k) == 0);
-                    x[r] = take_min ? (y < x[r] ? y : x[r]) : (y > x[r] ? y : x[r]);
-                }
-            }
+        for (int u = 0; u < kPwU; ++u) {
+            const int k = k0 + u * nt;
+            pk[u] = k < np ? src[k] : 0u;
+            if (stash && k < np) pairs[k] = pk[u];
         }
-}
-
-// One warp: keys of a tile with nc <= 32 R candidates into wk[0, 32 R), sorted.
-template <int R>
-__device__ __forceinline__ void warp_sort_keys(const DevGrid &g, const uint64_t *anchor, const uint32_t *cand,
-                                               int nc, const int lo[3], unsigned long long *wk, int lane) {
-    unsigned long long x[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const int e = 32 * r + lane;
-        x[r] = e < nc ? slot_key(g, anchor, cand[e], lo) : ~0ull;
+        for (int u = 0; u < kPwU; ++u) {
+            const PS<T> *w = wts + 12 * (size_t)(k0 + u * nt < np ? mark(pk[u] & 0xffff) : 0u);
+            wx[u] = w[(pk[u] >> 16) & 3];
+            wy[u] = w[4 + ((pk[u] >> 18) & 3)];
+            wz[u] = w[8 + ((pk[u] >> 20) & 3)];
+        }
+#pragma unroll
+        for (int u = 0; u < kPwU; ++u) {
+            const int k = k0 + u * nt;
+            if (k < np) pw[k] = pair_weight3(wx[u], wy[u], wz[u]);
+        }
     }
-    warp_bitonic<R>(x, lane);
-#pragma unroll
-    for (int r = 0; r < R; ++r) wk[32 * r + lane] = x[r];
-    __syncwarp();
 }
 
-__global__ void __launch_bounds__(kBlock) k_slot_sort(
+// One 32-candidate word of the tile's 24 bit sets, lane l < 24 returning set l's
+// word: columns, rows, planes covered by the lane's candidate, whose anchor is
+// at r - 3.
+template <int KW>
+__device__ __forceinline__ unsigned cover_word(int3 r, const int dim[3], int lane) {
+    unsigned mine = 0;
+#pragma unroll
+    for (int x = 0; x < kTile; ++x) {
+        const unsigned vx = __ballot_sync(0xffffffffu, (unsigned)(x + 3 - r.x) < (unsigned)KW && x < dim[0]);
+        const unsigned vy = __ballot_sync(0xffffffffu, (unsigned)(x + 3 - r.y) < (unsigned)KW && x < dim[1]);
+        const unsigned vz = __ballot_sync(0xffffffffu, (unsigned)(x + 3 - r.z) < (unsigned)KW && x < dim[2]);
+        if (lane == x) mine = vx;
+        if (lane == kTile + x) mine = vy;
+        if (lane == 2 * kTile + x) mine = vz;
+    }
+    return mine;
+}
+
+// A cell's list from the bit sets, nw words each: candidate | offset << 16.
+template <class Set, class First>
+__device__ __forceinline__ void emit_list(int c, int pos, int np, int nw, Set set, First first, uint32_t *out) {
+    const int x = c & 7, y = (c >> 3) & 7, z = c >> 6, code = x + 4 * y + 16 * z;
+    for (int w = 0; w < nw; ++w) {
+        unsigned m = set(x, w) & set(kTile + y, w) & set(2 * kTile + z, w);
+        while (m) {
+            const int i = 32 * w + __ffs((int)m) - 1;
+            m &= m - 1;
+            if (pos < np) out[pos] = (uint32_t)i | ((uint32_t)(code - first(i)) << 16);
+            ++pos;
+        }
+    }
+}
+
+template <typename T, int KW>
+__global__ void __launch_bounds__(kListThreads, kListCtas) k_tile_lists(
     CaseTab ct, int mode, int ncompact_cap, const int *__restrict__ ncompact_p, SlotGeom sg,
-    const uint32_t *__restrict__ dense_of, const uint32_t *__restrict__ start,
-    const uint64_t *__restrict__ anchor, const int *__restrict__ level, Slots sl, DevStatus *st) {
+    const uint32_t *__restrict__ dense_of, const uint32_t *__restrict__ start, const uint64_t *__restrict__ anchor,
+    const int *__restrict__ level, Slots sl, const PS<T> *__restrict__ wts, int *__restrict__ big,
+    int *__restrict__ nbig) {
+    constexpr int kSetPitch = kListCand / 32 + 1;  // odd: no bank conflicts
+    __shared__ __align__(16) unsigned long long s_keys[kListCand];  // or 32-bit keys
+    __shared__ uint32_t s_mark[kListCand], s_pair[kListStash];
+    __shared__ unsigned s_set[3 * kTile][kSetPitch];
+    __shared__ short s_first[kListCand];
+    __shared__ uint16_t s_rel[kListCand];  // anchor + 3, 4 bits an axis
+    __shared__ uint16_t s_cell[kTileCells], s_base[kTileCells + 2];
+    __shared__ uint32_t s_min[kListThreads / 32], s_max[kListThreads / 32];
+    __shared__ int s_w[kListThreads / 32];
     grid_dep_wait();
-    __shared__ unsigned long long keys[kMaxCand];  // also kBlock/32 warp regions of kWarpSort
     const int ncompact = min(*ncompact_p, ncompact_cap);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    // ---- phase 1: one warp per small tile
-    unsigned long long *wk = keys + warp * kWarpSort;
-    for (int cs = blockIdx.x * nwarp + warp; cs < ncompact; cs += gridDim.x * nwarp) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int kE = kListCand / kListThreads;  // candidates a thread
+    for (int cs = blockIdx.x; cs < ncompact; cs += gridDim.x) {
         const uint32_t d = dense_of[cs];
         const uint32_t b = start[d];
         const int nc = (int)(start[d + 1] - b);
-        if (nc > kWarpSort) continue;
+        if (nc > kListCand) {
+            if (tid == 0) big[atomicAdd(nbig, 1)] = cs;
+            continue;
+        }
+        const uint32_t pb = sl.poff[b];
+        const int room = (int)(sl.poff[b + nc] - pb);  // the tile's share of the pair arrays
         int lo[3], dim[3], lev;
         const int cse = slot_geometry(ct, mode, sg, sl, level, d, b, lo, dim, lev);
         const DevGrid &g = ct.get(cse).g;
-        static_assert(kWarpSort == 256, "warp sorts cover 64, 128 or 256 keys");
-        if (nc <= 64) warp_sort_keys<2>(g, anchor, sl.cand + b, nc, lo, wk, lane);
-        else if (nc <= 128) warp_sort_keys<4>(g, anchor, sl.cand + b, nc, lo, wk, lane);
-        else warp_sort_keys<8>(g, anchor, sl.cand + b, nc, lo, wk, lane);
-        slot_emit(g, anchor, wk, nc, b, cs, lo, sl, lane, 32);
-        if (lane == 0) {
+        uint32_t m[kE], mn = ~0u, mx = 0;
+        int bin[kE];
+#pragma unroll
+        for (int e = 0; e < kE; ++e) {
+            const int i = tid + e * kListThreads;
+            m[e] = 0;
+            bin[e] = 0;
+            if (i < nc) {
+                m[e] = sl.cand[b + i];
+                bin[e] = (int)(slot_key(g, anchor, m[e], lo) >> 32);
+                mn = min(mn, m[e]), mx = max(mx, m[e]);
+            }
+        }
+        mn = __reduce_min_sync(0xffffffffu, mn);
+        mx = __reduce_max_sync(0xffffffffu, mx);
+        if (lane == 0) s_min[warp] = mn, s_max[warp] = mx;
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < kListThreads / 32; ++w) mn = min(mn, s_min[w]), mx = max(mx, s_max[w]);
+        // ranks: keys padded with maxima to a multiple of the vector loads
+        int rank[kE];
+#pragma unroll
+        for (int e = 0; e < kE; ++e) rank[e] = 0;
+        const int ne = (nc + kListThreads - 1) / kListThreads;
+        if (mx - mn < (1u << kMarkBits)) {
+            uint32_t *keys = (uint32_t *)s_keys, key[kE];
+#pragma unroll
+            for (int e = 0; e < kE; ++e) {
+                const int i = tid + e * kListThreads;
+                key[e] = i < nc ? ((uint32_t)bin[e] << kMarkBits) | (m[e] - mn) : ~0u;
+                if (e < ne) keys[i] = key[e];
+            }
+            __syncthreads();
+            for (int j = 0; j < nc; j += 4) {
+                const uint4 q = *(const uint4 *)(keys + j);
+#pragma unroll
+                for (int e = 0; e < kE; ++e)
+                    if (e < ne) rank[e] += (q.x < key[e]) + (q.y < key[e]) + (q.z < key[e]) + (q.w < key[e]);
+            }
+        } else {
+            unsigned long long key[kE];
+#pragma unroll
+            for (int e = 0; e < kE; ++e) {
+                const int i = tid + e * kListThreads;
+                key[e] = i < nc ? ((unsigned long long)bin[e] << 32) | m[e] : ~0ull;
+                if (e < ne) s_keys[i] = key[e];
+            }
+            __syncthreads();
+            for (int j = 0; j < nc; ++j) {
+                const unsigned long long q = s_keys[j];
+#pragma unroll
+                for (int e = 0; e < kE; ++e)
+                    if (e < ne) rank[e] += q < key[e];
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < kE; ++e)
+            if (tid + e * kListThreads < nc) {
+                const int3 q = bin_anchor(bin[e]);
+                const int r = rank[e];
+                sl.cand[b + r] = s_mark[r] = m[e];
+                s_rel[r] = (uint16_t)(q.x | (q.y << 4) | (q.z << 8));
+                s_first[r] = (short)((q.x - 3) + 4 * (q.y - 3) + 16 * (q.z - 3));
+            }
+        __syncthreads();
+        if (sl.bins)
+            slot_bins(nc, cs, sl, tid, kListThreads, [&](int i) {
+                const int q = s_rel[i];
+                return ((q >> 8) * kRow + ((q >> 4) & 15)) * kBinsPerRow + (q & 15);
+            });
+        const int nw = (nc + 31) >> 5;
+        for (int w = warp; w < nw; w += kListThreads / 32) {
+            const int i = 32 * w + lane, q = i < nc ? s_rel[i] : 0xfff;  // past the tile
+            const unsigned mine = cover_word<KW>(make_int3(q & 15, (q >> 4) & 15, q >> 8), dim, lane);
+            if (lane < 3 * kTile) s_set[lane][w] = mine;
+        }
+        __syncthreads();
+        // pairs per cell: thread t owns cells 4t .. 4t + 3 (half a row)
+        int t[4] = {0, 0, 0, 0};
+        {
+            const int x = (4 * tid) & 7, y = (tid >> 1) & 7, z = tid >> 4;
+            for (int w = 0; w < nw; ++w) {
+                const unsigned yz = s_set[kTile + y][w] & s_set[2 * kTile + z][w];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) t[k] += __popc(yz & s_set[x + k][w]);
+            }
+        }
+        // pairs and cells in one scan (at most 512 cells, 512 * 64 pairs)
+        const int v = (t[0] + t[1] + t[2] + t[3]) |
+                      (((t[0] > 0) + (t[1] > 0) + (t[2] > 0) + (t[3] > 0)) << 20);
+        int s = v;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int p = __shfl_up_sync(0xffffffffu, s, o);
+            if (lane >= o) s += p;
+        }
+        if (lane == 31) s_w[warp] = s;
+        __syncthreads();
+        int before = s - v, all = 0;
+#pragma unroll
+        for (int w = 0; w < kListThreads / 32; ++w) {
+            if (w < warp) before += s_w[w];
+            all += s_w[w];
+        }
+        const int nb = all >> 20, np = min(all & 0xfffff, room);  // equal but for a box wider than its grid (reported)
+        int pos = before & 0xfffff, c0 = before >> 20;
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (t[k] > 0) {
+                s_cell[c0] = (uint16_t)(4 * tid + k);
+                s_base[c0++] = (uint16_t)pos;
+                pos += t[k];
+            }
+        if (tid == 0) s_base[nb] = (uint16_t)(all & 0xfffff);
+        __syncthreads();
+        // the lists: a cell's candidates in ascending order
+        const bool stash = np <= kListStash;
+        uint32_t *const pairs = sl.pairs + pb, *const out = stash ? s_pair : pairs;
+        int2 *const band = sl.band + pb;
+        for (int q = tid; q < nb; q += kListThreads) {
+            const int c = s_cell[q], p0 = s_base[q];
+            band[q] = make_int2(c | ((s_base[q + 1] - p0) << 16), p0);
+            emit_list(c, p0, np, nw, [&](int i, int w) { return s_set[i][w]; }, [&](int i) { return s_first[i]; }, out);
+        }
+        __syncthreads();
+        pair_weights<T>(out, pairs, (PS<T> *)sl.pw + pb, np, stash, wts, tid, kListThreads,
+                        [&](int i) { return s_mark[i]; });
+        if (tid == 0) {
             sl.geo_lo[cs] = make_int4(lo[0], lo[1], lo[2], lev);
             sl.geo_dim[cs] = make_int4(dim[0], dim[1], dim[2], (int)b);
             sl.geo_case[cs] = cse;
+            sl.nband[cs] = nb;
+            sl.tinfo[cs] = make_int4((int)pb, np, nb, nc);
         }
-        __syncwarp();
+        __syncthreads();  // the next tile overwrites the shared lists
     }
-    __syncthreads();
-    // ---- phase 2: one CTA per large tile.  The CTA's tiles (cs = blockIdx.x
-    // mod gridDim.x) are screened blockDim.x at a time, one load per thread,
-    // and only the large ones are walked.
-    __shared__ int s_big[kBlock];
-    __shared__ int s_nbig;
-    for (long long c0 = blockIdx.x; c0 < ncompact; c0 += (long long)gridDim.x * blockDim.x) {
-        if (threadIdx.x == 0) s_nbig = 0;
-        __syncthreads();
-        const long long ct_cs = c0 + (long long)threadIdx.x * gridDim.x;
-        if (ct_cs < ncompact) {
-            const uint32_t d = dense_of[ct_cs];
-            if ((int)(start[d + 1] - start[d]) > kWarpSort) s_big[atomicAdd(&s_nbig, 1)] = (int)ct_cs;
-        }
-        __syncthreads();
-        const int nbig = s_nbig;
-        for (int q = 0; q < nbig; ++q) {
-            const int cs = s_big[q];
+}
+
+// The tiles of more than kListCand candidates, one CTA each.
+template <typename T, int KW>
+__global__ void __launch_bounds__(kPairThreads) k_tile_lists_large(
+    CaseTab ct, int mode, SlotGeom sg, const uint32_t *__restrict__ dense_of, const uint32_t *__restrict__ start,
+    const uint64_t *__restrict__ anchor, const int *__restrict__ level, Slots sl, const PS<T> *__restrict__ wts,
+    const int *__restrict__ big, const int *__restrict__ nbig_p, DevStatus *st) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    grid_dep_wait();
+    PS<T> *const pwts = (PS<T> *)sl.pw;
+    const int nbig = *nbig_p, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    CtaLists &sh = *(CtaLists *)smem_raw;
+    {
+        for (int q = blockIdx.x; q < nbig; q += gridDim.x) {
+            const int cs = big[q];
             const uint32_t d = dense_of[cs];
             const uint32_t b = start[d];
-            const int nc = (int)(start[d + 1] - b);
+            int nc = (int)(start[d + 1] - b);
             int lo[3], dim[3], lev;
             const int cse = slot_geometry(ct, mode, sg, sl, level, d, b, lo, dim, lev);
             const DevGrid &g = ct.get(cse).g;
+            const uint32_t pb = sl.poff[b];
+            int room = (int)(sl.poff[b + nc] - pb);
             if (nc > kMaxCand) {
                 // report, and leave an empty tile (no bins, no cells)
-                if (sl.bins) {
-                    uint16_t *bs = sl.bins + (size_t)cs * kBins;
-                    for (int r = threadIdx.x; r < kBins; r += blockDim.x) bs[r] = 0;
-                }
-                if (threadIdx.x == 0) {
-                    raise_status(st, IB_ERR_UNSUPPORTED, nc);
-                    sl.geo_lo[cs] = make_int4(lo[0], lo[1], lo[2], lev);
-                    sl.geo_dim[cs] = make_int4(0, 0, 0, (int)b);
-                    sl.geo_case[cs] = cse;
-                }
-                __syncthreads();
-                continue;
+                if (tid == 0) raise_status(st, IB_ERR_UNSUPPORTED, nc);
+                nc = room = 0;
+                dim[0] = dim[1] = dim[2] = 0;
             }
             int np2 = 1;
             while (np2 < nc) np2 <<= 1;
-            for (int i = threadIdx.x; i < np2; i += blockDim.x)
-                keys[i] = i < nc ? slot_key(g, anchor, sl.cand[b + i], lo) : ~0ull;
+            for (int i = tid; i < np2; i += kPairThreads)
+                sh.keys[i] = i < nc ? slot_key(g, anchor, sl.cand[b + i], lo) : ~0ull;
             __syncthreads();
             for (int k = 2; k <= np2; k <<= 1)
                 for (int j = k >> 1; j > 0; j >>= 1) {
-                    for (int i = threadIdx.x; i < np2; i += blockDim.x) {
+                    for (int i = tid; i < np2; i += kPairThreads) {
                         const int ixj = i ^ j;
                         if (ixj > i) {
-                            const unsigned long long x = keys[i], y = keys[ixj];
+                            const unsigned long long x = sh.keys[i], y = sh.keys[ixj];
                             if ((x > y) == ((i & k) == 0)) {
-                                keys[i] = y;
-                                keys[ixj] = x;
+                                sh.keys[i] = y;
+                                sh.keys[ixj] = x;
                             }
                         }
                     }
                     __syncthreads();
                 }
-            slot_emit(g, anchor, keys, nc, b, cs, lo, sl, threadIdx.x, blockDim.x);
-            if (threadIdx.x == 0) {
+            if (sl.bins) slot_bins(nc, cs, sl, tid, kPairThreads, [&](int i) { return (int)(sh.keys[i] >> 32); });
+            // sorted candidates and the bit sets, one word per warp and step
+            const int nw = (nc + 31) >> 5;
+            for (int w = warp; w < nw; w += kPairWarps) {
+                const int i = 32 * w + lane;
+                int3 r = make_int3(15, 15, 15);
+                if (i < nc) {
+                    r = bin_anchor((int)(sh.keys[i] >> 32));
+                    sl.cand[b + i] = (uint32_t)(sh.keys[i] & 0xffffffffu);
+                    sh.first[i] = (short)((r.x - 3) + 4 * (r.y - 3) + 16 * (r.z - 3));
+                }
+                const unsigned mine = cover_word<KW>(r, dim, lane);
+                if (lane < 3 * kTile) sh.set[lane][w] = mine;
+            }
+            __syncthreads();
+            // pairs per cell: thread t owns cells 2t and 2t + 1
+            int t0 = 0, t1 = 0;
+            {
+                const int x = (2 * tid) & 7, y = (tid >> 2) & 7, z = tid >> 5;
+                for (int w = 0; w < nw; ++w) {
+                    const unsigned yz = sh.set[kTile + y][w] & sh.set[2 * kTile + z][w];
+                    t0 += __popc(yz & sh.set[x][w]);
+                    t1 += __popc(yz & sh.set[x + 1][w]);
+                }
+            }
+            int pv = t0 + t1, bv = (t0 > 0) + (t1 > 0);
+            for (int o = 1; o < 32; o <<= 1) {
+                const int yp = __shfl_up_sync(0xffffffffu, pv, o), yb = __shfl_up_sync(0xffffffffu, bv, o);
+                if (lane >= o) pv += yp, bv += yb;
+            }
+            if (lane == 31) sh.wp[warp] = pv, sh.wb[warp] = bv;
+            __syncthreads();
+            int wp = 0, wb = 0, nb = 0, np = 0;
+            for (int w = 0; w < kPairWarps; ++w) {
+                if (w < warp) wp += sh.wp[w], wb += sh.wb[w];
+                nb += sh.wb[w];
+                np += sh.wp[w];
+            }
+            np = min(np, room);
+            const int p0 = wp + pv - (t0 + t1), b0 = wb + bv - ((t0 > 0) + (t1 > 0));
+            if (t0 > 0) sh.band[b0] = make_int2((2 * tid) | (t0 << 16), p0);
+            if (t1 > 0) sh.band[b0 + (t0 > 0)] = make_int2((2 * tid + 1) | (t1 << 16), p0 + t0);
+            __syncthreads();
+            const bool stash = np <= kPairStash;
+            uint32_t *const pairs = sl.pairs + pb, *const spair = (uint32_t *)sh.keys;
+            int2 *const band = sl.band + pb;
+            for (int qb = tid; qb < nb; qb += kPairThreads) {
+                const int2 e = sh.band[qb];
+                band[qb] = e;
+                emit_list(e.x & 0xffff, e.y, np, nw, [&](int i, int w) { return sh.set[i][w]; },
+                          [&](int i) { return sh.first[i]; }, stash ? spair : pairs);
+            }
+            __syncthreads();
+            const uint32_t *cand = sl.cand + b;
+            pair_weights<T>(stash ? spair : pairs, pairs, pwts + pb, np, stash, wts, tid, kPairThreads,
+                            [&](int i) { return cand[i]; });
+            if (tid == 0) {
                 sl.geo_lo[cs] = make_int4(lo[0], lo[1], lo[2], lev);
                 sl.geo_dim[cs] = make_int4(dim[0], dim[1], dim[2], (int)b);
                 sl.geo_case[cs] = cse;
+                sl.nband[cs] = nb;
+                sl.tinfo[cs] = make_int4((int)pb, np, nb, nc);
             }
             __syncthreads();
-        }
-        __syncthreads();  // s_big and s_nbig are reused by the next screen
-    }
-}
-
-// ---------------------------------------------------------------------------
-// per-cell gather lists.  One CTA of 8 warps per compact tile (grid-stride).
-// A cell's contributions are the candidates whose stencil covers it.  The
-// bin walk of gather_cell visits a tile's bins in ascending (anchor z, y, x)
-// order and a bin's candidates in index order -- in ascending candidate
-// index, the order the tile's candidates are sorted in -- so listing every
-// cell's candidates in ascending index reproduces its summation order.
-// The (candidate, stencil cell) pairs are scattered by a stable counting sort
-// on the cell: each warp counts the pairs of a contiguous range of candidates
-// (one candidate per step, one lane per stencil offset, so the cells of a
-// step are distinct), a scan over (cell, warp) gives every warp its base in
-// every cell's list, and each warp then places its pairs candidate by
-// candidate.
-// ---------------------------------------------------------------------------
-constexpr int kPairThreads = 256;
-constexpr int kPairWarps = kPairThreads / 32;
-static_assert(kTileCells == 2 * kPairThreads, "each thread of k_tile_pairs owns two cells");
-
-template <typename T, int KW>
-__global__ void __launch_bounds__(kPairThreads, 5) k_tile_pairs(CaseTab ct, int ncompact_cap,
-                                                             const int *__restrict__ ncompact_p, Slots sl,
-                                                             const uint64_t *__restrict__ anchor,
-                                                             const PS<T> *__restrict__ wts) {
-    PS<T> *const pwts = (PS<T> *)sl.pw;
-    grid_dep_wait();
-    constexpr int KW3 = KW * KW * KW;
-    // per candidate: the in-tile stencil offsets per axis (bits 0-3 x, 4-7 y,
-    // 8-11 z) and its first stencil cell relative to the tile, x + 8 y + 64 z
-    // + 256, from bit 12
-    __shared__ unsigned int s_anc[kMaxCand];
-    __shared__ __align__(16) unsigned int s_cnt[kPairWarps][kTileCells];  // counts, then list cursors
-    __shared__ int s_wp[kPairWarps], s_wb[kPairWarps];
-    const int ncompact = min(*ncompact_p, ncompact_cap);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    // this lane's stencil offsets k = lane + 32 q
-    // (ox | oy << 2 | oz << 4, or ~0u past the stencil)
-    constexpr int kSub = (KW3 + 31) / 32;
-    unsigned kcode[kSub];
-    int koff[kSub];  // the offset's cell step x + 8 y + 64 z
-#pragma unroll
-    for (int q = 0; q < kSub; ++q) {
-        const int k = lane + 32 * q;
-        kcode[q] = k < KW3 ? (unsigned)((k % KW) | (((k / KW) % KW) << 2) | ((k / (KW * KW)) << 4)) : ~0u;
-        koff[q] = (k % KW) + kTile * ((k / KW) % KW) + kTile * kTile * (k / (KW * KW));
-    }
-    for (int cs = blockIdx.x; cs < ncompact; cs += gridDim.x) {
-        const int4 lo = sl.geo_lo[cs], dim = sl.geo_dim[cs];
-        const DevGrid g = ct.get(sl.geo_case[cs]).g;
-        const int b = dim.w;
-        const uint32_t dn = sl.dense_of[cs];
-        int nc = (int)(sl.start[dn + 1] - sl.start[dn]);
-        if (nc > kMaxCand) nc = 0;  // left empty by the sort (status raised there)
-        int2 *band = sl.band + sl.poff[b];
-        uint32_t *pairs = sl.pairs + sl.poff[b];
-        PS<T> *pw = pwts ? pwts + sl.poff[b] : nullptr;
-        for (int i = tid; i < nc; i += blockDim.x) {
-            const uint64_t an = anchor[sl.cand[b + i]];
-            int d[3] = {anchor_x(an) - lo.x + 3, anchor_y(an) - lo.y + 3, anchor_z(an) - lo.z + 3};
-            const int dm[3] = {dim.x, dim.y, dim.z};
-            unsigned code = 0;
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                if (d[q] < 0) d[q] += g.n[q];
-                if (d[q] >= g.n[q]) d[q] -= g.n[q];
-                d[q] = min(d[q], 15) - 3;  // a candidate's anchor lies within [-3, 8) of the tile
-                unsigned mq = 0;
-#pragma unroll
-                for (int k = 0; k < KW; ++k) mq |= (d[q] + k >= 0 && d[q] + k < dm[q]) ? 1u << k : 0u;
-                code |= mq << (4 * q);
-            }
-            s_anc[i] = code | (unsigned)(d[0] + kTile * d[1] + kTile * kTile * d[2] + 256) << 12;
-        }
-        for (int c = tid; c < kPairWarps * kTileCells / 4; c += blockDim.x)
-            ((uint4 *)&s_cnt[0][0])[c] = make_uint4(0u, 0u, 0u, 0u);
-        __syncthreads();
-        // Each warp walks a contiguous range of candidates, one candidate per
-        // step, lane l taking the stencil offsets k = l + 32 q: the cells of
-        // one step are distinct, so counts and list slots need no ranking.
-        const int seg = (nc + kPairWarps - 1) / kPairWarps;
-        const int i0 = min(nc, warp * seg), i1 = min(nc, i0 + seg);
-        // cell of candidate i's stencil offset (lane, q), or -1
-        auto cell_of = [&](unsigned pk, int q) {
-            const unsigned o = kcode[q];
-            const unsigned in = (pk >> (o & 3)) & (pk >> (4 + ((o >> 2) & 3))) & (pk >> (8 + ((o >> 4) & 3)));
-            return (o != ~0u && (in & 1u)) ? (int)(pk >> 12) - 256 + koff[q] : -1;
-        };
-        for (int i = i0; i < i1; ++i) {
-            const unsigned pk = s_anc[i];
-#pragma unroll
-            for (int q = 0; q < kSub; ++q) {
-                const int c = cell_of(pk, q);
-                if (c >= 0) atomicAdd(&s_cnt[warp][c], 1u);
-            }
-        }
-        __syncthreads();
-        // (cell, warp) scan: thread t owns cells 2t and 2t + 1
-        int tot[2] = {0, 0}, pre[2][kPairWarps];
-#pragma unroll
-        for (int w = 0; w < kPairWarps; ++w) {
-            const uint2 cw = ((const uint2 *)s_cnt[w])[tid];
-            pre[0][w] = tot[0];
-            pre[1][w] = tot[1];
-            tot[0] += (int)cw.x;
-            tot[1] += (int)cw.y;
-        }
-        int pv = tot[0] + tot[1], bv = (tot[0] > 0) + (tot[1] > 0);
-        for (int o = 1; o < 32; o <<= 1) {
-            const int yp = __shfl_up_sync(0xffffffffu, pv, o), yb = __shfl_up_sync(0xffffffffu, bv, o);
-            if (lane >= o) pv += yp, bv += yb;
-        }
-        if (lane == 31) s_wp[warp] = pv, s_wb[warp] = bv;
-        __syncthreads();
-        int wp = 0, wb = 0;
-        for (int w = 0; w < warp; ++w) wp += s_wp[w], wb += s_wb[w];
-        const int cp0 = wp + pv - (tot[0] + tot[1]), cb0 = wb + bv - ((tot[0] > 0) + (tot[1] > 0));
-        const int cbase[2] = {cp0, cp0 + tot[0]};
-        if (tot[0] > 0) band[cb0] = make_int2((2 * tid) | (tot[0] << 16), cbase[0]);
-        if (tot[1] > 0) band[cb0 + (tot[0] > 0)] = make_int2((2 * tid + 1) | (tot[1] << 16), cbase[1]);
-        if (tid == blockDim.x - 1) {
-            const int nbd = cb0 + (tot[0] > 0) + (tot[1] > 0);
-            sl.nband[cs] = nbd;
-            sl.tinfo[cs] = make_int4((int)sl.poff[b], (int)(sl.poff[b + nc] - sl.poff[b]), nbd, nc);
-        }
-#pragma unroll
-        for (int w = 0; w < kPairWarps; ++w)
-            ((uint2 *)s_cnt[w])[tid] = make_uint2((unsigned)(cbase[0] + pre[0][w]), (unsigned)(cbase[1] + pre[1][w]));
-        __syncthreads();
-        // placement in candidate order: a cell's list ascends in candidate
-        // index (one step's cells are distinct; the warp barrier orders steps)
-        for (int i = i0; i < i1; ++i) {
-            const unsigned pk = s_anc[i];
-#pragma unroll
-            for (int q = 0; q < kSub; ++q) {
-                const int c = cell_of(pk, q);
-                if (c >= 0) pairs[atomicAdd(&s_cnt[warp][c], 1u)] = (unsigned)i | (kcode[q] << 16);
-            }
-            __syncwarp();
-        }
-        __syncthreads();
-        // every pair's weight product, one pair per thread (the pair words
-        // written above are visible to the whole CTA after the barrier), kPwU
-        // pairs per thread at a time: the pair words, then the candidates'
-        // marker indices, then their axis weights are each loaded together,
-        // three dependent rounds of loads instead of three per pair
-        if (pw) {
-            const int np = (int)(sl.poff[b + nc] - sl.poff[b]);
-            constexpr int kPwU = 4;
-            for (int k0 = tid; k0 < np; k0 += kPwU * kPairThreads) {
-                unsigned pk[kPwU];
-                uint32_t mk[kPwU];
-#pragma unroll
-                for (int u = 0; u < kPwU; ++u) {
-                    const int k = k0 + u * kPairThreads;
-                    pk[u] = k < np ? pairs[k] : 0u;
-                }
-#pragma unroll
-                for (int u = 0; u < kPwU; ++u) mk[u] = k0 + u * kPairThreads < np ? sl.cand[b + (pk[u] & 0xffff)] : 0u;
-                PS<T> wx[kPwU], wy[kPwU], wz[kPwU];
-#pragma unroll
-                for (int u = 0; u < kPwU; ++u) {
-                    const PS<T> *w = wts + 12 * (size_t)mk[u];
-                    wx[u] = w[(pk[u] >> 16) & 3];
-                    wy[u] = w[4 + ((pk[u] >> 18) & 3)];
-                    wz[u] = w[8 + ((pk[u] >> 20) & 3)];
-                }
-#pragma unroll
-                for (int u = 0; u < kPwU; ++u) {
-                    const int k = k0 + u * kPairThreads;
-                    if (k < np) pw[k] = pair_weight3(wx[u], wy[u], wz[u]);
-                }
-            }
         }
     }
 }
@@ -1266,19 +1332,6 @@ __global__ void __launch_bounds__(kPairThreads, 5) k_tile_pairs(CaseTab ct, int 
 // sums then read shared memory only.  Tiles with more than Stage<T>::N
 // candidates read the same values from global memory instead.
 // ---------------------------------------------------------------------------
-// Spreading (ib_spread) over the tiles' per-cell lists: the case's u slot
-// holds the field spread into, its f slot is null.
-template <typename T, int KER>
-__global__ void __launch_bounds__(256) k_spread_gather(CaseTab ct, const int *__restrict__ ncompact_p, Slots sl,
-                                                       const PS<T> *__restrict__ wts, const PS<T> *__restrict__ A) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    PS<T> *sw = (PS<T> *)smem_raw;
-    PS<T> *sA = sw + (size_t)TileStage<T>::N * 12;
-    const int nc = *ncompact_p;
-    for (int cs = blockIdx.x; cs < nc; cs += gridDim.x)
-        gather_tile_lists<T, Kernel<KER>::W, false>(ct, cs, sl, wts, A, 0.0, sw, sA);
-}
-
 // Spreading (ib_spread) with warp-aggregated atomics: one lane per marker,
 // weights formed on the fly, no binning.
 template <typename T, int KER>
@@ -1804,6 +1857,27 @@ __global__ void __launch_bounds__(kGatherThreads, sizeof(T) == 4 ? 5 : 4) k_gath
     cp_async_wait_all();  // (a prefetch is only issued for a tile that follows)
 }
 
+// Spreading (ib_spread) over the tiles' per-cell lists, as a wavefront gather
+// over every tile: the case's u slot holds the field spread into, its f slot
+// is null.
+template <typename T, int KER>
+__global__ void __launch_bounds__(kGatherThreads, sizeof(T) == 4 ? 5 : 4)
+k_spread_gather(CaseTab ct, const int *__restrict__ ncompact_p, Slots sl, const PS<T> *__restrict__ A) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr int stage = TileStage<T>::N;
+    PS<T> *sA = (PS<T> *)smem_raw;
+    uint32_t *sp = (uint32_t *)(sA + (size_t)stage * 4);
+    PS<T> *spw = (PS<T> *)(sp + kLevPairs);
+    int2 *sband = (int2 *)(spw + kLevPairs);
+    grid_dep_wait();
+    const int nc = *ncompact_p;
+    GatherPipe pipe{0, false};
+    for (int cs = blockIdx.x; cs < nc; cs += gridDim.x)
+        gather_tile_level<T, Kernel<KER>::W>(ct, cs, sl, A, 0.0, sA, sp, spw, sband, stage, [] { return true; }, pipe,
+                                             cs + (int)gridDim.x < nc ? cs + (int)gridDim.x : -1);
+    cp_async_wait_all();
+}
+
 // The atomic form of a wavefront's spreading (ib_ctx_set_spread_mode):
 // every marker of the wavefront adds S A to the field with warp-aggregated
 // atomics.  Its position data are loaded before the wait; the sources after.
@@ -1932,7 +2006,8 @@ struct SlotScratch {
     int ncompact_cap;
     int lb_tiles[2];              // look-back tiles of the slot scan and of the pair-count scan
     unsigned long long *lb_stat;  // [lb_tiles[0] + lb_tiles[1]] tile words
-    unsigned int *lb_ticket;      // [2]
+    unsigned int *lb_ticket;      // [2], then the number of large tiles
+    int *big;                     // [ncompact_cap] large tiles
 };
 
 // Workspace of the slot lists, and the zeroing they need.
@@ -1951,7 +2026,8 @@ static int slots_alloc(Arena &ar, int M, int ndense, int mode, Slots &sl, SlotSc
     sc.lb_tiles[0] = ndense / kLbTile + 1;
     sc.lb_tiles[1] = with_pairs ? (int)(sc.cand_cap / kLbTile) + 1 : 0;
     sc.lb_stat = ar.take<unsigned long long>((size_t)sc.lb_tiles[0] + sc.lb_tiles[1]);
-    sc.lb_ticket = ar.take<unsigned int>(2);
+    sc.lb_ticket = ar.take<unsigned int>(3);
+    sc.big = ar.take<int>(ncap);
     sl.dense_of = ar.take<uint32_t>(ncap);
     sl.cand = ar.take<uint32_t>(sc.cand_cap);
     // bin tables: only the particle-resident form walks them
@@ -1982,7 +2058,7 @@ static int slots_alloc(Arena &ar, int M, int ndense, int mode, Slots &sl, SlotSc
     cudaMemsetAsync(sl.count, 0, sizeof(uint32_t) * ndense, s);
     cudaMemsetAsync(sl.cursor, 0, sizeof(uint32_t) * ndense, s);
     cudaMemsetAsync(sc.lb_stat, 0, sizeof(unsigned long long) * (sc.lb_tiles[0] + sc.lb_tiles[1]), s);
-    cudaMemsetAsync(sc.lb_ticket, 0, 2 * sizeof(unsigned int), s);
+    cudaMemsetAsync(sc.lb_ticket, 0, 3 * sizeof(unsigned int), s);
     return IB_OK;
 }
 
@@ -2003,19 +2079,14 @@ static int slots_build(ib_ctx *ctx, const CaseTab &ct, int M, int ndense, SlotGe
                    (int)sc.cand_cap, (const uint32_t *)(sl.start + ndense), sl.poff, sc.lb_stat + sc.lb_tiles[0],
                    sc.lb_ticket + 1, ctx->status);
     ncompact_dev = (int *)(sl.flag_scan + ndense);
-    // one resident wave (a second wave would only repeat the screening)
-    int sper = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&sper, k_slot_sort, kBlock, 0);
-    launch_pdl(k_slot_sort, dim3(ctx->sm_count * (sper > 0 ? sper : 1)), dim3(kBlock), 0, s, ct, sg.mode,
-               sc.ncompact_cap, (const int *)ncompact_dev, sg, (const uint32_t *)sl.dense_of,
-               (const uint32_t *)sl.start, anchor, level, sl, ctx->status);
-    if (with_pairs) {
-        // one resident wave
-        int pper = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pper, k_tile_pairs<T, KW>, kPairThreads, 0);
-        launch_pdl(k_tile_pairs<T, KW>, dim3(ctx->sm_count * (pper > 0 ? pper : 1)), dim3(kPairThreads), 0, s, ct,
-                   sc.ncompact_cap, (const int *)ncompact_dev, sl, anchor, wts);
-    }
+    launch_pdl(k_tile_lists<T, KW>, dim3(ctx->sm_count * kListCtas), dim3(kListThreads), 0, s, ct, sg.mode, sc.ncompact_cap,
+               (const int *)ncompact_dev, sg, (const uint32_t *)sl.dense_of, (const uint32_t *)sl.start, anchor, level, sl,
+               wts, sc.big, (int *)sc.lb_ticket + 2);
+    auto large = k_tile_lists_large<T, KW>;
+    cudaFuncSetAttribute(large, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CtaLists));
+    launch_pdl(large, dim3(ctx->sm_count), dim3(kPairThreads), sizeof(CtaLists), s, ct, sg.mode, sg,
+               (const uint32_t *)sl.dense_of, (const uint32_t *)sl.start, anchor, level, sl, wts, (const int *)sc.big,
+               (const int *)sc.lb_ticket + 2, ctx->status);
     return check_launch("slot lists");
 }
 
@@ -2061,9 +2132,10 @@ static int run_spread(ib_ctx *ctx, const ib_grid *grid, int M, const double *X, 
     rc = slots_build<T, KW>(ctx, ct, M, (int)ndense, sg, ms.anchor, (const PS<T> *)ms.wts, nullptr, sl, sc, ncompact, s,
                             true);
     if (rc) return rc;
-    cudaFuncSetAttribute(k_spread_gather<T, KER>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)tile_stage_bytes<T>());
-    k_spread_gather<T, KER><<<ctx->sm_count * 4, 256, tile_stage_bytes<T>(), s>>>(ct, ncompact, sl, ms.wts, ms.A);
+    const size_t smem = level_stage_bytes<T>(TileStage<T>::N);
+    cudaFuncSetAttribute(k_spread_gather<T, KER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    launch_pdl(k_spread_gather<T, KER>, dim3(ctx->sm_count * (sizeof(T) == 4 ? 5 : 4)), dim3(kGatherThreads), smem, s, ct,
+               (const int *)ncompact, sl, (const PS<T> *)ms.A);
     return check_launch("ib_spread");
 }
 
