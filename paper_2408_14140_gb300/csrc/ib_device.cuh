@@ -130,15 +130,17 @@ struct Slots {
     int4 *geo_lo;      // [ncompact_max] tile first cell (wrapped), w = level
     int4 *geo_dim;     // [ncompact_max] tile dims, w = first candidate
     int *geo_case;     // [ncompact_max] case of the tile
-    // per-cell gather lists (built once per call, see k_tile_pairs).  A
+    // per-cell gather lists (built once per call, see k_tile_lists).  A
     // candidate contributes one pair per stencil cell inside its tile;
     // poff[i] is the exclusive prefix of those counts over candidate
     // positions, so tile cs with first candidate b owns pairs
     // [poff[b], poff[b + nc]) -- KW^3 M in total.  band[poff[b] + q] =
     // {cell | count << 16, first pair relative to poff[b]} for its q-th band
-    // cell (cells in index order), and pairs[poff[b] + k] = candidate | ox << 16
-    // | oy << 18 | oz << 20, each cell's pairs in ascending candidate order
-    // (the gather order).
+    // cell, cells ordered by count, largest first.  Wavefront form: the first
+    // pair of the cell's slice of 32, whose rows of pairs[] are markers (jagged
+    // rows, see k_tile_lists).  Group form: the cell's own first pair, its
+    // pairs contiguous, candidate | ox << 16 | oy << 18 | oz << 20.  Each
+    // cell's pairs ascend in candidate order (the gather order).
     uint32_t *pcnt;    // [cand_cap] in-tile stencil cells of each candidate
     uint32_t *poff;    // [cand_cap + 1] exclusive scan of pcnt
     int2 *band;
@@ -147,6 +149,7 @@ struct Slots {
     // [ncompact_max] the tile's list record {first pair poff[b], pairs,
     // band cells, candidates}, one load for the wavefront gather
     int4 *tinfo;
+    uint4 *slen;       // [ncompact_max] rows of the tile's slices (a byte each, at most 255)
     // [KW^3 M] per pair, its weight product pair_weight(w, ox, oy, oz) in the
     // pass-sum type PS<T> (parallel to pairs; nullable)
     void *pw;

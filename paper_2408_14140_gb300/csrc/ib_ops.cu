@@ -805,28 +805,46 @@ __global__ void k_level_slots(int mode, const int *__restrict__ nlev_p, const in
     }
 }
 
-// Per wavefront, its tiles in decreasing number of band cells (a counting
-// sort; equal sizes in any order).  The wavefront gather takes its tiles in
-// this order, so when a wavefront has more tiles than resident CTAs the
-// second round gets the smallest ones.  Only the launch order changes: every
-// tile's sums are the same whichever CTA computes them.
-__global__ void __launch_bounds__(512) k_level_tile_order(const int *__restrict__ nlev_p,
-                                                           const int *__restrict__ lev_sbeg,
-                                                           const int *__restrict__ nband, int *__restrict__ tperm) {
+// Per wavefront, the slices of its tiles, longest first (a counting sort by
+// their rows; equal ones in any order): one warp of the wavefront gather takes
+// a slice, and the last round of warps then has the shortest.  Only the order
+// of work changes.  Wavefront L's list starts at lev_slice[L].x, a bound of what
+// the wavefronts before it need (a slice has at least one pair), and has
+// lev_slice[L].y entries {tile, slice, first pair of the tile, cells}.
+constexpr int kSliceOrderThreads = 1024;
+__global__ void __launch_bounds__(kSliceOrderThreads) k_level_slices(const int *__restrict__ nlev_p,
+                                                                     const int *__restrict__ lev_sbeg, Slots sl,
+                                                                     int2 *__restrict__ lev_slice,
+                                                                     int4 *__restrict__ slices) {
     grid_dep_wait();
-    __shared__ int s_hist[kTileCells + 1];
+    __shared__ int s_hist[256];
     const int nl = *nlev_p;
     for (int L = blockIdx.x; L < nl; L += gridDim.x) {  // one CTA per wavefront
         const int s0 = lev_sbeg[L], s1 = lev_sbeg[L + 1];
-        for (int k = threadIdx.x; k <= kTileCells; k += blockDim.x) s_hist[k] = 0;
+        const int base = s0 < s1 ? (int)((uint32_t)sl.tinfo[s0].x >> 5) + s0 : 0;
+        for (int k = threadIdx.x; k < 256; k += blockDim.x) s_hist[k] = 0;
         __syncthreads();
-        for (int t = s0 + threadIdx.x; t < s1; t += blockDim.x)
-            atomicAdd(&s_hist[kTileCells - min(max(nband[t], 0), kTileCells)], 1);
-        __syncthreads();
-        block_scan_chunked(kTileCells + 1, [&](int k) { return s_hist[k]; }, [&](int k, int pre) { s_hist[k] = pre; });
-        __syncthreads();
-        for (int t = s0 + threadIdx.x; t < s1; t += blockDim.x)
-            tperm[s0 + atomicAdd(&s_hist[kTileCells - min(max(nband[t], 0), kTileCells)], 1)] = t;
+        for (int pass = 0; pass < 2; ++pass) {
+            for (int t = s0 + threadIdx.x; t < s1; t += blockDim.x) {
+                const int4 ti = sl.tinfo[t];
+                const uint4 l4 = sl.slen[t];
+                const unsigned lw[4] = {l4.x, l4.y, l4.z, l4.w};
+                const int ns = (ti.z + 31) >> 5;
+#pragma unroll
+                for (int s = 0; s < 16; ++s)
+                    if (s < ns) {
+                        const int j = atomicAdd(&s_hist[255 - ((lw[s >> 2] >> (8 * (s & 3))) & 255u)], 1);
+                        if (pass) slices[base + j] = make_int4(t, s, ti.x, ti.z);
+                    }
+            }
+            __syncthreads();
+            if (pass == 0) {
+                block_scan_chunked(256, [&](int k) { return s_hist[k]; }, [&](int k, int pre) { s_hist[k] = pre; });
+                __syncthreads();
+            } else if (threadIdx.x == 0) {
+                lev_slice[L] = make_int2(base, s_hist[255]);  // every slice counted: the last bucket's end
+            }
+        }
         __syncthreads();
     }
 }
@@ -948,63 +966,43 @@ __device__ __forceinline__ void slot_bins(int nc, int cs, const Slots &sl, int l
 // tile's first one (64 where that does not fit).  Tiles of more than kListCand
 // candidates go to a second kernel, whose CTAs sort them by a bitonic network.
 // ---------------------------------------------------------------------------
+// The lists' layout.  The wavefront gather takes 32 cells a warp (a slice), so
+// a tile's cells are ordered by list length, longest first, and a slice's
+// pairs lie row by row: row k holds the k-th pair of every cell that has one,
+// in lane order, with no padding (jagged diagonal storage; a lane's place in a
+// row is its rank among the lanes with more than k pairs).  A pair is its
+// marker and its weight.  The group kernels walk a cell's pairs alone: for
+// them each list is contiguous and a pair is candidate | offset << 16.
 constexpr int kListThreads = 128;
-constexpr int kListCtas = 10;               // CTAs of an SM
+constexpr int kListCtas = 10;              // CTAs of an SM
 constexpr int kListCand = 512;
-constexpr int kListStash = 1792;           // pairs a CTA stages in shared memory (more: memory)
 constexpr int kPairThreads = 256;          // the large tiles' CTAs
-constexpr int kPairWarps = kPairThreads / 32;
 constexpr int kPairWords = kMaxCand / 32;  // words of a bit set
-constexpr int kPairStash = 4096;
 constexpr int kMarkBits = 21;
-static_assert(kTileCells == 4 * kListThreads && kTileCells == 2 * kPairThreads && kBins <= 1 << (32 - kMarkBits),
+constexpr int kSlices = kTileCells / 32;   // slices of a tile
+constexpr int kLenBins = 128;              // list lengths told apart in the order (longer: any order)
+static_assert(kTileCells == 4 * kListThreads && kTileCells == 2 * kPairThreads && kBins <= 1 << (32 - kMarkBits) &&
+                  kSlices == 16,
               "tile lists");
 
+struct ListShared {
+    int hist[kLenBins];
+    int sum[kSlices];                      // pairs of each slice
+    uint16_t cell[kTileCells], cnt[kTileCells];
+    unsigned char len[kSlices];            // rows of each slice (at most 255 told)
+    int nb;
+};
 struct CtaLists {
     unsigned long long keys[kMaxCand];
     unsigned set[3 * kTile][kPairWords + 1];
-    int2 band[kTileCells];
     short first[kMaxCand];
-    int wp[kPairWarps], wb[kPairWarps];
+    ListShared ls;
 };
-// (the pairs replace the keys)
-static_assert(sizeof(uint32_t) * kPairStash <= sizeof(unsigned long long) * kMaxCand, "stash");
 
 // Tile coordinates + 3 of a bin's anchor (past the tile for the last bin).
 __device__ __forceinline__ int3 bin_anchor(int bin) {
     const int row = bin / kBinsPerRow;
     return make_int3(bin - row * kBinsPerRow, row % kRow, row / kRow);
-}
-
-// Pair words [0, np) from `src` (the staged list, or memory) and the weights.
-template <typename T, class Mark>
-__device__ __forceinline__ void pair_weights(const uint32_t *src, uint32_t *pairs, PS<T> *pw, int np, bool stash,
-                                             const PS<T> *__restrict__ wts, int t0, int nt, Mark mark) {
-    // kPwU pairs per thread at a time: the axis weights of a batch are loaded
-    // together
-    constexpr int kPwU = 4;
-    for (int k0 = t0; k0 < np; k0 += kPwU * nt) {
-        unsigned pk[kPwU];
-        PS<T> wx[kPwU], wy[kPwU], wz[kPwU];
-#pragma unroll
-        for (int u = 0; u < kPwU; ++u) {
-            const int k = k0 + u * nt;
-            pk[u] = k < np ? src[k] : 0u;
-            if (stash && k < np) pairs[k] = pk[u];
-        }
-#pragma unroll
-        for (int u = 0; u < kPwU; ++u) {
-            const PS<T> *w = wts + 12 * (size_t)(k0 + u * nt < np ? mark(pk[u] & 0xffff) : 0u);
-            wx[u] = w[(pk[u] >> 16) & 3];
-            wy[u] = w[4 + ((pk[u] >> 18) & 3)];
-            wz[u] = w[8 + ((pk[u] >> 20) & 3)];
-        }
-#pragma unroll
-        for (int u = 0; u < kPwU; ++u) {
-            const int k = k0 + u * nt;
-            if (k < np) pw[k] = pair_weight3(wx[u], wy[u], wz[u]);
-        }
-    }
 }
 
 // One 32-candidate word of the tile's 24 bit sets, lane l < 24 returning set l's
@@ -1025,18 +1023,131 @@ __device__ __forceinline__ unsigned cover_word(int3 r, const int dim[3], int lan
     return mine;
 }
 
-// A cell's list from the bit sets, nw words each: candidate | offset << 16.
-template <class Set, class First>
-__device__ __forceinline__ void emit_list(int c, int pos, int np, int nw, Set set, First first, uint32_t *out) {
-    const int x = c & 7, y = (c >> 3) & 7, z = c >> 6, code = x + 4 * y + 16 * z;
-    for (int w = 0; w < nw; ++w) {
-        unsigned m = set(x, w) & set(kTile + y, w) & set(2 * kTile + z, w);
-        while (m) {
-            const int i = 32 * w + __ffs((int)m) - 1;
-            m &= m - 1;
-            if (pos < np) out[pos] = (uint32_t)i | ((uint32_t)(code - first(i)) << 16);
-            ++pos;
+// A tile's lists from its bit sets of nw words (set(i, w): columns, rows, planes
+// for i from 0, 8, 16), by a CTA of NT threads.  The caller has zeroed ls.hist
+// and ls.len before a barrier.
+template <typename T, int NT, class Set, class First, class Mark>
+__device__ __forceinline__ void build_lists(const Slots &sl, int cs, uint32_t pb, int room, int nc, int nw, bool jagged,
+                                            const PS<T> *__restrict__ wts, ListShared &ls, Set set, First first,
+                                            Mark mark) {
+    constexpr int C = kTileCells / NT;  // cells a thread, neighbours along x
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int t[C], r[C];
+    {
+        const int x = (C * tid) & 7, y = ((C * tid) >> 3) & 7, z = (C * tid) >> 6;
+#pragma unroll
+        for (int k = 0; k < C; ++k) t[k] = 0;
+        for (int w = 0; w < nw; ++w) {
+            const unsigned yz = set(kTile + y, w) & set(2 * kTile + z, w);
+#pragma unroll
+            for (int k = 0; k < C; ++k) t[k] += __popc(yz & set(x + k, w));
         }
+    }
+    // counting sort of the cells by list length
+    auto bucket = [](int n) { return kLenBins - 1 - min(n, kLenBins - 1); };
+#pragma unroll
+    for (int k = 0; k < C; ++k) r[k] = t[k] > 0 ? atomicAdd(&ls.hist[bucket(t[k])], 1) : 0;
+    __syncthreads();
+    if (warp == 0) {
+        int h[kLenBins / 32], s = 0;
+#pragma unroll
+        for (int k = 0; k < kLenBins / 32; ++k) {
+            h[k] = ls.hist[kLenBins / 32 * lane + k];
+            s += h[k];
+        }
+        int inc = s;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += v;
+        }
+        int run = inc - s;
+#pragma unroll
+        for (int k = 0; k < kLenBins / 32; ++k) {
+            ls.hist[kLenBins / 32 * lane + k] = run;
+            run += h[k];
+        }
+        if (lane == 31) ls.nb = inc;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < C; ++k)
+        if (t[k] > 0) {
+            const int q = ls.hist[bucket(t[k])] + r[k];
+            ls.cell[q] = (uint16_t)(C * tid + k);
+            ls.cnt[q] = (uint16_t)t[k];
+        }
+    __syncthreads();
+    const int nb = ls.nb, ns = (nb + 31) >> 5;
+    for (int s = warp; s < ns; s += NT / 32) {
+        const int n = 32 * s + lane < nb ? ls.cnt[32 * s + lane] : 0;
+        const int sum = __reduce_add_sync(0xffffffffu, n), len = __reduce_max_sync(0xffffffffu, n);
+        if (lane == 0) ls.sum[s] = sum, ls.len[s] = (unsigned char)min(len, 255);
+    }
+    __syncthreads();
+    uint32_t *const pairs = sl.pairs + pb;
+    PS<T> *const pw = (PS<T> *)sl.pw + pb;
+    int2 *const band = sl.band + pb;
+    int np = 0;
+    for (int s = 0; s < ns; ++s) np += ls.sum[s];
+    for (int s = warp; s < ns; s += NT / 32) {
+        const int q = 32 * s + lane;
+        const int c = q < nb ? ls.cell[q] : 0, n = q < nb ? ls.cnt[q] : 0;
+        int base = 0;
+        for (int j = 0; j < s; ++j) base += ls.sum[j];
+        int own = n;  // the list's first pair where lists are contiguous
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, own, o);
+            if (lane >= o) own += v;
+        }
+        own += base - n;
+        if (q < nb) band[q] = make_int2(c | (n << 16), jagged ? base : own);
+        const int x = c & 7, y = (c >> 3) & 7, z = c >> 6, code = x + 4 * y + 16 * z;
+        const int rows = __reduce_max_sync(0xffffffffu, n);
+        int w = -1, off = base;
+        unsigned m = 0;
+        constexpr int kU = 4;  // rows whose loads are in flight together
+        for (int k0 = 0; k0 < rows; k0 += kU) {
+            int i[kU], pos[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const bool act = k0 + u < n;
+                const unsigned a = __ballot_sync(0xffffffffu, act);
+                pos[u] = act ? (jagged ? off + __popc(a & ((1u << lane) - 1u)) : own + k0 + u) : room;
+                off += __popc(a);
+                i[u] = 0;
+                if (act) {
+                    while (!m) {
+                        ++w;
+                        m = set(x, w) & set(kTile + y, w) & set(2 * kTile + z, w);
+                    }
+                    i[u] = 32 * w + __ffs((int)m) - 1;
+                    m &= m - 1;
+                }
+            }
+            uint32_t mk[kU];
+            int oc[kU];
+            PS<T> wx[kU], wy[kU], wz[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                mk[u] = mark(i[u]);
+                oc[u] = pos[u] < room ? code - first(i[u]) : 0;
+                const PS<T> *wm = wts + 12 * (size_t)mk[u];
+                wx[u] = wm[oc[u] & 3];
+                wy[u] = wm[4 + ((oc[u] >> 2) & 3)];
+                wz[u] = wm[8 + (oc[u] >> 4)];
+            }
+#pragma unroll
+            for (int u = 0; u < kU; ++u)
+                if (pos[u] < room) {  // (more than the room only with a box wider than its grid, reported)
+                    pairs[pos[u]] = jagged ? mk[u] : (uint32_t)i[u] | ((uint32_t)oc[u] << 16);
+                    pw[pos[u]] = pair_weight3(wx[u], wy[u], wz[u]);
+                }
+        }
+    }
+    if (tid == 0) {
+        sl.nband[cs] = nb;
+        sl.tinfo[cs] = make_int4((int)pb, min(np, room), nb, nc);
+        sl.slen[cs] = *(const uint4 *)ls.len;
     }
 }
 
@@ -1044,17 +1155,16 @@ template <typename T, int KW>
 __global__ void __launch_bounds__(kListThreads, kListCtas) k_tile_lists(
     CaseTab ct, int mode, int ncompact_cap, const int *__restrict__ ncompact_p, SlotGeom sg,
     const uint32_t *__restrict__ dense_of, const uint32_t *__restrict__ start, const uint64_t *__restrict__ anchor,
-    const int *__restrict__ level, Slots sl, const PS<T> *__restrict__ wts, int *__restrict__ big,
+    const int *__restrict__ level, Slots sl, const PS<T> *__restrict__ wts, int jagged, int *__restrict__ big,
     int *__restrict__ nbig) {
     constexpr int kSetPitch = kListCand / 32 + 1;  // odd: no bank conflicts
     __shared__ __align__(16) unsigned long long s_keys[kListCand];  // or 32-bit keys
-    __shared__ uint32_t s_mark[kListCand], s_pair[kListStash];
+    __shared__ uint32_t s_mark[kListCand];
     __shared__ unsigned s_set[3 * kTile][kSetPitch];
     __shared__ short s_first[kListCand];
     __shared__ uint16_t s_rel[kListCand];  // anchor + 3, 4 bits an axis
-    __shared__ uint16_t s_cell[kTileCells], s_base[kTileCells + 2];
     __shared__ uint32_t s_min[kListThreads / 32], s_max[kListThreads / 32];
-    __shared__ int s_w[kListThreads / 32];
+    __shared__ __align__(16) ListShared s_ls;
     grid_dep_wait();
     const int ncompact = min(*ncompact_p, ncompact_cap);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1148,62 +1258,16 @@ __global__ void __launch_bounds__(kListThreads, kListCtas) k_tile_lists(
             const unsigned mine = cover_word<KW>(make_int3(q & 15, (q >> 4) & 15, q >> 8), dim, lane);
             if (lane < 3 * kTile) s_set[lane][w] = mine;
         }
+        s_ls.hist[tid] = 0;
+        if (tid < kSlices) s_ls.len[tid] = 0;
         __syncthreads();
-        // pairs per cell: thread t owns cells 4t .. 4t + 3 (half a row)
-        int t[4] = {0, 0, 0, 0};
-        {
-            const int x = (4 * tid) & 7, y = (tid >> 1) & 7, z = tid >> 4;
-            for (int w = 0; w < nw; ++w) {
-                const unsigned yz = s_set[kTile + y][w] & s_set[2 * kTile + z][w];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) t[k] += __popc(yz & s_set[x + k][w]);
-            }
-        }
-        // pairs and cells in one scan (at most 512 cells, 512 * 64 pairs)
-        const int v = (t[0] + t[1] + t[2] + t[3]) |
-                      (((t[0] > 0) + (t[1] > 0) + (t[2] > 0) + (t[3] > 0)) << 20);
-        int s = v;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int p = __shfl_up_sync(0xffffffffu, s, o);
-            if (lane >= o) s += p;
-        }
-        if (lane == 31) s_w[warp] = s;
-        __syncthreads();
-        int before = s - v, all = 0;
-#pragma unroll
-        for (int w = 0; w < kListThreads / 32; ++w) {
-            if (w < warp) before += s_w[w];
-            all += s_w[w];
-        }
-        const int nb = all >> 20, np = min(all & 0xfffff, room);  // equal but for a box wider than its grid (reported)
-        int pos = before & 0xfffff, c0 = before >> 20;
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-            if (t[k] > 0) {
-                s_cell[c0] = (uint16_t)(4 * tid + k);
-                s_base[c0++] = (uint16_t)pos;
-                pos += t[k];
-            }
-        if (tid == 0) s_base[nb] = (uint16_t)(all & 0xfffff);
-        __syncthreads();
-        // the lists: a cell's candidates in ascending order
-        const bool stash = np <= kListStash;
-        uint32_t *const pairs = sl.pairs + pb, *const out = stash ? s_pair : pairs;
-        int2 *const band = sl.band + pb;
-        for (int q = tid; q < nb; q += kListThreads) {
-            const int c = s_cell[q], p0 = s_base[q];
-            band[q] = make_int2(c | ((s_base[q + 1] - p0) << 16), p0);
-            emit_list(c, p0, np, nw, [&](int i, int w) { return s_set[i][w]; }, [&](int i) { return s_first[i]; }, out);
-        }
-        __syncthreads();
-        pair_weights<T>(out, pairs, (PS<T> *)sl.pw + pb, np, stash, wts, tid, kListThreads,
-                        [&](int i) { return s_mark[i]; });
+        build_lists<T, kListThreads>(sl, cs, pb, room, nc, nw, jagged != 0, wts, s_ls,
+                                     [&](int i, int w) { return s_set[i][w]; }, [&](int i) { return s_first[i]; },
+                                     [&](int i) { return s_mark[i]; });
         if (tid == 0) {
             sl.geo_lo[cs] = make_int4(lo[0], lo[1], lo[2], lev);
             sl.geo_dim[cs] = make_int4(dim[0], dim[1], dim[2], (int)b);
             sl.geo_case[cs] = cse;
-            sl.nband[cs] = nb;
-            sl.tinfo[cs] = make_int4((int)pb, np, nb, nc);
         }
         __syncthreads();  // the next tile overwrites the shared lists
     }
@@ -1214,10 +1278,9 @@ template <typename T, int KW>
 __global__ void __launch_bounds__(kPairThreads) k_tile_lists_large(
     CaseTab ct, int mode, SlotGeom sg, const uint32_t *__restrict__ dense_of, const uint32_t *__restrict__ start,
     const uint64_t *__restrict__ anchor, const int *__restrict__ level, Slots sl, const PS<T> *__restrict__ wts,
-    const int *__restrict__ big, const int *__restrict__ nbig_p, DevStatus *st) {
+    int jagged, const int *__restrict__ big, const int *__restrict__ nbig_p, DevStatus *st) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     grid_dep_wait();
-    PS<T> *const pwts = (PS<T> *)sl.pw;
     const int nbig = *nbig_p, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     CtaLists &sh = *(CtaLists *)smem_raw;
     {
@@ -1259,7 +1322,7 @@ __global__ void __launch_bounds__(kPairThreads) k_tile_lists_large(
             if (sl.bins) slot_bins(nc, cs, sl, tid, kPairThreads, [&](int i) { return (int)(sh.keys[i] >> 32); });
             // sorted candidates and the bit sets, one word per warp and step
             const int nw = (nc + 31) >> 5;
-            for (int w = warp; w < nw; w += kPairWarps) {
+            for (int w = warp; w < nw; w += kPairThreads / 32) {
                 const int i = 32 * w + lane;
                 int3 r = make_int3(15, 15, 15);
                 if (i < nc) {
@@ -1270,54 +1333,16 @@ __global__ void __launch_bounds__(kPairThreads) k_tile_lists_large(
                 const unsigned mine = cover_word<KW>(r, dim, lane);
                 if (lane < 3 * kTile) sh.set[lane][w] = mine;
             }
+            if (tid < kLenBins) sh.ls.hist[tid] = 0;
+            if (tid < kSlices) sh.ls.len[tid] = 0;
             __syncthreads();
-            // pairs per cell: thread t owns cells 2t and 2t + 1
-            int t0 = 0, t1 = 0;
-            {
-                const int x = (2 * tid) & 7, y = (tid >> 2) & 7, z = tid >> 5;
-                for (int w = 0; w < nw; ++w) {
-                    const unsigned yz = sh.set[kTile + y][w] & sh.set[2 * kTile + z][w];
-                    t0 += __popc(yz & sh.set[x][w]);
-                    t1 += __popc(yz & sh.set[x + 1][w]);
-                }
-            }
-            int pv = t0 + t1, bv = (t0 > 0) + (t1 > 0);
-            for (int o = 1; o < 32; o <<= 1) {
-                const int yp = __shfl_up_sync(0xffffffffu, pv, o), yb = __shfl_up_sync(0xffffffffu, bv, o);
-                if (lane >= o) pv += yp, bv += yb;
-            }
-            if (lane == 31) sh.wp[warp] = pv, sh.wb[warp] = bv;
-            __syncthreads();
-            int wp = 0, wb = 0, nb = 0, np = 0;
-            for (int w = 0; w < kPairWarps; ++w) {
-                if (w < warp) wp += sh.wp[w], wb += sh.wb[w];
-                nb += sh.wb[w];
-                np += sh.wp[w];
-            }
-            np = min(np, room);
-            const int p0 = wp + pv - (t0 + t1), b0 = wb + bv - ((t0 > 0) + (t1 > 0));
-            if (t0 > 0) sh.band[b0] = make_int2((2 * tid) | (t0 << 16), p0);
-            if (t1 > 0) sh.band[b0 + (t0 > 0)] = make_int2((2 * tid + 1) | (t1 << 16), p0 + t0);
-            __syncthreads();
-            const bool stash = np <= kPairStash;
-            uint32_t *const pairs = sl.pairs + pb, *const spair = (uint32_t *)sh.keys;
-            int2 *const band = sl.band + pb;
-            for (int qb = tid; qb < nb; qb += kPairThreads) {
-                const int2 e = sh.band[qb];
-                band[qb] = e;
-                emit_list(e.x & 0xffff, e.y, np, nw, [&](int i, int w) { return sh.set[i][w]; },
-                          [&](int i) { return sh.first[i]; }, stash ? spair : pairs);
-            }
-            __syncthreads();
-            const uint32_t *cand = sl.cand + b;
-            pair_weights<T>(stash ? spair : pairs, pairs, pwts + pb, np, stash, wts, tid, kPairThreads,
-                            [&](int i) { return cand[i]; });
+            build_lists<T, kPairThreads>(sl, cs, pb, room, nc, nw, jagged != 0, wts, sh.ls,
+                                         [&](int i, int w) { return sh.set[i][w]; }, [&](int i) { return sh.first[i]; },
+                                         [&](int i) { return (uint32_t)(sh.keys[i] & 0xffffffffu); });
             if (tid == 0) {
                 sl.geo_lo[cs] = make_int4(lo[0], lo[1], lo[2], lev);
                 sl.geo_dim[cs] = make_int4(dim[0], dim[1], dim[2], (int)b);
                 sl.geo_case[cs] = cse;
-                sl.nband[cs] = nb;
-                sl.tinfo[cs] = make_int4((int)pb, np, nb, nc);
             }
             __syncthreads();
         }
@@ -1415,7 +1440,6 @@ __device__ __forceinline__ bool grid_sync(Barrier b, DevStatus *st) {
 // persistent multidirect-forcing passes (cooperative launch)
 // ---------------------------------------------------------------------------
 constexpr int kInterpThreads = 256;  // level interpolation CTA
-constexpr int kGatherThreads = 256;  // level gather CTA (one tile at a time)
 
 template <typename T>
 struct PassArgs {
@@ -1427,13 +1451,12 @@ struct PassArgs {
     Slots sl;
     const int *mperm;
     const int *lev_mbeg;
-    const int *lev_sbeg;
-    const int *tperm;  // per wavefront, its tiles largest first (wavefront gather order)
+    const int2 *lev_slice;  // per wavefront, its slices' first entry and number
+    const int4 *slices;     // (k_level_slices)
     const int *nlev;
     int Ns;
     int L0;  // first wavefront the persistent kernel processes
     int atomic;  // spread with warp-aggregated atomics instead of the tile gather
-    int stage;   // candidates a gather CTA stages in shared memory (larger tiles read memory)
     double dt, inv_dt;  // inv_dt = 1 / dt, formed on the host
     Barrier bar;
     DevStatus *st;
@@ -1587,295 +1610,127 @@ __global__ void __launch_bounds__(kInterpThreads) k_interp_level_c3(PassArgs<T> 
     }
 }
 
-// The wavefront gather, one CTA per tile (grid-stride), many CTAs per SM,
-// over the tiles' per-cell lists (sums bitwise those of the bin walk).
+// The wavefront gather: one warp per slice of 32 band cells, a lane per cell,
+// over the slices' jagged rows.  Pair words and weights come in coalesced rows
+// straight from memory (they stay in L2 through a wavefront's passes), the
+// sources from L2 and L1 (a marker's is read by the 27 cells of its stencil);
+// no shared memory, no barrier, and kSliceRows rows in flight a warp.  A tile
+// per CTA with its lists staged in shared memory spent most of its time in
+// staging round trips and barriers: 17.0 us a launch on the 256^3 cluster in
+// FP64 (50 on its first wavefront).
 //
-// Before the wait (nothing here is written by the interpolation): the tile's
-// pair words and pair weights (the weight products, formed once per call by
-// k_tile_pairs) are staged in shared memory, and each thread loads the list
-// heads and field values of its (at most two) band cells.  After the wait
-// only the spread sources are loaded; the sums then run from shared memory
-// and registers.  Each cell's pairs are added in list order with the same
-// weight products as gather_tile_lists forms on the fly, so the sums are
-// bitwise the same.
-constexpr int kLevPairs = 3072;  // pairs staged per tile (more: read from memory)
+// Before the wait (nothing here is written by the interpolation): the slice's
+// record and cells, the cells' field values and the first rows.  Each cell's
+// pairs are added in ascending candidate order, as in the bin walk.
+constexpr int kSliceThreads = 128;
+template <typename T> constexpr int kSliceCtas = sizeof(T) == 4 ? 8 : 6;  // CTAs of an SM
+constexpr int kSliceRows = 4;
 
-constexpr int kLevHalf = kLevPairs / 2;  // a tile this small can be prefetched into half the buffer
-constexpr int kLevBand = kTileCells;      // band records of a prefetched tile (at most one per cell)
-
-// Shared memory of a level gather CTA staging `stage` candidates: their
-// spread sources, the tile's pair words and pair weights (two halves), and
-// two buffers of band records for prefetched tiles.
-// FP32 fields only: there the staging round trips of a CTA's later tiles are
-// on the critical path (prefetching measured 566 -> 553 us per step); the
-// FP64 gather is bound by its double-float sums and measured no gain.
-template <typename T>
-constexpr bool kLevPrefetch = sizeof(T) == 4;
-
-template <typename T>
-size_t level_stage_bytes(int stage) {
-    return (size_t)stage * 4 * sizeof(PS<T>) + (size_t)kLevPairs * (sizeof(uint32_t) + sizeof(PS<T>)) +
-           (kLevPrefetch<T> ? (size_t)2 * kLevBand * sizeof(int2) : 0);
+__device__ __forceinline__ void load_source(const float *A, uint32_t m, float a[3]) {
+    const float4 v = ((const float4 *)A)[m];
+    a[0] = v.x, a[1] = v.y, a[2] = v.z;
+}
+__device__ __forceinline__ void load_source(const float2 *A, uint32_t m, float2 a[3]) {
+    const float4 v = ((const float4 *)A)[2 * (size_t)m];
+    a[0] = make_float2(v.x, v.y), a[1] = make_float2(v.z, v.w);
+    a[2] = A[4 * (size_t)m + 2];
 }
 
-// Asynchronous global -> shared copies (cp.async, completed by
-// cp_async_wait_all and made visible to the CTA by a barrier).
-template <int B>
-__device__ __forceinline__ void cp_async(void *smem, const void *gmem) {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(sa), "l"(gmem), "n"(B) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-// Where a gather CTA's next tile stands: its lists prefetched into half
-// `half` of the staging buffers (pre), or not.
-struct GatherPipe {
-    int half;
-    bool pre;
-};
-
-// `wait` runs between the staging of what the interpolation does not write
-// and the loads of the spread sources; false (a wait that gave up) leaves the
-// tile untouched, CTA-uniformly.  Each pair's weight product comes from the
-// per-pair weights k_tile_pairs formed (the value pair_weight gives).
-// `pipe` says whether this tile's lists (pair words, pair weights, band
-// records) were prefetched by the CTA's previous tile; on return it says the
-// same of the next tile `cs_next` (-1: none), whose lists this tile
-// prefetches into the other half while it works when both fit a half.
-template <typename T, int KW, class Wait>
-__device__ __forceinline__ bool gather_tile_level(const CaseTab &ct, int cs, const Slots &sl, const PS<T> *A_src,
-                                                  double inv_dt, PS<T> *sA, uint32_t *sp_all, PS<T> *spw_all,
-                                                  int2 *sband, int stage, Wait wait, GatherPipe &pipe,
-                                                  int cs_next) {
+template <typename T, class Wait>
+__device__ __forceinline__ void gather_slice(const CaseTab &ct, int4 rec, const Slots &sl, const PS<T> *A, double inv_dt,
+                                             Wait wait) {
     using S = PS<T>;
-    // the tile's record, geometry and case: independent loads
-    const int4 ti = sl.tinfo[cs];
-    const int4 lo = sl.geo_lo[cs], dim = sl.geo_dim[cs];
+    constexpr int U = kSliceRows;
+    const int lane = threadIdx.x & 31, q = 32 * rec.y + lane, cs = rec.x;
+    const uint32_t pb = (uint32_t)rec.z;
+    const bool has = q < rec.w;
+    const int2 e = has ? sl.band[pb + q] : make_int2(0, 0);
+    const int4 lo = sl.geo_lo[cs];
     const DevCase cd = ct.get(sl.geo_case[cs]);
     const DevGrid &g = cd.g;
     const long long N = (long long)g.n[0] * g.n[1] * g.n[2];
     T *const u = (T *)cd.u;
-    T *const f_out = (T *)cd.f;
-    const uint32_t pb = (uint32_t)ti.x;
-    const int np = ti.y, nb = ti.z, nc = ti.w;
-    const uint32_t *cand = sl.cand + dim.w;
-    const int2 *band = sl.band + pb;
-    const uint32_t *pairs = sl.pairs + pb;
-    const S *pwg = (const S *)sl.pw + pb;
-    const bool pre = pipe.pre;
-    const bool staged = nc <= stage, pstaged = pre || np <= kLevPairs;
-    // this tile's lists: the prefetched half, or from the start of the buffer
-    const int lbase = pre ? pipe.half * kLevHalf : 0;
-    uint32_t *const sp = sp_all + lbase;
-    S *const spw = spw_all + lbase;
-    const int2 *const sb = sband + (pre ? pipe.half : 0) * kLevBand;
-    if (pre) {
-        cp_async_wait_all();
-        __syncthreads();
-    }
-    // prefetch the next tile's lists into the other half when both tiles fit one
-    pipe.pre = false;
-    if (kLevPrefetch<T> && cs_next >= 0 && (pre || np <= kLevHalf)) {
-        const int4 tn = sl.tinfo[cs_next];
-        if (tn.y <= kLevHalf && tn.z <= kLevBand) {
-            const int h = pre ? 1 - pipe.half : 1;
-            const uint32_t *pn = sl.pairs + tn.x;
-            const S *wn = (const S *)sl.pw + tn.x;
-            const int2 *bn = sl.band + tn.x;
-            for (int k = threadIdx.x; k < tn.y; k += blockDim.x) {
-                cp_async<4>(sp_all + h * kLevHalf + k, pn + k);
-                cp_async<(int)sizeof(S)>(spw_all + h * kLevHalf + k, wn + k);
-            }
-            for (int q = threadIdx.x; q < tn.z; q += blockDim.x) cp_async<8>(sband + h * kLevBand + q, bn + q);
-            cp_async_commit();
-            pipe.pre = true;
-            pipe.half = h;
+    const int cnt = e.x >> 16, cell = e.x & 0xffff;
+    const long long c = ((long long)wrap_add(lo.z, cell >> 6, g.n[2]) * g.n[1] + wrap_add(lo.y, (cell >> 3) & 7, g.n[1])) *
+                            g.n[0] +
+                        wrap_add(lo.x, cell & 7, g.n[0]);
+    T v[3] = {T(0), T(0), T(0)};
+    if (has) v[0] = u[c], v[1] = u[N + c], v[2] = u[2 * N + c];
+    const uint32_t *const pairs = sl.pairs + pb;
+    const S *const pw = (const S *)sl.pw + pb;
+    int off = __shfl_sync(0xffffffffu, e.y, 0);
+    const int rows = __reduce_max_sync(0xffffffffu, cnt);
+    uint32_t mk[U];
+    S wt[U];
+    auto load_rows = [&](int k0) {
+#pragma unroll
+        for (int r = 0; r < U; ++r) {
+            const bool act = k0 + r < cnt;
+            const unsigned a = __ballot_sync(0xffffffffu, act);
+            const int pos = off + __popc(a & ((1u << lane) - 1u));
+            off += __popc(a);
+            mk[r] = act ? __ldg(pairs + pos) : 0u;
+            wt[r] = act ? __ldg(pw + pos) : S();
         }
-    }
-    auto cell_index = [&](int cell) {
-        const int tx = cell & 7, ty = (cell >> 3) & 7, tz = cell >> 6;
-        return ((long long)wrap_add(lo.z, tz, g.n[2]) * g.n[1] + wrap_add(lo.y, ty, g.n[1])) * g.n[0] +
-               wrap_add(lo.x, tx, g.n[0]);
     };
-    // ---- before the wait
-    int2 e[2];
-    long long c[2];
-    T v[2][3];
+    load_rows(0);
+    wait();
+    SumAcc<T> acc[3];
+    for (int k0 = 0; k0 < rows; k0 += U) {
+        S a[U][3], w[U];
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        const int q = threadIdx.x + j * blockDim.x;
-        e[j] = make_int2(0, 0);
-        c[j] = 0;
-        v[j][0] = v[j][1] = v[j][2] = T(0);
-        if (q < nb) {
-            e[j] = pre ? sb[q] : band[q];
-            c[j] = cell_index(e[j].x & 0xffff);
-            v[j][0] = u[c[j]];
-            v[j][1] = u[N + c[j]];
-            v[j][2] = u[2 * N + c[j]];
+        for (int r = 0; r < U; ++r) {
+            w[r] = wt[r];
+            a[r][0] = a[r][1] = a[r][2] = S();
+            if (k0 + r < cnt) load_source(A, mk[r], a[r]);
+        }
+        if (k0 + U < rows) load_rows(k0 + U);
+#pragma unroll
+        for (int r = 0; r < U; ++r)
+            if (k0 + r < cnt) {
+                acc[0].add(w[r], a[r][0]);
+                acc[1].add(w[r], a[r][1]);
+                acc[2].add(w[r], a[r][2]);
+            }
+    }
+    if (has) {
+        T *const f_out = (T *)cd.f;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const T s = acc[k].value();
+            u[k * N + c] = v[k] + s;
+            if (f_out) f_out[k * N + c] += (T)(s * inv_dt);
         }
     }
-    if (pstaged && !pre)
-        for (int k = threadIdx.x; k < np; k += blockDim.x) {
-            sp[k] = __ldg(pairs + k);
-            spw[k] = __ldg(pwg + k);
-        }
-    const uint32_t m0 = (staged && (int)threadIdx.x < nc) ? cand[threadIdx.x] : 0u;
-    // ---- the interpolation's sources
-    if (!wait()) return false;
-    if (staged)
-        for (int i = threadIdx.x; i < nc; i += blockDim.x) {
-            const uint32_t m = i == (int)threadIdx.x ? m0 : cand[i];
-#pragma unroll
-            for (int q = 0; q < 3; ++q) sA[4 * i + q] = A_src[4 * (size_t)m + q];
-        }
-    __syncthreads();
-    auto cell_sum = [&](int2 ee, T out[3]) {
-        const int cnt = ee.x >> 16;
-        SumAcc<T> acc[3];
-        auto done = [&]() {
-#pragma unroll
-            for (int q = 0; q < 3; ++q) out[q] = acc[q].value();
-        };
-        if (staged && pstaged) {
-            // batches of kSB pairs: every shared-memory load of a batch is
-            // issued before its sums, which are added in list order
-            constexpr int kSB = 4;
-            for (int k0 = 0; k0 < cnt; k0 += kSB) {
-                uint32_t pk[kSB];
-                S wt[kSB], a[kSB][3];
-#pragma unroll
-                for (int j = 0; j < kSB; ++j) {
-                    const bool in = k0 + j < cnt;
-                    pk[j] = in ? sp[ee.y + k0 + j] : 0u;
-                    wt[j] = in ? spw[ee.y + k0 + j] : S();
-                }
-#pragma unroll
-                for (int j = 0; j < kSB; ++j) {
-                    const S *Ai = sA + 4 * (pk[j] & 0xffff);
-                    a[j][0] = Ai[0], a[j][1] = Ai[1], a[j][2] = Ai[2];
-                }
-#pragma unroll
-                for (int j = 0; j < kSB; ++j)
-                    if (k0 + j < cnt) {
-                        acc[0].add(wt[j], a[j][0]);
-                        acc[1].add(wt[j], a[j][1]);
-                        acc[2].add(wt[j], a[j][2]);
-                    }
-            }
-            done();
-            return;
-        }
-        for (int k = 0; k < cnt; ++k) {
-            const uint32_t pk = pstaged ? sp[ee.y + k] : __ldg(pairs + ee.y + k);
-            const S wt = pstaged ? spw[ee.y + k] : __ldg(pwg + ee.y + k);
-            const int i = pk & 0xffff;
-            S a0, a1, a2;
-            if (staged) {
-                const S *Ai = sA + 4 * i;
-                a0 = Ai[0], a1 = Ai[1], a2 = Ai[2];
-            } else {
-                const S *Ai = A_src + 4 * (size_t)cand[i];
-                a0 = Ai[0], a1 = Ai[1], a2 = Ai[2];
-            }
-            acc[0].add(wt, a0);
-            acc[1].add(wt, a1);
-            acc[2].add(wt, a2);
-        }
-        done();
-    };
-    auto update = [&](long long cc, const T vv[3], const T acc[3]) {
-#pragma unroll
-        for (int q = 0; q < 3; ++q) u[q * N + cc] = vv[q] + acc[q];
-        if (f_out)
-#pragma unroll
-            for (int q = 0; q < 3; ++q) f_out[q * N + cc] += (T)(acc[q] * inv_dt);
-    };
-#pragma unroll
-    for (int j = 0; j < 2; ++j)
-        if ((int)threadIdx.x + j * (int)blockDim.x < nb) {
-            T acc[3];
-            cell_sum(e[j], acc);
-            update(c[j], v[j], acc);
-        }
-    // cells beyond two per thread (blocks smaller than half a tile)
-    for (int q = threadIdx.x + 2 * blockDim.x; q < nb; q += blockDim.x) {
-        const int2 ee = pre ? sb[q] : band[q];
-        const long long cc = cell_index(ee.x & 0xffff);
-        T acc[3];
-        cell_sum(ee, acc);
-        const T vv[3] = {u[cc], u[N + cc], u[2 * N + cc]};
-        update(cc, vv, acc);
-    }
-    __syncthreads();
-    return true;
 }
 
 template <typename T, int KER>
-__global__ void __launch_bounds__(kGatherThreads, sizeof(T) == 4 ? 5 : 4) k_gather_level(PassArgs<T> a, int L) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int stage = a.stage;                             // staged candidates per tile
-    PS<T> *sA = (PS<T> *)smem_raw;                         // [stage][4]
-    uint32_t *sp = (uint32_t *)(sA + (size_t)stage * 4);   // [kLevPairs]
-    PS<T> *spw = (PS<T> *)(sp + kLevPairs);                // [kLevPairs]
-    int2 *sband = (int2 *)(spw + kLevPairs);               // [2][kLevBand]
+__global__ void __launch_bounds__(kSliceThreads, kSliceCtas<T>) k_gather_level(PassArgs<T> a, int L) {
     const int nl = *a.nlev;
-    const int s0 = L < nl ? a.lev_sbeg[L] : 0, s1 = L < nl ? a.lev_sbeg[L + 1] : 0;
-    if (s0 + (int)blockIdx.x >= s1) {
-        grid_dep_wait();
-        return;
+    const int2 ls = L < nl ? a.lev_slice[L] : make_int2(0, 0);
+    const int step = gridDim.x * (kSliceThreads / 32);
+    for (int j = blockIdx.x * (kSliceThreads / 32) + (threadIdx.x >> 5); j < ls.y; j += step) {
+        // FP64 fields: at its last slice a warp lets the next interpolation be
+        // scheduled, so its CTAs load their marker data while the last slices sum
+        if (sizeof(T) == 8 && j + step >= ls.y) grid_dep_launch();
+        gather_slice<T>(a.ct, a.slices[ls.x + j], a.sl, a.ms.A, a.inv_dt, [] { grid_dep_wait(); });
     }
-    // Tiles come largest first.  FP64 sums are bound by FP64 issue, so their
-    // rounds alternate direction (boustrophedon): the CTA with the largest tile
-    // of one round takes the smallest of the next (measured 4 % faster per
-    // step).  FP32 tiles are latency-bound and finish sooner in plain
-    // grid-stride order (measured 0.5 %).  Either way, once a round's index
-    // passes the end, every later round's does too.
-    // (the wait inside returns at once after the first tile)
-    constexpr bool kSnake = sizeof(T) == 8;
-    const int G = gridDim.x, i = blockIdx.x, nt = s1 - s0;
-    auto tile_of = [&](int r) { return (kSnake && (r & 1)) ? (r + 1) * G - 1 - i : r * G + i; };
-    GatherPipe pipe{0, false};
-    for (int r = 0;; ++r) {
-        const int j = tile_of(r);
-        if (j >= nt) break;
-        const int jn = tile_of(r + 1);
-        // FP64 fields: at its last tile the CTA lets the next interpolation be
-        // scheduled, so its CTAs load their marker data while the last tiles
-        // sum (measured 762 -> 739 us per step; FP32 fields, whose gather
-        // ends sooner, measured 553 -> 567 us and keep the trigger at exit)
-        if (sizeof(T) == 8 && jn >= nt) grid_dep_launch();
-        gather_tile_level<T, Kernel<KER>::W>(
-            a.ct, a.tperm[s0 + j], a.sl, a.ms.A, a.inv_dt, sA, sp, spw, sband, stage,
-            [] {
-                grid_dep_wait();
-                return true;
-            },
-            pipe, jn < nt ? a.tperm[s0 + jn] : -1);
-    }
-    cp_async_wait_all();  // (a prefetch is only issued for a tile that follows)
+    grid_dep_wait();  // every CTA waits before it exits
 }
 
-// Spreading (ib_spread) over the tiles' per-cell lists, as a wavefront gather
-// over every tile: the case's u slot holds the field spread into, its f slot
+// Spreading (ib_spread) over the tiles' lists, a CTA per tile, its warps taking
+// the tile's slices: the case's u slot holds the field spread into, its f slot
 // is null.
 template <typename T, int KER>
-__global__ void __launch_bounds__(kGatherThreads, sizeof(T) == 4 ? 5 : 4)
-k_spread_gather(CaseTab ct, const int *__restrict__ ncompact_p, Slots sl, const PS<T> *__restrict__ A) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr int stage = TileStage<T>::N;
-    PS<T> *sA = (PS<T> *)smem_raw;
-    uint32_t *sp = (uint32_t *)(sA + (size_t)stage * 4);
-    PS<T> *spw = (PS<T> *)(sp + kLevPairs);
-    int2 *sband = (int2 *)(spw + kLevPairs);
+__global__ void __launch_bounds__(kSliceThreads, kSliceCtas<T>)
+k_spread_gather(CaseTab ct, const int *ncompact_p, Slots sl, const PS<T> *A) {
     grid_dep_wait();
     const int nc = *ncompact_p;
-    GatherPipe pipe{0, false};
-    for (int cs = blockIdx.x; cs < nc; cs += gridDim.x)
-        gather_tile_level<T, Kernel<KER>::W>(ct, cs, sl, A, 0.0, sA, sp, spw, sband, stage, [] { return true; }, pipe,
-                                             cs + (int)gridDim.x < nc ? cs + (int)gridDim.x : -1);
-    cp_async_wait_all();
+    for (int cs = blockIdx.x; cs < nc; cs += gridDim.x) {
+        const int4 ti = sl.tinfo[cs];
+        for (int s = threadIdx.x >> 5; 32 * s < ti.z; s += kSliceThreads / 32)
+            gather_slice<T>(ct, make_int4(cs, s, ti.x, ti.z), sl, A, 0.0, [] {});
+    }
 }
 
 // The atomic form of a wavefront's spreading (ib_ctx_set_spread_mode):
@@ -1914,16 +1769,13 @@ __global__ void __launch_bounds__(256) k_scatter_level(PassArgs<T> a, int L) {
 template <typename T, int KER>
 __global__ void __launch_bounds__(256) k_mdf_passes(PassArgs<T> a) {
     constexpr int KW = Kernel<KER>::W;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    PS<T> *sw = (PS<T> *)smem_raw;                      // [N][12]
-    PS<T> *sA = sw + (size_t)TileStage<T>::N * 12;      // [N][4]
     const int nl = *a.nlev;
     const double inv_dt = a.inv_dt;
     const int gtid = blockIdx.x * blockDim.x + threadIdx.x;
     const int gsz = gridDim.x * blockDim.x;
     for (int L = a.L0; L < nl; ++L) {
         const int m0 = a.lev_mbeg[L], m1 = a.lev_mbeg[L + 1];
-        const int s0 = a.lev_sbeg[L], s1 = a.lev_sbeg[L + 1];
+        const int2 ls = a.atomic ? make_int2(0, 0) : a.lev_slice[L];
         for (int m = 0; m < a.Ns; ++m) {
             // interpolation phase: U = J u, F += (U^d - U)/dt, A = (U^d - U) dV / h^3
             for (int i = m0 + gtid; i < m1; i += gsz) {
@@ -1962,9 +1814,9 @@ __global__ void __launch_bounds__(256) k_mdf_passes(PassArgs<T> a) {
                     scatter_marker<T, KW>((T *)cd.u, (T *)cd.f, cd.g, N, a.ms.anchor[l], w, A, valid, inv_dt);
                 }
             } else {
-                // gather phase over the wavefront's tiles (their per-cell lists)
-                for (int cs = s0 + blockIdx.x; cs < s1; cs += gridDim.x)
-                    gather_tile_lists<T, KW, true>(a.ct, cs, a.sl, a.ms.wts, a.ms.A, inv_dt, sw, sA);
+                // gather phase over the wavefront's slices
+                for (int j = gtid >> 5; j < ls.y; j += gsz >> 5)
+                    gather_slice<T>(a.ct, a.slices[ls.x + j], a.sl, a.ms.A, inv_dt, [] {});
             }
             if (!grid_sync(a.bar, a.st)) return;
         }
@@ -2045,12 +1897,14 @@ static int slots_alloc(Arena &ar, int M, int ndense, int mode, Slots &sl, SlotSc
         sl.pw = ar.take<PS<T>>((size_t)KW3 * M);
         sl.nband = ar.take<int>(ncap);
         sl.tinfo = ar.take<int4>(ncap);
+        sl.slen = ar.take<uint4>(ncap);
     } else {
         sl.pcnt = sl.poff = nullptr;
         sl.band = nullptr;
         sl.pairs = nullptr;
         sl.nband = nullptr;
         sl.tinfo = nullptr;
+        sl.slen = nullptr;
         sl.pw = nullptr;
     }
     if (!ar.ok())
@@ -2066,7 +1920,7 @@ static int slots_alloc(Arena &ar, int M, int ndense, int mode, Slots &sl, SlotSc
 template <typename T, int KW>
 static int slots_build(ib_ctx *ctx, const CaseTab &ct, int M, int ndense, SlotGeom sg, const uint64_t *anchor,
                        const PS<T> *wts, const int *level, Slots &sl, const SlotScratch &sc, int *&ncompact_dev,
-                       cudaStream_t s, bool with_pairs, bool pdl_first = true) {
+                       cudaStream_t s, bool with_pairs, bool jagged, bool pdl_first = true) {
     const int nb = grid_blocks(M, 256, ctx->sm_count);
     launch_dep(pdl_first, k_slot_count<KW>, dim3(nb), dim3(256), 0, s, ct, M, sg, anchor, sl.count);
     launch_pdl(k_slot_scan, dim3(sc.lb_tiles[0]), dim3(kLbThreads), 0, s, (const uint32_t *)sl.count, ndense,
@@ -2081,11 +1935,12 @@ static int slots_build(ib_ctx *ctx, const CaseTab &ct, int M, int ndense, SlotGe
     ncompact_dev = (int *)(sl.flag_scan + ndense);
     launch_pdl(k_tile_lists<T, KW>, dim3(ctx->sm_count * kListCtas), dim3(kListThreads), 0, s, ct, sg.mode, sc.ncompact_cap,
                (const int *)ncompact_dev, sg, (const uint32_t *)sl.dense_of, (const uint32_t *)sl.start, anchor, level, sl,
-               wts, sc.big, (int *)sc.lb_ticket + 2);
+               wts, jagged ? 1 : 0, sc.big, (int *)sc.lb_ticket + 2);
     auto large = k_tile_lists_large<T, KW>;
     cudaFuncSetAttribute(large, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CtaLists));
     launch_pdl(large, dim3(ctx->sm_count), dim3(kPairThreads), sizeof(CtaLists), s, ct, sg.mode, sg,
-               (const uint32_t *)sl.dense_of, (const uint32_t *)sl.start, anchor, level, sl, wts, (const int *)sc.big,
+               (const uint32_t *)sl.dense_of, (const uint32_t *)sl.start, anchor, level, sl, wts, jagged ? 1 : 0,
+               (const int *)sc.big,
                (const int *)sc.lb_ticket + 2, ctx->status);
     return check_launch("slot lists");
 }
@@ -2130,11 +1985,9 @@ static int run_spread(ib_ctx *ctx, const ib_grid *grid, int M, const double *X, 
     PhaseTimer tm(ctx, IB_PHASE_SPREAD, s);
     k_prep_spread<T, KER><<<nb, 256, 0, s>>>(g, M, X, F, dV, ms, ctx->status);
     rc = slots_build<T, KW>(ctx, ct, M, (int)ndense, sg, ms.anchor, (const PS<T> *)ms.wts, nullptr, sl, sc, ncompact, s,
-                            true);
+                            true, true);
     if (rc) return rc;
-    const size_t smem = level_stage_bytes<T>(TileStage<T>::N);
-    cudaFuncSetAttribute(k_spread_gather<T, KER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    launch_pdl(k_spread_gather<T, KER>, dim3(ctx->sm_count * (sizeof(T) == 4 ? 5 : 4)), dim3(kGatherThreads), smem, s, ct,
+    launch_pdl(k_spread_gather<T, KER>, dim3(ctx->sm_count * kSliceCtas<T>), dim3(kSliceThreads), 0, s, ct,
                (const int *)ncompact, sl, (const PS<T> *)ms.A);
     return check_launch("ib_spread");
 }
@@ -2188,11 +2041,14 @@ static int run_mdf(ib_ctx *ctx, Arena &ar, const CaseTab &ct, const ib_particles
     Slots sl{};
     SlotScratch sc{};
     int rc = IB_OK;
-    int *tperm = nullptr;
+    int2 *lev_slice = nullptr;
+    int4 *slices = nullptr;
     if (!atomic) {
         rc = slots_alloc<T, KW>(ar, M, (int)ndense, sg.mode, sl, sc, s, true, resident);
         if (rc) return rc;
-        tperm = ar.take<int>(sc.ncompact_cap);
+        lev_slice = ar.take<int2>(P + 1);
+        // a tile of p pairs has at most p / 32 + 1 slices
+        slices = ar.take<int4>((size_t)KW * KW * KW * M / 32 + sc.ncompact_cap + 1);
     }
     if (!ar.ok())
         return oom_error(ar.used, ar.cap);
@@ -2205,8 +2061,8 @@ static int run_mdf(ib_ctx *ctx, Arena &ar, const CaseTab &ct, const ib_particles
     a.sl = sl;
     a.mperm = mperm;
     a.lev_mbeg = lo.lev_mbeg;
-    a.lev_sbeg = lev_sbeg;
-    a.tperm = tperm;
+    a.lev_slice = lev_slice;
+    a.slices = slices;
     a.nlev = lo.nlev;
     a.Ns = Ns;
     a.dt = dt;
@@ -2214,9 +2070,6 @@ static int run_mdf(ib_ctx *ctx, Arena &ar, const CaseTab &ct, const ib_particles
     a.bar = bar;
     a.st = ctx->status;
     a.atomic = atomic ? 1 : 0;
-    // staging capacity of the wavefront gather (a layout choice: the sums
-    // are the same staged or not)
-    a.stage = ctx->gather_stage > 0 && ctx->gather_stage < TileStage<T>::N ? ctx->gather_stage : TileStage<T>::N;
     // wavefronts enqueued as separate kernels: the count the last call on this
     // context copied to a pinned host word (read without synchronising: an
     // aligned 4-byte word is either the old or the new count; a short count
@@ -2291,7 +2144,7 @@ static int run_mdf(ib_ctx *ctx, Arena &ar, const CaseTab &ct, const ib_particles
     int *ncompact = nullptr;
     if (!atomic) {
         rc = slots_build<T, KW>(ctx, ct, M, (int)ndense, sg, ms.anchor, (const PS<T> *)ms.wts, lo.level, sl, sc,
-                                ncompact, s, true, false);
+                                ncompact, s, true, level_path, false);
         if (rc) return rc;
         a.sl = sl;
     }
@@ -2341,8 +2194,8 @@ static int run_mdf(ib_ctx *ctx, Arena &ar, const CaseTab &ct, const ib_particles
     if (!atomic) {
         launch_pdl(k_level_slots, dim3(1), dim3(256), 0, s, sg.mode, (const int *)lo.nlev,
                    (const int *)lo.lev_pbeg, (const uint32_t *)sl.flag_scan, (int)ndense, lev_sbeg);
-        launch_pdl(k_level_tile_order, dim3(P < 64 ? P : 64), dim3(512), 0, s, (const int *)lo.nlev,
-                   (const int *)lev_sbeg, (const int *)sl.nband, tperm);
+        launch_pdl(k_level_slices, dim3(P < 64 ? P : 64), dim3(kSliceOrderThreads), 0, s, (const int *)lo.nlev,
+                   (const int *)lev_sbeg, sl, lev_slice, slices);
     }
     tprep.stop();
     // (the field is first read and written by the pass kernels below)
@@ -2350,27 +2203,21 @@ static int run_mdf(ib_ctx *ctx, Arena &ar, const CaseTab &ct, const ib_particles
     // one timed phase: the wavefront kernels and the persistent remainder
     PhaseTimer tpass(ctx, IB_PHASE_MDF_PASSES, s);
     {
-        const size_t gsm = level_stage_bytes<T>(a.stage);
-        cudaFuncSetAttribute(k_gather_level<T, KER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm);
-        // one resident wave of gather CTAs (grid-stride over the wavefront's tiles)
-        int gper = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&gper, k_gather_level<T, KER>, kGatherThreads, gsm);
-        if (gper < 1) gper = 1;
+        // one resident wave of gather CTAs (grid-stride over the wavefront's slices)
+        int gper = kSliceCtas<T>;
         if (ctx->gather_ctas > 0 && ctx->gather_ctas < gper) gper = ctx->gather_ctas;
         // every level kernel after the first is a programmatic dependent of
         // the one before it (see k_interp_level); the first gather instead
         // waits for the interpolation on the second stream
         cudaLaunchConfig_t cg = {};
         cg.gridDim = dim3(ctx->sm_count * gper);
-        cg.blockDim = dim3(kGatherThreads);
-        cg.dynamicSmemBytes = gsm;
+        cg.blockDim = dim3(kSliceThreads);
         cg.stream = s;
         cg.attrs = pdl;
         // the atomic form: one lane per marker of the largest wavefront at most
         cudaLaunchConfig_t cs = cg;
         cs.gridDim = dim3(grid_blocks(M, 256, ctx->sm_count));
         cs.blockDim = dim3(256);
-        cs.dynamicSmemBytes = 0;
         if (fork) cudaStreamWaitEvent(s, ctx->fork_ev[1], 0);
         for (int L = 0; L < Lenq; ++L)
             for (int m = 0; m < Ns; ++m) {
@@ -2388,14 +2235,12 @@ static int run_mdf(ib_ctx *ctx, Arena &ar, const CaseTab &ct, const ib_particles
             }
     }
     int per_sm = 0;
-    const size_t smem = tile_stage_bytes<T>();
-    cudaFuncSetAttribute(k_mdf_passes<T, KER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mdf_passes<T, KER>, 256, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mdf_passes<T, KER>, 256, 0);
     if (per_sm < 1) return set_error(IB_ERR_CUDA, "mdf kernel cannot be resident");
     int nblocks = per_sm * ctx->sm_count;
     void *args[] = {&a};
     cudaError_t e =
-        cudaLaunchCooperativeKernel((const void *)k_mdf_passes<T, KER>, nblocks, 256, args, smem, s);
+        cudaLaunchCooperativeKernel((const void *)k_mdf_passes<T, KER>, nblocks, 256, args, 0, s);
     if (e != cudaSuccess) return set_error(IB_ERR_CUDA, "mdf launch: %s", cudaGetErrorString(e));
     tpass.stop();
     cudaMemcpyAsync(ctx->h_nlev, lo.nlev, sizeof(int), cudaMemcpyDeviceToHost, s);
