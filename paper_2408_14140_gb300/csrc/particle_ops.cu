@@ -922,26 +922,54 @@ __global__ void __launch_bounds__(kVolThreads, 2) k_volume_plan(CaseTab ct, int 
 // Volume integrals of axis-aligned ellipsoids (semi-axes a, b, c), through
 // the level set of Eq. (level-set function of spheroidal geometries).  Grid =
 // P * nsplit CTAs, CTA (p, s) walks a slab of cell planes of particle p's
-// box: the level set is evaluated once per node into two rolling node planes
-// in shared memory, and every cell of the plane forms alpha from its eight
-// corners (cells with alpha = 0 are skipped).  Boxes wider than kEllAx - 1
-// cells evaluate the corners per cell.  The same sums as the oracle, grouped
-// per CTA then per slab.
+// box.  The kernel is bound by the FP64 pipe (2 operations per clock and SM), so
+// FP64 is kept for what needs it: FP32 squares of the scaled cell centres tell
+// the cells with every corner inside (alpha = 1: five FP64 operations) and
+// outside (none) from those the surface may cut, and the level set is evaluated
+// only at nodes near the surface, once per node into two rolling node planes in
+// shared memory.  An FP64 instruction costs the same for one lane as for 32:
+// the CTA lists a plane's near nodes and cut cells (a list a warp, in the order
+// of its rows) and runs the lists end to end, and what is the same for the CTA
+// or a plane is computed by one warp.  48 ellipsoids of FP32 fields in boxes of
+// up to 28 cells an axis: 64 us; 167 us with the level set at every node and
+// alpha for every cell, 99 us with each warp running its own rows' lists.
+// Boxes wider than kEllAx - 1 cells in x or y evaluate the corners per cell.
+// The same sums as the oracle, grouped per lane, CTA and slab.
 // ---------------------------------------------------------------------------
 constexpr int kEllAx = 65;
-constexpr size_t kEllSmem = 2 * (size_t)kEllAx * kEllAx * sizeof(double);
-static_assert(kEllSmem >= 7 * kVolThreads * sizeof(double) && kVolSmem >= 7 * kVolThreads * sizeof(double),
-              "the CTA sum reuses the dynamic shared memory");
+constexpr int kEllWarps = kVolThreads / 32;
+struct EllBox {
+    double c[3], ia[3];  // centre, inverse semi-axes
+    int lo[3], dims[3];  // first cell and cells per axis
+    bool ok;
+};
+struct EllShared {
+    double plane[2][kEllAx * kEllAx];
+    double sq[3][kEllAx];                  // squares of the nodes' scaled coordinates
+    double r[3][kEllAx];                   // the cells' distances from the centre
+    float nsq[3][kEllAx], csq[3][kEllAx];  // FP32 squares: nodes, cell centres
+    int off[3][kEllAx];                    // the cells' wrapped grid indices
+    EllBox box;
+    int count[2][kEllWarps];  // entries of the warps' lists: near nodes, cut cells
+    uint16_t list[2][kEllWarps][(kEllAx + kEllWarps - 1) / kEllWarps * kEllAx];
+};
+constexpr size_t kEllSmem = sizeof(EllShared);
+static_assert(kEllSmem >= 7 * kVolThreads * sizeof(double), "the CTA sum reuses the dynamic shared memory");
 
 __device__ __forceinline__ double pvf_alpha8(const double ph[8]) {
     double num = 0.0, den = 0.0;
 #pragma unroll
     for (int m = 0; m < 8; ++m) {
-        num += fmax(-ph[m], 0.0);
-        den += fabs(ph[m]);
+        // max(-phi, 0) and |phi| by the sign bit
+        const double mag = fabs(ph[m]);
+        num += __double_as_longlong(ph[m]) < 0 ? mag : 0.0;
+        den += mag;
     }
     return den > 0.0 ? num / den : 0.5;
 }
+// an FP32 field value widened on the integer pipe
+__device__ __forceinline__ double widened(float x) { return df_widen(x); }
+__device__ __forceinline__ double widened(double x) { return x; }
 
 template <typename T>
 __global__ void __launch_bounds__(kVolThreads) k_volume_ellipsoid(CaseTab ct, int P, int nsplit,
@@ -951,76 +979,198 @@ __global__ void __launch_bounds__(kVolThreads) k_volume_ellipsoid(CaseTab ct, in
                                                                   unsigned int *__restrict__ done, double *Iu,
                                                                   double *Irxu, double *vol, DevStatus *st) {
     extern __shared__ __align__(16) double s_phi[];
+    EllShared &s = *(EllShared *)s_phi;
     const int p = blockIdx.x / nsplit, split = blockIdx.x % nsplit;
     if (p >= P) return;
     const DevCase cd = ct.of_particle(p);
     const DevGrid g = cd.g;
     const T *__restrict__ u = (const T *)cd.u;
-    const double c[3] = {Xr[3 * p], Xr[3 * p + 1], Xr[3 * p + 2]};
-    const double ax[3] = {axes[3 * p], axes[3 * p + 1], axes[3 * p + 2]};
-    double acc[7] = {0, 0, 0, 0, 0, 0, 0};
-    bool ok = finite3(c) && finite3(ax) && ax[0] > 0.0 && ax[1] > 0.0 && ax[2] > 0.0;
-    if (!ok && threadIdx.x == 0 && split == 0) raise_status(st, IB_ERR_NONFINITE, p);
-    int lo[3] = {0, 0, 0}, dims[3] = {0, 0, 0};
-    if (ok) {
-        for (int a = 0; a < 3; ++a) {
-            const long long l = (long long)floor((c[a] - ax[a] - g.org[a]) * g.inv_h) - 1;
-            const long long hg = (long long)floor((c[a] + ax[a] - g.org[a]) * g.inv_h) + 1;
-            lo[a] = (int)l;
-            dims[a] = (int)(hg - l + 1);
-            if (dims[a] > g.n[a] || l < INT_MIN / 2 || l > INT_MAX / 2) ok = false;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp == 0) {
+        const double ctr[3] = {Xr[3 * p], Xr[3 * p + 1], Xr[3 * p + 2]};
+        const double ax[3] = {axes[3 * p], axes[3 * p + 1], axes[3 * p + 2]};
+        bool ok = finite3(ctr) && finite3(ax) && ax[0] > 0.0 && ax[1] > 0.0 && ax[2] > 0.0;
+        if (!ok && lane == 0 && split == 0) raise_status(st, IB_ERR_NONFINITE, p);
+        if (ok) {
+            bool fits = true;
+            for (int a = 0; a < 3; ++a) {
+                const long long l = (long long)floor((ctr[a] - ax[a] - g.org[a]) * g.inv_h) - 1;
+                const long long hg = (long long)floor((ctr[a] + ax[a] - g.org[a]) * g.inv_h) + 1;
+                const int d = (int)(hg - l + 1);
+                if (d > g.n[a] || l < INT_MIN / 2 || l > INT_MAX / 2) fits = false;
+                if (lane == 0) {
+                    s.box.c[a] = ctr[a];
+                    s.box.ia[a] = 1.0 / ax[a];
+                    s.box.lo[a] = (int)l;
+                    s.box.dims[a] = d;
+                }
+            }
+            if (!fits && lane == 0 && split == 0) raise_status(st, IB_ERR_UNSUPPORTED, p);
+            ok = fits;
         }
-        if (!ok && threadIdx.x == 0 && split == 0) raise_status(st, IB_ERR_UNSUPPORTED, p);
+        if (lane == 0) s.box.ok = ok;
     }
+    __syncthreads();
+    double acc[7] = {0, 0, 0, 0, 0, 0, 0};
+    const EllBox &bx = s.box;
+    const bool ok = bx.ok;
+    const int lo[3] = {ok ? bx.lo[0] : 0, ok ? bx.lo[1] : 0, ok ? bx.lo[2] : 0};
+    const int dims[3] = {ok ? bx.dims[0] : 0, ok ? bx.dims[1] : 0, ok ? bx.dims[2] : 0};
     const int t = (dims[2] + nsplit - 1) / nsplit;
     const int z0 = split * t, z1 = min(dims[2], z0 + t);
     if (ok && z0 < z1) {
         const long long N = (long long)g.n[0] * g.n[1] * g.n[2];
         const double h = g.h;
-        const double ia[3] = {1.0 / ax[0], 1.0 / ax[1], 1.0 / ax[2]};
-        auto level = [&](int i, int j, int k) {  // node (lo + (i, j, k)): x_node = org + index h
-            const double x = (g.org[0] + (double)(lo[0] + i) * h - c[0]) * ia[0];
-            const double y = (g.org[1] + (double)(lo[1] + j) * h - c[1]) * ia[1];
-            const double z = (g.org[2] + (double)(lo[2] + k) * h - c[2]) * ia[2];
-            return sqrt(x * x + y * y + z * z) - 1.0;
-        };
-        auto add_cell = [&](int i, int j, int k, double al) {
-            const long long cc = ((long long)wrap_int(lo[2] + k, g.n[2]) * g.n[1] + wrap_int(lo[1] + j, g.n[1])) *
-                                     g.n[0] + wrap_int(lo[0] + i, g.n[0]);
-            const double r[3] = {g.org[0] + ((double)(lo[0] + i) + 0.5) * h - c[0],
-                                 g.org[1] + ((double)(lo[1] + j) + 0.5) * h - c[1],
-                                 g.org[2] + ((double)(lo[2] + k) + 0.5) * h - c[2]};
-            const double u0 = (double)u[cc], u1 = (double)u[N + cc], u2 = (double)u[2 * N + cc];
-            acc[0] += al * u0;
-            acc[1] += al * u1;
-            acc[2] += al * u2;
-            acc[3] += al * (r[1] * u2 - r[2] * u1);
-            acc[4] += al * (r[2] * u0 - r[0] * u2);
-            acc[5] += al * (r[0] * u1 - r[1] * u0);
-            acc[6] += al;
-        };
         const int nx = dims[0] + 1, ny = dims[1] + 1;
         if (nx <= kEllAx && ny <= kEllAx) {
-            const int plane = nx * ny;
-            auto node_plane = [&](int kn, double *buf) {
-                for (int q = threadIdx.x; q < plane; q += blockDim.x) buf[q] = level(q % nx, q / nx, kn);
+            // axis a's entries of nodes and cells first, first + 1, ... (at most
+            // kEllAx, none beyond the box)
+            auto table = [&](int a, int first) {
+                const double ia = bx.ia[a], ca = bx.c[a];
+                for (int i = lane; i < kEllAx && first + i <= dims[a]; i += 32) {
+                    const double x = (g.org[a] + (double)(lo[a] + first + i) * h - ca) * ia;
+                    const double r = g.org[a] + ((double)(lo[a] + first + i) + 0.5) * h - ca;
+                    s.sq[a][i] = x * x;
+                    s.nsq[a][i] = (float)(x * x);
+                    s.r[a][i] = r;
+                    s.csq[a][i] = (float)(r * ia * (r * ia));
+                    s.off[a][i] = wrap_int(lo[a] + first + i, g.n[a]);
+                }
             };
-            node_plane(z0, s_phi + (z0 & 1) * plane);
+            // a corner lies within del of its cell's centre in scaled
+            // coordinates; the margin is far above the FP32 squares' rounding
+            const float fa[3] = {(float)h * (float)bx.ia[0], (float)h * (float)bx.ia[1], (float)h * (float)bx.ia[2]};
+            const float del = 0.5f * sqrtf(fa[0] * fa[0] + fa[1] * fa[1] + fa[2] * fa[2]) * 1.0001f + 1e-5f;
+            const float in = 1.0f - del, out = 1.0f + del, nin = 1.0f - 2.0f * del, nout = 1.0f + 2.0f * del;
+            const float in2 = in > 0.0f ? in * in * 0.9999f : -1.0f, out2 = out * out * 1.0001f;
+            const float nin2 = nin > 0.0f ? nin * nin * 0.9999f : -1.0f, nout2 = nout * nout * 1.0001f;
+            // append the lanes' flagged entries to the warp's list
+            auto push = [&](uint16_t *list, int &cnt, bool flag, int code) {
+                const unsigned b = __ballot_sync(0xffffffffu, flag);
+                if (flag) list[cnt + __popc(b & ((1u << lane) - 1u))] = (uint16_t)code;
+                cnt += __popc(b);
+            };
+            // run(entry) over the warps' lists end to end, 32 entries a warp
+            auto run_lists = [&](int which, auto &&run) {
+                int start = 0, w = 0, n = s.count[which][0];
+                for (int e = threadIdx.x;; e += kVolThreads) {
+                    while (w < kEllWarps && e >= start + n) {
+                        start += n;
+                        ++w;
+                        n = w < kEllWarps ? s.count[which][w] : 0;
+                    }
+                    if (w == kEllWarps) break;
+                    const int code = s.list[which][w][e - start];
+                    run(code & 255, code >> 8);
+                }
+            };
+            // the tables hold the z planes zt, ..., zt + kEllAx - 1
+            int zt = z0;
+            auto list_nodes = [&](int kn) {
+                const float z2 = s.nsq[2][kn - zt];
+                int cnt = 0;
+                for (int i0 = 0; i0 < nx; i0 += 32) {
+                    const int i = i0 + lane;
+                    const float x2 = i < nx ? s.nsq[0][i] + z2 : -1.0f;
+                    for (int j = warp; j < ny; j += kEllWarps) {
+                        const float q = x2 + s.nsq[1][j];
+                        push(s.list[0][warp], cnt, x2 >= 0.0f && q >= nin2 && q <= nout2, j << 8 | i);
+                    }
+                }
+                if (lane == 0) s.count[0][warp] = cnt;
+            };
+            auto eval_nodes = [&](int kn) {
+                double *const buf = s.plane[kn & 1];
+                const double zz = s.sq[2][kn - zt];
+                run_lists(0, [&](int i, int j) { buf[j * nx + i] = sqrt(s.sq[0][i] + s.sq[1][j] + zz) - 1.0; });
+            };
+            if (warp < 3) table(warp, warp == 2 ? z0 : 0);
+            __syncthreads();
+            list_nodes(z0);
+            __syncthreads();
+            eval_nodes(z0);
+            __syncthreads();
+            list_nodes(z0 + 1);
+            __syncthreads();
+            int inside = 0;  // cells of alpha 1
             for (int kz = z0; kz < z1; ++kz) {
-                node_plane(kz + 1, s_phi + ((kz + 1) & 1) * plane);
+                eval_nodes(kz + 1);
+                const float z2 = s.csq[2][kz - zt];
+                const double rz = s.r[2][kz - zt];
+                const long long zrow = (long long)s.off[2][kz - zt] * g.n[1];
+                // list the cut cells; sum a lane's cells of alpha 1 per column step
+                int cuts = 0;
+                for (int i0 = 0; i0 < dims[0]; i0 += 32) {
+                    const int i = i0 + lane;
+                    const bool cell = i < dims[0];
+                    const float x2 = cell ? s.csq[0][i] + z2 : 0.0f;
+                    const int ox = cell ? s.off[0][i] : 0;
+                    double pu[3] = {0, 0, 0}, yu0 = 0.0, yu2 = 0.0;
+                    const int before = inside;
+                    for (int j = warp; j < dims[1]; j += kEllWarps) {
+                        const float q = x2 + s.csq[1][j];
+                        if (cell && q < in2) {
+                            const long long cc = (zrow + s.off[1][j]) * g.n[0] + ox;
+                            const double u0 = widened(u[cc]), u1 = widened(u[N + cc]), u2 = widened(u[2 * N + cc]);
+                            const double ry = s.r[1][j];
+                            pu[0] += u0, pu[1] += u1, pu[2] += u2;
+                            yu0 = fma(ry, u0, yu0);
+                            yu2 = fma(ry, u2, yu2);
+                            ++inside;
+                        }
+                        push(s.list[1][warp], cuts, cell && q >= in2 && q <= out2, j << 8 | i);
+                    }
+                    if (inside != before) {
+                        const double rx = s.r[0][i];
+                        acc[0] += pu[0];
+                        acc[1] += pu[1];
+                        acc[2] += pu[2];
+                        acc[3] += fma(-rz, pu[1], yu2);
+                        acc[4] = fma(rz, pu[0], fma(-rx, pu[2], acc[4]));
+                        acc[5] += fma(rx, pu[1], -yu0);
+                    }
+                }
+                if (lane == 0) s.count[1][warp] = cuts;
                 __syncthreads();
-                const double *b0 = s_phi + (kz & 1) * plane, *b1 = s_phi + ((kz + 1) & 1) * plane;
-                for (int q = threadIdx.x; q < dims[0] * dims[1]; q += blockDim.x) {
-                    const int j = q / dims[0], i = q - j * dims[0];
+                const double *b0 = s.plane[kz & 1], *b1 = s.plane[(kz + 1) & 1];
+                run_lists(1, [&](int i, int j) {
                     const int qn = j * nx + i;
                     const double ph[8] = {b0[qn], b0[qn + 1], b0[qn + nx], b0[qn + nx + 1],
                                           b1[qn], b1[qn + 1], b1[qn + nx], b1[qn + nx + 1]};
                     const double al = pvf_alpha8(ph);
-                    if (al != 0.0) add_cell(i, j, kz, al);
+                    if (al == 0.0) return;
+                    const long long cc = (zrow + s.off[1][j]) * g.n[0] + s.off[0][i];
+                    const double u0 = al * widened(u[cc]), u1 = al * widened(u[N + cc]),
+                                 u2 = al * widened(u[2 * N + cc]);
+                    const double rx = s.r[0][i], ry = s.r[1][j];
+                    acc[0] += u0;
+                    acc[1] += u1;
+                    acc[2] += u2;
+                    acc[3] = fma(ry, u2, fma(-rz, u1, acc[3]));
+                    acc[4] = fma(rz, u0, fma(-rx, u2, acc[4]));
+                    acc[5] = fma(rx, u1, fma(-ry, u0, acc[5]));
+                    acc[6] += al;
+                });
+                if (kz + 1 < z1) {
+                    if (kz + 2 - zt == kEllAx) {  // the next planes' table
+                        __syncthreads();
+                        zt = kz + 1;
+                        if (warp == 2) table(2, zt);
+                        __syncthreads();
+                    }
+                    list_nodes(kz + 2);
                 }
                 __syncthreads();
             }
+            acc[6] += (double)inside;
         } else {
+            const double c[3] = {bx.c[0], bx.c[1], bx.c[2]}, ia[3] = {bx.ia[0], bx.ia[1], bx.ia[2]};
+            auto level = [&](int i, int j, int k) {  // node (lo + (i, j, k)): x_node = org + index h
+                const double x = (g.org[0] + (double)(lo[0] + i) * h - c[0]) * ia[0];
+                const double y = (g.org[1] + (double)(lo[1] + j) * h - c[1]) * ia[1];
+                const double z = (g.org[2] + (double)(lo[2] + k) * h - c[2]) * ia[2];
+                return sqrt(x * x + y * y + z * z) - 1.0;
+            };
             for (int kz = z0; kz < z1; ++kz)
                 for (int q = threadIdx.x; q < dims[0] * dims[1]; q += blockDim.x) {
                     const int j = q / dims[0], i = q - j * dims[0];
@@ -1028,7 +1178,20 @@ __global__ void __launch_bounds__(kVolThreads) k_volume_ellipsoid(CaseTab ct, in
 #pragma unroll
                     for (int m = 0; m < 8; ++m) ph[m] = level(i + (m & 1), j + ((m >> 1) & 1), kz + ((m >> 2) & 1));
                     const double al = pvf_alpha8(ph);
-                    if (al != 0.0) add_cell(i, j, kz, al);
+                    if (al == 0.0) continue;
+                    const long long cc = ((long long)wrap_int(lo[2] + kz, g.n[2]) * g.n[1] + wrap_int(lo[1] + j, g.n[1])) *
+                                             g.n[0] + wrap_int(lo[0] + i, g.n[0]);
+                    const double r[3] = {g.org[0] + ((double)(lo[0] + i) + 0.5) * h - c[0],
+                                         g.org[1] + ((double)(lo[1] + j) + 0.5) * h - c[1],
+                                         g.org[2] + ((double)(lo[2] + kz) + 0.5) * h - c[2]};
+                    const double u0 = (double)u[cc], u1 = (double)u[N + cc], u2 = (double)u[2 * N + cc];
+                    acc[0] += al * u0;
+                    acc[1] += al * u1;
+                    acc[2] += al * u2;
+                    acc[3] += al * (r[1] * u2 - r[2] * u1);
+                    acc[4] += al * (r[2] * u0 - r[0] * u2);
+                    acc[5] += al * (r[0] * u1 - r[1] * u0);
+                    acc[6] += al;
                 }
         }
     }

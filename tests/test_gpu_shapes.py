@@ -115,3 +115,31 @@ def test_drag_force_matches_oracle(api):
     ref = oracle.drag_force(Fib, Inew, Iold, 1.3, 2e-3)
     assert nerr(FD, ref) <= 1e-15
     ctx.close()
+
+
+# boxes of 40/41 cells (one and a half warps of a row), of 64 cells (the widest
+# with node planes) and 65, tall and flat ones, an ellipsoid below a cell, and
+# a whole box per CTA or a plane or two per CTA
+@pytest.mark.parametrize("split", [0, 1, 32])
+def test_cell_classes_and_box_sizes(api, split):
+    N = 80
+    h = 1.0 / N
+    rng = synth.SplitMix64(21)
+    u = synth.fourier_field((N,) * 3, 4, rng, h)
+    half = np.array([[18.5, 18.9, 2.2], [31.0, 3.0, 31.9], [2.0, 30.6, 31.4], [1.5, 2.5, 37.0],
+                     [0.2, 0.4, 0.3], [4.0, 4.0, 4.0]])
+    X = np.array([[40, 40, 40], [40.5, 40.25, 12], [0.3, 40, 79.9], [20, 60.1, 40], [33.2, 41.9, 7.5], [16, 16, 16]])
+    ctx = api.Context()
+    ctx.set_volume_split(split)
+    out = ctx.particle_volume_integrals_ellipsoid(torch.tensor(u, device="cuda"), h, t64(X * h), t64(half * h))
+    ctx.status()
+    ref = oracle.volume_integrals_ellipsoid((N,) * 3, h, (0, 0, 0), u, X * h, half * h)
+    for g, r in zip(out, ref):
+        assert nerr(g, r) <= TOL[0]
+    # cells outside take no part, whatever they hold
+    v = torch.full((3, N, N, N), float("nan"), device="cuda", dtype=torch.float64)
+    v[:, 8:24, 8:24, 8:24] = torch.tensor(u[:, 8:24, 8:24, 8:24], device="cuda")
+    part = ctx.particle_volume_integrals_ellipsoid(v, h, t64(X[5:] * h), t64(half[5:] * h))
+    for g, r in zip(part, out):
+        assert torch.equal(g[0], r[5])
+    ctx.close()
