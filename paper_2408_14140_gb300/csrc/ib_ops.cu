@@ -1711,9 +1711,13 @@ __global__ void __launch_bounds__(kSliceThreads, kSliceCtas<T>) k_gather_level(P
     const int step = gridDim.x * (kSliceThreads / 32);
     for (int j = blockIdx.x * (kSliceThreads / 32) + (threadIdx.x >> 5); j < ls.y; j += step) {
         // FP64 fields: at its last slice a warp lets the next interpolation be
-        // scheduled, so its CTAs load their marker data while the last slices sum
-        if (sizeof(T) == 8 && j + step >= ls.y) grid_dep_launch();
-        gather_slice<T>(a.ct, a.slices[ls.x + j], a.sl, a.ms.A, a.inv_dt, [] { grid_dep_wait(); });
+        // scheduled, so its CTAs load their marker data while the last slices
+        // sum (after the wait: that data includes the forces that the
+        // interpolation before this kernel wrote)
+        gather_slice<T>(a.ct, a.slices[ls.x + j], a.sl, a.ms.A, a.inv_dt, [&] {
+            grid_dep_wait();
+            if (sizeof(T) == 8 && j + step >= ls.y) grid_dep_launch();
+        });
     }
     grid_dep_wait();  // every CTA waits before it exits
 }

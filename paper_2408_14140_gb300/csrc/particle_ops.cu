@@ -967,8 +967,10 @@ __device__ __forceinline__ double pvf_alpha8(const double ph[8]) {
     }
     return den > 0.0 ? num / den : 0.5;
 }
-// an FP32 field value widened on the integer pipe
-__device__ __forceinline__ double widened(float x) { return df_widen(x); }
+// an FP32 field value, exact, widened on the integer pipe (which takes subnormals as 0)
+__device__ __forceinline__ double widened(float x) {
+    return (__float_as_uint(x) << 1) - 1u < 0xffffffu ? (double)x : df_widen(x);
+}
 __device__ __forceinline__ double widened(double x) { return x; }
 
 template <typename T>
