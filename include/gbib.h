@@ -283,13 +283,12 @@ GBIB_API int particle_volume_integrals(ib_ctx *ctx, const ib_grid *grid, const v
  * after the forcing (Eqs. particle1/particle2, Sec. 3.2.2) with the particles
  * where they are: the cells and their volume fractions alpha are the same.
  * particle_volume_integrals_keep computes what particle_volume_integrals
- * computes (bitwise) and keeps in `plan` the cells each CTA visited, plane by
- * plane, with the boundary cells' alpha; particle_volume_integrals_plan then
- * integrates another field u (same grid, same particles) over the kept cells
- * with the kept alpha and the same per-cell arithmetic, without evaluating a
- * level set: each particle's kept cells are one list spread evenly over the
- * context's split of CTAs per particle (ib_ctx_set_volume_split; automatic:
- * one resident wave), so its sums agree with particle_volume_integrals on
+ * computes (bitwise) and keeps in `plan` the cells the surface cuts with their
+ * alpha; particle_volume_integrals_plan then integrates another field u (same
+ * grid, same particles) over the kept cells and the cells of alpha 1 (which
+ * follow from the positions) with the same per-cell arithmetic, without
+ * evaluating a level set, over the context's split of CTAs per particle
+ * (ib_ctx_set_volume_split; automatic: one resident wave), so its sums agree with particle_volume_integrals on
  * that field to rounding (another summation order; deterministic for a given
  * split).  A plan holds up to P particles
  * whose stencil boxes have at most max_box_cells cells (at most 40 cells per

@@ -27,27 +27,26 @@
 
 namespace gbib {
 
-// double -> (hi, lo), integer pipe only.
+// double -> (hi, lo), integer pipe only.  Outside [2^-74, 2^128): below 2^-126
+// a zero, below 2^-74 no low part, above (and Inf, NaN) the class is kept.
 __device__ __forceinline__ float2 df_split(double x) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     const unsigned h32 = (unsigned)(b >> 32), l32 = (unsigned)b;
-    const unsigned sgn = h32 & 0x80000000u;
-    const int e = (int)((h32 >> 20) & 0x7ffu);  // biased exponent (bias 1023)
-    const unsigned mh = ((h32 & 0xfffffu) << 3) | (l32 >> 29);  // top 23 stored bits
-    if (e <= 896) return make_float2(__uint_as_float(sgn), __uint_as_float(sgn));  // |x| < 2^-126
-    if (e >= 1151) {  // beyond float range, Inf or NaN: keep the class
+    const unsigned mag = h32 & 0x7fffffffu, sgn = h32 & 0x80000000u;
+    // the exponent rebiased from 1023 to 127 and the top 23 stored bits
+    const unsigned hi = __funnelshift_l(l32, mag - (896u << 20), 3) | sgn;
+    if (mag - (949u << 20) < (202u << 20)) {
+        // the remaining 29 bits r, worth r * 2^(e - 1075), e the double's exponent
+        const float scale = __uint_as_float((hi & 0xff800000u) - (52u << 23));
+        return make_float2(__uint_as_float(hi), __fmul_rn(__uint2float_rn(l32 & 0x1fffffffu), scale));
+    }
+    const unsigned e = mag >> 20;
+    if (e <= 896) return make_float2(__uint_as_float(sgn), __uint_as_float(sgn));
+    if (e >= 1151) {
         const unsigned nan = (e == 2047 && ((h32 & 0xfffffu) | l32)) ? 0x400000u : 0u;
         return make_float2(__uint_as_float(sgn | 0x7f800000u | nan), 0.0f);
     }
-    const float hi = __uint_as_float(sgn | ((unsigned)(e - 896) << 23) | mh);
-    float lo = 0.0f;
-    if (e >= 949) {
-        // remaining 29 bits r, worth r * 2^(e - 1075)
-        const unsigned r = l32 & 0x1fffffffu;
-        const float scale = __uint_as_float((unsigned)(e - 948) << 23);
-        lo = __uint_as_float(__float_as_uint(__fmul_rn(__uint2float_rn(r), scale)) | sgn);
-    }
-    return make_float2(hi, lo);
+    return make_float2(__uint_as_float(hi), 0.0f);
 }
 
 // float -> double, exact, integer pipe only (float subnormals become 0).

@@ -48,25 +48,36 @@ __device__ __forceinline__ void block_sum(double v[NV]) {
 
 // ---------------------------------------------------------------------------
 // volume integrals.  Grid = P * nsplit CTAs; CTA (p, s) walks a slab of
-// cell planes of particle p's box.  Per plane it evaluates the level set
-// phi = |x - X_r|/R - 1 once per node (only for nodes within 1.75 h of the
-// surface: the corners of every cell whose centre lies within 0.8661 h of the
-// surface), keeps two node planes in shared memory, and then visits, row by
-// row, only the cells whose centre lies within R + 0.8661 h.  Cells whose
-// centre lies deeper than R - 0.8661 h have all corners inside (alpha = 1);
-// the others form alpha from their eight corner values.  The last CTA of a
-// particle (completion counter) adds the nsplit partial sums in slab order.
+// cell planes of particle p's box.  Cells whose centre lies deeper than
+// R - 0.8661 h have all corners inside (alpha = 1) and are summed by columns;
+// those within R + 0.8661 h form alpha from their eight corner values, the level
+// set phi = |x - X_r|/R - 1, evaluated once per node (only for nodes within
+// 1.75 h of the surface: the corners of every such cell) into two rolling node
+// planes in shared memory.  The last CTA of a particle (completion counter)
+// adds the nsplit partial sums in slab order.
 // ---------------------------------------------------------------------------
 constexpr int kVolSplit = 8;       // CTAs per particle of the allocation-free entry point
 constexpr int kVolMaxSplit = 32;
 constexpr int kVolThreads = 256;   // 8 warps
 constexpr int kVolMaxBox = 40;     // cells per axis of one particle's box (tabulated path)
 constexpr int kVolAx = kVolMaxBox + 1;
-// two node planes of (max(-phi, 0), max(phi, 0)) pairs + per-row grid
-// offsets + per-axis tables (cell offsets and node squares as float pairs,
-// cell squares in FP32)
-constexpr size_t kVolSmem = 2 * kVolAx * kVolAx * sizeof(double2) + kVolAx * sizeof(long long) +
-                            6 * kVolAx * sizeof(float2) + 3 * kVolAx * sizeof(float);
+constexpr int kVolWarps = kVolThreads / 32;
+// What the interior sums read: grid offsets of rows and planes, the cells'
+// offsets from X_r as float pairs and their squares in FP32, per axis.
+struct VolTables {
+    long long row_off[kVolAx], plane_off[kVolAx];
+    float2 tbf[3][kVolAx];
+    float tcf[3][kVolAx];
+};
+struct VolShared {
+    float4 phi[2][kVolAx * kVolAx];  // node planes: (max(-phi, 0), max(phi, 0)) as float pairs
+    VolTables tb;
+    float2 tsq[3][kVolAx];           // squares of the nodes' offsets as float pairs
+    int count[2][kVolWarps];         // entries of the warps' lists: near nodes, cut cells
+    uint16_t list[2][kVolWarps][(kVolAx + kVolWarps - 1) / kVolWarps * kVolAx];
+};
+constexpr size_t kVolSmem = sizeof(VolShared);
+static_assert(kVolSmem >= 10 * kVolThreads * sizeof(double), "the CTA sums reuse the dynamic shared memory");
 
 // Double-float accumulation: a sum kept as the unevaluated pair hi + lo of two
 // floats -- Knuth's TwoSum for the addition error and the fused multiply-add
@@ -130,6 +141,182 @@ __device__ __forceinline__ DF df_phi(DF x2, float2 iR) {
     const float q = r * iR.x;
     const float qe = fmaf(r, iR.x, -q) + fmaf(r, iR.y, corr * iR.x);
     return df_sum(DF{q, qe}, DF{-1.0f, 0.0f});
+}
+
+// A thread's double-float sums of w = alpha u, of the six products ry w2,
+// rz w1, rz w0, rx w2, rx w1, ry w0 (r x w = (ry w2 - rz w1, rz w0 - rx w2,
+// rx w1 - ry w0)), of the cut cells' alpha, and its number of cells of alpha 1.
+struct VolSums {
+    DF W[3] = {}, Pm[6] = {}, V = {};
+    unsigned inside = 0;
+};
+// one cell's share: its alpha, field values and centre offsets as float pairs
+template <typename T>
+__device__ __forceinline__ void add_cut_cell(VolSums &s, float2 a2, const float2 v[3], float2 fx, float2 fy, float2 fz) {
+    df_add2(s.V, a2.x, a2.y);
+    float wh[3], wl[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        // alpha u with the product's rounding error and the cross terms
+        wh[c] = a2.x * v[c].x;
+        wl[c] = fmaf(a2.x, v[c].x, -wh[c]) + a2.y * v[c].x;
+        if constexpr (sizeof(T) == 8) wl[c] = fmaf(a2.x, v[c].y, wl[c]);
+        df_add2(s.W[c], wh[c], wl[c]);
+    }
+    df_add_prod(s.Pm[0], fy.x, fy.y, wh[2], wl[2]);
+    df_add_prod(s.Pm[1], fz.x, fz.y, wh[1], wl[1]);
+    df_add_prod(s.Pm[2], fz.x, fz.y, wh[0], wl[0]);
+    df_add_prod(s.Pm[3], fx.x, fx.y, wh[2], wl[2]);
+    df_add_prod(s.Pm[4], fx.x, fx.y, wh[1], wl[1]);
+    df_add_prod(s.Pm[5], fy.x, fy.y, wh[0], wl[0]);
+}
+
+// The tables of a box (its first cell lo, centre c), by warps 0 to 5.
+__device__ __forceinline__ void volume_tables(VolTables &tb, const DevGrid &g, const int lo[3], const int dims[3],
+                                              const double c[3]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp < 3) {
+        for (int i = lane; i < dims[warp]; i += 32) {
+            const double xc = g.org[warp] + ((double)(lo[warp] + i) + 0.5) * g.h - c[warp];
+            tb.tbf[warp][i] = df_split_rn(xc);
+            tb.tcf[warp][i] = (float)(xc * xc);
+        }
+    } else if (warp == 3) {
+        for (int j = lane; j < dims[1]; j += 32) tb.row_off[j] = (long long)wrap_int(lo[1] + j, g.n[1]) * g.n[0];
+    } else if (warp == 4) {
+        for (int k = lane; k < dims[2]; k += 32)
+            tb.plane_off[k] = (long long)wrap_int(lo[2] + k, g.n[2]) * g.n[1] * g.n[0];
+    }
+}
+// squared distance of a cell's centre from X_r in FP32 (one order everywhere)
+__device__ __forceinline__ float centre_sq(float xy, float z) { return __fadd_rn(xy, z); }
+
+// The cells of alpha 1 (squared distance below rin2) in planes [z0, z1): a thread
+// takes columns of the slab, so that a cell costs three sums and the two
+// products with its z offset; those with x and y are taken once a column.
+// DEPTH planes' field values are loaded together (two of an FP64 field where four
+// would not fit the registers of k_volume: 41 against 38 us).
+template <int DEPTH, typename T>
+__device__ __forceinline__ void interior_columns(VolSums &s, const T *__restrict__ u, const DevGrid &g, const VolTables &tb,
+                                                 int lo0w, const int dims[3], int z0, int z1, float rin2) {
+    const long long N = (long long)g.n[0] * g.n[1] * g.n[2];
+    for (int q = threadIdx.x; q < dims[0] * dims[1]; q += kVolThreads) {
+        const int j = q / dims[0], i = q - j * dims[0];
+        const float xy = __fadd_rn(tb.tcf[0][i], tb.tcf[1][j]);
+        if (!(xy < rin2)) continue;
+        const T *const col = u + tb.row_off[j] + wrap_add(lo0w, i, g.n[0]);
+        DF S[3] = {}, Z0 = {}, Z1 = {};
+        unsigned n = 0;
+        for (int k0 = z0; k0 < z1; k0 += DEPTH) {
+            bool in[DEPTH];
+            T v[DEPTH][3];
+#pragma unroll
+            for (int r = 0; r < DEPTH; ++r) {
+                in[r] = k0 + r < z1 && centre_sq(xy, tb.tcf[2][k0 + r]) < rin2;
+                if (in[r])
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) v[r][c] = col[c * N + tb.plane_off[k0 + r]];
+            }
+#pragma unroll
+            for (int r = 0; r < DEPTH; ++r) {
+                if (!in[r]) continue;
+                const float2 fz = tb.tbf[2][k0 + r];
+                const float2 v0 = field_pair(v[r][0]), v1 = field_pair(v[r][1]), v2 = field_pair(v[r][2]);
+                df_add2(S[0], v0.x, v0.y);
+                df_add2(S[1], v1.x, v1.y);
+                df_add2(S[2], v2.x, v2.y);
+                df_add_prod(Z0, fz.x, fz.y, v0.x, v0.y);
+                df_add_prod(Z1, fz.x, fz.y, v1.x, v1.y);
+                ++n;
+            }
+        }
+        if (n == 0) continue;
+        const float2 fx = tb.tbf[0][i], fy = tb.tbf[1][j];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) df_add2(s.W[c], S[c].hi, S[c].lo);
+        df_add_prod(s.Pm[0], fy.x, fy.y, S[2].hi, S[2].lo);
+        df_add2(s.Pm[1], Z1.hi, Z1.lo);
+        df_add2(s.Pm[2], Z0.hi, Z0.lo);
+        df_add_prod(s.Pm[3], fx.x, fx.y, S[2].hi, S[2].lo);
+        df_add_prod(s.Pm[4], fx.x, fx.y, S[1].hi, S[1].lo);
+        df_add_prod(s.Pm[5], fy.x, fy.y, S[0].hi, S[0].lo);
+        s.inside += n;
+    }
+}
+
+// End of a CTA of the double-float sums: the CTA's sums in double-float, one
+// conversion to FP64 per quantity, and the particle's nsplit CTA sums in FP64, in
+// order, by the last CTA of the particle to finish (FP64 issue is scarce on this
+// part: no FP64 operation per warp).  The threads' sums go through shared memory
+// (s_sum, free again once every thread is here): a warp adds a quantity, its
+// lanes kVolWarps entries each before the shuffles, a third of the instructions of
+// shuffle trees in every warp.
+struct VolFinish {
+    float2 sum[10][kVolThreads];
+};
+__device__ __forceinline__ void volume_finish_df(VolSums &s, double h, int p, int split, int nsplit,
+                                                 double *__restrict__ partial, unsigned int *__restrict__ done,
+                                                 double *Iu, double *Irxu, double *vol, VolFinish &f) {
+    __shared__ unsigned s_ncell[kVolWarps];
+    __shared__ double s_q[10];
+    __shared__ int s_last_df;
+    const unsigned ncell = __reduce_add_sync(0xffffffffu, s.inside);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (lane == 0) s_ncell[wid] = ncell;
+    __syncthreads();  // every thread is done with the shared memory reused here
+#pragma unroll
+    for (int q = 0; q < 10; ++q) {
+        const DF x = q < 3 ? s.W[q] : q < 9 ? s.Pm[q < 3 || q > 8 ? 0 : q - 3] : s.V;
+        f.sum[q][threadIdx.x] = make_float2(x.hi, x.lo);
+    }
+    __syncthreads();
+    for (int q = wid; q < 10; q += kVolWarps) {
+        DF x = {0.f, 0.f};
+#pragma unroll
+        for (int m = 0; m < kVolWarps; ++m) {
+            const float2 y = f.sum[q][lane + 32 * m];
+            df_add2(x, y.x, y.y);
+        }
+        df_warp_sum(x);
+        if (lane == 0) s_q[q] = df_to_double(make_float2(x.hi, x.lo));
+    }
+    __syncthreads();
+    if (threadIdx.x < 7) {
+        const int k = threadIdx.x;
+        double x;
+        if (k < 3) {
+            x = s_q[k];
+        } else if (k < 6) {
+            x = s_q[3 + 2 * (k - 3)] - s_q[4 + 2 * (k - 3)];  // (ry w2 - rz w1, rz w0 - rx w2, rx w1 - ry w0)
+        } else {
+            unsigned n = 0;
+            for (int w = 0; w < kVolWarps; ++w) n += s_ncell[w];
+            x = (double)n + s_q[9];
+        }
+        const double h3 = h * h * h;
+        partial[((size_t)p * nsplit + split) * 7 + k] = x * h3;
+        __threadfence();  // release: partials before the count
+    }
+    __syncwarp();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last_df = atomicAdd(done + p, 1u) == (unsigned int)nsplit - 1;
+        __threadfence();  // acquire: the count before the other partials
+    }
+    __syncthreads();
+    if (s_last_df && threadIdx.x < 7) {
+        const int k = threadIdx.x;
+        double x = 0.0;
+        for (int sp = 0; sp < nsplit; ++sp) x += __ldcg(partial + ((size_t)p * nsplit + sp) * 7 + k);
+        if (k < 3) {
+            if (Iu) Iu[3 * p + k] = x;
+        } else if (k < 6) {
+            if (Irxu) Irxu[3 * p + k - 3] = x;
+        } else if (vol) {
+            vol[p] = x;
+        }
+        if (k == 0) done[p] = 0;  // ready for the next call
+    }
 }
 
 // |x| from x^2 to within a few units of FP64 rounding: an FP32 square root
@@ -241,29 +428,25 @@ __device__ void volume_finish(double acc[7], double h, int p, int split, int nsp
     }
 }
 
-// Most of this kernel's cost is GB300's low FP64 rate, and FP64 pipe time is
-// charged per warp instruction whatever the number of active lanes.  So each
-// plane is walked as flat lists that keep warps full and uniform:
-//   * shell nodes (|x - X_r| within 1.75 h of the surface): phi in FP64;
-//   * interior cells (centre deeper than R - 0.8661 h, shrunk by one cell,
-//     all corners inside: alpha = 1): plain sums;
-//   * boundary cells (the rest within R + 0.8661 h): alpha from the corners.
-// Per-row index ranges come from FP32 square roots widened by a cell; every
-// node and boundary cell is still tested exactly in FP64.
+// Per plane the CTA lists the near nodes and the cut cells (a list a warp, from
+// ballots over its rows, tested on FP32 squares of the tables) and runs the
+// lists end to end, a thread an entry, two barriers a plane; everything per
+// node and cell is double-float on the FP32 pipes.  64 spheres of 24 cells in an
+// FP64 field: 39 us; 57 us with per-row index ranges, row scans and a row search
+// per entry (five barriers a plane) and the interior cells listed as well.
+//
 // A kept volume plan (particle_volume_integrals_keep / _plan): per particle,
-// the cells each CTA visits plane by plane in its visiting order -- interior
-// cells (alpha = 1) and boundary cells with their alpha, or a skip mark --
-// so that a second call at the same particle positions sums another field
-// over the same cells with the same alpha without evaluating a level set.
-// Capacity `cap` entries per particle and list; a keeping CTA's slab starts
-// at dims0 dims1 z0, and each plane's header gives its lists' counts and
-// first entries.
+// the cut cells plane by plane in visiting order, with their alpha or a skip
+// mark, so that a second call at the same particle positions sums another field
+// over the same cells with the same alpha without evaluating a level set (the
+// cells of alpha 1 follow from the positions).  Capacity `cap` entries per
+// particle; a keeping CTA's slab starts at dims0 dims1 z0, and each plane's
+// header gives its list's count and first entry.
 struct PvfPlanDev {
     int cap;
-    int4 *hdr;        // [P][kVolAx] per plane: interior and boundary counts, first entries
-    unsigned *ient;   // [P][cap] interior cell i | j << 16
-    unsigned *bent;   // [P][cap] boundary cell i | j << 16, or kPvfSkip
-    float2 *balpha;   // [P][cap] boundary alpha as a float pair
+    int2 *hdr;        // [P][kVolAx] per plane: cut cells, first entry
+    unsigned *bent;   // [P][cap] cut cell i | j << 8, or kPvfSkip
+    float2 *balpha;   // [P][cap] its alpha as a float pair
     double *pos;      // [P][4] X_r and R the plan was kept for
 };
 constexpr unsigned kPvfSkip = 0x80000000u;
@@ -278,346 +461,225 @@ __global__ void __launch_bounds__(kVolThreads, 3) k_volume(CaseTab ct, int P, in
                                                         double *Irxu, double *vol, DevStatus *st,
                                                         PvfPlanDev pl = PvfPlanDev{}) {
     extern __shared__ __align__(16) double s_vol[];
-    // per-row work lists (rows <= kVolAx)
-    __shared__ int r_na[kVolAx], r_nb[kVolAx], r_nc[2][kVolAx], r_ca[kVolAx], r_cb[kVolAx];
-    __shared__ int r_ia[kVolAx], r_ib[kVolAx], r_ic[kVolAx];
-    __shared__ int p_node[kVolAx + 1], p_int[kVolAx + 1], p_bnd[kVolAx + 1];
-    __shared__ int c_node[kVolAx], c_int[kVolAx], c_bnd[kVolAx];
+    VolShared &s = *(VolShared *)s_vol;
     const int p = blockIdx.x / nsplit, split = blockIdx.x % nsplit;
     if (p >= P) return;
     const DevCase &cd = ct.of_particle(p);
     const DevGrid g = cd.g;
     const T *__restrict__ u = (const T *)cd.u;
-    // the particle's scalars, formed once by thread 0 (FP64 is scarce here:
-    // 256 threads each forming them cost more than a slab's cells)
-    __shared__ double s_c[3], s_d[6];
-    __shared__ float s_f[4];  // x of node 0 and of cell 0, 1/R as a float pair
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // the particle's scalars, formed once by warp 0 (FP64 is scarce here: 256
+    // threads each forming them cost more than a slab's cells)
+    __shared__ double s_c[3], s_sq[4], s_iR;
+    __shared__ float s_fsq[4];
+    __shared__ float2 s_iRf;
     __shared__ int s_box[7];
-    if (threadIdx.x == 0) {
+    if (warp == 0) {
         const double cc[3] = {Xr[3 * p], Xr[3 * p + 1], Xr[3 * p + 2]};
         const double R0 = radius[p];
         bool okk = finite3(cc) && isfinite(R0) && R0 > 0.0;
-        if (!okk && split == 0) raise_status(st, IB_ERR_NONFINITE, p);
-        int lo0[3] = {0, 0, 0}, dm0[3] = {0, 0, 0};
+        if (!okk && lane == 0 && split == 0) raise_status(st, IB_ERR_NONFINITE, p);
         if (okk) {
-            for (int a = 0; a < 3; ++a) {
-                long long l = (long long)floor((cc[a] - R0 - g.org[a]) * g.inv_h) - 1;
-                long long hgh = (long long)floor((cc[a] + R0 - g.org[a]) * g.inv_h) + 1;
-                lo0[a] = (int)l;
-                dm0[a] = (int)(hgh - l + 1);
-                if (dm0[a] > g.n[a] || l < INT_MIN / 2 || l > INT_MAX / 2) okk = false;
+            // a lane an axis
+            const int a = lane < 3 ? lane : 0;
+            const double ca = a == 0 ? cc[0] : a == 1 ? cc[1] : cc[2];
+            const long long l = (long long)floor((ca - R0 - g.org[a]) * g.inv_h) - 1;
+            const long long hgh = (long long)floor((ca + R0 - g.org[a]) * g.inv_h) + 1;
+            const int d = (int)(hgh - l + 1);
+            if (lane < 3) {
+                s_box[a] = (int)l;
+                s_box[3 + a] = d;
             }
-            if (!okk && split == 0) raise_status(st, IB_ERR_UNSUPPORTED, p);
-        }
-        for (int a = 0; a < 3; ++a) {
-            s_c[a] = cc[a];
-            s_box[a] = lo0[a];
-            s_box[3 + a] = dm0[a];
-        }
-        if constexpr (MODE != 0) {
-            const bool tabbed = dm0[0] <= kVolMaxBox && dm0[1] <= kVolMaxBox && dm0[2] <= kVolMaxBox;
-            if (okk && (!tabbed || (long long)dm0[0] * dm0[1] * dm0[2] > pl.cap)) {
-                if (split == 0) raise_status(st, IB_ERR_UNSUPPORTED, p);
-                okk = false;
+            okk = __all_sync(0xffffffffu, !(d > g.n[a] || l < INT_MIN / 2 || l > INT_MAX / 2));
+            if (!okk && lane == 0 && split == 0) raise_status(st, IB_ERR_UNSUPPORTED, p);
+            if constexpr (MODE != 0) {
+                const bool tabbed = __all_sync(0xffffffffu, d <= kVolMaxBox);
+                __syncwarp();
+                if (okk && (!tabbed || (long long)s_box[3] * s_box[4] * s_box[5] > pl.cap)) {
+                    if (lane == 0 && split == 0) raise_status(st, IB_ERR_UNSUPPORTED, p);
+                    okk = false;
+                }
             }
-            if (split == 0) {
-                pl.pos[4 * p] = cc[0], pl.pos[4 * p + 1] = cc[1], pl.pos[4 * p + 2] = cc[2];
-                pl.pos[4 * p + 3] = R0;
+            // squares of the bounds: cells surely inside, cells of alpha 0, the
+            // node shell (a lane a bound)
+            const double off = lane == 0 ? -0.8661 : lane == 1 ? 0.8661 : lane == 2 ? -1.75 : 1.75;
+            const double b = R0 + off * g.h;
+            if (lane < 4) {
+                // in FP32 with a relative margin far above the rounding of the
+                // squares (the nodes and cells that matter lie 0.01 h inside the
+                // node shell and 8e-5 h inside the cell bounds); cells in the
+                // margin take the corner formula, exact for them too
+                const double sq = b > 0.0 ? b * b : (lane == 0 ? -1.0 : 0.0);
+                s_sq[lane] = sq;
+                s_fsq[lane] = sq < 0.0 ? -1.0f : (float)sq * (lane & 1 ? 1.0f + 1e-5f : 1.0f - 1e-5f);
             }
+            const double ir = 1.0 / R0;
+            if (lane == 0) s_iR = ir, s_iRf = df_split_rn(ir);
         }
-        s_box[6] = okk;
-        if (okk) {
-            const double hh = g.h;
-            const double rin = R0 - 0.8661 * hh, rout = R0 + 0.8661 * hh;
-            const double sl = fmax(0.0, R0 - 1.75 * hh), sh = R0 + 1.75 * hh;
-            s_d[0] = R0;
-            s_d[1] = 1.0 / R0;
-            s_d[2] = rin > 0 ? rin * rin : -1.0;
-            s_d[3] = rout * rout;
-            s_d[4] = sl * sl;
-            s_d[5] = sh * sh;
-            s_f[0] = (float)(g.org[0] + (double)lo0[0] * hh - cc[0]);
-            s_f[1] = (float)(g.org[0] + ((double)lo0[0] + 0.5) * hh - cc[0]);
-            const float2 ir = df_split_rn(s_d[1]);
-            s_f[2] = ir.x;
-            s_f[3] = ir.y;
+        if (lane < 3) s_c[lane] = lane == 0 ? cc[0] : lane == 1 ? cc[1] : cc[2];
+        if (MODE != 0 && split == 0 && lane == 0) {
+            pl.pos[4 * p] = cc[0], pl.pos[4 * p + 1] = cc[1], pl.pos[4 * p + 2] = cc[2];
+            pl.pos[4 * p + 3] = R0;
         }
+        if (lane == 0) s_box[6] = okk;
     }
     __syncthreads();
     const double c[3] = {s_c[0], s_c[1], s_c[2]};
-    double acc[7] = {0, 0, 0, 0, 0, 0, 0};
     const bool ok = s_box[6] != 0;
-    const int lo[3] = {s_box[0], s_box[1], s_box[2]}, dims[3] = {s_box[3], s_box[4], s_box[5]};
+    const int lo[3] = {ok ? s_box[0] : 0, ok ? s_box[1] : 0, ok ? s_box[2] : 0};
+    const int dims[3] = {ok ? s_box[3] : 0, ok ? s_box[4] : 0, ok ? s_box[5] : 0};
     const int t = (dims[2] + nsplit - 1) / nsplit;
     const int z0 = split * t, z1 = min(dims[2], z0 + t);
-    if (ok && z0 < z1) {
-        const long long N = (long long)g.n[0] * g.n[1] * g.n[2];
-        const double h = g.h, iR = s_d[1];
-        const double rin2 = s_d[2], rout2 = s_d[3];
-        const double sl2 = s_d[4], sh2 = s_d[5];
-        const int lo0w = wrap_int(lo[0], g.n[0]);
-        const bool tab = dims[0] <= kVolMaxBox && dims[1] <= kVolMaxBox && dims[2] <= kVolMaxBox;
-        if (tab) {
-            const int nx = dims[0] + 1, plane = nx * (dims[1] + 1);
-            double2 *phi2 = (double2 *)s_vol;  // node planes: (max(-phi, 0), max(phi, 0))
-            long long *row_off = (long long *)(phi2 + 2 * kVolAx * kVolAx);
-            float2 *tbf = (float2 *)(row_off + kVolAx);  // cell offsets as float pairs
-            float2 *tsq = tbf + 3 * kVolAx;               // node offset squares as float pairs
-            float *tcf = (float *)(tsq + 3 * kVolAx);     // cell offset squares in FP32
-            for (int a = 0; a < 3; ++a)
-                for (int i = threadIdx.x; i <= dims[a]; i += blockDim.x) {
-                    const double xc = g.org[a] + ((double)(lo[a] + i) + 0.5) * h - c[a];
-                    const double xn = g.org[a] + (double)(lo[a] + i) * h - c[a];
-                    tbf[a * kVolAx + i] = df_split_rn(xc);
-                    tsq[a * kVolAx + i] = df_split_rn(xn * xn);
-                    tcf[a * kVolAx + i] = (float)(xc * xc);
+    const int lo0w = ok ? wrap_int(lo[0], g.n[0]) : 0;
+    if (dims[0] <= kVolMaxBox && dims[1] <= kVolMaxBox && dims[2] <= kVolMaxBox) {
+        VolSums sums;
+        if (ok && z0 < z1) {
+            const int nx = dims[0] + 1, ny = dims[1] + 1;
+            volume_tables(s.tb, g, lo, dims, c);
+            if (warp >= 5) {  // (warps 0 to 4 fill the other tables)
+                const int a = warp - 5;
+                for (int i = lane; i <= dims[a]; i += 32) {
+                    const double xn = g.org[a] + (double)(lo[a] + i) * g.h - c[a];
+                    s.tsq[a][i] = df_split_rn(xn * xn);
                 }
-            const float2 iRf = make_float2(s_f[2], s_f[3]);
-            // FP32 centre tests with a relative margin far above their rounding;
-            // cells in the margin take the corner formula, exact for them too
-            const float rout2f = (float)rout2 * (1.0f + 1e-5f);
-            const float rin2f = rin2 > 0 ? (float)rin2 * (1.0f - 1e-5f) : -1.0f;
-            for (int j = threadIdx.x; j < dims[1]; j += blockDim.x)
-                row_off[j] = (long long)wrap_int(lo[1] + j, g.n[1]) * g.n[0];
+            }
+            const float rin2 = s_fsq[0], rout2 = s_fsq[1], sl2 = s_fsq[2], sh2 = s_fsq[3];
+            const float2 iRf = s_iRf;
             __syncthreads();
-            const float fih = (float)g.inv_h;
-            // Index ranges of positions x_i = base + i h, i in [0, n), from FP32
-            // bounds with a margin of kEps cells -- far above the FP32 error of
-            // the bounds (< 1e-4 cells on grids up to 1024^3), so that every
-            // exact member is listed (range_out: |x_i| <= w) or every listed
-            // index is an exact member (range_in: |x_i| < w); empty when
-            // first > last.  Exact FP64 tests decide the cells in the margin.
-            constexpr float kEps = 1e-3f;
-            auto range_out = [&](float base, float w, int n, int &first, int &last) {
-                first = max(0, (int)ceilf((-w - base) * fih - kEps));
-                last = min(n - 1, (int)floorf((w - base) * fih + kEps));
+            auto push = [&](uint16_t *list, int &cnt, bool flag, int code) {
+                const unsigned b = __ballot_sync(0xffffffffu, flag);
+                if (flag) list[cnt + __popc(b & ((1u << lane) - 1u))] = (uint16_t)code;
+                cnt += __popc(b);
             };
-            auto range_in = [&](float base, float w, int n, int &first, int &last) {
-                first = max(0, (int)floorf((-w - base) * fih + kEps) + 1);
-                last = min(n - 1, (int)ceilf((w - base) * fih - kEps) - 1);
-            };
-            const float xbf = s_f[0], xcbf = s_f[1];  // x of node 0 and of cell 0
-            // FP32 fields: the per-row ranges from FP32 squares, the shell and
-            // the cell bounds widened by a relative 1e-5 (the rows and cells
-            // that matter lie 0.01 h inside the node shell and 8e-5 h inside
-            // the cell bounds, far beyond the FP32 error of the squares)
-            const float sh2f = (float)sh2 * (1.0f + 1e-5f), sl2f = (float)sl2 * (1.0f - 1e-5f);
-            auto node_plane = [&](int kn, double2 *buf) {
-                const int rows = dims[1] + 1;
-                for (int j = threadIdx.x; j < rows; j += blockDim.x) {
-                    bool in_shell, beyond_sl;
-                    float wo, wi;
-                    {
-                        const float dyz = tsq[kVolAx + j].x + tsq[2 * kVolAx + kn].x;
-                        in_shell = dyz < sh2f;
-                        beyond_sl = sl2f > dyz;
-                        wo = sqrtf(fmaxf(sh2f - dyz, 0.f));
-                        wi = sqrtf(fmaxf(sl2f - dyz, 0.f));
+            // run(entry's place, i, j) over the warps' lists end to end
+            auto run_lists = [&](int which, auto &&run) {
+                int start = 0, w = 0, n = s.count[which][0];
+                for (int e = threadIdx.x;; e += kVolThreads) {
+                    while (w < kVolWarps && e >= start + n) {
+                        start += n;
+                        ++w;
+                        n = w < kVolWarps ? s.count[which][w] : 0;
                     }
-                    int a0 = 0, n0 = 0, a1 = 0, n1 = 0;
-                    if (in_shell) {
-                        // nodes of the shell sl <= |x| <= sh: the outer range minus
-                        // the nodes surely inside sl
-                        int f, l, fi = 1, li = 0;
-                        range_out(xbf, wo, nx, f, l);
-                        if (beyond_sl) range_in(xbf, wi, nx, fi, li);
-                        if (li >= fi && l >= f) {
-                            a0 = f;
-                            n0 = max(0, min(l, fi - 1) - f + 1);
-                            a1 = max(li + 1, f);
-                            n1 = max(0, l - a1 + 1);
-                        } else {
-                            a0 = f;
-                            n0 = max(0, l - f + 1);
-                        }
-                    }
-                    r_na[j] = a0, r_nc[0][j] = n0, r_nb[j] = a1, r_nc[1][j] = n1;
-                    c_node[j] = n0 + n1;
-                }
-                __syncthreads();
-                warp0_scan(c_node, p_node, rows);
-                __syncthreads();
-                const int tot = p_node[rows];
-                for (int q = threadIdx.x; q < tot; q += blockDim.x) {
-                    const int j = find_row(p_node, rows, q);
-                    const int k = q - p_node[j];
-                    const int i = k < r_nc[0][j] ? r_na[j] + k : r_nb[j] + (k - r_nc[0][j]);
-                    // every listed node gets its level set value (nodes slightly
-                    // outside the shell too: the values stay exact)
-                    {
-                        // double-float level set, stored as
-                        // (max(-phi, 0), max(phi, 0)) float pairs
-                        const DF x2 = df_sum(DF{tsq[i].x, tsq[i].y},
-                                             df_sum(DF{tsq[kVolAx + j].x, tsq[kVolAx + j].y},
-                                                    DF{tsq[2 * kVolAx + kn].x, tsq[2 * kVolAx + kn].y}));
-                        const DF ph = x2.hi > 0.0f ? df_phi(x2, iRf) : DF{-1.0f, 0.0f};
-                        ((float4 *)buf)[j * nx + i] = ph.hi < 0.0f ? make_float4(-ph.hi, -ph.lo, 0.f, 0.f)
-                                                                   : make_float4(0.f, 0.f, ph.hi, ph.lo);
-                    }
+                    if (w == kVolWarps) break;
+                    const int code = s.list[which][w][e - start];
+                    run(e, code & 255, code >> 8);
                 }
             };
-            node_plane(z0, phi2 + (z0 & 1) * plane);
+            auto list_nodes = [&](int kn) {
+                const float z2 = s.tsq[2][kn].x;
+                int cnt = 0;
+                for (int i0 = 0; i0 < nx; i0 += 32) {
+                    const int i = i0 + lane;
+                    const float xz = i < nx ? s.tsq[0][i].x + z2 : 0.0f;
+                    for (int j = warp; j < ny; j += kVolWarps) {
+                        const float q = xz + s.tsq[1][j].x;
+                        push(s.list[0][warp], cnt, i < nx && q >= sl2 && q <= sh2, j << 8 | i);
+                    }
+                }
+                if (lane == 0) s.count[0][warp] = cnt;
+            };
+            // a listed node's level set value in double-float
+            auto eval_nodes = [&](int kn) {
+                float4 *const buf = s.phi[kn & 1];
+                const DF z2 = {s.tsq[2][kn].x, s.tsq[2][kn].y};
+                run_lists(0, [&](int, int i, int j) {
+                    const DF x2 = df_sum(DF{s.tsq[0][i].x, s.tsq[0][i].y},
+                                         df_sum(DF{s.tsq[1][j].x, s.tsq[1][j].y}, z2));
+                    const DF ph = x2.hi > 0.0f ? df_phi(x2, iRf) : DF{-1.0f, 0.0f};
+                    buf[j * nx + i] = ph.hi < 0.0f ? make_float4(-ph.hi, -ph.lo, 0.f, 0.f)
+                                                   : make_float4(0.f, 0.f, ph.hi, ph.lo);
+                });
+            };
+            auto list_cells = [&](int kz) {
+                const float z2 = s.tb.tcf[2][kz];
+                int cnt = 0;
+                for (int i0 = 0; i0 < dims[0]; i0 += 32) {
+                    const int i = i0 + lane;
+                    const bool cell = i < dims[0];
+                    const float x2 = cell ? s.tb.tcf[0][i] : 0.0f;
+                    for (int j = warp; j < dims[1]; j += kVolWarps) {
+                        const float q = centre_sq(__fadd_rn(x2, s.tb.tcf[1][j]), z2);
+                        push(s.list[1][warp], cnt, cell && !(q < rin2) && q <= rout2, j << 8 | i);
+                    }
+                }
+                if (lane == 0) s.count[1][warp] = cnt;
+            };
+            list_nodes(z0);
+            __syncthreads();
+            eval_nodes(z0);
+            __syncthreads();
+            list_nodes(z0 + 1);
+            interior_columns<sizeof(T) == 8 ? 2 : 4>(sums, u, g, s.tb, lo0w, dims, z0, z1, rin2);
             // the CTA's entries in the plan: from dims0 dims1 z0 on, plane by plane
-            long long pi = (long long)p * pl.cap + (long long)dims[0] * dims[1] * z0, pb = pi;
-            // per-thread double-float sums of w = alpha u, of the six products
-            // ry w2, rz w1, rz w0, rx w2, rx w1, ry w0 (r x w = (ry w2 - rz w1,
-            // rz w0 - rx w2, rx w1 - ry w0)) and of the boundary cells' alpha;
-            // no FP64 operation per cell in either field precision
-            long long nint_cells = 0;
-            DF W[3] = {}, Pm[6] = {}, V = {};
+            const long long N = (long long)g.n[0] * g.n[1] * g.n[2];
+            long long pb = (long long)p * pl.cap + (long long)dims[0] * dims[1] * z0;
             for (int kz = z0; kz < z1; ++kz) {
-                node_plane(kz + 1, phi2 + ((kz + 1) & 1) * plane);
-                // cell rows of plane kz: interior range and the boundary ranges around it
-                for (int j = threadIdx.x; j < dims[1]; j += blockDim.x) {
-                    bool in_out, in_in;
-                    float wo, wi;
-                    {
-                        const float ryz2 = tcf[kVolAx + j] + tcf[2 * kVolAx + kz];
-                        in_out = ryz2 <= rout2f;
-                        in_in = ryz2 < rin2f;
-                        wo = sqrtf(fmaxf(rout2f - ryz2, 0.f));
-                        wi = sqrtf(fmaxf(rin2f - ryz2, 0.f));
-                    }
-                    int ia = 0, ib = -1, ja = 0, jb = -1;
-                    if (in_out) {
-                        range_out(xcbf, wo, dims[0], ia, ib);
-                        if (in_in) range_in(xcbf, wi, dims[0], ja, jb);
-                        ja = max(ja, ia);  // interior within the outer range
-                        jb = min(jb, ib);
-                    }
-                    if (jb < ja) {
-                        ja = ib + 1;  // no interior: one boundary interval [ia, ib]
-                        jb = ib;
-                    }
-                    r_ia[j] = ia;
-                    r_ib[j] = ib;
-                    r_ic[j] = ja;  // interior [ja, jb] with jb stored implicitly by count
-                    c_int[j] = jb >= ja ? jb - ja + 1 : 0;
-                    r_ca[j] = max(0, min(ja - 1, ib) - ia + 1);   // left boundary [ia, ja-1]
-                    r_cb[j] = jb >= ja ? max(0, ib - jb) : 0;      // right boundary [jb+1, ib]
-                    c_bnd[j] = r_ca[j] + r_cb[j];
-                }
                 __syncthreads();
-                warp0_scan(c_int, p_int, dims[1]);
-                warp0_scan(c_bnd, p_bnd, dims[1]);
+                eval_nodes(kz + 1);
+                list_cells(kz);
                 __syncthreads();
-                const int nint = p_int[dims[1]], nbnd = p_bnd[dims[1]];
-                if (MODE == 1 && threadIdx.x == 0)
-                    pl.hdr[p * kVolAx + kz] =
-                        make_int4(nint, nbnd, (int)(pi - (long long)p * pl.cap), (int)(pb - (long long)p * pl.cap));
-                const double2 *b0 = phi2 + (kz & 1) * plane, *b1 = phi2 + ((kz + 1) & 1) * plane;
-                const float2 fz = tbf[2 * kVolAx + kz];
-                const float rz2f = tcf[2 * kVolAx + kz];
-                const long long plane_off = (long long)wrap_int(lo[2] + kz, g.n[2]) * g.n[1] * g.n[0];
-                // interior cells: alpha = 1
-                for (int q = threadIdx.x; q < nint; q += blockDim.x) {
-                    const int j = find_row(p_int, dims[1], q);
-                    const int i = r_ic[j] + (q - p_int[j]);
-                    if (MODE == 1) pl.ient[pi + q] = (unsigned)i | ((unsigned)j << 16);
-                    const long long cc = plane_off + row_off[j] + wrap_add(lo0w, i, g.n[0]);
-                    const float2 fx = tbf[i], fy = tbf[kVolAx + j];
-                    const float2 v0 = field_pair(u[cc]), v1 = field_pair(u[N + cc]), v2 = field_pair(u[2 * N + cc]);
-                    df_add2(W[0], v0.x, v0.y);
-                    df_add2(W[1], v1.x, v1.y);
-                    df_add2(W[2], v2.x, v2.y);
-                    df_add_prod(Pm[0], fy.x, fy.y, v2.x, v2.y);
-                    df_add_prod(Pm[1], fz.x, fz.y, v1.x, v1.y);
-                    df_add_prod(Pm[2], fz.x, fz.y, v0.x, v0.y);
-                    df_add_prod(Pm[3], fx.x, fx.y, v2.x, v2.y);
-                    df_add_prod(Pm[4], fx.x, fx.y, v1.x, v1.y);
-                    df_add_prod(Pm[5], fy.x, fy.y, v0.x, v0.y);
+                int ncut = 0;
+                if constexpr (MODE == 1) {
+                    for (int w = 0; w < kVolWarps; ++w) ncut += s.count[1][w];
+                    if (threadIdx.x == 0) pl.hdr[p * kVolAx + kz] = make_int2(ncut, (int)(pb - (long long)p * pl.cap));
                 }
-                nint_cells += (nint + (int)blockDim.x - 1 - (int)threadIdx.x) / (int)blockDim.x;
-                // boundary cells: alpha = sum of max(-phi, 0) / sum |phi| over the corners
-                for (int q = threadIdx.x; q < nbnd; q += blockDim.x) {
+                const float4 *const f0 = s.phi[kz & 1], *const f1 = s.phi[(kz + 1) & 1];
+                const float2 fz = s.tb.tbf[2][kz];
+                const T *const up = u + s.tb.plane_off[kz];
+                // alpha = sum of max(-phi, 0) / sum |phi| over the corners, in double-float
+                run_lists(1, [&](int e, int i, int j) {
+                    if (MODE == 1) pl.bent[pb + e] = kPvfSkip;  // until the cell counts
+                    // (loaded before alpha is known: its latency overlaps the sums)
+                    const T *const uc = up + s.tb.row_off[j] + wrap_add(lo0w, i, g.n[0]);
+                    const T u3[3] = {uc[0], uc[N], uc[2 * N]};
+                    const int qn = j * nx + i;
+                    const float4 cn[8] = {f0[qn], f0[qn + 1], f0[qn + nx], f0[qn + nx + 1],
+                                          f1[qn], f1[qn + 1], f1[qn + nx], f1[qn + nx + 1]};
+                    DF num = {0.f, 0.f}, neg = {0.f, 0.f};
+#pragma unroll
+                    for (int m = 0; m < 8; ++m) {
+                        df_add2(num, cn[m].x, cn[m].y);
+                        df_add2(neg, cn[m].z, cn[m].w);
+                    }
+                    num = df_sum(num, DF{0.f, 0.f});
+                    neg = df_sum(neg, DF{0.f, 0.f});
+                    if (num.hi == 0.0f && neg.hi > 0.0f) return;  // alpha = 0
                     float2 a2 = make_float2(1.f, 0.f);
-                    const int j = find_row(p_bnd, dims[1], q);
-                    const int k = q - p_bnd[j];
-                    const int i = k < r_ca[j] ? r_ia[j] + k : r_ic[j] + c_int[j] + (k - r_ca[j]);
-                    if (MODE == 1) pl.bent[pb + q] = kPvfSkip;  // until the cell counts
-                    {
-                        // the cell's alpha in double-float (both field precisions)
-                        const float d2f = tcf[i] + tcf[kVolAx + j] + rz2f;
-                        if (d2f > rout2f) continue;
-                        if (!(d2f < rin2f)) {
-                            const int qn = j * nx + i;
-                            const float4 *f0 = (const float4 *)b0, *f1 = (const float4 *)b1;
-                            const float4 cn[8] = {f0[qn], f0[qn + 1], f0[qn + nx], f0[qn + nx + 1],
-                                                  f1[qn], f1[qn + 1], f1[qn + nx], f1[qn + nx + 1]};
-                            DF num = {0.f, 0.f}, neg = {0.f, 0.f};
-#pragma unroll
-                            for (int m = 0; m < 8; ++m) {
-                                df_add2(num, cn[m].x, cn[m].y);
-                                df_add2(neg, cn[m].z, cn[m].w);
-                            }
-                            num = df_sum(num, DF{0.f, 0.f});
-                            neg = df_sum(neg, DF{0.f, 0.f});
-                            if (num.hi == 0.0f && neg.hi > 0.0f) continue;  // alpha = 0
-                            const DF den = df_sum(num, neg);
-                            if (den.hi == 0.0f) {
-                                a2 = make_float2(0.5f, 0.f);
-                            } else if (neg.hi != 0.0f) {
-                                if (den.hi < 1e-30f) {
-                                    a2 = df_split_rn(((double)num.hi + num.lo) / ((double)den.hi + den.lo));
-                                } else {
-                                    // num / den: a quotient and one remainder correction
-                                    const float rd = __frcp_rn(den.hi);
-                                    const float q1 = num.hi * rd;
-                                    const float pr = q1 * den.hi;
-                                    const float pe = fmaf(q1, den.hi, -pr);
-                                    const float rr = ((num.hi - pr) - pe) + fmaf(-q1, den.lo, num.lo);
-                                    a2 = make_float2(q1, rr * rd);
-                                }
-                            }
+                    const DF den = df_sum(num, neg);
+                    if (den.hi == 0.0f) {
+                        a2 = make_float2(0.5f, 0.f);
+                    } else if (neg.hi != 0.0f) {
+                        if (den.hi < 1e-30f) {
+                            a2 = df_split_rn(((double)num.hi + num.lo) / ((double)den.hi + den.lo));
+                        } else {
+                            // num / den: a quotient and one remainder correction
+                            const float rd = __frcp_rn(den.hi);
+                            const float q1 = num.hi * rd;
+                            const float pr = q1 * den.hi;
+                            const float pe = fmaf(q1, den.hi, -pr);
+                            const float rr = ((num.hi - pr) - pe) + fmaf(-q1, den.lo, num.lo);
+                            a2 = make_float2(q1, rr * rd);
                         }
-                        if constexpr (MODE == 1) {
-                            pl.bent[pb + q] = (unsigned)i | ((unsigned)j << 16);
-                            pl.balpha[pb + q] = a2;
-                        }
-                        const long long cc = plane_off + row_off[j] + wrap_add(lo0w, i, g.n[0]);
-                        df_add2(V, a2.x, a2.y);
-                        const float2 fx = tbf[i], fy = tbf[kVolAx + j];
-                        const float2 v[3] = {field_pair(u[cc]), field_pair(u[N + cc]), field_pair(u[2 * N + cc])};
-                        float wh[3], wl[3];
-#pragma unroll
-                        for (int q3 = 0; q3 < 3; ++q3) {
-                            // alpha u with the product's rounding error and the cross terms
-                            wh[q3] = a2.x * v[q3].x;
-                            wl[q3] = fmaf(a2.x, v[q3].x, -wh[q3]) + a2.y * v[q3].x;
-                            if constexpr (sizeof(T) == 8) wl[q3] = fmaf(a2.x, v[q3].y, wl[q3]);
-                            df_add2(W[q3], wh[q3], wl[q3]);
-                        }
-                        df_add_prod(Pm[0], fy.x, fy.y, wh[2], wl[2]);
-                        df_add_prod(Pm[1], fz.x, fz.y, wh[1], wl[1]);
-                        df_add_prod(Pm[2], fz.x, fz.y, wh[0], wl[0]);
-                        df_add_prod(Pm[3], fx.x, fx.y, wh[2], wl[2]);
-                        df_add_prod(Pm[4], fx.x, fx.y, wh[1], wl[1]);
-                        df_add_prod(Pm[5], fy.x, fy.y, wh[0], wl[0]);
                     }
-                }
-                pi += nint;
-                pb += nbnd;
-                __syncthreads();
+                    if constexpr (MODE == 1) {
+                        pl.bent[pb + e] = (unsigned)i | ((unsigned)j << 8);
+                        pl.balpha[pb + e] = a2;
+                    }
+                    const float2 v[3] = {field_pair(u3[0]), field_pair(u3[1]), field_pair(u3[2])};
+                    add_cut_cell<T>(sums, a2, v, s.tb.tbf[0][i], s.tb.tbf[1][j], fz);
+                });
+                pb += ncut;
+                if (kz + 1 < z1) list_nodes(kz + 2);
             }
-            acc[6] += (double)nint_cells;
-            // warp sums in double-float, then FP64 in lane 0 only
-#pragma unroll
-            for (int q = 0; q < 3; ++q) df_warp_sum(W[q]);
-#pragma unroll
-            for (int q = 0; q < 6; ++q) df_warp_sum(Pm[q]);
-            df_warp_sum(V);
-            if ((threadIdx.x & 31) == 0) {
-                acc[6] += (double)V.hi + (double)V.lo;
-                double pm[6];
-#pragma unroll
-                for (int q = 0; q < 6; ++q) pm[q] = (double)Pm[q].hi + (double)Pm[q].lo;
-#pragma unroll
-                for (int q = 0; q < 3; ++q) acc[q] = (double)W[q].hi + (double)W[q].lo;
-                acc[3] = pm[0] - pm[1];
-                acc[4] = pm[2] - pm[3];
-                acc[5] = pm[4] - pm[5];
-            }
-        } else {
+        }
+        volume_finish_df(sums, g.h, p, split, nsplit, partial, done, Iu, Irxu, vol, *(VolFinish *)s_vol);
+        return;
+    }
+    double acc[7] = {0, 0, 0, 0, 0, 0, 0};
+    {
+        const long long N = (long long)g.n[0] * g.n[1] * g.n[2];
+        const double h = g.h, iR = s_iR, rin2 = s_sq[0], rout2 = s_sq[1];
+        {
             // boxes wider than kVolMaxBox: every cell of the slab, corners evaluated directly
             for (int kz = z0; kz < z1; ++kz) {
                 const int k = lo[2] + kz;
@@ -661,19 +723,15 @@ __global__ void __launch_bounds__(kVolThreads, 3) k_volume(CaseTab ct, int P, in
 }
 
 // ---------------------------------------------------------------------------
-// Volume integrals from a kept plan.  The particle's kept cells -- interior
-// cells, and boundary cells with their double-float alpha -- are read as one
-// list per particle (the planes' lists in plane order), split evenly over
-// nsplit CTAs, each taking a contiguous range.  A thread sums its cells in
-// double-float exactly as k_volume does per cell, kPlanUnroll cells at a
-// time with their list entries and field values loaded together, so no chain
-// of dependent loads runs plane by plane; then warp sums in double-float and
-// the CTA's warp sums and the particle's CTA sums in FP64, in order.  The same
-// cells, alpha and per-cell arithmetic as k_volume, in another summation
-// order.
+// Volume integrals from a kept plan: the cells of alpha 1 by columns of a slab of
+// planes, as in k_volume, and the particle's kept cut cells with their alpha, one
+// list per particle (the planes' lists in plane order), split evenly over nsplit
+// CTAs, each taking a contiguous range, kPlanUnroll cells at a time with their
+// list entries and field values loaded together.  The same cells, alpha and
+// per-cell arithmetic as k_volume, in another summation order.  64 spheres of 24
+// cells in an FP64 field: 27 us; 32 us with the interior cells read from a list.
 // ---------------------------------------------------------------------------
 constexpr int kPlanUnroll = 4;
-constexpr size_t kPlanSmem = 10 * (kVolThreads / 32) * sizeof(float2);  // the warps' sums
 
 template <typename T>
 __global__ void __launch_bounds__(kVolThreads, 2) k_volume_plan(CaseTab ct, int P, int nsplit,
@@ -683,136 +741,84 @@ __global__ void __launch_bounds__(kVolThreads, 2) k_volume_plan(CaseTab ct, int 
                                                               unsigned int *__restrict__ done, double *Iu,
                                                               double *Irxu, double *vol, DevStatus *st,
                                                               PvfPlanDev pl) {
-    extern __shared__ __align__(16) double s_vol[];
-    __shared__ float2 tbf[3 * kVolAx];  // cell-centre offsets from X_r as float pairs
-    __shared__ long long row_off[kVolAx], plane_off[kVolAx];
-    __shared__ int c_int[kVolAx], c_bnd[kVolAx], b_int[kVolAx], b_bnd[kVolAx];
-    __shared__ int p_int[kVolAx + 1], p_bnd[kVolAx + 1];
+    __shared__ VolTables tb;
+    __shared__ VolFinish fin;
+    __shared__ int c_cut[kVolAx], b_cut[kVolAx], p_cut[kVolAx + 1];
     __shared__ double s_c[3];
+    __shared__ float s_rin2;
     __shared__ int s_box[7];
     const int p = blockIdx.x / nsplit, split = blockIdx.x % nsplit;
     if (p >= P) return;
     const DevCase &cd = ct.of_particle(p);
     const DevGrid g = cd.g;
     const T *__restrict__ u = (const T *)cd.u;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // the plan's plane headers, loaded beside the particle's scalars (every
     // particle has kVolAx header slots; only the box's planes are read)
-    for (int k = threadIdx.x; k < kVolAx; k += blockDim.x) {
-        const int4 hc = pl.hdr[p * kVolAx + k];
-        c_int[k] = hc.x;
-        c_bnd[k] = hc.y;
-        b_int[k] = hc.z;
-        b_bnd[k] = hc.w;
-    }
-    if (threadIdx.x == 0) {
+    if (warp > 0)
+        for (int k = threadIdx.x - 32; k < kVolAx; k += kVolThreads - 32) {
+            const int2 hc = pl.hdr[p * kVolAx + k];
+            c_cut[k] = hc.x;
+            b_cut[k] = hc.y;
+        }
+    else {
         // the particle's box as the keeping call formed it, once the plan is
-        // known to be this particle's
+        // known to be this particle's; a lane an axis
         const double cc[3] = {Xr[3 * p], Xr[3 * p + 1], Xr[3 * p + 2]};
         const double R0 = radius[p];
         const double *q = pl.pos + 4 * p;
         bool okk = q[0] == cc[0] && q[1] == cc[1] && q[2] == cc[2] && q[3] == R0;
-        if (!okk && split == 0) raise_status(st, IB_ERR_INVALID, p);  // not the plan's particle
-        int lo0[3] = {0, 0, 0}, dm0[3] = {0, 0, 0};
+        if (!okk && lane == 0 && split == 0) raise_status(st, IB_ERR_INVALID, p);  // not the plan's particle
         okk = okk && finite3(cc) && isfinite(R0) && R0 > 0.0;
-        if (okk)
-            for (int a = 0; a < 3; ++a) {
-                const long long l = (long long)floor((cc[a] - R0 - g.org[a]) * g.inv_h) - 1;
-                const long long hgh = (long long)floor((cc[a] + R0 - g.org[a]) * g.inv_h) + 1;
-                lo0[a] = (int)l;
-                dm0[a] = (int)(hgh - l + 1);
-                // the keeping call kept only boxes of the tabulated size
-                if (dm0[a] > g.n[a] || dm0[a] > kVolMaxBox || l < INT_MIN / 2 || l > INT_MAX / 2) okk = false;
+        if (okk) {
+            const int a = lane < 3 ? lane : 0;
+            const double ca = a == 0 ? cc[0] : a == 1 ? cc[1] : cc[2];
+            const long long l = (long long)floor((ca - R0 - g.org[a]) * g.inv_h) - 1;
+            const long long hgh = (long long)floor((ca + R0 - g.org[a]) * g.inv_h) + 1;
+            const int d = (int)(hgh - l + 1);
+            if (lane < 3) {
+                s_box[a] = (int)l;
+                s_box[3 + a] = d;
+                s_c[a] = ca;
             }
-        if (okk && (long long)dm0[0] * dm0[1] * dm0[2] > pl.cap) okk = false;  // not kept (reported then)
-        for (int a = 0; a < 3; ++a) {
-            s_c[a] = cc[a];
-            s_box[a] = lo0[a];
-            s_box[3 + a] = dm0[a];
+            // the keeping call kept only boxes of the tabulated size
+            okk = __all_sync(0xffffffffu, !(d > g.n[a] || d > kVolMaxBox || l < INT_MIN / 2 || l > INT_MAX / 2));
+            __syncwarp();
+            if (okk && (long long)s_box[3] * s_box[4] * s_box[5] > pl.cap) okk = false;  // not kept (reported then)
+            const double b = R0 - 0.8661 * g.h;
+            if (lane == 0) s_rin2 = b > 0.0 ? (float)(b * b) * (1.0f - 1e-5f) : -1.0f;
         }
-        s_box[6] = okk;
+        if (lane == 0) s_box[6] = okk;
     }
     __syncthreads();
-    const bool ok = s_box[6] != 0;
-    const int lo[3] = {s_box[0], s_box[1], s_box[2]}, dims[3] = {s_box[3], s_box[4], s_box[5]};
-    const long long N = (long long)g.n[0] * g.n[1] * g.n[2];
-    if (ok) {
-        const double h = g.h;
-        for (int a = 0; a < 3; ++a)
-            for (int i = threadIdx.x; i <= dims[a]; i += blockDim.x)
-                tbf[a * kVolAx + i] = df_split_rn(g.org[a] + ((double)(lo[a] + i) + 0.5) * h - s_c[a]);
-        for (int j = threadIdx.x; j < dims[1]; j += blockDim.x)
-            row_off[j] = (long long)wrap_int(lo[1] + j, g.n[1]) * g.n[0];
-        for (int k = threadIdx.x; k < dims[2]; k += blockDim.x)
-            plane_off[k] = (long long)wrap_int(lo[2] + k, g.n[2]) * g.n[1] * g.n[0];
-    }
-    __syncthreads();
-    if (ok) {
-        warp0_scan(c_int, p_int, dims[2]);
-        warp0_scan(c_bnd, p_bnd, dims[2]);
-    }
-    __syncthreads();
-    DF W[3] = {}, Pm[6] = {}, V = {};
-    long long nint_cells = 0;
-    if (ok) {
+    VolSums sums;
+    if (s_box[6]) {
+        const int lo[3] = {s_box[0], s_box[1], s_box[2]}, dims[3] = {s_box[3], s_box[4], s_box[5]};
+        const double c[3] = {s_c[0], s_c[1], s_c[2]};
+        const long long N = (long long)g.n[0] * g.n[1] * g.n[2];
         const int lo0w = wrap_int(lo[0], g.n[0]);
+        volume_tables(tb, g, lo, dims, c);
+        warp0_scan(c_cut, p_cut, dims[2]);
+        __syncthreads();
+        const int t = (dims[2] + nsplit - 1) / nsplit;
+        interior_columns<4>(sums, u, g, tb, lo0w, dims, min(dims[2], split * t), min(dims[2], (split + 1) * t), s_rin2);
+        // cut cells: the kept alpha (entries of cells with alpha = 0 are marked)
         const long long base = (long long)p * pl.cap;
-        const int NI = p_int[dims[2]], NB = p_bnd[dims[2]];
-        // interior cells: alpha = 1
-        const int i0 = (int)((long long)NI * split / nsplit), i1 = (int)((long long)NI * (split + 1) / nsplit);
-        // a thread's entries ascend, so its plane only moves forward
-        int kzc = i0 + (int)threadIdx.x < i1 ? find_row(p_int, dims[2], i0 + threadIdx.x) : 0;
-        for (int e0 = i0 + threadIdx.x; e0 < i1; e0 += kPlanUnroll * blockDim.x) {
-            long long cc[kPlanUnroll];
-            int kz[kPlanUnroll];
-            unsigned ent[kPlanUnroll];
-#pragma unroll
-            for (int t = 0; t < kPlanUnroll; ++t) {
-                const int e = e0 + t * blockDim.x;
-                if (e < i1)
-                    while (p_int[kzc + 1] <= e) ++kzc;
-                kz[t] = kzc;
-                ent[t] = e < i1 ? pl.ient[base + b_int[kzc] + (e - p_int[kzc])] : 0u;
-            }
-            float2 v[kPlanUnroll][3];
-#pragma unroll
-            for (int t = 0; t < kPlanUnroll; ++t) {
-                const int i = (int)(ent[t] & 0xffffu), j = (int)(ent[t] >> 16);
-                cc[t] = plane_off[kz[t]] + row_off[j] + wrap_add(lo0w, i, g.n[0]);
-                if (e0 + t * (int)blockDim.x < i1)
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) v[t][c] = field_pair(u[c * N + cc[t]]);
-            }
-#pragma unroll
-            for (int t = 0; t < kPlanUnroll; ++t) {
-                if (e0 + t * (int)blockDim.x >= i1) break;
-                const int i = (int)(ent[t] & 0xffffu), j = (int)(ent[t] >> 16);
-                const float2 fx = tbf[i], fy = tbf[kVolAx + j], fz = tbf[2 * kVolAx + kz[t]];
-                df_add2(W[0], v[t][0].x, v[t][0].y);
-                df_add2(W[1], v[t][1].x, v[t][1].y);
-                df_add2(W[2], v[t][2].x, v[t][2].y);
-                df_add_prod(Pm[0], fy.x, fy.y, v[t][2].x, v[t][2].y);
-                df_add_prod(Pm[1], fz.x, fz.y, v[t][1].x, v[t][1].y);
-                df_add_prod(Pm[2], fz.x, fz.y, v[t][0].x, v[t][0].y);
-                df_add_prod(Pm[3], fx.x, fx.y, v[t][2].x, v[t][2].y);
-                df_add_prod(Pm[4], fx.x, fx.y, v[t][1].x, v[t][1].y);
-                df_add_prod(Pm[5], fy.x, fy.y, v[t][0].x, v[t][0].y);
-                ++nint_cells;
-            }
-        }
-        // boundary cells: the kept alpha (entries of cells with alpha = 0 are marked)
+        const int NB = p_cut[dims[2]];
         const int j0 = (int)((long long)NB * split / nsplit), j1 = (int)((long long)NB * (split + 1) / nsplit);
-        int kzb = j0 + (int)threadIdx.x < j1 ? find_row(p_bnd, dims[2], j0 + threadIdx.x) : 0;
-        for (int e0 = j0 + threadIdx.x; e0 < j1; e0 += kPlanUnroll * blockDim.x) {
+        // a thread's entries ascend, so its plane only moves forward
+        int kzb = j0 + (int)threadIdx.x < j1 ? find_row(p_cut, dims[2], j0 + threadIdx.x) : 0;
+        for (int e0 = j0 + threadIdx.x; e0 < j1; e0 += kPlanUnroll * kVolThreads) {
             int kz[kPlanUnroll];
             unsigned ent[kPlanUnroll];
             float2 al[kPlanUnroll];
 #pragma unroll
             for (int t = 0; t < kPlanUnroll; ++t) {
-                const int e = e0 + t * blockDim.x;
+                const int e = e0 + t * kVolThreads;
                 if (e < j1)
-                    while (p_bnd[kzb + 1] <= e) ++kzb;
+                    while (p_cut[kzb + 1] <= e) ++kzb;
                 kz[t] = kzb;
-                const long long at = base + b_bnd[kz[t]] + (e - p_bnd[kz[t]]);
+                const long long at = base + b_cut[kz[t]] + (e - p_cut[kz[t]]);
                 ent[t] = e < j1 ? pl.bent[at] : kPvfSkip;
                 al[t] = e < j1 ? pl.balpha[at] : make_float2(0.f, 0.f);
             }
@@ -820,102 +826,20 @@ __global__ void __launch_bounds__(kVolThreads, 2) k_volume_plan(CaseTab ct, int 
 #pragma unroll
             for (int t = 0; t < kPlanUnroll; ++t) {
                 if (ent[t] == kPvfSkip) continue;
-                const int i = (int)(ent[t] & 0xffffu), j = (int)(ent[t] >> 16);
-                const long long cc = plane_off[kz[t]] + row_off[j] + wrap_add(lo0w, i, g.n[0]);
+                const int i = (int)(ent[t] & 255u), j = (int)(ent[t] >> 8);
+                const long long cc = tb.plane_off[kz[t]] + tb.row_off[j] + wrap_add(lo0w, i, g.n[0]);
 #pragma unroll
                 for (int c = 0; c < 3; ++c) v[t][c] = field_pair(u[c * N + cc]);
             }
 #pragma unroll
             for (int t = 0; t < kPlanUnroll; ++t) {
                 if (ent[t] == kPvfSkip) continue;
-                const float2 a2 = al[t];
-                const int i = (int)(ent[t] & 0xffffu), j = (int)(ent[t] >> 16);
-                df_add2(V, a2.x, a2.y);
-                const float2 fx = tbf[i], fy = tbf[kVolAx + j], fz = tbf[2 * kVolAx + kz[t]];
-                float wh[3], wl[3];
-#pragma unroll
-                for (int q3 = 0; q3 < 3; ++q3) {
-                    wh[q3] = a2.x * v[t][q3].x;
-                    wl[q3] = fmaf(a2.x, v[t][q3].x, -wh[q3]) + a2.y * v[t][q3].x;
-                    if constexpr (sizeof(T) == 8) wl[q3] = fmaf(a2.x, v[t][q3].y, wl[q3]);
-                    df_add2(W[q3], wh[q3], wl[q3]);
-                }
-                df_add_prod(Pm[0], fy.x, fy.y, wh[2], wl[2]);
-                df_add_prod(Pm[1], fz.x, fz.y, wh[1], wl[1]);
-                df_add_prod(Pm[2], fz.x, fz.y, wh[0], wl[0]);
-                df_add_prod(Pm[3], fx.x, fx.y, wh[2], wl[2]);
-                df_add_prod(Pm[4], fx.x, fx.y, wh[1], wl[1]);
-                df_add_prod(Pm[5], fy.x, fy.y, wh[0], wl[0]);
+                const int i = (int)(ent[t] & 255u), j = (int)(ent[t] >> 8);
+                add_cut_cell<T>(sums, al[t], v[t], tb.tbf[0][i], tb.tbf[1][j], tb.tbf[2][kz[t]]);
             }
         }
     }
-    // warp sums (double-float; the interior count exactly), the CTA's eight
-    // warp sums in double-float too, one conversion to FP64 per quantity, and
-    // the particle's nsplit CTA sums in FP64, in order (FP64 issue is scarce
-    // on this part: no FP64 operation per warp)
-#pragma unroll
-    for (int q = 0; q < 3; ++q) df_warp_sum(W[q]);
-#pragma unroll
-    for (int q = 0; q < 6; ++q) df_warp_sum(Pm[q]);
-    df_warp_sum(V);
-    const unsigned ncell = __reduce_add_sync(0xffffffffu, (unsigned)nint_cells);
-    float2 *s_w = (float2 *)s_vol;  // [warps][10] double-float warp sums
-    __shared__ unsigned s_ncell[kVolThreads / 32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) {
-#pragma unroll
-        for (int q = 0; q < 3; ++q) s_w[wid * 10 + q] = make_float2(W[q].hi, W[q].lo);
-#pragma unroll
-        for (int q = 0; q < 6; ++q) s_w[wid * 10 + 3 + q] = make_float2(Pm[q].hi, Pm[q].lo);
-        s_w[wid * 10 + 9] = make_float2(V.hi, V.lo);
-        s_ncell[wid] = ncell;
-    }
-    __syncthreads();
-    __shared__ double s_q[10];
-    if (threadIdx.x < 10) {
-        const int k = threadIdx.x;
-        DF x = {0.f, 0.f};
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) x = df_sum(x, DF{s_w[w * 10 + k].x, s_w[w * 10 + k].y});
-        s_q[k] = df_to_double(make_float2(x.hi, x.lo));
-    }
-    __syncthreads();
-    if (threadIdx.x < 7) {
-        const int k = threadIdx.x;
-        double x;
-        if (k < 3) {
-            x = s_q[k];
-        } else if (k < 6) {
-            x = s_q[3 + 2 * (k - 3)] - s_q[4 + 2 * (k - 3)];  // (ry w2 - rz w1, rz w0 - rx w2, rx w1 - ry w0)
-        } else {
-            unsigned n = 0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) n += s_ncell[w];
-            x = (double)n + s_q[9];
-        }
-        const double h3 = g.h * g.h * g.h;
-        partial[((size_t)p * nsplit + split) * 7 + k] = x * h3;
-        __threadfence();  // release: partials before the count
-    }
-    __shared__ int s_last;
-    if (threadIdx.x == 0) {
-        __threadfence();
-        s_last = atomicAdd(done + p, 1u) == (unsigned int)nsplit - 1;
-        __threadfence();  // acquire: the count before the other partials
-    }
-    __syncthreads();
-    if (s_last && threadIdx.x < 7) {
-        // the particle's last CTA adds the CTA sums in CTA order
-        const int k = threadIdx.x;
-        double x = 0.0;
-        for (int sp = 0; sp < nsplit; ++sp) x += __ldcg(partial + ((size_t)p * nsplit + sp) * 7 + k);
-        if (k < 3) {
-            if (Iu) Iu[3 * p + k] = x;
-        } else if (k < 6) {
-            if (Irxu) Irxu[3 * p + k - 3] = x;
-        } else if (vol) {
-            vol[p] = x;
-        }
-        if (k == 0) done[p] = 0;  // ready for the next call
-    }
+    volume_finish_df(sums, g.h, p, split, nsplit, partial, done, Iu, Irxu, vol, fin);
 }
 
 // ---------------------------------------------------------------------------
@@ -1450,14 +1374,14 @@ static int run_volume_plan(ib_ctx *ctx, Arena &ar, const CaseTab &ct, const ib_p
 template <typename T>
 static int run_plan_sums(ib_ctx *ctx, Arena &ar, const CaseTab &ct, const ib_particles *pp, const PvfPlanDev &pl,
                          double *Iu, double *Irxu, double *vol, cudaStream_t s) {
-    const int nsplit = volume_split(ctx, (const void *)k_volume_plan<T>, kPlanSmem, pp->P);
+    const int nsplit = volume_split(ctx, (const void *)k_volume_plan<T>, 0, pp->P);
     double *partial = ar.take<double>((size_t)pp->P * nsplit * 7);
     unsigned int *done = ar.take<unsigned int>(pp->P);
     if (!ar.ok())
         return oom_error(ar.used, ar.cap);
     PhaseTimer tm(ctx, IB_PHASE_VOLUME, s);
     cudaMemsetAsync(done, 0, sizeof(unsigned int) * pp->P, s);
-    k_volume_plan<T><<<pp->P * nsplit, kVolThreads, kPlanSmem, s>>>(ct, pp->P, nsplit, pp->Xr, pp->radius, partial,
+    k_volume_plan<T><<<pp->P * nsplit, kVolThreads, 0, s>>>(ct, pp->P, nsplit, pp->Xr, pp->radius, partial,
                                                                     done, Iu, Irxu, vol, ctx->status, pl);
     return check_launch("particle_volume_integrals_plan");
 }
@@ -1490,26 +1414,25 @@ int ib_pvf_plan_create(ib_ctx *ctx, int P, int max_box_cells, ib_pvf_plan **plan
         return set_error(IB_ERR_INVALID, "bad plan size (P %d, max_box_cells %d)", P, max_box_cells);
     const size_t cap = (size_t)max_box_cells;
     auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
-    const size_t b_hdr = up(sizeof(int4) * (size_t)P * kVolAx), b_ient = up(sizeof(unsigned) * P * cap),
-                 b_bent = b_ient, b_alpha = up(sizeof(float2) * P * cap), b_pos = up(sizeof(double) * 4 * (size_t)P);
+    const size_t b_hdr = up(sizeof(int2) * (size_t)P * kVolAx), b_bent = up(sizeof(unsigned) * P * cap),
+                 b_alpha = up(sizeof(float2) * P * cap), b_pos = up(sizeof(double) * 4 * (size_t)P);
     ib_pvf_plan *pl = new (std::nothrow) ib_pvf_plan();
     if (!pl) return set_error(IB_ERR_OOM, "plan object");
     pl->device = ctx->device;
     pl->P = P;
     pl->cap = max_box_cells;
     pl->nsplit = 0;
-    if (cudaMalloc(&pl->mem, b_hdr + b_ient + b_bent + b_alpha + b_pos) != cudaSuccess) {
+    if (cudaMalloc(&pl->mem, b_hdr + b_bent + b_alpha + b_pos) != cudaSuccess) {
         cudaGetLastError();
         delete pl;
-        return set_error(IB_ERR_OOM, "plan of %zu bytes", b_hdr + b_ient + b_bent + b_alpha + b_pos);
+        return set_error(IB_ERR_OOM, "plan of %zu bytes", b_hdr + b_bent + b_alpha + b_pos);
     }
     char *m = (char *)pl->mem;
     pl->dev.cap = max_box_cells;
-    pl->dev.hdr = (int4 *)m;
-    pl->dev.ient = (unsigned *)(m + b_hdr);
-    pl->dev.bent = (unsigned *)(m + b_hdr + b_ient);
-    pl->dev.balpha = (float2 *)(m + b_hdr + b_ient + b_bent);
-    pl->dev.pos = (double *)(m + b_hdr + b_ient + b_bent + b_alpha);
+    pl->dev.hdr = (int2 *)m;
+    pl->dev.bent = (unsigned *)(m + b_hdr);
+    pl->dev.balpha = (float2 *)(m + b_hdr + b_bent);
+    pl->dev.pos = (double *)(m + b_hdr + b_bent + b_alpha);
     *plan = pl;
     return IB_OK;
 }

@@ -143,3 +143,30 @@ def test_cell_classes_and_box_sizes(api, split):
     for g, r in zip(part, out):
         assert torch.equal(g[0], r[5])
     ctx.close()
+
+
+# spheres: boxes of 40 cells (the widest tabulated) and 41 to 43, a box of more
+# than a warp's width with seams, one of a few cells, one below a cell
+@pytest.mark.parametrize("split", [0, 1, 32])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_sphere_box_sizes(api, prec, split):
+    N = 48
+    h = 1.0 / N
+    rng = synth.SplitMix64(33)
+    u = synth.fourier_field((N,) * 3, 4, rng, h)
+    if prec == 1:
+        u = u.astype(np.float32).astype(np.float64)
+    half = np.array([18.9, 19.6, 16.3, 3.0, 1.6, 0.3])
+    X = np.array([[24, 24, 24], [24, 23.5, 24.2], [0.1, 47.8, 30.3], [12, 12, 12], [40.2, 7.7, 9.1], [30.4, 5.6, 20.1]])
+    P = len(half)
+    z3 = torch.zeros((P, 3), device="cuda", dtype=torch.float64)
+    parts = dict(Xr=t64(X * h), Ur=z3, Wr=z3, radius=t64(half * h), rho_p=torch.ones(P, device="cuda", dtype=torch.float64),
+                 moff=torch.zeros(P + 1, device="cuda", dtype=torch.int32))
+    ctx = api.Context()
+    ctx.set_volume_split(split)
+    out = ctx.particle_volume_integrals(torch.tensor(u, device="cuda", dtype=api.field_dtype(prec)), h, parts)
+    ctx.status()
+    ref = oracle.volume_integrals((N,) * 3, h, (0, 0, 0), u, X * h, half * h)
+    for g, r in zip(out, ref):
+        assert nerr(g, r) <= 1e-12
+    ctx.close()
