@@ -154,15 +154,22 @@ def load(path: str = LIB_PATH):
 
 
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else None
+    # (the argument types turn the integer into a pointer)
+    return t.data_ptr() if t is not None else None
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    # the current stream's handle, without building a Stream object around it
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _need(t, name, dtype, shape=None):
+    # (the usual case in one pass: a call's checks cost as much as its launches)
+    if isinstance(t, torch.Tensor) and t.is_cuda and t.dtype == dtype and t.is_contiguous() and \
+            (shape is None or t.shape == shape):
+        return t
     if not isinstance(t, torch.Tensor):
         raise TypeError("%s must be a torch.Tensor" % name)
     if not t.is_cuda:

@@ -51,6 +51,23 @@ int validate_grid(const ib_grid *g, int need_prec) {
     return IB_OK;
 }
 
+int resident_ctas(ib_ctx *ctx, const void *kern, int threads, size_t smem) {
+    for (int i = 0; i < ctx->nprep; ++i)
+        if (ctx->prep_kern[i] == kern) return ctx->prep_ctas[i];
+    int n = 0;
+    if ((smem > 48 * 1024 &&
+         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, threads, smem) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    if (n > 0 && ctx->nprep < ib_ctx::kPrepared) {
+        ctx->prep_kern[ctx->nprep] = kern;
+        ctx->prep_ctas[ctx->nprep++] = n;
+    }
+    return n;
+}
+
 DevGrid make_dev_grid(const ib_grid *g) {
     DevGrid d;
     for (int a = 0; a < 3; ++a) {

@@ -246,7 +246,21 @@ struct ib_ctx {
     cudaEvent_t stage_ev[kStageSlots];
     int stage_next;
     gbib::FftTables *fft_tab;  // device: roots of unity of the fluid step's transforms
+    // kernels this context has prepared and their resident CTAs per SM (see
+    // gbib::resident_ctas)
+    static constexpr int kPrepared = 24;
+    const void *prep_kern[kPrepared];
+    int prep_ctas[kPrepared];
+    int nprep;
 };
+
+namespace gbib {
+// A kernel's resident CTAs per SM at one launch shape (a kernel is always asked
+// for with the same one), its dynamic shared memory limit raised to `smem` on the
+// way; 0 when it cannot be resident.  Both are asked of the driver once per
+// context and kernel: they took a quarter of a small call's host time.
+int resident_ctas(ib_ctx *ctx, const void *kern, int threads, size_t smem);
+}  // namespace gbib
 
 // A batch's case table uploaded once (ib_batch_table_create): device memory
 // owned by the table, so calls that take it stage nothing on the host.

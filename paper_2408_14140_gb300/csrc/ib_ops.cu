@@ -1941,7 +1941,7 @@ static int slots_build(ib_ctx *ctx, const CaseTab &ct, int M, int ndense, SlotGe
                (const int *)ncompact_dev, sg, (const uint32_t *)sl.dense_of, (const uint32_t *)sl.start, anchor, level, sl,
                wts, jagged ? 1 : 0, sc.big, (int *)sc.lb_ticket + 2);
     auto large = k_tile_lists_large<T, KW>;
-    cudaFuncSetAttribute(large, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CtaLists));
+    resident_ctas(ctx, (const void *)large, kPairThreads, sizeof(CtaLists));  // (its shared memory limit)
     launch_pdl(large, dim3(ctx->sm_count), dim3(kPairThreads), sizeof(CtaLists), s, ct, sg.mode, sg,
                (const uint32_t *)sl.dense_of, (const uint32_t *)sl.start, anchor, level, sl, wts, jagged ? 1 : 0,
                (const int *)sc.big,
@@ -2117,7 +2117,7 @@ static int run_mdf(ib_ctx *ctx, Arena &ar, const CaseTab &ct, const ib_particles
     if (order == IB_ORDER_SEQUENTIAL)
         launch_pdl(k_conflicts, dim3(grid_blocks(32 * P, 256, ctx->sm_count)), dim3(256), 0, fs, ct, P, KW,
                    (const double *)pp->Xr, (const double *)rho, nbr_cnt, nbr);
-    cudaFuncSetAttribute(k_levels, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLevSmem);
+    resident_ctas(ctx, (const void *)k_levels, kLevThreads, kLevSmem);  // (its shared memory limit)
     launch_pdl(k_levels, dim3(1), dim3(kLevThreads), kLevSmem, fs, ct, P, order, KW, (const double *)pp->Xr,
                (const double *)rho, (const int *)pp->marker_offset, (const int *)nbr_cnt, (const int *)nbr, lo,
                lev_work, lev_cur);
@@ -2238,8 +2238,7 @@ static int run_mdf(ib_ctx *ctx, Arena &ar, const CaseTab &ct, const ib_particles
                     cudaLaunchKernelEx(&cg, k_gather_level<T, KER>, a, L);
             }
     }
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mdf_passes<T, KER>, 256, 0);
+    const int per_sm = resident_ctas(ctx, (const void *)k_mdf_passes<T, KER>, 256, 0);
     if (per_sm < 1) return set_error(IB_ERR_CUDA, "mdf kernel cannot be resident");
     int nblocks = per_sm * ctx->sm_count;
     void *args[] = {&a};

@@ -1276,18 +1276,18 @@ __global__ void k_newton_euler(CollideArgs a, const double *__restrict__ Fc, Dev
 // CTAs per particle: the context's choice, or (0) as many as fill one resident
 // wave of `kern` for P particles, within [1, kVolMaxSplit].
 static int volume_split(ib_ctx *ctx, const void *kern, size_t smem, int P) {
-    if (ctx->vol_split > 0) return ctx->vol_split;
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kVolThreads, smem) != cudaSuccess || per_sm < 1)
-        per_sm = 1;
-    const long long n = (long long)per_sm * ctx->sm_count / (P > 0 ? P : 1);
+    if (ctx->vol_split > 0) {
+        resident_ctas(ctx, kern, kVolThreads, smem);  // (raises its shared memory limit)
+        return ctx->vol_split;
+    }
+    const int per_sm = resident_ctas(ctx, kern, kVolThreads, smem);
+    const long long n = (long long)(per_sm < 1 ? 1 : per_sm) * ctx->sm_count / (P > 0 ? P : 1);
     return (int)(n < 1 ? 1 : (n > kVolMaxSplit ? kVolMaxSplit : n));
 }
 
 template <typename T>
 static int run_volume(ib_ctx *ctx, Arena &ar, const CaseTab &ct, const ib_particles *pp, double *Iu,
                       double *Irxu, double *vol, cudaStream_t s) {
-    cudaFuncSetAttribute(k_volume<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVolSmem);
     const int nsplit = volume_split(ctx, (const void *)k_volume<T>, kVolSmem, pp->P);
     double *partial = ar.take<double>((size_t)pp->P * nsplit * 7);
     unsigned int *done = ar.take<unsigned int>(pp->P);
@@ -1359,7 +1359,6 @@ static int run_volume_static(const CaseTab &ct, const ib_particles *pp, double *
 template <typename T, int MODE>
 static int run_volume_plan(ib_ctx *ctx, Arena &ar, const CaseTab &ct, const ib_particles *pp, int nsplit,
                            const PvfPlanDev &pl, double *Iu, double *Irxu, double *vol, cudaStream_t s) {
-    cudaFuncSetAttribute(k_volume<T, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVolSmem);
     double *partial = ar.take<double>((size_t)pp->P * nsplit * 7);
     unsigned int *done = ar.take<unsigned int>(pp->P);
     if (!ar.ok())
@@ -1456,13 +1455,10 @@ int particle_volume_integrals_keep(ib_ctx *ctx, const ib_grid *grid, const void 
     const CaseTab ct = single_case(grid, (void *)u, nullptr, parts->P);
     Arena ar(ctx);
     int nsplit;
-    if (grid->prec == IB_F64) {
-        cudaFuncSetAttribute(k_volume<double, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVolSmem);
+    if (grid->prec == IB_F64)
         nsplit = volume_split(ctx, (const void *)k_volume<double, 1>, kVolSmem, parts->P);
-    } else {
-        cudaFuncSetAttribute(k_volume<float, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVolSmem);
+    else
         nsplit = volume_split(ctx, (const void *)k_volume<float, 1>, kVolSmem, parts->P);
-    }
     plan->nsplit = nsplit;
     plan->grid = *grid;
     if (grid->prec == IB_F64)
@@ -1549,7 +1545,6 @@ int particle_volume_integrals_ellipsoid(ib_ctx *ctx, const ib_grid *grid, const 
     const CaseTab ct = single_case(grid, (void *)u, nullptr, P);
     Arena ar(ctx);
     const void *ek = grid->prec == IB_F64 ? (const void *)k_volume_ellipsoid<double> : (const void *)k_volume_ellipsoid<float>;
-    cudaFuncSetAttribute(ek, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEllSmem);
     const int nsplit = volume_split(ctx, ek, kEllSmem, P);
     double *partial = ar.take<double>((size_t)P * nsplit * 7);
     unsigned int *done = ar.take<unsigned int>(P);
@@ -1558,11 +1553,9 @@ int particle_volume_integrals_ellipsoid(ib_ctx *ctx, const ib_grid *grid, const 
     PhaseTimer tm(ctx, IB_PHASE_VOLUME, s);
     cudaMemsetAsync(done, 0, sizeof(unsigned int) * P, s);
     if (grid->prec == IB_F64) {
-        cudaFuncSetAttribute(k_volume_ellipsoid<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEllSmem);
         k_volume_ellipsoid<double><<<P * nsplit, kVolThreads, kEllSmem, s>>>(ct, P, nsplit, Xr, axes, partial, done,
                                                                              Iu, Irxu, vol, ctx->status);
     } else {
-        cudaFuncSetAttribute(k_volume_ellipsoid<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEllSmem);
         k_volume_ellipsoid<float><<<P * nsplit, kVolThreads, kEllSmem, s>>>(ct, P, nsplit, Xr, axes, partial, done,
                                                                             Iu, Irxu, vol, ctx->status);
     }
