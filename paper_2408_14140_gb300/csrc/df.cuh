@@ -49,6 +49,44 @@ __device__ __forceinline__ float2 df_split(double x) {
     return make_float2(__uint_as_float(hi), 0.0f);
 }
 
+// (float)x, and that with the rest (float)(x - (float)x): round to nearest, the
+// bits the conversions give, on the integer pipe (a double's conversions run at
+// the FP64 rate; the conversions serve what is outside FP32's normal range,
+// out of line, where the compiler cannot run them for every value).
+static __device__ __noinline__ float df_round_rare(double x) { return (float)x; }
+static __device__ __noinline__ float2 df_round_pair_rare(double x) {
+    const float h = (float)x;
+    return make_float2(h, (float)(x - (double)h));
+}
+// the magnitude's top 24 bits rounded to nearest (even), exponent rebiased to
+// FP32's; mag and l32 the double's words, its sign cleared
+__device__ __forceinline__ unsigned df_round_bits(unsigned mag, unsigned l32, unsigned &up) {
+    const unsigned t = __funnelshift_l(l32, mag - (896u << 20), 3);
+    up = (l32 & 0x1fffffffu) + (t & 1u) > 0x10000000u ? 1u : 0u;
+    return t + up;
+}
+__device__ __forceinline__ float df_round(double x) {
+    const unsigned h32 = (unsigned)__double2hiint(x), l32 = (unsigned)__double2loint(x);
+    const unsigned mag = h32 & 0x7fffffffu, sgn = h32 & 0x80000000u;
+    if ((mag | l32) == 0) return __uint_as_float(sgn);
+    if (mag - (897u << 20) >= (253u << 20)) return df_round_rare(x);
+    unsigned up;
+    return __uint_as_float(df_round_bits(mag, l32, up) | sgn);
+}
+__device__ __forceinline__ float2 df_round_pair(double x) {
+    const unsigned h32 = (unsigned)__double2hiint(x), l32 = (unsigned)__double2loint(x);
+    const unsigned mag = h32 & 0x7fffffffu, sgn = h32 & 0x80000000u;
+    if ((mag | l32) == 0) return make_float2(__uint_as_float(sgn), 0.0f);
+    if (mag - (949u << 20) >= (201u << 20)) return df_round_pair_rare(x);
+    unsigned up;
+    const unsigned r = df_round_bits(mag, l32, up);
+    // what rounding left, in units of 2^(e - 1075), e the double's exponent
+    int rest = (int)(l32 & 0x1fffffffu) - (int)(up << 29);
+    rest = sgn ? -rest : rest;
+    const float scale = __uint_as_float(((mag >> 20) - 948u) << 23);
+    return make_float2(__uint_as_float(r | sgn), __fmul_rn(__int2float_rn(rest), scale));
+}
+
 // float -> double, exact, integer pipe only (float subnormals become 0).
 __device__ __forceinline__ double df_widen(float f) {
     const unsigned b = __float_as_uint(f);

@@ -94,6 +94,37 @@ template <int KER> struct Kernel;
 template <> struct Kernel<IB_DELTA_ROMA3> { static constexpr int W = 3; };
 template <> struct Kernel<IB_DELTA_PESKIN4> { static constexpr int W = 4; };
 
+// The first stencil cell along an axis: unwrapped (held within 2^30) and modulo n.
+struct FirstCell {
+    int cell, wrapped;
+};
+// floor(t), and the first cell floor(t) - 1.  Within 30 bits the floor is one
+// addition of 1.5 * 2^52 rounded down, whose low word is the integer, and one
+// subtraction, and the indices stay 32 bits wide: an FP64 rounding and a conversion
+// take the FP64 pipe, which bounds the marker preparation.
+static __device__ __noinline__ double floor_of_rare(double t, int n, FirstCell *f) {
+    const double b = floor(t);
+    const long long i = (long long)b - 1;
+    f->cell = (int)(i < -(1LL << 30) ? -(1LL << 30) : (i > (1LL << 30) ? (1LL << 30) : i));
+    f->wrapped = wrap_int(i, n);
+    return b;
+}
+__device__ __forceinline__ double floor_of(double t, int n, FirstCell &f) {
+    if (((unsigned)__double2hiint(t) & 0x7fffffffu) < (1023u + 30u) << 20) {
+        const double m = __dadd_rd(t, 6755399441055744.0);
+        const int i = __double2loint(m) - 1;
+        int v = i < 0 ? i + n : (i >= n ? i - n : i);
+        if ((unsigned)v >= (unsigned)n) v = ((i % n) + n) % n;  // more than a period away
+        f.cell = i;
+        f.wrapped = v;
+        return __dadd_rn(m, -6755399441055744.0);
+    }
+    FirstCell far;
+    const double b = floor_of_rare(t, n, &far);
+    f = far;
+    return b;
+}
+
 // One axis of the regularised delta kernel.  s is the position in units of
 // h measured from the first cell centre; returns the first stencil cell
 // (unwrapped) and the kernel weights of the W cells from there.  All
@@ -106,25 +137,26 @@ template <> struct Kernel<IB_DELTA_PESKIN4> { static constexpr int W = 4; };
 // s, the stencil cell and r are FP64 (r = s - b is exact); the weights are
 // FP32 for FP32 fields.
 template <int KER>
-__device__ __forceinline__ long long axis_weights(double s, float w[4]) {
+__device__ __forceinline__ FirstCell axis_weights(double s, int n, float w[4]) {
+    FirstCell f;
     if (KER == IB_DELTA_ROMA3) {
-        double b = floor(s + 0.5);
-        float r = (float)(s - b);
+        const double b = floor_of(s + 0.5, n, f);
+        const float r = df_round(s - b);
         float q = sqrtf(1.0f - 3.0f * r * r);
         w[0] = (2.0f - 3.0f * r - q) * (float)(1.0 / 6.0);
         w[1] = (1.0f + q) * (float)(1.0 / 3.0);
         w[2] = (2.0f + 3.0f * r - q) * (float)(1.0 / 6.0);
         w[3] = 0.0f;
-        return (long long)b - 1;
+        return f;
     } else {
-        double b = floor(s);
-        float r = (float)(s - b);
+        const double b = floor_of(s, n, f);
+        const float r = df_round(s - b);
         float q = sqrtf(1.0f + 4.0f * r - 4.0f * r * r);
         w[0] = (3.0f - 2.0f * r - q) * 0.125f;
         w[1] = (3.0f - 2.0f * r + q) * 0.125f;
         w[2] = (1.0f + 2.0f * r + q) * 0.125f;
         w[3] = (1.0f + 2.0f * r - q) * 0.125f;
-        return (long long)b - 1;
+        return f;
     }
 }
 
@@ -136,9 +168,10 @@ __device__ __forceinline__ long long axis_weights(double s, float w[4]) {
 // the factors 2 and 4 are exact).  Each weight is within a few 2^-47 of the
 // FP64 formula, which keeps only the first stencil cell's FP64 arithmetic.
 template <int KER>
-__device__ __forceinline__ long long axis_weights(double s, float2 w[4]) {
+__device__ __forceinline__ FirstCell axis_weights(double s, int n, float2 w[4]) {
+    FirstCell f;
     if (KER == IB_DELTA_ROMA3) {
-        const double b = floor(s + 0.5);
+        const double b = floor_of(s + 0.5, n, f);
         const float2 r = df_split(s - b);
         const float2 r3 = df_mul(r, make_float2(3.0f, 0.0f));
         const float2 q = df_sqrt(df_add(make_float2(1.0f, 0.0f), df_neg(df_mul(r3, r))));
@@ -149,9 +182,9 @@ __device__ __forceinline__ long long axis_weights(double s, float2 w[4]) {
         w[1] = df_mul(df_add(make_float2(1.0f, 0.0f), q), c3);
         w[2] = df_mul(df_add(df_add(make_float2(2.0f, 0.0f), r3), df_neg(q)), c6);
         w[3] = make_float2(0.0f, 0.0f);
-        return (long long)b - 1;
+        return f;
     } else {
-        const double b = floor(s);
+        const double b = floor_of(s, n, f);
         const float2 r = df_split(s - b);
         const float2 r2 = df_scale(r, 2.0f);
         // 1 + 4r - 4r^2 = 1 + 2 (2r) - (2r)^2
@@ -161,7 +194,7 @@ __device__ __forceinline__ long long axis_weights(double s, float2 w[4]) {
         w[1] = df_scale(df_add(a, q), 0.125f);
         w[2] = df_scale(df_add(c, q), 0.125f);
         w[3] = df_scale(df_add(c, df_neg(q)), 0.125f);
-        return (long long)b - 1;
+        return f;
     }
 }
 

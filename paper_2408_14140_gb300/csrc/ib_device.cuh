@@ -74,7 +74,7 @@ struct MarkerState {
     uint64_t *anchor;  // [M] wrapped first stencil cell
     PS<T> *wts;        // [M][12] per-axis weights (x 0..3, y 4..7, z 8..11)
     PS<T> *A;          // [M][4] spread source of the current pass
-    double *Ud;        // [M][3] desired velocity
+    double *Ud;        // FP64 fields only: [M][3] desired velocity
     // FP32 fields only: [M][8] the desired velocity as float pairs, hi
     // (0..2) + lo (4..6), and dV / h^3 (3)
     float *Ud32;

@@ -31,15 +31,28 @@ namespace gbib {
 // form (FP32, or double-float pairs for FP64 fields).
 template <typename T, int KER>
 __device__ __forceinline__ uint64_t marker_weights(const DevGrid &g, const double X[3],
-                                                   PS<T> w[12], long long first[3]) {
+                                                   PS<T> w[12], int first[3]) {
     int a[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        double s = (X[d] - g.org[d]) * g.inv_h - 0.5;
-        first[d] = axis_weights<KER>(s, w + 4 * d);
-        a[d] = wrap_int(first[d], g.n[d]);
+        const double s = (X[d] - g.org[d]) * g.inv_h - 0.5;
+        const FirstCell f = axis_weights<KER>(s, g.n[d], w + 4 * d);
+        first[d] = f.cell;
+        a[d] = f.wrapped;
     }
     return pack_anchor(a[0], a[1], a[2]);
+}
+
+// A marker's weights to the workspace, 16 bytes a store.
+__device__ __forceinline__ void store_weights(float *dst, const float w[12]) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+        ((float4 *)dst)[k] = make_float4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]);
+}
+__device__ __forceinline__ void store_weights(float2 *dst, const float2 w[12]) {
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+        ((float4 *)dst)[k] = make_float4(w[2 * k].x, w[2 * k].y, w[2 * k + 1].x, w[2 * k + 1].y);
 }
 
 // ---------------------------------------------------------------------------
@@ -59,7 +72,7 @@ __global__ void __launch_bounds__(256) k_interpolate(DevGrid g, const T *__restr
             continue;
         }
         PS<T> ws[12];
-        long long first[3];
+        int first[3];
         uint64_t anc = marker_weights<T, KER>(g, x, ws, first);
         T o[3];
         interp_marker<T, KW>(u, g, N, anc, ws, o);
@@ -91,10 +104,9 @@ __global__ void k_prep_spread(DevGrid g, int M, const double *__restrict__ X,
             dv = 0.0;
         }
         PS<T> w[12];
-        long long first[3];
+        int first[3];
         ms.anchor[l] = marker_weights<T, KER>(g, x, w, first);
-#pragma unroll
-        for (int k = 0; k < 12; ++k) ms.wts[12 * l + k] = w[k];
+        store_weights(ms.wts + 12 * (size_t)l, w);
         double q = dv * g.inv_h3;
         ms.A[4 * l + 0] = to_store((T)(f[0] * q));
         ms.A[4 * l + 1] = to_store((T)(f[1] * q));
@@ -147,8 +159,14 @@ __global__ void __launch_bounds__(kRadiusThreads) k_marker_radius(int P, const d
 // cross-CTA reductions: per particle the stencil box bounds (lo starts at a
 // huge value, hi at a very negative one: memset 0x7f / 0x80 bytes) and a
 // completion count (0).
+//
+// Bound by the FP64 pipe: FP64 is kept for the position, the first stencil cell
+// and the desired velocity; roundings to FP32 run on the integer pipe, a warp
+// reduces its box bounds before the atomics, and the weights leave in 16-byte
+// stores.  512 spheres of 800 markers, FP32 fields: 76 -> 51 us (20 us for 64
+// spheres of 1800 in FP64, as before: few warps, bound by their latency).
 struct PrepScratch {
-    long long *lo, *hi;          // [P][3]
+    int *lo, *hi;                // [P][3], from the particle's centre cell
     unsigned int *done;          // [P]
 };
 constexpr int kPrepSplit = 4;    // CTAs per particle
@@ -161,14 +179,14 @@ __global__ void __launch_bounds__(256) k_prep_particles(
     int4 *__restrict__ box_lo, int4 *__restrict__ box_dim,
     int *__restrict__ part_of, PrepScratch ps, DevStatus *st) {
     constexpr int KW = Kernel<KER>::W;
-    __shared__ long long s_lo[3], s_hi[3];
+    __shared__ int s_lo[3], s_hi[3];
     __shared__ int s_last;
     const int p = blockIdx.x / kPrepSplit, part = blockIdx.x % kPrepSplit;
     if (p >= P) return;
     const DevGrid g = ct.of_particle(p).g;
     if (threadIdx.x < 3) {
-        s_lo[threadIdx.x] = LLONG_MAX;
-        s_hi[threadIdx.x] = LLONG_MIN;
+        s_lo[threadIdx.x] = INT_MAX;
+        s_hi[threadIdx.x] = INT_MIN;
     }
     __syncthreads();
     double xc[3] = {Xr[3 * p], Xr[3 * p + 1], Xr[3 * p + 2]};
@@ -179,7 +197,15 @@ __global__ void __launch_bounds__(256) k_prep_particles(
     const int m0 = moff[p], m1 = moff[p + 1];
     const int nm = m1 - m0;
     const int l0 = m0 + (int)((long long)part * nm / kPrepSplit), l1 = m0 + (int)((long long)(part + 1) * nm / kPrepSplit);
-    long long lo[3] = {LLONG_MAX, LLONG_MAX, LLONG_MAX}, hi[3] = {LLONG_MIN, LLONG_MIN, LLONG_MIN};
+    // the box bounds are counted from about the particle's centre cell (the same
+    // in all its CTAs), so that they fit 32 bits; a marker further off saturates
+    // (its box is too wide either way)
+    constexpr int kFar = 1 << 28;
+    int cell[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+        cell[d] = pok ? max(-kFar, min(kFar, __float2int_rd((df_round(xc[d]) - df_round(g.org[d])) * df_round(g.inv_h)))) : 0;
+    int lo[3] = {INT_MAX, INT_MAX, INT_MAX}, hi[3] = {INT_MIN, INT_MIN, INT_MIN};
     for (int l = l0 + threadIdx.x; l < l1; l += blockDim.x) {
         double r[3] = {R[3 * l], R[3 * l + 1], R[3 * l + 2]};
         double dv = dV[l];
@@ -190,35 +216,36 @@ __global__ void __launch_bounds__(256) k_prep_particles(
         double x[3] = {xc[0] + r[0], xc[1] + r[1], xc[2] + r[2]};
         if (!pok) x[0] = g.org[0], x[1] = g.org[1], x[2] = g.org[2];
         PS<T> w[12];
-        long long first[3];
+        int first[3];
         ms.anchor[l] = marker_weights<T, KER>(g, x, w, first);
-#pragma unroll
-        for (int k = 0; k < 12; ++k) ms.wts[12 * l + k] = w[k];
+        store_weights(ms.wts + 12 * (size_t)l, w);
         const double ud[3] = {uc[0] + (wc[1] * r[2] - wc[2] * r[1]), uc[1] + (wc[2] * r[0] - wc[0] * r[2]),
                               uc[2] + (wc[0] * r[1] - wc[1] * r[0])};
+        if constexpr (sizeof(T) == 4) {
+            const float2 a = df_round_pair(ud[0]), b = df_round_pair(ud[1]), c = df_round_pair(ud[2]);
+            ((float4 *)(ms.Ud32 + 8 * (size_t)l))[0] = make_float4(a.x, b.x, c.x, df_round(dv * g.inv_h3));
+            ((float4 *)(ms.Ud32 + 8 * (size_t)l))[1] = make_float4(a.y, b.y, c.y, 0.f);
+        } else {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) ms.Ud[3 * l + c] = ud[c];
-        if (sizeof(T) == 4) {
-            float4 h, o;
-            h.x = (float)ud[0], h.y = (float)ud[1], h.z = (float)ud[2];
-            h.w = (float)(dv * g.inv_h3);
-            o.x = (float)(ud[0] - (double)h.x), o.y = (float)(ud[1] - (double)h.y);
-            o.z = (float)(ud[2] - (double)h.z), o.w = 0.f;
-            ((float4 *)(ms.Ud32 + 8 * (size_t)l))[0] = h;
-            ((float4 *)(ms.Ud32 + 8 * (size_t)l))[1] = o;
+            for (int c = 0; c < 3; ++c) ms.Ud[3 * l + c] = ud[c];
         }
         F[3 * l] = F[3 * l + 1] = F[3 * l + 2] = 0.0;
         part_of[l] = p;
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-            lo[d] = min(lo[d], first[d]);
-            hi[d] = max(hi[d], first[d] + KW - 1);
+            const int off = max(-kFar, min(kFar, first[d] - cell[d]));
+            lo[d] = min(lo[d], off);
+            hi[d] = max(hi[d], off + KW - 1);
         }
     }
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        atomicMin(&s_lo[d], lo[d]);
-        atomicMax(&s_hi[d], hi[d]);
+        lo[d] = __reduce_min_sync(0xffffffffu, lo[d]);
+        hi[d] = __reduce_max_sync(0xffffffffu, hi[d]);
+        if ((threadIdx.x & 31) == 0) {
+            atomicMin(&s_lo[d], lo[d]);
+            atomicMax(&s_hi[d], hi[d]);
+        }
     }
     __syncthreads();
     // combine the particle's CTAs; the last one to finish writes the results
@@ -233,14 +260,13 @@ __global__ void __launch_bounds__(256) k_prep_particles(
     }
     __syncthreads();
     if (threadIdx.x == 0 && s_last) {
-        long long blo[3], bhi[3];
+        int blo[3], dims[3];
         for (int d = 0; d < 3; ++d) {
-            blo[d] = atomicAdd((unsigned long long *)&ps.lo[3 * p + d], 0ull);
-            bhi[d] = atomicAdd((unsigned long long *)&ps.hi[3 * p + d], 0ull);
+            const int l = atomicAdd(&ps.lo[3 * p + d], 0), h = atomicAdd(&ps.hi[3 * p + d], 0);
+            blo[d] = cell[d] + l;
+            dims[d] = h - l + 1;
         }
         if (m1 > m0) {
-            int dims[3];
-            for (int d = 0; d < 3; ++d) dims[d] = (int)(bhi[d] - blo[d] + 1);
             box_lo[p] = make_int4(wrap_int(blo[0], g.n[0]), wrap_int(blo[1], g.n[1]), wrap_int(blo[2], g.n[2]), 0);
             box_dim[p] = make_int4(dims[0], dims[1], dims[2], 0);
             for (int d = 0; d < 3; ++d)
@@ -1384,7 +1410,7 @@ __global__ void __launch_bounds__(256) k_spread_atomic(DevGrid g, int M, const d
         }
         if (!valid) x[0] = g.org[0], x[1] = g.org[1], x[2] = g.org[2];
         PS<T> ws[12], A[3];
-        long long first[3];
+        int first[3];
         const uint64_t anc = marker_weights<T, KER>(g, x, ws, first);
         const double q = dv * g.inv_h3;
 #pragma unroll
@@ -1848,7 +1874,7 @@ static bool take_markers(Arena &ar, int M, MarkerState<T> &ms) {
     ms.anchor = ar.take<uint64_t>(M > 0 ? M : 1);
     ms.wts = ar.take<PS<T>>((size_t)12 * (M > 0 ? M : 1));
     ms.A = ar.take<PS<T>>((size_t)4 * (M > 0 ? M : 1));
-    ms.Ud = ar.take<double>((size_t)3 * (M > 0 ? M : 1));
+    ms.Ud = sizeof(T) == 8 ? ar.take<double>((size_t)3 * (M > 0 ? M : 1)) : nullptr;
     ms.Ud32 = sizeof(T) == 4 ? ar.take<float>((size_t)8 * (M > 0 ? M : 1)) : nullptr;
     return ar.ok();
 }
@@ -2008,8 +2034,8 @@ static int run_mdf(ib_ctx *ctx, Arena &ar, const CaseTab &ct, const ib_particles
     int4 *box_dim = ar.take<int4>(P);
     int *part_of = ar.take<int>(M > 0 ? M : 1);
     PrepScratch prep_ps;
-    prep_ps.lo = ar.take<long long>((size_t)3 * P);
-    prep_ps.hi = ar.take<long long>((size_t)3 * P);
+    prep_ps.lo = ar.take<int>((size_t)3 * P);
+    prep_ps.hi = ar.take<int>((size_t)3 * P);
     prep_ps.done = ar.take<unsigned int>(P);
     LevelOut lo;
     lo.level = ar.take<int>(P);
@@ -2125,8 +2151,8 @@ static int run_mdf(ib_ctx *ctx, Arena &ar, const CaseTab &ct, const ib_particles
                (const int *)pp->marker_offset, (const int *)lo.mbase, mperm);
     cudaEventRecord(ctx->fork_ev[3], fs);
     cudaMemsetAsync(bar.count, 0, 2 * sizeof(unsigned int), s);
-    cudaMemsetAsync(prep_ps.lo, 0x7f, sizeof(long long) * 3 * P, s);
-    cudaMemsetAsync(prep_ps.hi, 0x80, sizeof(long long) * 3 * P, s);
+    cudaMemsetAsync(prep_ps.lo, 0x7f, sizeof(int) * 3 * P, s);
+    cudaMemsetAsync(prep_ps.hi, 0x80, sizeof(int) * 3 * P, s);
     cudaMemsetAsync(prep_ps.done, 0, sizeof(unsigned int) * P, s);
     k_prep_particles<T, KER><<<P * kPrepSplit, 256, 0, s>>>(ct, P, pp->Xr, pp->Ur, pp->Wr, pp->marker_offset, mk->R,
                                                  mk->dV, ms, F_out, box_lo, box_dim, part_of, prep_ps,
