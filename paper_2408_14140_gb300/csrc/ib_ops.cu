@@ -1001,6 +1001,7 @@ __device__ __forceinline__ void slot_bins(int nc, int cs, const Slots &sl, int l
 // them each list is contiguous and a pair is candidate | offset << 16.
 constexpr int kListThreads = 128;
 constexpr int kListCtas = 10;              // CTAs of an SM
+constexpr int kSpreadCtas = 6;             // of the summing form (5 and 8: 90 and 99 us)
 constexpr int kListCand = 512;
 constexpr int kPairThreads = 256;          // the large tiles' CTAs
 constexpr int kPairWords = kMaxCand / 32;  // words of a bit set
@@ -1049,13 +1050,37 @@ __device__ __forceinline__ unsigned cover_word(int3 r, const int dim[3], int lan
     return mine;
 }
 
+// a marker's spread source
+__device__ __forceinline__ void load_source(const float *A, uint32_t m, float a[3]) {
+    const float4 v = ((const float4 *)A)[m];
+    a[0] = v.x, a[1] = v.y, a[2] = v.z;
+}
+__device__ __forceinline__ void load_source(const float2 *A, uint32_t m, float2 a[3]) {
+    const float4 v = ((const float4 *)A)[2 * (size_t)m];
+    a[0] = make_float2(v.x, v.y), a[1] = make_float2(v.z, v.w);
+    a[2] = A[4 * (size_t)m + 2];
+}
+
+// Standalone spreading sums a tile's cells where the lists would be written: its
+// lists are read once, so writing and reading them cost more than the sums (64
+// spheres of 1800 markers, FP64: lists and gather 63 + 53 us, 84 us together).
+template <typename T>
+struct SpreadSum {
+    const PS<T> *A;  // [M][4] sources
+    T *f;            // null: write the lists
+    DevGrid g;
+    int lo[3];
+};
+
 // A tile's lists from its bit sets of nw words (set(i, w): columns, rows, planes
 // for i from 0, 8, 16), by a CTA of NT threads.  The caller has zeroed ls.hist
 // and ls.len before a barrier.
-template <typename T, int NT, class Set, class First, class Mark>
+// With SUM every cell's sum is added to the field instead (a lane a cell, the
+// pairs in the same order).
+template <typename T, int NT, bool SUM, class Set, class First, class Mark>
 __device__ __forceinline__ void build_lists(const Slots &sl, int cs, uint32_t pb, int room, int nc, int nw, bool jagged,
                                             const PS<T> *__restrict__ wts, ListShared &ls, Set set, First first,
-                                            Mark mark) {
+                                            Mark mark, const SpreadSum<T> &sp) {
     constexpr int C = kTileCells / NT;  // cells a thread, neighbours along x
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int t[C], r[C];
@@ -1110,6 +1135,58 @@ __device__ __forceinline__ void build_lists(const Slots &sl, int cs, uint32_t pb
         if (lane == 0) ls.sum[s] = sum, ls.len[s] = (unsigned char)min(len, 255);
     }
     __syncthreads();
+    if constexpr (SUM) {
+        const DevGrid &g = sp.g;
+        const long long N = (long long)g.n[0] * g.n[1] * g.n[2];
+        for (int s = warp; s < ns; s += NT / 32) {
+            const int q = 32 * s + lane;
+            const int c = q < nb ? ls.cell[q] : 0, n = q < nb ? ls.cnt[q] : 0;
+            const int x = c & 7, y = (c >> 3) & 7, z = c >> 6, code = x + 4 * y + 16 * z;
+            T *const f = sp.f +
+                         ((long long)wrap_add(sp.lo[2], z, g.n[2]) * g.n[1] + wrap_add(sp.lo[1], y, g.n[1])) * g.n[0] +
+                         wrap_add(sp.lo[0], x, g.n[0]);
+            T v[3] = {T(0), T(0), T(0)};
+            if (n > 0) v[0] = f[0], v[1] = f[N], v[2] = f[2 * N];
+            const int rows = __reduce_max_sync(0xffffffffu, n);
+            SumAcc<T> acc[3];
+            int w = -1;
+            unsigned m = 0;
+            constexpr int kU = 4;  // rows whose loads are in flight together
+            for (int k0 = 0; k0 < rows; k0 += kU) {
+                PS<T> wx[kU], wy[kU], wz[kU], a[kU][3];
+#pragma unroll
+                for (int u = 0; u < kU; ++u)
+                    if (k0 + u < n) {
+                        while (!m) {
+                            ++w;
+                            m = set(x, w) & set(kTile + y, w) & set(2 * kTile + z, w);
+                        }
+                        const int i = 32 * w + __ffs((int)m) - 1, oc = code - first(i);
+                        m &= m - 1;
+                        const uint32_t mk = mark(i);
+                        const PS<T> *wm = wts + 12 * (size_t)mk;
+                        wx[u] = wm[oc & 3];
+                        wy[u] = wm[4 + ((oc >> 2) & 3)];
+                        wz[u] = wm[8 + (oc >> 4)];
+                        load_source(sp.A, mk, a[u]);
+                    }
+#pragma unroll
+                for (int u = 0; u < kU; ++u)
+                    if (k0 + u < n) {
+                        const PS<T> wt = pair_weight3(wx[u], wy[u], wz[u]);
+                        acc[0].add(wt, a[u][0]);
+                        acc[1].add(wt, a[u][1]);
+                        acc[2].add(wt, a[u][2]);
+                    }
+            }
+            if (n > 0) {
+                f[0] = v[0] + acc[0].value();
+                f[N] = v[1] + acc[1].value();
+                f[2 * N] = v[2] + acc[2].value();
+            }
+        }
+        return;
+    }
     uint32_t *const pairs = sl.pairs + pb;
     PS<T> *const pw = (PS<T> *)sl.pw + pb;
     int2 *const band = sl.band + pb;
@@ -1177,12 +1254,12 @@ __device__ __forceinline__ void build_lists(const Slots &sl, int cs, uint32_t pb
     }
 }
 
-template <typename T, int KW>
-__global__ void __launch_bounds__(kListThreads, kListCtas) k_tile_lists(
+template <typename T, int KW, bool SUM>
+__global__ void __launch_bounds__(kListThreads, SUM ? kSpreadCtas : kListCtas) k_tile_lists(
     CaseTab ct, int mode, int ncompact_cap, const int *__restrict__ ncompact_p, SlotGeom sg,
     const uint32_t *__restrict__ dense_of, const uint32_t *__restrict__ start, const uint64_t *__restrict__ anchor,
     const int *__restrict__ level, Slots sl, const PS<T> *__restrict__ wts, int jagged, int *__restrict__ big,
-    int *__restrict__ nbig) {
+    int *__restrict__ nbig, SpreadSum<T> sp) {
     constexpr int kSetPitch = kListCand / 32 + 1;  // odd: no bank conflicts
     __shared__ __align__(16) unsigned long long s_keys[kListCand];  // or 32-bit keys
     __shared__ uint32_t s_mark[kListCand];
@@ -1203,8 +1280,8 @@ __global__ void __launch_bounds__(kListThreads, kListCtas) k_tile_lists(
             if (tid == 0) big[atomicAdd(nbig, 1)] = cs;
             continue;
         }
-        const uint32_t pb = sl.poff[b];
-        const int room = (int)(sl.poff[b + nc] - pb);  // the tile's share of the pair arrays
+        const uint32_t pb = SUM ? 0u : sl.poff[b];
+        const int room = SUM ? 0 : (int)(sl.poff[b + nc] - pb);  // the tile's share of the pair arrays
         int lo[3], dim[3], lev;
         const int cse = slot_geometry(ct, mode, sg, sl, level, d, b, lo, dim, lev);
         const DevGrid &g = ct.get(cse).g;
@@ -1268,7 +1345,8 @@ __global__ void __launch_bounds__(kListThreads, kListCtas) k_tile_lists(
             if (tid + e * kListThreads < nc) {
                 const int3 q = bin_anchor(bin[e]);
                 const int r = rank[e];
-                sl.cand[b + r] = s_mark[r] = m[e];
+                s_mark[r] = m[e];
+                if (!SUM) sl.cand[b + r] = m[e];
                 s_rel[r] = (uint16_t)(q.x | (q.y << 4) | (q.z << 8));
                 s_first[r] = (short)((q.x - 3) + 4 * (q.y - 3) + 16 * (q.z - 3));
             }
@@ -1287,10 +1365,11 @@ __global__ void __launch_bounds__(kListThreads, kListCtas) k_tile_lists(
         s_ls.hist[tid] = 0;
         if (tid < kSlices) s_ls.len[tid] = 0;
         __syncthreads();
-        build_lists<T, kListThreads>(sl, cs, pb, room, nc, nw, jagged != 0, wts, s_ls,
-                                     [&](int i, int w) { return s_set[i][w]; }, [&](int i) { return s_first[i]; },
-                                     [&](int i) { return s_mark[i]; });
-        if (tid == 0) {
+        if (SUM) sp.lo[0] = lo[0], sp.lo[1] = lo[1], sp.lo[2] = lo[2], sp.g = g;
+        build_lists<T, kListThreads, SUM>(sl, cs, pb, room, nc, nw, jagged != 0, wts, s_ls,
+                                          [&](int i, int w) { return s_set[i][w]; }, [&](int i) { return s_first[i]; },
+                                          [&](int i) { return s_mark[i]; }, sp);
+        if (!SUM && tid == 0) {
             sl.geo_lo[cs] = make_int4(lo[0], lo[1], lo[2], lev);
             sl.geo_dim[cs] = make_int4(dim[0], dim[1], dim[2], (int)b);
             sl.geo_case[cs] = cse;
@@ -1300,11 +1379,11 @@ __global__ void __launch_bounds__(kListThreads, kListCtas) k_tile_lists(
 }
 
 // The tiles of more than kListCand candidates, one CTA each.
-template <typename T, int KW>
+template <typename T, int KW, bool SUM>
 __global__ void __launch_bounds__(kPairThreads) k_tile_lists_large(
     CaseTab ct, int mode, SlotGeom sg, const uint32_t *__restrict__ dense_of, const uint32_t *__restrict__ start,
     const uint64_t *__restrict__ anchor, const int *__restrict__ level, Slots sl, const PS<T> *__restrict__ wts,
-    int jagged, const int *__restrict__ big, const int *__restrict__ nbig_p, DevStatus *st) {
+    int jagged, const int *__restrict__ big, const int *__restrict__ nbig_p, DevStatus *st, SpreadSum<T> sp) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     grid_dep_wait();
     const int nbig = *nbig_p, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1318,8 +1397,8 @@ __global__ void __launch_bounds__(kPairThreads) k_tile_lists_large(
             int lo[3], dim[3], lev;
             const int cse = slot_geometry(ct, mode, sg, sl, level, d, b, lo, dim, lev);
             const DevGrid &g = ct.get(cse).g;
-            const uint32_t pb = sl.poff[b];
-            int room = (int)(sl.poff[b + nc] - pb);
+            const uint32_t pb = SUM ? 0u : sl.poff[b];
+            int room = SUM ? 0 : (int)(sl.poff[b + nc] - pb);
             if (nc > kMaxCand) {
                 // report, and leave an empty tile (no bins, no cells)
                 if (tid == 0) raise_status(st, IB_ERR_UNSUPPORTED, nc);
@@ -1353,7 +1432,7 @@ __global__ void __launch_bounds__(kPairThreads) k_tile_lists_large(
                 int3 r = make_int3(15, 15, 15);
                 if (i < nc) {
                     r = bin_anchor((int)(sh.keys[i] >> 32));
-                    sl.cand[b + i] = (uint32_t)(sh.keys[i] & 0xffffffffu);
+                    if (!SUM) sl.cand[b + i] = (uint32_t)(sh.keys[i] & 0xffffffffu);
                     sh.first[i] = (short)((r.x - 3) + 4 * (r.y - 3) + 16 * (r.z - 3));
                 }
                 const unsigned mine = cover_word<KW>(r, dim, lane);
@@ -1362,10 +1441,12 @@ __global__ void __launch_bounds__(kPairThreads) k_tile_lists_large(
             if (tid < kLenBins) sh.ls.hist[tid] = 0;
             if (tid < kSlices) sh.ls.len[tid] = 0;
             __syncthreads();
-            build_lists<T, kPairThreads>(sl, cs, pb, room, nc, nw, jagged != 0, wts, sh.ls,
-                                         [&](int i, int w) { return sh.set[i][w]; }, [&](int i) { return sh.first[i]; },
-                                         [&](int i) { return (uint32_t)(sh.keys[i] & 0xffffffffu); });
-            if (tid == 0) {
+            if (SUM) sp.lo[0] = lo[0], sp.lo[1] = lo[1], sp.lo[2] = lo[2], sp.g = g;
+            build_lists<T, kPairThreads, SUM>(sl, cs, pb, room, nc, nw, jagged != 0, wts, sh.ls,
+                                              [&](int i, int w) { return sh.set[i][w]; },
+                                              [&](int i) { return sh.first[i]; },
+                                              [&](int i) { return (uint32_t)(sh.keys[i] & 0xffffffffu); }, sp);
+            if (!SUM && tid == 0) {
                 sl.geo_lo[cs] = make_int4(lo[0], lo[1], lo[2], lev);
                 sl.geo_dim[cs] = make_int4(dim[0], dim[1], dim[2], (int)b);
                 sl.geo_case[cs] = cse;
@@ -1652,16 +1733,6 @@ constexpr int kSliceThreads = 128;
 template <typename T> constexpr int kSliceCtas = sizeof(T) == 4 ? 8 : 6;  // CTAs of an SM
 constexpr int kSliceRows = 4;
 
-__device__ __forceinline__ void load_source(const float *A, uint32_t m, float a[3]) {
-    const float4 v = ((const float4 *)A)[m];
-    a[0] = v.x, a[1] = v.y, a[2] = v.z;
-}
-__device__ __forceinline__ void load_source(const float2 *A, uint32_t m, float2 a[3]) {
-    const float4 v = ((const float4 *)A)[2 * (size_t)m];
-    a[0] = make_float2(v.x, v.y), a[1] = make_float2(v.z, v.w);
-    a[2] = A[4 * (size_t)m + 2];
-}
-
 template <typename T, class Wait>
 __device__ __forceinline__ void gather_slice(const CaseTab &ct, int4 rec, const Slots &sl, const PS<T> *A, double inv_dt,
                                              Wait wait) {
@@ -1746,21 +1817,6 @@ __global__ void __launch_bounds__(kSliceThreads, kSliceCtas<T>) k_gather_level(P
         });
     }
     grid_dep_wait();  // every CTA waits before it exits
-}
-
-// Spreading (ib_spread) over the tiles' lists, a CTA per tile, its warps taking
-// the tile's slices: the case's u slot holds the field spread into, its f slot
-// is null.
-template <typename T, int KER>
-__global__ void __launch_bounds__(kSliceThreads, kSliceCtas<T>)
-k_spread_gather(CaseTab ct, const int *ncompact_p, Slots sl, const PS<T> *A) {
-    grid_dep_wait();
-    const int nc = *ncompact_p;
-    for (int cs = blockIdx.x; cs < nc; cs += gridDim.x) {
-        const int4 ti = sl.tinfo[cs];
-        for (int s = threadIdx.x >> 5; 32 * s < ti.z; s += kSliceThreads / 32)
-            gather_slice<T>(ct, make_int4(cs, s, ti.x, ti.z), sl, A, 0.0, [] {});
-    }
 }
 
 // The atomic form of a wavefront's spreading (ib_ctx_set_spread_mode):
@@ -1946,11 +2002,12 @@ static int slots_alloc(Arena &ar, int M, int ndense, int mode, Slots &sl, SlotSc
     return IB_OK;
 }
 
-// The kernel chain: count, scan, compact, fill, scan, sort, per-cell lists.
+// The kernel chain: count, scan, compact, fill, scan, sort, per-cell lists -- or,
+// given a field to spread into (sp.f), the cells' sums.
 template <typename T, int KW>
 static int slots_build(ib_ctx *ctx, const CaseTab &ct, int M, int ndense, SlotGeom sg, const uint64_t *anchor,
                        const PS<T> *wts, const int *level, Slots &sl, const SlotScratch &sc, int *&ncompact_dev,
-                       cudaStream_t s, bool with_pairs, bool jagged, bool pdl_first = true) {
+                       cudaStream_t s, bool jagged, bool pdl_first = true, SpreadSum<T> sp = {}) {
     const int nb = grid_blocks(M, 256, ctx->sm_count);
     launch_dep(pdl_first, k_slot_count<KW>, dim3(nb), dim3(256), 0, s, ct, M, sg, anchor, sl.count);
     launch_pdl(k_slot_scan, dim3(sc.lb_tiles[0]), dim3(kLbThreads), 0, s, (const uint32_t *)sl.count, ndense,
@@ -1958,20 +2015,22 @@ static int slots_build(ib_ctx *ctx, const CaseTab &ct, int M, int ndense, SlotGe
     launch_pdl(k_slot_fill<KW>, dim3(nb), dim3(256), 0, s, ct, M, sg, anchor, (const uint32_t *)sl.start,
                sl.cursor, sl.cand, sl.pcnt);
     // the pair counts of the filled candidate positions [0, start[ndense])
-    if (with_pairs)
+    if (!sp.f)
         launch_pdl(k_scan_lb, dim3(sc.lb_tiles[1]), dim3(kLbThreads), 0, s, (const uint32_t *)sl.pcnt,
                    (int)sc.cand_cap, (const uint32_t *)(sl.start + ndense), sl.poff, sc.lb_stat + sc.lb_tiles[0],
                    sc.lb_ticket + 1, ctx->status);
     ncompact_dev = (int *)(sl.flag_scan + ndense);
-    launch_pdl(k_tile_lists<T, KW>, dim3(ctx->sm_count * kListCtas), dim3(kListThreads), 0, s, ct, sg.mode, sc.ncompact_cap,
-               (const int *)ncompact_dev, sg, (const uint32_t *)sl.dense_of, (const uint32_t *)sl.start, anchor, level, sl,
-               wts, jagged ? 1 : 0, sc.big, (int *)sc.lb_ticket + 2);
-    auto large = k_tile_lists_large<T, KW>;
-    resident_ctas(ctx, (const void *)large, kPairThreads, sizeof(CtaLists));  // (its shared memory limit)
-    launch_pdl(large, dim3(ctx->sm_count), dim3(kPairThreads), sizeof(CtaLists), s, ct, sg.mode, sg,
-               (const uint32_t *)sl.dense_of, (const uint32_t *)sl.start, anchor, level, sl, wts, jagged ? 1 : 0,
-               (const int *)sc.big,
-               (const int *)sc.lb_ticket + 2, ctx->status);
+    auto lists = [&](auto small, auto large, int ctas) {
+        launch_pdl(small, dim3(ctx->sm_count * ctas), dim3(kListThreads), 0, s, ct, sg.mode, sc.ncompact_cap,
+                   (const int *)ncompact_dev, sg, (const uint32_t *)sl.dense_of, (const uint32_t *)sl.start, anchor,
+                   level, sl, wts, jagged ? 1 : 0, sc.big, (int *)sc.lb_ticket + 2, sp);
+        resident_ctas(ctx, (const void *)large, kPairThreads, sizeof(CtaLists));  // (its shared memory limit)
+        launch_pdl(large, dim3(ctx->sm_count), dim3(kPairThreads), sizeof(CtaLists), s, ct, sg.mode, sg,
+                   (const uint32_t *)sl.dense_of, (const uint32_t *)sl.start, anchor, level, sl, wts, jagged ? 1 : 0,
+                   (const int *)sc.big, (const int *)sc.lb_ticket + 2, ctx->status, sp);
+    };
+    if (sp.f) lists(k_tile_lists<T, KW, true>, k_tile_lists_large<T, KW, true>, kSpreadCtas);
+    else lists(k_tile_lists<T, KW, false>, k_tile_lists_large<T, KW, false>, kListCtas);
     return check_launch("slot lists");
 }
 
@@ -2010,15 +2069,13 @@ static int run_spread(ib_ctx *ctx, const ib_grid *grid, int M, const double *X, 
     Slots sl;
     SlotScratch sc;
     int *ncompact = nullptr;
-    int rc = slots_alloc<T, KW>(ar, M, (int)ndense, sg.mode, sl, sc, s, true, false);
+    int rc = slots_alloc<T, KW>(ar, M, (int)ndense, sg.mode, sl, sc, s, false, false);
     if (rc) return rc;
     PhaseTimer tm(ctx, IB_PHASE_SPREAD, s);
     k_prep_spread<T, KER><<<nb, 256, 0, s>>>(g, M, X, F, dV, ms, ctx->status);
     rc = slots_build<T, KW>(ctx, ct, M, (int)ndense, sg, ms.anchor, (const PS<T> *)ms.wts, nullptr, sl, sc, ncompact, s,
-                            true, true);
+                            true, true, SpreadSum<T>{ms.A, (T *)f});
     if (rc) return rc;
-    launch_pdl(k_spread_gather<T, KER>, dim3(ctx->sm_count * kSliceCtas<T>), dim3(kSliceThreads), 0, s, ct,
-               (const int *)ncompact, sl, (const PS<T> *)ms.A);
     return check_launch("ib_spread");
 }
 
@@ -2174,7 +2231,7 @@ static int run_mdf(ib_ctx *ctx, Arena &ar, const CaseTab &ct, const ib_particles
     int *ncompact = nullptr;
     if (!atomic) {
         rc = slots_build<T, KW>(ctx, ct, M, (int)ndense, sg, ms.anchor, (const PS<T> *)ms.wts, lo.level, sl, sc,
-                                ncompact, s, true, level_path, false);
+                                ncompact, s, level_path, false);
         if (rc) return rc;
         a.sl = sl;
     }

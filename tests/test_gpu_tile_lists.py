@@ -9,6 +9,7 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 from paper_2408_14140_gb300 import synth
 
 pytestmark = pytest.mark.gpu
@@ -60,4 +61,12 @@ def test_forms_agree_bitwise(api, n, P, per, rad, prec, delta, order):
         assert torch.equal(u, out[0][0])
         assert torch.equal(F, out[0][1])
     assert not torch.equal(out[0][0], u0)
+    # standalone spreading sums in the list kernels themselves
+    Xm = np.repeat(X, per, axis=0) + R
+    F = rng.uniforms(3 * P * per).reshape(P * per, 3) - 0.5
+    f = u0.clone()
+    ctx.ib_spread(f, t(Xm), t(F), marks["dV"], h, delta=delta)
+    ctx.status()
+    ref = oracle.spread(n, h, (0, 0, 0), Xm, F, np.full(P * per, h ** 3), delta, f=u0.double().cpu().numpy())
+    assert np.max(np.abs(f.double().cpu().numpy() - ref)) <= (1e-12 if prec == 0 else 2e-5) * np.max(np.abs(ref))
     ctx.close()
