@@ -131,22 +131,20 @@ struct Slots {
     int4 *geo_dim;     // [ncompact_max] tile dims, w = first candidate
     int *geo_case;     // [ncompact_max] case of the tile
     // per-cell gather lists (built once per call, see k_tile_lists).  A
-    // candidate contributes one pair per stencil cell inside its tile;
-    // poff[i] is the exclusive prefix of those counts over candidate
-    // positions, so tile cs with first candidate b owns pairs
-    // [poff[b], poff[b + nc]) -- KW^3 M in total.  band[poff[b] + q] =
-    // {cell | count << 16, first pair relative to poff[b]} for its q-th band
+    // candidate contributes one pair per stencil cell inside its tile, KW^3 M in
+    // total; tile cs owns the pairs from pb = tinfo[cs].x on.  band[pb + q] =
+    // {cell | count << 16, first pair relative to pb} for its q-th band
     // cell, cells ordered by count, largest first.  Wavefront form: the first
     // pair of the cell's slice of 32, whose rows of pairs[] are markers (jagged
     // rows, see k_tile_lists).  Group form: the cell's own first pair, its
     // pairs contiguous, candidate | ox << 16 | oy << 18 | oz << 20.  Each
     // cell's pairs ascend in candidate order (the gather order).
-    uint32_t *pcnt;    // [cand_cap] in-tile stencil cells of each candidate
-    uint32_t *poff;    // [cand_cap + 1] exclusive scan of pcnt
+    unsigned int *pair_cursor;    // pairs given out
+    unsigned long long pair_cap;  // KW^3 M
     int2 *band;
     uint32_t *pairs;
     int *nband;        // [ncompact_max] band cells of the tile
-    // [ncompact_max] the tile's list record {first pair poff[b], pairs,
+    // [ncompact_max] the tile's list record {first pair, pairs,
     // band cells, candidates}, one load for the wavefront gather
     int4 *tinfo;
     uint4 *slen;       // [ncompact_max] rows of the tile's slices (a byte each, at most 255)
@@ -376,8 +374,9 @@ __device__ __forceinline__ void gather_tile_lists(const CaseTab &ct, int cs, con
     const int nc = (int)(sl.start[d + 1] - sl.start[d]);
     const int nb = sl.nband[cs];
     const uint32_t *cand = sl.cand + dim.w;
-    const int2 *band = sl.band + sl.poff[dim.w];
-    const uint32_t *pairs = sl.pairs + sl.poff[dim.w];
+    const uint32_t pb = (uint32_t)sl.tinfo[cs].x;
+    const int2 *band = sl.band + pb;
+    const uint32_t *pairs = sl.pairs + pb;
     const bool staged = nc <= TileStage<T>::N;
     auto cell_index = [&](int cell) {
         const int tx = cell & 7, ty = (cell >> 3) & 7, tz = cell >> 6;
@@ -530,8 +529,7 @@ __device__ __forceinline__ void gather_tiles_lists(const CaseTab &ct, int cs0, i
         while (k + 1 < nt && s_boff[k + 1] <= qq) ++k;
         const int cs = cs0 + k;
         const int4 lo = sl.geo_lo[cs];
-        const int b = sl.geo_dim[cs].w;
-        const size_t pb = sl.poff[b];
+        const size_t pb = (uint32_t)sl.tinfo[cs].x;
         const int2 e = sl.band[pb + (qq - s_boff[k])];
         const int cell = e.x & 0xffff, cnt = e.x >> 16;
         const uint32_t *pr = sl.pairs + pb + e.y;

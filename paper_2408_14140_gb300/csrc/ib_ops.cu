@@ -542,35 +542,23 @@ __global__ void __launch_bounds__(kLevThreads) k_levels(CaseTab ct, int P, int o
 // the KW cells from `first`.  Global tiles use wrapped cells; local tiles use
 // cells relative to the particle box (no wrap, box <= grid).
 template <int KW>
-__device__ __forceinline__ int axis_tiles_global(int first, int n, int t[3], int c[3]) {
+__device__ __forceinline__ int axis_tiles_global(int first, int n, int t[3]) {
     int cnt = 0;
 #pragma unroll
     for (int k = 0; k < KW; ++k) {
-        int cc = wrap_add(first, k, n);
-        int tt = cc / kTile;
+        const int tt = wrap_add(first, k, n) / kTile;
         int j = 0;
         while (j < cnt && t[j] != tt) ++j;
-        if (j < cnt) ++c[j];
-        else if (cnt < 3) {
-            t[cnt] = tt;
-            c[cnt++] = 1;
-        }
+        if (j == cnt && cnt < 3) t[cnt++] = tt;
     }
     return cnt;
 }
 
 template <int KW>
-__device__ __forceinline__ int axis_tiles_local(long long first_rel, int t[3], int c[3]) {
-    int a = (int)(first_rel / kTile), b = (int)((first_rel + KW - 1) / kTile);
-    t[0] = a;
-    if (b != a) {
-        t[1] = b;
-        c[0] = (int)((long long)(a + 1) * kTile - first_rel);
-        c[1] = KW - c[0];
-        return 2;
-    }
-    c[0] = KW;
-    return 1;
+__device__ __forceinline__ int axis_tiles_local(int first_rel, int t[3]) {
+    t[0] = first_rel / kTile;
+    t[1] = (first_rel + KW - 1) / kTile;
+    return t[1] != t[0] ? 2 : 1;
 }
 
 struct SlotGeom {
@@ -586,25 +574,24 @@ template <int KW, typename Fn>
 __device__ __forceinline__ void for_marker_slots(const CaseTab &ct, const SlotGeom &sg, int l,
                                                  uint64_t anc, Fn f) {
     int tx[3], ty[3], tz[3], nx, ny, nz;
-    int cx[3] = {0, 0, 0}, cy[3] = {0, 0, 0}, cz[3] = {0, 0, 0};  // stencil cells per axis tile
     uint32_t base = 0;
     const DevCase &cd = ct.get(sg.part_of ? ct.case_of(sg.part_of[l]) : 0);
     const DevGrid &g = cd.g;
     if (sg.mode == 0) {
-        nx = axis_tiles_global<KW>(anchor_x(anc), g.n[0], tx, cx);
-        ny = axis_tiles_global<KW>(anchor_y(anc), g.n[1], ty, cy);
-        nz = axis_tiles_global<KW>(anchor_z(anc), g.n[2], tz, cz);
+        nx = axis_tiles_global<KW>(anchor_x(anc), g.n[0], tx);
+        ny = axis_tiles_global<KW>(anchor_y(anc), g.n[1], ty);
+        nz = axis_tiles_global<KW>(anchor_z(anc), g.n[2], tz);
     } else {
         int p = sg.part_of[l];
         int4 blo = sg.box_lo[p];
         // relative first cell: (anchor - box_lo) mod n, < box dims
         // box_lo is wrapped by the preparation kernel: [0, n)
-        long long rx = wrap_diff(anchor_x(anc), blo.x, g.n[0]);
-        long long ry = wrap_diff(anchor_y(anc), blo.y, g.n[1]);
-        long long rz = wrap_diff(anchor_z(anc), blo.z, g.n[2]);
-        nx = axis_tiles_local<KW>(rx, tx, cx);
-        ny = axis_tiles_local<KW>(ry, ty, cy);
-        nz = axis_tiles_local<KW>(rz, tz, cz);
+        const int rx = wrap_diff(anchor_x(anc), blo.x, g.n[0]);
+        const int ry = wrap_diff(anchor_y(anc), blo.y, g.n[1]);
+        const int rz = wrap_diff(anchor_z(anc), blo.z, g.n[2]);
+        nx = axis_tiles_local<KW>(rx, tx);
+        ny = axis_tiles_local<KW>(ry, ty);
+        nz = axis_tiles_local<KW>(rz, tz);
         // a box wider than kMaxBox is reported by the preparation kernel;
         // keep every slot id in range regardless
         if (tx[nx - 1] >= kLocalTiles || ty[ny - 1] >= kLocalTiles || tz[nz - 1] >= kLocalTiles) return;
@@ -618,7 +605,7 @@ __device__ __forceinline__ void for_marker_slots(const CaseTab &ct, const SlotGe
                     s = cd.tile_off + ((uint32_t)tz[k] * cd.tiles[1] + ty[j]) * cd.tiles[0] + tx[i];
                 else
                     s = base + ((uint32_t)tz[k] * kLocalTiles + ty[j]) * kLocalTiles + tx[i];
-                f(s, (uint32_t)(cx[i] * cy[j] * cz[k]));
+                f(s);
             }
 }
 
@@ -627,19 +614,17 @@ __global__ void k_slot_count(CaseTab ct, int M, SlotGeom sg, const uint64_t *__r
                              uint32_t *__restrict__ count) {
     grid_dep_wait();
     for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < M; l += gridDim.x * blockDim.x)
-        for_marker_slots<KW>(ct, sg, l, anchor[l], [&](uint32_t s, uint32_t) { atomicAdd(count + s, 1u); });
+        for_marker_slots<KW>(ct, sg, l, anchor[l], [&](uint32_t s) { atomicAdd(count + s, 1u); });
 }
 
 template <int KW>
 __global__ void k_slot_fill(CaseTab ct, int M, SlotGeom sg, const uint64_t *__restrict__ anchor,
                             const uint32_t *__restrict__ start, uint32_t *__restrict__ cursor,
-                            uint32_t *__restrict__ cand, uint32_t *__restrict__ pcnt) {
+                            uint32_t *__restrict__ cand) {
     grid_dep_wait();
     for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < M; l += gridDim.x * blockDim.x)
-        for_marker_slots<KW>(ct, sg, l, anchor[l], [&](uint32_t s, uint32_t ncell) {
-            uint32_t pos = start[s] + atomicAdd(cursor + s, 1u);
-            cand[pos] = (uint32_t)l;
-            if (pcnt) pcnt[pos] = ncell;
+        for_marker_slots<KW>(ct, sg, l, anchor[l], [&](uint32_t s) {
+            cand[start[s] + atomicAdd(cursor + s, 1u)] = (uint32_t)l;
         });
 }
 
@@ -784,70 +769,30 @@ __global__ void __launch_bounds__(kLbThreads) k_slot_scan(const uint32_t *__rest
     }
 }
 
-// out = exclusive scan of in[0, n'), n' = min(n, *n_dev); out[n'] = total.
-// Tiles past n' return at once.
-__global__ void __launch_bounds__(kLbThreads) k_scan_lb(const uint32_t *__restrict__ in, int n,
-                                                        const uint32_t *__restrict__ n_dev,
-                                                        uint32_t *__restrict__ out, unsigned long long *tstat,
-                                                        unsigned int *ticket, DevStatus *st) {
-    __shared__ int s_tile;
-    grid_dep_wait();
-    const int nn = min(n, (int)*n_dev);
-    if (threadIdx.x == 0) s_tile = (int)atomicAdd(ticket, 1u);
-    __syncthreads();
-    const int tile = s_tile;
-    if (tile * kLbTile > nn) return;  // no element, and not the tile of the total either
-    const int i0 = tile * kLbTile + threadIdx.x * kLbItems;
-    uint32_t v[kLbItems];
-    unsigned long long sum = 0;
-#pragma unroll
-    for (int k = 0; k < kLbItems; ++k) {
-        v[k] = i0 + k < nn ? in[i0 + k] : 0u;
-        sum += v[k];
-    }
-    unsigned long long tot, base;
-    const unsigned long long ex = lb_block_scan(sum, &tot);
-    if (!lb_tile_base(tile, tot, tstat, st, base)) return;
-    unsigned long long run = base + ex;
-#pragma unroll
-    for (int k = 0; k < kLbItems; ++k) {
-        if (i0 + k < nn) out[i0 + k] = (uint32_t)run;
-        run += v[k];
-    }
-    if (i0 <= nn && nn < i0 + kLbItems) out[nn] = (uint32_t)run;
-}
-
-__global__ void k_level_slots(int mode, const int *__restrict__ nlev_p, const int *__restrict__ lev_pbeg,
-                              const uint32_t *__restrict__ fscan, int ndense, int *__restrict__ lev_sbeg) {
-    grid_dep_wait();
-    int nl = *nlev_p;
-    for (int L = threadIdx.x; L <= nl; L += blockDim.x) {
-        if (mode == 0) {
-            lev_sbeg[L] = L == 0 ? 0 : (int)fscan[ndense];
-        } else {
-            long long d = (long long)lev_pbeg[L] * kLocalSlots;
-            lev_sbeg[L] = (int)fscan[d < ndense ? d : ndense];
-        }
-    }
-}
-
 // Per wavefront, the slices of its tiles, longest first (a counting sort by
 // their rows; equal ones in any order): one warp of the wavefront gather takes
 // a slice, and the last round of warps then has the shortest.  Only the order
-// of work changes.  Wavefront L's list starts at lev_slice[L].x, a bound of what
-// the wavefronts before it need (a slice has at least one pair), and has
-// lev_slice[L].y entries {tile, slice, first pair of the tile, cells}.
+// of work changes.  Wavefront L's list starts at lev_slice[L].x, taken from the
+// cursor in whatever order the wavefronts come, and has lev_slice[L].y entries
+// {tile, slice, first pair of the tile, cells}.  A wavefront's tiles are consecutive:
+// global tiles form one, a particle's local tiles follow its rank.
 constexpr int kSliceOrderThreads = 1024;
-__global__ void __launch_bounds__(kSliceOrderThreads) k_level_slices(const int *__restrict__ nlev_p,
-                                                                     const int *__restrict__ lev_sbeg, Slots sl,
+__global__ void __launch_bounds__(kSliceOrderThreads) k_level_slices(int mode, const int *__restrict__ nlev_p,
+                                                                     const int *__restrict__ lev_pbeg, int ndense,
+                                                                     Slots sl, unsigned int *__restrict__ cursor,
                                                                      int2 *__restrict__ lev_slice,
                                                                      int4 *__restrict__ slices) {
     grid_dep_wait();
-    __shared__ int s_hist[256];
+    __shared__ int s_hist[256], s_base;
     const int nl = *nlev_p;
+    auto first_tile = [&](int L) {
+        if (mode == 0) return L == 0 ? 0 : (int)sl.flag_scan[ndense];
+        const long long d = (long long)lev_pbeg[L] * kLocalSlots;
+        return (int)sl.flag_scan[d < ndense ? d : ndense];
+    };
     for (int L = blockIdx.x; L < nl; L += gridDim.x) {  // one CTA per wavefront
-        const int s0 = lev_sbeg[L], s1 = lev_sbeg[L + 1];
-        const int base = s0 < s1 ? (int)((uint32_t)sl.tinfo[s0].x >> 5) + s0 : 0;
+        const int s0 = first_tile(L), s1 = first_tile(L + 1);
+        int base = 0;
         for (int k = threadIdx.x; k < 256; k += blockDim.x) s_hist[k] = 0;
         __syncthreads();
         for (int pass = 0; pass < 2; ++pass) {
@@ -865,10 +810,14 @@ __global__ void __launch_bounds__(kSliceOrderThreads) k_level_slices(const int *
             }
             __syncthreads();
             if (pass == 0) {
-                block_scan_chunked(256, [&](int k) { return s_hist[k]; }, [&](int k, int pre) { s_hist[k] = pre; });
+                const int total =
+                    block_scan_chunked(256, [&](int k) { return s_hist[k]; }, [&](int k, int pre) { s_hist[k] = pre; });
+                if (threadIdx.x == 0) {
+                    s_base = (int)atomicAdd(cursor, (unsigned)total);
+                    lev_slice[L] = make_int2(s_base, total);
+                }
                 __syncthreads();
-            } else if (threadIdx.x == 0) {
-                lev_slice[L] = make_int2(base, s_hist[255]);  // every slice counted: the last bucket's end
+                base = s_base;
             }
         }
         __syncthreads();
@@ -1016,9 +965,13 @@ struct ListShared {
     int hist[kLenBins];
     int sum[kSlices];                      // pairs of each slice
     uint16_t cell[kTileCells], cnt[kTileCells];
-    unsigned char len[kSlices];            // rows of each slice (at most 255 told)
-    int nb;
+    // rows of each slice (at most 255 told), read as one 16-byte word
+    alignas(16) unsigned char len[kSlices];
+    int nb;                                // band cells
+    int np;                                // pairs of the tile
+    uint32_t base;                         // its first pair
 };
+static_assert(offsetof(ListShared, len) % 16 == 0 && alignof(ListShared) == 16, "16-byte read");
 struct CtaLists {
     unsigned long long keys[kMaxCand];
     unsigned set[3 * kTile][kPairWords + 1];
@@ -1073,12 +1026,14 @@ struct SpreadSum {
 };
 
 // A tile's lists from its bit sets of nw words (set(i, w): columns, rows, planes
-// for i from 0, 8, 16), by a CTA of NT threads.  The caller has zeroed ls.hist
-// and ls.len before a barrier.
+// for i from 0, 8, 16), by a CTA of NT threads.  The caller has zeroed ls.hist,
+// ls.np and ls.len before a barrier.  The tile takes its share of the pair arrays
+// from a cursor, so no scan of the candidates' pair counts is needed (5 to 16 us a
+// call); where it lies changes no sum.
 // With SUM every cell's sum is added to the field instead (a lane a cell, the
 // pairs in the same order).
 template <typename T, int NT, bool SUM, class Set, class First, class Mark>
-__device__ __forceinline__ void build_lists(const Slots &sl, int cs, uint32_t pb, int room, int nc, int nw, bool jagged,
+__device__ __forceinline__ void build_lists(const Slots &sl, int cs, int nc, int nw, bool jagged,
                                             const PS<T> *__restrict__ wts, ListShared &ls, Set set, First first,
                                             Mark mark, const SpreadSum<T> &sp) {
     constexpr int C = kTileCells / NT;  // cells a thread, neighbours along x
@@ -1098,7 +1053,15 @@ __device__ __forceinline__ void build_lists(const Slots &sl, int cs, uint32_t pb
     auto bucket = [](int n) { return kLenBins - 1 - min(n, kLenBins - 1); };
 #pragma unroll
     for (int k = 0; k < C; ++k) r[k] = t[k] > 0 ? atomicAdd(&ls.hist[bucket(t[k])], 1) : 0;
+    if constexpr (!SUM) {
+        int sum = 0;
+#pragma unroll
+        for (int k = 0; k < C; ++k) sum += t[k];
+        sum = __reduce_add_sync(0xffffffffu, sum);
+        if (lane == 0) atomicAdd(&ls.np, sum);
+    }
     __syncthreads();
+    if (!SUM && tid == 32) ls.base = atomicAdd(sl.pair_cursor, (unsigned)ls.np);
     if (warp == 0) {
         int h[kLenBins / 32], s = 0;
 #pragma unroll
@@ -1187,12 +1150,14 @@ __device__ __forceinline__ void build_lists(const Slots &sl, int cs, uint32_t pb
         }
         return;
     }
+    const uint32_t pb = ls.base;
+    // (more pairs than the arrays hold only with a box wider than its grid, which is
+    // reported: such a tile is left empty)
+    const bool fits = (unsigned long long)pb + ls.np <= sl.pair_cap;
     uint32_t *const pairs = sl.pairs + pb;
     PS<T> *const pw = (PS<T> *)sl.pw + pb;
     int2 *const band = sl.band + pb;
-    int np = 0;
-    for (int s = 0; s < ns; ++s) np += ls.sum[s];
-    for (int s = warp; s < ns; s += NT / 32) {
+    for (int s = fits ? warp : ns; s < ns; s += NT / 32) {
         const int q = 32 * s + lane;
         const int c = q < nb ? ls.cell[q] : 0, n = q < nb ? ls.cnt[q] : 0;
         int base = 0;
@@ -1215,7 +1180,7 @@ __device__ __forceinline__ void build_lists(const Slots &sl, int cs, uint32_t pb
             for (int u = 0; u < kU; ++u) {
                 const bool act = k0 + u < n;
                 const unsigned a = __ballot_sync(0xffffffffu, act);
-                pos[u] = act ? (jagged ? off + __popc(a & ((1u << lane) - 1u)) : own + k0 + u) : room;
+                pos[u] = act ? (jagged ? off + __popc(a & ((1u << lane) - 1u)) : own + k0 + u) : -1;
                 off += __popc(a);
                 i[u] = 0;
                 if (act) {
@@ -1233,7 +1198,7 @@ __device__ __forceinline__ void build_lists(const Slots &sl, int cs, uint32_t pb
 #pragma unroll
             for (int u = 0; u < kU; ++u) {
                 mk[u] = mark(i[u]);
-                oc[u] = pos[u] < room ? code - first(i[u]) : 0;
+                oc[u] = pos[u] >= 0 ? code - first(i[u]) : 0;
                 const PS<T> *wm = wts + 12 * (size_t)mk[u];
                 wx[u] = wm[oc[u] & 3];
                 wy[u] = wm[4 + ((oc[u] >> 2) & 3)];
@@ -1241,15 +1206,15 @@ __device__ __forceinline__ void build_lists(const Slots &sl, int cs, uint32_t pb
             }
 #pragma unroll
             for (int u = 0; u < kU; ++u)
-                if (pos[u] < room) {  // (more than the room only with a box wider than its grid, reported)
+                if (pos[u] >= 0) {
                     pairs[pos[u]] = jagged ? mk[u] : (uint32_t)i[u] | ((uint32_t)oc[u] << 16);
                     pw[pos[u]] = pair_weight3(wx[u], wy[u], wz[u]);
                 }
         }
     }
     if (tid == 0) {
-        sl.nband[cs] = nb;
-        sl.tinfo[cs] = make_int4((int)pb, min(np, room), nb, nc);
+        sl.nband[cs] = fits ? nb : 0;
+        sl.tinfo[cs] = make_int4((int)pb, fits ? ls.np : 0, fits ? nb : 0, nc);
         sl.slen[cs] = *(const uint4 *)ls.len;
     }
 }
@@ -1280,8 +1245,6 @@ __global__ void __launch_bounds__(kListThreads, SUM ? kSpreadCtas : kListCtas) k
             if (tid == 0) big[atomicAdd(nbig, 1)] = cs;
             continue;
         }
-        const uint32_t pb = SUM ? 0u : sl.poff[b];
-        const int room = SUM ? 0 : (int)(sl.poff[b + nc] - pb);  // the tile's share of the pair arrays
         int lo[3], dim[3], lev;
         const int cse = slot_geometry(ct, mode, sg, sl, level, d, b, lo, dim, lev);
         const DevGrid &g = ct.get(cse).g;
@@ -1363,10 +1326,11 @@ __global__ void __launch_bounds__(kListThreads, SUM ? kSpreadCtas : kListCtas) k
             if (lane < 3 * kTile) s_set[lane][w] = mine;
         }
         s_ls.hist[tid] = 0;
+        if (tid == 0) s_ls.np = 0;
         if (tid < kSlices) s_ls.len[tid] = 0;
         __syncthreads();
         if (SUM) sp.lo[0] = lo[0], sp.lo[1] = lo[1], sp.lo[2] = lo[2], sp.g = g;
-        build_lists<T, kListThreads, SUM>(sl, cs, pb, room, nc, nw, jagged != 0, wts, s_ls,
+        build_lists<T, kListThreads, SUM>(sl, cs, nc, nw, jagged != 0, wts, s_ls,
                                           [&](int i, int w) { return s_set[i][w]; }, [&](int i) { return s_first[i]; },
                                           [&](int i) { return s_mark[i]; }, sp);
         if (!SUM && tid == 0) {
@@ -1397,12 +1361,10 @@ __global__ void __launch_bounds__(kPairThreads) k_tile_lists_large(
             int lo[3], dim[3], lev;
             const int cse = slot_geometry(ct, mode, sg, sl, level, d, b, lo, dim, lev);
             const DevGrid &g = ct.get(cse).g;
-            const uint32_t pb = SUM ? 0u : sl.poff[b];
-            int room = SUM ? 0 : (int)(sl.poff[b + nc] - pb);
             if (nc > kMaxCand) {
                 // report, and leave an empty tile (no bins, no cells)
                 if (tid == 0) raise_status(st, IB_ERR_UNSUPPORTED, nc);
-                nc = room = 0;
+                nc = 0;
                 dim[0] = dim[1] = dim[2] = 0;
             }
             int np2 = 1;
@@ -1439,10 +1401,11 @@ __global__ void __launch_bounds__(kPairThreads) k_tile_lists_large(
                 if (lane < 3 * kTile) sh.set[lane][w] = mine;
             }
             if (tid < kLenBins) sh.ls.hist[tid] = 0;
+            if (tid == 0) sh.ls.np = 0;
             if (tid < kSlices) sh.ls.len[tid] = 0;
             __syncthreads();
             if (SUM) sp.lo[0] = lo[0], sp.lo[1] = lo[1], sp.lo[2] = lo[2], sp.g = g;
-            build_lists<T, kPairThreads, SUM>(sl, cs, pb, room, nc, nw, jagged != 0, wts, sh.ls,
+            build_lists<T, kPairThreads, SUM>(sl, cs, nc, nw, jagged != 0, wts, sh.ls,
                                               [&](int i, int w) { return sh.set[i][w]; },
                                               [&](int i) { return sh.first[i]; },
                                               [&](int i) { return (uint32_t)(sh.keys[i] & 0xffffffffu); }, sp);
@@ -1942,9 +1905,11 @@ static bool take_markers(Arena &ar, int M, MarkerState<T> &ms) {
 struct SlotScratch {
     size_t cand_cap;
     int ncompact_cap;
-    int lb_tiles[2];              // look-back tiles of the slot scan and of the pair-count scan
-    unsigned long long *lb_stat;  // [lb_tiles[0] + lb_tiles[1]] tile words
-    unsigned int *lb_ticket;      // [2], then the number of large tiles
+    int lb_tiles;                 // look-back tiles of the slot scan
+    unsigned long long *lb_stat;  // [lb_tiles] tile words
+    // [4] the scan's ticket, the cursors of the pairs and of the slices, the number
+    // of large tiles
+    unsigned int *words;
     int *big;                     // [ncompact_cap] large tiles
 };
 
@@ -1961,10 +1926,9 @@ static int slots_alloc(Arena &ar, int M, int ndense, int mode, Slots &sl, SlotSc
     sl.start = ar.take<uint32_t>(ndense + 1);
     sl.cursor = ar.take<uint32_t>(ndense);
     sl.flag_scan = ar.take<uint32_t>(ndense + 1);
-    sc.lb_tiles[0] = ndense / kLbTile + 1;
-    sc.lb_tiles[1] = with_pairs ? (int)(sc.cand_cap / kLbTile) + 1 : 0;
-    sc.lb_stat = ar.take<unsigned long long>((size_t)sc.lb_tiles[0] + sc.lb_tiles[1]);
-    sc.lb_ticket = ar.take<unsigned int>(3);
+    sc.lb_tiles = ndense / kLbTile + 1;
+    sc.lb_stat = ar.take<unsigned long long>(sc.lb_tiles);
+    sc.words = ar.take<unsigned int>(4);
     sc.big = ar.take<int>(ncap);
     sl.dense_of = ar.take<uint32_t>(ncap);
     sl.cand = ar.take<uint32_t>(sc.cand_cap);
@@ -1976,8 +1940,8 @@ static int slots_alloc(Arena &ar, int M, int ndense, int mode, Slots &sl, SlotSc
     constexpr int KW3 = KW * KW * KW;
     if (with_pairs) {
         // every stencil cell of every marker is one pair: KW^3 M in total
-        sl.pcnt = ar.take<uint32_t>(sc.cand_cap);
-        sl.poff = ar.take<uint32_t>(sc.cand_cap + 1);
+        sl.pair_cursor = sc.words + 1;
+        sl.pair_cap = (unsigned long long)KW3 * M;
         sl.band = ar.take<int2>((size_t)KW3 * M);
         sl.pairs = ar.take<uint32_t>((size_t)KW3 * M);
         sl.pw = ar.take<PS<T>>((size_t)KW3 * M);
@@ -1985,7 +1949,8 @@ static int slots_alloc(Arena &ar, int M, int ndense, int mode, Slots &sl, SlotSc
         sl.tinfo = ar.take<int4>(ncap);
         sl.slen = ar.take<uint4>(ncap);
     } else {
-        sl.pcnt = sl.poff = nullptr;
+        sl.pair_cursor = nullptr;
+        sl.pair_cap = 0;
         sl.band = nullptr;
         sl.pairs = nullptr;
         sl.nband = nullptr;
@@ -1997,12 +1962,12 @@ static int slots_alloc(Arena &ar, int M, int ndense, int mode, Slots &sl, SlotSc
         return oom_error(ar.used, ar.cap);
     cudaMemsetAsync(sl.count, 0, sizeof(uint32_t) * ndense, s);
     cudaMemsetAsync(sl.cursor, 0, sizeof(uint32_t) * ndense, s);
-    cudaMemsetAsync(sc.lb_stat, 0, sizeof(unsigned long long) * (sc.lb_tiles[0] + sc.lb_tiles[1]), s);
-    cudaMemsetAsync(sc.lb_ticket, 0, 3 * sizeof(unsigned int), s);
+    cudaMemsetAsync(sc.lb_stat, 0, sizeof(unsigned long long) * sc.lb_tiles, s);
+    cudaMemsetAsync(sc.words, 0, 4 * sizeof(unsigned int), s);
     return IB_OK;
 }
 
-// The kernel chain: count, scan, compact, fill, scan, sort, per-cell lists -- or,
+// The kernel chain: count, scan and compact, fill, sort and per-cell lists -- or,
 // given a field to spread into (sp.f), the cells' sums.
 template <typename T, int KW>
 static int slots_build(ib_ctx *ctx, const CaseTab &ct, int M, int ndense, SlotGeom sg, const uint64_t *anchor,
@@ -2010,24 +1975,19 @@ static int slots_build(ib_ctx *ctx, const CaseTab &ct, int M, int ndense, SlotGe
                        cudaStream_t s, bool jagged, bool pdl_first = true, SpreadSum<T> sp = {}) {
     const int nb = grid_blocks(M, 256, ctx->sm_count);
     launch_dep(pdl_first, k_slot_count<KW>, dim3(nb), dim3(256), 0, s, ct, M, sg, anchor, sl.count);
-    launch_pdl(k_slot_scan, dim3(sc.lb_tiles[0]), dim3(kLbThreads), 0, s, (const uint32_t *)sl.count, ndense,
-               sl.start, sl.flag_scan, sl.dense_of, sc.lb_stat, sc.lb_ticket, ctx->status);
+    launch_pdl(k_slot_scan, dim3(sc.lb_tiles), dim3(kLbThreads), 0, s, (const uint32_t *)sl.count, ndense,
+               sl.start, sl.flag_scan, sl.dense_of, sc.lb_stat, sc.words, ctx->status);
     launch_pdl(k_slot_fill<KW>, dim3(nb), dim3(256), 0, s, ct, M, sg, anchor, (const uint32_t *)sl.start,
-               sl.cursor, sl.cand, sl.pcnt);
-    // the pair counts of the filled candidate positions [0, start[ndense])
-    if (!sp.f)
-        launch_pdl(k_scan_lb, dim3(sc.lb_tiles[1]), dim3(kLbThreads), 0, s, (const uint32_t *)sl.pcnt,
-                   (int)sc.cand_cap, (const uint32_t *)(sl.start + ndense), sl.poff, sc.lb_stat + sc.lb_tiles[0],
-                   sc.lb_ticket + 1, ctx->status);
+               sl.cursor, sl.cand);
     ncompact_dev = (int *)(sl.flag_scan + ndense);
     auto lists = [&](auto small, auto large, int ctas) {
         launch_pdl(small, dim3(ctx->sm_count * ctas), dim3(kListThreads), 0, s, ct, sg.mode, sc.ncompact_cap,
                    (const int *)ncompact_dev, sg, (const uint32_t *)sl.dense_of, (const uint32_t *)sl.start, anchor,
-                   level, sl, wts, jagged ? 1 : 0, sc.big, (int *)sc.lb_ticket + 2, sp);
+                   level, sl, wts, jagged ? 1 : 0, sc.big, (int *)sc.words + 3, sp);
         resident_ctas(ctx, (const void *)large, kPairThreads, sizeof(CtaLists));  // (its shared memory limit)
         launch_pdl(large, dim3(ctx->sm_count), dim3(kPairThreads), sizeof(CtaLists), s, ct, sg.mode, sg,
                    (const uint32_t *)sl.dense_of, (const uint32_t *)sl.start, anchor, level, sl, wts, jagged ? 1 : 0,
-                   (const int *)sc.big, (const int *)sc.lb_ticket + 2, ctx->status, sp);
+                   (const int *)sc.big, (const int *)sc.words + 3, ctx->status, sp);
     };
     if (sp.f) lists(k_tile_lists<T, KW, true>, k_tile_lists_large<T, KW, true>, kSpreadCtas);
     else lists(k_tile_lists<T, KW, false>, k_tile_lists_large<T, KW, false>, kListCtas);
@@ -2105,7 +2065,6 @@ static int run_mdf(ib_ctx *ctx, Arena &ar, const CaseTab &ct, const ib_particles
     int *lev_cur = ar.take<int>(P + 1);
     int *nbr_cnt = ar.take<int>(P);
     int *nbr = ar.take<int>((size_t)P * kMaxNbr);
-    int *lev_sbeg = ar.take<int>(P + 1);
     int *mperm = ar.take<int>(M > 0 ? M : 1);
     unsigned int *sched = ar.take<unsigned int>(P + 1);  // done counters + ticket
     Barrier bar;
@@ -2279,10 +2238,8 @@ static int run_mdf(ib_ctx *ctx, Arena &ar, const CaseTab &ct, const ib_particles
     }
     }
     if (!atomic) {
-        launch_pdl(k_level_slots, dim3(1), dim3(256), 0, s, sg.mode, (const int *)lo.nlev,
-                   (const int *)lo.lev_pbeg, (const uint32_t *)sl.flag_scan, (int)ndense, lev_sbeg);
-        launch_pdl(k_level_slices, dim3(P < 64 ? P : 64), dim3(kSliceOrderThreads), 0, s, (const int *)lo.nlev,
-                   (const int *)lev_sbeg, sl, lev_slice, slices);
+        launch_pdl(k_level_slices, dim3(P < 64 ? P : 64), dim3(kSliceOrderThreads), 0, s, sg.mode,
+                   (const int *)lo.nlev, (const int *)lo.lev_pbeg, (int)ndense, sl, sc.words + 2, lev_slice, slices);
     }
     tprep.stop();
     // (the field is first read and written by the pass kernels below)
