@@ -202,12 +202,10 @@ GBIB_API int ib_ctx_set_volume_split(ib_ctx *ctx, int ctas_per_particle);
 
 /* ---- wavefront gather layout (tuning knobs) ------------------------------
  * ctas_per_sm: resident gather CTAs per SM (0, the default: as many as fit;
- * 1..32 caps it).  stage: the candidates of a tile that a gather CTA stages
- * in shared memory (0, the default: the largest capacity, 256 for FP32 and
- * 192 for FP64 fields; else a multiple of 32 in [32, 256], capped at the
- * largest); a tile with more candidates reads them from memory, and a smaller
- * capacity lets more CTAs share an SM.  Neither changes a result: every cell
- * adds the same values in the same order.  IB_ERR_INVALID otherwise.       */
+ * 1..32 caps it).  stage: 0 or a multiple of 32 in [32, 256]; accepted for
+ * callers that set it, without effect (the gather stages nothing in shared
+ * memory).  Neither changes a result: every cell adds the same values in the
+ * same order.  IB_ERR_INVALID otherwise.                                   */
 GBIB_API int ib_ctx_set_gather(ib_ctx *ctx, int ctas_per_sm, int stage);
 
 /* ---- overlap: a dependency before the field is written ------------------
@@ -458,7 +456,12 @@ GBIB_API int particle_volume_integrals_static(const ib_grid *grid, const void *u
  * differences across the cell; the divergence of a cell field at a node is
  * its negative adjoint.  The implicit solves are exact in Fourier space, so
  * every n[a] must be a power of two in [16, 1024] (else IB_ERR_UNSUPPORTED).
- * Workspace: two complex grid fields (predictor), one (projection).
+ * Workspace: three half spectra (predictor: n0/2 complex numbers a line in x)
+ * or one and a scalar field (projection), and for each spectrum a column of
+ * n1 n2 complex numbers beside it.  FP64 fields are transformed in 64-bit fixed
+ * point scaled line by line, with errors no larger than an FP64 transform's;
+ * fields whose values do not fit it (not finite, or too far apart in magnitude)
+ * take FP64 stencils.
  *
  * fluid_predictor -- Step 1, Eq. (31): writes u_star = u~*,n+1 from
  *   (I - nu dt/2 L) u~* = u^n + dt (-div(u u)^{n+1/2} - grad p^{n-1/2} / rho_f

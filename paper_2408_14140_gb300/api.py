@@ -259,8 +259,9 @@ class Context:
         self._check(self.lib.ib_ctx_set_spread_mode(self.handle, SPREAD_MODES[mode]))
 
     def set_gather(self, ctas_per_sm: int = 0, stage: int = 0):
-        """Wavefront gather layout: resident CTAs per SM and staged candidates
-        per tile (0: the defaults; see gbib.h).  Results do not change."""
+        """Wavefront gather layout: resident CTAs per SM (0: as many as fit);
+        ``stage`` is accepted without effect (see gbib.h).  Results do not
+        change."""
         self._check(self.lib.ib_ctx_set_gather(self.handle, int(ctas_per_sm), int(stage)))
 
     def fluid_predictor(self, u, p, h, rho_f, mu, g, dt, u_star=None, origin=(0.0, 0.0, 0.0), stream=None):

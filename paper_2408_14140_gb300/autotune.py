@@ -10,10 +10,8 @@ laid out on the GPU, never the results:
 * ``volume_split``: the CTAs per particle of the volume integrals (slabs of
   cell planes; 0: one resident wave) -- the same sums, grouped differently;
 * ``gather_ctas``: resident wavefront-gather CTAs per SM (0: as many as fit);
-* ``gather_stage``: the candidates of a spreading tile that a gather CTA
-  stages in shared memory -- the tile's bin capacity on chip; larger tiles
-  read their candidates from memory, a smaller capacity lets more CTAs share
-  an SM (0: the largest).  Both gather choices leave every sum unchanged.
+* ``gather_stage``: a knob the gather accepts without effect (it stages
+  nothing in shared memory).  Both gather choices leave every sum unchanged.
 
 :func:`tune` times a caller-supplied step (the call sequence of the
 workload) on the device -- CUDA events on the current stream, warm-up steps

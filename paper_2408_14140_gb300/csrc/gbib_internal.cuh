@@ -265,7 +265,7 @@ struct ib_ctx {
     int vol_split;       // CTAs per particle of the volume integrals (0: one resident wave)
     int spread_mode;     // IB_SPREAD_GATHER (deterministic) or IB_SPREAD_ATOMIC
     int gather_ctas;     // wavefront gather CTAs per SM (0: as many as fit)
-    int gather_stage;    // candidates a gather CTA stages (0: the largest capacity)
+    int gather_stage;    // accepted, without effect
     void *field_wait;    // cudaEvent_t waited on before the forcing passes (nullable)
     // a second stream and two events: the first interpolation of a forcing
     // call runs on it beside the slot-list kernels (fork and join)

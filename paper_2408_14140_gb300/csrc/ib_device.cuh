@@ -346,7 +346,6 @@ namespace gbib {
 // Candidates of one tile staged in shared memory by the list gathers.
 template <typename T> struct TileStage;
 template <> struct TileStage<float> { static constexpr int N = 256; };
-template <> struct TileStage<double> { static constexpr int N = 192; };
 
 template <typename T>
 constexpr size_t tile_stage_bytes() {

@@ -12,10 +12,11 @@
 //     order).  Each tile's list is sorted by (anchor row, marker index) once,
 //     which fixes the summation order of every cell: spreading is a
 //     deterministic gather over marker bins, with no floating-point atomics.
-//  3. Passes: one persistent cooperative kernel runs, per wavefront of
-//     non-conflicting particles and per forcing pass m, an interpolation
-//     phase over markers (U, F += (U^d - U)/dt) and a gather phase over tiles
-//     (u += S (U^d - U) dV / h^3, the increment of Algorithm 1's correction),
+//  3. Passes: per wavefront of non-conflicting particles and per forcing pass
+//     m, an interpolation over markers (U, F += (U^d - U)/dt) and a gather over
+//     the tiles' cells (u += S (U^d - U) dV / h^3, the increment of Algorithm
+//     1's correction), a kernel each; wavefronts beyond the count of the call
+//     before run in one persistent cooperative kernel, whose phases are
 //     separated by grid-wide barriers with bounded waits.
 //
 // The correction is applied incrementally, u(m) = u(m-1) + dt S(F^m - F^{m-1}),
@@ -1420,13 +1421,6 @@ __global__ void __launch_bounds__(kPairThreads) k_tile_lists_large(
 }
 
 // ---------------------------------------------------------------------------
-// gather of one tile: every cell sums w * A over the markers whose stencil
-// covers it, rows in (z, y) order, markers in index order within a row.
-// The tile's candidates (their per-axis weights, spread source and x offset)
-// are first staged in shared memory with independent loads; the per-cell
-// sums then read shared memory only.  Tiles with more than Stage<T>::N
-// candidates read the same values from global memory instead.
-// ---------------------------------------------------------------------------
 // Spreading (ib_spread) with warp-aggregated atomics: one lane per marker,
 // weights formed on the fly, no binning.
 template <typename T, int KER>
@@ -1535,20 +1529,19 @@ struct PassArgs {
 // ---------------------------------------------------------------------------
 // one wavefront pass as two ordinary kernels (the form CUDA-graph replay runs
 // back to back): interpolation over the wavefront's markers, then a gather
-// with one CTA per tile (grid-stride), many CTAs per SM hiding latency.
+// with one warp per slice of 32 cells, many warps per SM hiding latency.
 //
 // Every level kernel but the first of a call is launched as a programmatic
 // dependent of the one before it: it starts while its predecessor finishes,
 // loads what the predecessor does not write (marker weights, anchors, desired
-// velocities, forces; tile lists, candidate weights, the first band cell's
-// field values), then waits for the predecessor and reads what it wrote (the
+// velocities, forces; the slice's record, field values and first pairs), then waits for the predecessor and reads what it wrote (the
 // field for an interpolation, the spread sources for a gather).  Every CTA
 // waits before it exits, so a level kernel completes only after its
 // predecessor.  An interpolation lets its gather start right after its own
-// wait (the gather's CTAs stage their lists meanwhile); for FP32 fields a
+// wait (the gather's warps load theirs meanwhile); for FP32 fields a
 // gather lets the next interpolation start only as its CTAs exit, so that
 // interpolation's CTAs land on idle SMs (measured faster than an early start),
-// and for FP64 fields once each of its CTAs has reached its last tile.
+// and for FP64 fields once each of its CTAs has waited and reached a last slice.
 // ---------------------------------------------------------------------------
 template <typename T, int KER>
 __global__ void __launch_bounds__(kInterpThreads) k_interp_level(PassArgs<T> a, int L) {

@@ -319,26 +319,6 @@ __device__ __forceinline__ void volume_finish_df(VolSums &s, double h, int p, in
     }
 }
 
-// |x| from x^2 to within a few units of FP64 rounding: an FP32 square root
-// refined by one Newton step in FP64 (s = s0 + (x2 - s0^2) / (2 s0), the
-// classical Heron/Newton iteration; the FP32 start has relative error below
-// 2^-22, so one step leaves an error below 2^-44 relative to the FP64 root).
-// Cheaper than a full FP64 square root on parts whose FP64 rate is low.
-__device__ __forceinline__ double norm_from_square(double x2) {
-    const float sf = sqrtf((float)x2);
-    if (!(sf > 0.0f)) return sqrt(x2);  // zero, or an FP32 under/overflow: exact path
-    const double s0 = (double)sf;
-    const double r = fma(-s0, s0, x2);
-    return fma(r, (double)(0.5f / sf), s0);
-}
-
-// 1/x to within a few units of FP64 rounding: an FP32 reciprocal refined by
-// one Newton step (r = r0 + r0 (1 - x r0)), for x in the FP32 normal range.
-__device__ __forceinline__ double recip_refined(double x) {
-    const double r0 = (double)(1.0f / (float)x);
-    return fma(r0, fma(-x, r0, 1.0), r0);
-}
-
 // Exclusive scan of cnt[0..n) into pre[0..n] by warp 0 (n may exceed 32).
 __device__ __forceinline__ void warp0_scan(const int *cnt, int *pre, int n) {
     if (threadIdx.x >= 32) return;
