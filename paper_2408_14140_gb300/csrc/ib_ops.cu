@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(kRadiusThreads) k_marker_radius(int P, const d
 // Per particle (kPrepSplit CTAs): marker positions, desired velocities,
 // anchors, weights, and the particle's unwrapped stencil box.  Scratch of the
 // cross-CTA reductions: per particle the stencil box bounds (lo starts at a
-// huge value, hi at a very negative one: memset 0x7f / 0x80 bytes) and a
+// huge value, hi at a very negative one) and a
 // completion count (0).
 //
 // Bound by the FP64 pipe: FP64 is kept for the position, the first stencil cell
@@ -1891,6 +1891,24 @@ static bool take_markers(Arena &ar, int M, MarkerState<T> &ms) {
     return ar.ok();
 }
 
+// A call's counters and cursors set in one launch: four memsets of a few words to
+// a megabyte each were four more steps of the preparation's chain.
+struct Fill {
+    unsigned *p[4];
+    unsigned n[4], value[4];  // 32-bit words
+};
+__global__ void __launch_bounds__(256) k_fill(Fill f) {
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+        for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < f.n[a]; i += gridDim.x * blockDim.x)
+            f.p[a][i] = f.value[a];
+}
+static void launch_fill(ib_ctx *ctx, const Fill &f, cudaStream_t s) {
+    unsigned most = 0;
+    for (int a = 0; a < 4; ++a) most = f.n[a] > most ? f.n[a] : most;
+    k_fill<<<grid_blocks(most, 256, ctx->sm_count), 256, 0, s>>>(f);
+}
+
 // Slot lists for `M` prepared markers over ndense dense slots, in two steps
 // so that a call issues every memset before its kernel chain (the chain's
 // kernels are programmatic dependents of one another; a memset in between
@@ -1908,7 +1926,7 @@ struct SlotScratch {
 
 // Workspace of the slot lists, and the zeroing they need.
 template <typename T, int KW>
-static int slots_alloc(Arena &ar, int M, int ndense, int mode, Slots &sl, SlotScratch &sc, cudaStream_t s,
+static int slots_alloc(ib_ctx *ctx, Arena &ar, int M, int ndense, int mode, Slots &sl, SlotScratch &sc, cudaStream_t s,
                        bool with_pairs, bool with_bins) {
     const size_t per = mode == 0 ? 27 : 8;
     sc.cand_cap = (size_t)M * per + 1;
@@ -1953,10 +1971,8 @@ static int slots_alloc(Arena &ar, int M, int ndense, int mode, Slots &sl, SlotSc
     }
     if (!ar.ok())
         return oom_error(ar.used, ar.cap);
-    cudaMemsetAsync(sl.count, 0, sizeof(uint32_t) * ndense, s);
-    cudaMemsetAsync(sl.cursor, 0, sizeof(uint32_t) * ndense, s);
-    cudaMemsetAsync(sc.lb_stat, 0, sizeof(unsigned long long) * sc.lb_tiles, s);
-    cudaMemsetAsync(sc.words, 0, 4 * sizeof(unsigned int), s);
+    launch_fill(ctx, Fill{{sl.count, sl.cursor, (unsigned *)sc.lb_stat, sc.words},
+                          {(unsigned)ndense, (unsigned)ndense, 2u * (unsigned)sc.lb_tiles, 4u}, {0, 0, 0, 0}}, s);
     return IB_OK;
 }
 
@@ -2022,7 +2038,7 @@ static int run_spread(ib_ctx *ctx, const ib_grid *grid, int M, const double *X, 
     Slots sl;
     SlotScratch sc;
     int *ncompact = nullptr;
-    int rc = slots_alloc<T, KW>(ar, M, (int)ndense, sg.mode, sl, sc, s, false, false);
+    int rc = slots_alloc<T, KW>(ctx, ar, M, (int)ndense, sg.mode, sl, sc, s, false, false);
     if (rc) return rc;
     PhaseTimer tm(ctx, IB_PHASE_SPREAD, s);
     k_prep_spread<T, KER><<<nb, 256, 0, s>>>(g, M, X, F, dV, ms, ctx->status);
@@ -2083,7 +2099,7 @@ static int run_mdf(ib_ctx *ctx, Arena &ar, const CaseTab &ct, const ib_particles
     int2 *lev_slice = nullptr;
     int4 *slices = nullptr;
     if (!atomic) {
-        rc = slots_alloc<T, KW>(ar, M, (int)ndense, sg.mode, sl, sc, s, true, resident);
+        rc = slots_alloc<T, KW>(ctx, ar, M, (int)ndense, sg.mode, sl, sc, s, true, resident);
         if (rc) return rc;
         lev_slice = ar.take<int2>(P + 1);
         // a tile of p pairs has at most p / 32 + 1 slices
@@ -2159,10 +2175,10 @@ static int run_mdf(ib_ctx *ctx, Arena &ar, const CaseTab &ct, const ib_particles
     launch_pdl(k_marker_order, dim3(P < ctx->sm_count * 4 ? P : ctx->sm_count * 4), dim3(256), 0, fs, P,
                (const int *)pp->marker_offset, (const int *)lo.mbase, mperm);
     cudaEventRecord(ctx->fork_ev[3], fs);
-    cudaMemsetAsync(bar.count, 0, 2 * sizeof(unsigned int), s);
-    cudaMemsetAsync(prep_ps.lo, 0x7f, sizeof(int) * 3 * P, s);
-    cudaMemsetAsync(prep_ps.hi, 0x80, sizeof(int) * 3 * P, s);
-    cudaMemsetAsync(prep_ps.done, 0, sizeof(unsigned int) * P, s);
+    // (box bounds far above and far below any cell)
+    launch_fill(ctx, Fill{{bar.count, (unsigned *)prep_ps.lo, (unsigned *)prep_ps.hi, prep_ps.done},
+                          {2u, 3u * (unsigned)P, 3u * (unsigned)P, (unsigned)P},
+                          {0u, 0x7f7f7f7fu, 0x80808080u, 0u}}, s);
     k_prep_particles<T, KER><<<P * kPrepSplit, 256, 0, s>>>(ct, P, pp->Xr, pp->Ur, pp->Wr, pp->marker_offset, mk->R,
                                                  mk->dV, ms, F_out, box_lo, box_dim, part_of, prep_ps,
                                                  ctx->status);
