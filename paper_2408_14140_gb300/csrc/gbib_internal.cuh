@@ -290,7 +290,7 @@ struct ib_ctx {
 namespace gbib {
 // A kernel's resident CTAs per SM at one launch shape (a kernel is always asked
 // for with the same one), its dynamic shared memory limit raised to `smem` on the
-// way; 0 when it cannot be resident.  Both are asked of the driver once per
+// way; 0 when it cannot be resident.  Both are asked of the CUDA runtime once per
 // context and kernel: they took a quarter of a small call's host time.
 int resident_ctas(ib_ctx *ctx, const void *kern, int threads, size_t smem);
 }  // namespace gbib
