@@ -28,6 +28,12 @@
 
 namespace gbib {
 
+// A position along an axis in cells from the first cell's centre (rounded the same
+// wherever it is formed).
+__device__ __forceinline__ double cell_position(double X, double org, double inv_h) {
+    return __fma_rn(__dsub_rn(X, org), inv_h, -0.5);
+}
+
 // A marker's wrapped anchor and its per-axis weights in the pass storage
 // form (FP32, or double-float pairs for FP64 fields).
 template <typename T, int KER>
@@ -36,7 +42,7 @@ __device__ __forceinline__ uint64_t marker_weights(const DevGrid &g, const doubl
     int a[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        const double s = (X[d] - g.org[d]) * g.inv_h - 0.5;
+        const double s = cell_position(X[d], g.org[d], g.inv_h);
         const FirstCell f = axis_weights<KER>(s, g.n[d], w + 4 * d);
         first[d] = f.cell;
         a[d] = f.wrapped;
@@ -172,6 +178,32 @@ struct PrepScratch {
 };
 constexpr int kPrepSplit = 4;    // CTAs per particle
 
+// A particle's box bounds are counted in 32 bits from about its centre's cell.  Of
+// a centre 2^27 cells or more from the origin that cell, and the markers' first
+// cells along the axis, take 64 bits: by these calls, after the markers' loop (in
+// it, and with the loop's arithmetic modulo 2^32 instead, the kernel took 57 to 60
+// us, not 51: other registers, fewer CTAs).  A marker kFar cells or more from its
+// centre makes the box too wide.
+constexpr int kFar = 1 << 28;
+static __device__ __noinline__ long long far_cell(double x, double org, double inv_h) {
+    return (long long)floor((x - org) * inv_h);
+}
+template <int KER>
+static __device__ __noinline__ int2 far_bounds(const double *R, const double *dV, int l0, int l1, int d, double xc, double org,
+                                               double inv_h) {
+    const long long cell = far_cell(xc, org, inv_h);
+    int2 b = make_int2(INT_MAX, INT_MIN);
+    for (int l = l0; l < l1; l += blockDim.x) {
+        const double r = finite3(R + 3 * l) && finite_bits(dV[l]) ? R[3 * l + d] : 0.0;
+        const double s = cell_position(xc + r, org, inv_h);
+        const long long off = (long long)floor(KER == IB_DELTA_ROMA3 ? s + 0.5 : s) - 1 - cell;
+        const bool near = off > -kFar && off < kFar;
+        b.x = min(b.x, near ? (int)off : -2 * kFar);
+        b.y = max(b.y, near ? (int)off + Kernel<KER>::W - 1 : 2 * kFar);
+    }
+    return b;
+}
+
 template <typename T, int KER>
 __global__ void __launch_bounds__(256) k_prep_particles(
     CaseTab ct, int P, const double *__restrict__ Xr, const double *__restrict__ Ur,
@@ -198,14 +230,14 @@ __global__ void __launch_bounds__(256) k_prep_particles(
     const int m0 = moff[p], m1 = moff[p + 1];
     const int nm = m1 - m0;
     const int l0 = m0 + (int)((long long)part * nm / kPrepSplit), l1 = m0 + (int)((long long)(part + 1) * nm / kPrepSplit);
-    // the box bounds are counted from about the particle's centre cell (the same
-    // in all its CTAs), so that they fit 32 bits; a marker further off saturates
-    // (its box is too wide either way)
-    constexpr int kFar = 1 << 28;
-    int cell[3];
+    int cell[3];  // the bounds' base, the same in all of the particle's CTAs
+    bool far = false;
 #pragma unroll
-    for (int d = 0; d < 3; ++d)
-        cell[d] = pok ? max(-kFar, min(kFar, __float2int_rd((df_round(xc[d]) - df_round(g.org[d])) * df_round(g.inv_h)))) : 0;
+    for (int d = 0; d < 3; ++d) {
+        const float c = pok ? (df_round(xc[d]) - df_round(g.org[d])) * df_round(g.inv_h) : 0.0f;
+        far = far || !(fabsf(c) < 0x1p27f);
+        cell[d] = max(-kFar, min(kFar, __float2int_rd(c)));
+    }
     int lo[3] = {INT_MAX, INT_MAX, INT_MAX}, hi[3] = {INT_MIN, INT_MIN, INT_MIN};
     for (int l = l0 + threadIdx.x; l < l1; l += blockDim.x) {
         double r[3] = {R[3 * l], R[3 * l + 1], R[3 * l + 2]};
@@ -239,6 +271,15 @@ __global__ void __launch_bounds__(256) k_prep_particles(
             hi[d] = max(hi[d], off + KW - 1);
         }
     }
+    const bool wide = min(min(lo[0], lo[1]), lo[2]) <= -kFar || max(max(hi[0], hi[1]), hi[2]) >= kFar;
+    if (far || wide) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const int2 b = far ? far_bounds<KER>(R, dV, l0 + threadIdx.x, l1, d, xc[d], g.org[d], g.inv_h)
+                               : make_int2(-2 * kFar, 2 * kFar);
+            lo[d] = b.x, hi[d] = b.y;
+        }
+    }
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
         lo[d] = __reduce_min_sync(0xffffffffu, lo[d]);
@@ -261,10 +302,11 @@ __global__ void __launch_bounds__(256) k_prep_particles(
     }
     __syncthreads();
     if (threadIdx.x == 0 && s_last) {
-        int blo[3], dims[3];
+        long long blo[3];
+        int dims[3];
         for (int d = 0; d < 3; ++d) {
             const int l = atomicAdd(&ps.lo[3 * p + d], 0), h = atomicAdd(&ps.hi[3 * p + d], 0);
-            blo[d] = cell[d] + l;
+            blo[d] = (far ? far_cell(xc[d], g.org[d], g.inv_h) : cell[d]) + l;
             dims[d] = h - l + 1;
         }
         if (m1 > m0) {
