@@ -454,8 +454,9 @@ GBIB_API int particle_volume_integrals_static(const ib_grid *grid, const void *u
  * precision; node (i, j, k) is the lower corner of cell (i, j, k)).  The
  * gradient of a nodal field at a cell centre averages the four node
  * differences across the cell; the divergence of a cell field at a node is
- * its negative adjoint.  The implicit solves are exact in Fourier space, so
- * every n[a] must be a power of two in [16, 1024] (else IB_ERR_UNSUPPORTED).
+ * its negative adjoint.  u, p and u_star may start on any element (16-byte
+ * aligned ones are read faster).  The implicit solves are exact in Fourier
+ * space, so every n[a] must be a power of two in [16, 1024] (else IB_ERR_UNSUPPORTED).
  * Workspace: three half spectra (predictor: n0/2 complex numbers a line in x)
  * or one and a scalar field (projection), and for each spectrum a column of
  * n1 n2 complex numbers beside it.  FP64 fields are transformed in 64-bit fixed

@@ -425,10 +425,14 @@ k_predictor_rhs(LevelDims d, const typename Q::T *__restrict__ u, const typename
 }
 
 // The largest magnitudes (high words) of an FP64 velocity field and a nodal
-// field, into words that are zero before.
+// field, into words that are zero before.  16-byte loads (V double2) where both
+// fields start on 16 bytes; a caller's view that starts on 8 takes V double.
 constexpr int kMaxThreads = 512;
-__global__ void __launch_bounds__(kMaxThreads) k_field_maxima(long long N, const double2 *__restrict__ u,
-                                                              const double2 *__restrict__ p, int *__restrict__ maxima) {
+__device__ __forceinline__ int largest(double v) { return magnitude(v); }
+__device__ __forceinline__ int largest(double2 v) { return max(magnitude(v.x), magnitude(v.y)); }
+template <typename V>
+__global__ void __launch_bounds__(kMaxThreads) k_field_maxima(long long N, const V *__restrict__ u, const V *__restrict__ p,
+                                                              int *__restrict__ maxima) {
     __shared__ int s_max[2];
     if (threadIdx.x < 2) s_max[threadIdx.x] = 0;
     __syncthreads();
@@ -437,14 +441,11 @@ __global__ void __launch_bounds__(kMaxThreads) k_field_maxima(long long N, const
     const long long first = (long long)blockIdx.x * kMaxThreads + threadIdx.x;
 #pragma unroll
     for (int f = 0; f < 2; ++f) {
-        const double2 *v = f ? p : u;
-        const long long n = f ? N / 2 : 3 * (N / 2);
+        const V *v = f ? p : u;
+        const long long n = N * (long long)sizeof(double) / (long long)sizeof(V) * (f ? 1 : 3);
         int x = 0;
 #pragma unroll 8
-        for (long long i = first; i < n; i += step) {
-            const double2 w = v[i];
-            x = max(x, max(magnitude(w.x), magnitude(w.y)));
-        }
+        for (long long i = first; i < n; i += step) x = max(x, largest(v[i]));
         m[f] = __reduce_max_sync(0xffffffffu, x);
     }
     if ((threadIdx.x & 31) == 0) {
@@ -805,7 +806,11 @@ static cudaError_t field_maxima(ib_ctx *ctx, size_t N, const double *u, const do
                                 cudaStream_t s) {
     const cudaError_t e = cudaMemsetAsync(maxima, 0, words * sizeof(int), s);
     if (e != cudaSuccess) return e;
-    k_field_maxima<<<2 * ctx->sm_count, kMaxThreads, 0, s>>>((long long)N, (const double2 *)u, (const double2 *)p, maxima);
+    const dim3 grid(2 * ctx->sm_count);
+    if ((((uintptr_t)u | (uintptr_t)p) & 15) == 0)
+        k_field_maxima<<<grid, kMaxThreads, 0, s>>>((long long)N, (const double2 *)u, (const double2 *)p, maxima);
+    else
+        k_field_maxima<<<grid, kMaxThreads, 0, s>>>((long long)N, u, p, maxima);
     return cudaGetLastError();
 }
 
