@@ -324,23 +324,7 @@ template <typename R> struct LineSymbol {
     __device__ __forceinline__ R inverse(R sz, R cz) const {
         const R d = helmholtz ? fma(q, sz, p) : fma(p, cz, q * sz);
         if (!helmholtz && d <= (R)3e-13) return (R)0;
-        return quotient(scale, d);
-    }
-    __device__ static __forceinline__ float quotient(float a, float d) {
-        if (!(d < 1e37f)) return a / d;
-        const float y = __fdividef(1.0f, d), x = a * y;
-        return fmaf(fmaf(-d, x, a), y, x);
-    }
-    // The FP64 pipe bounds the z pass (16 clocks an operation), so the
-    // reciprocal comes from the 20-bit approximation by one step of third
-    // order, y (1 + e + e^2) with e = 1 - d y, and the quotient's remainder
-    // corrects it: six operations, within an ulp of the division's.
-    __device__ static __forceinline__ double quotient(double a, double d) {
-        if (!(d < 1e300)) return a / d;
-        double y;
-        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-        const double e = fma(-d, y, 1.0), r = fma(y, fma(e, e, e), y), x = a * r;
-        return fma(fma(-d, x, a), r, x);
+        return scale / d;
     }
 };
 
