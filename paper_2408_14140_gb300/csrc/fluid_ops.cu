@@ -103,8 +103,9 @@ template <typename R> struct PlainNum {
 // FP64 fields in 64-bit fixed point: u in units of 2^(eu), p of 2^(ep), so that
 // the field's largest |u| and |p| have 59 bits; differences and sums are then
 // exact, and what a small value loses in its conversion is 2^-60 of the
-// field's largest one.  Products round to one unit.  The FP64 pipe (a warp
-// instruction in 16 clocks of an SM) forms only the final sum.
+// field's largest one.  A product is off by half a unit and the low halves' product
+// that it leaves out: at most 0.75 units in mul<64>, 1.5 in mul<62>, 2.5 in mul<61>.
+// The FP64 pipe (a warp instruction in 16 clocks of an SM) forms only the final sum.
 struct FixedNum {
     using T = double;
     using V = long long;
