@@ -192,13 +192,42 @@ template <int R, bool INV, typename C> __device__ __forceinline__ void radix(C *
 }
 
 // ---------------------------------------------------------------------------
+// a line's scale
+// ---------------------------------------------------------------------------
+// A line's fixed-point units before its first pass and after its last one.  With
+// S the sum of its points' magnitudes and X their largest, no value after passes
+// of radices R1 ... Rk exceeds min(S, R1 ... Rk X); `sum` and a pass's growth
+// are these two as bits above the largest component's exponent, and the unit
+// keeps the smaller one below 2^61.  Lines of 256 points and more start in the
+// unit of their first pass and are shifted, rounded, to the next pass's: S alone
+// left a flat line's points 51 bits of 256 points and 49 of 1024, and the
+// rounding of the input was then 0.9 and 2.6 times an FP64 transform's whole
+// error (now 0.4 and 0.6).  A line of a few large points has S near X, and its
+// shifts are zero.  Shorter lines keep one unit (at most 0.6 times).
+struct LineScale {
+    int first, last, sum;
+};
+template <class A, int LOGN> constexpr bool scaled_passes() { return A::kFixed && LOGN >= 8; }
+// bits of the bound after passes over sub-transforms of length NS; PAIR: the line
+// is the sum of two
+template <bool PAIR> constexpr int growth_bits(int ns) {
+    int l = 0;
+    while ((1 << l) < ns) ++l;
+    return l + (PAIR ? 3 : 2);  // |z| <= sqrt 2 of the larger component, that below 2 of its exponent
+}
+__device__ __forceinline__ longlong2 shift_rounded(longlong2 a, int s) {
+    const long long half = (1LL << s) >> 1;
+    return {(a.x + half) >> s, (a.y + half) >> s};
+}
+
+// ---------------------------------------------------------------------------
 // a line's transform: v[m] is the point t + TPL m on entry and on exit
 // ---------------------------------------------------------------------------
 // `at(p)`: index of the line's point p in the CTA's shared buffer (every
 // thread of the CTA calls this together).
-template <class A, int LOGN, bool INV, int NS, typename At>
+template <class A, int LOGN, bool INV, bool PAIR, int NS, typename At>
 __device__ __forceinline__ void fft_passes(typename A::C *v, int t, typename A::C *sm, At at,
-                                           const typename A::W *__restrict__ tw) {
+                                           const typename A::W *__restrict__ tw, int sum) {
     using C = typename A::C;
     constexpr int N = 1 << LOGN, E = A::points(LOGN), TPL = N / E, R = N / NS < E ? N / NS : E, B = E / R;
 #pragma unroll
@@ -217,6 +246,12 @@ __device__ __forceinline__ void fft_passes(typename A::C *v, int t, typename A::
     }
     static_assert(NS == 1 || twiddle_offset(NS, R) >= 0, "a pass without twiddle factors");
     if constexpr (NS * R < N) {
+        if constexpr (scaled_passes<A, LOGN>()) {
+            constexpr int NEXT = N / (NS * R) < E ? N : NS * R * E;  // the next pass's sub-transforms
+            const int shift = min(sum, growth_bits<PAIR>(NEXT)) - min(sum, growth_bits<PAIR>(NS * R));
+#pragma unroll
+            for (int m = 0; m < E; ++m) v[m] = shift_rounded(v[m], shift);
+        }
         __syncthreads();
 #pragma unroll
         for (int b = 0; b < B; ++b) {
@@ -227,13 +262,14 @@ __device__ __forceinline__ void fft_passes(typename A::C *v, int t, typename A::
         __syncthreads();
 #pragma unroll
         for (int m = 0; m < E; ++m) v[m] = sm[at(t + TPL * m)];
-        fft_passes<A, LOGN, INV, NS * R>(v, t, sm, at, tw);
+        fft_passes<A, LOGN, INV, PAIR, NS * R>(v, t, sm, at, tw, sum);
     }
 }
-template <class A, int LOGN, bool INV, typename At>
+// `sum`: the line's LineScale::sum; PAIR as in its line_scale
+template <class A, int LOGN, bool INV, bool PAIR = false, typename At>
 __device__ __forceinline__ void fft_line(typename A::C *v, int t, typename A::C *sm, At at,
-                                         const typename A::W *__restrict__ tw) {
-    fft_passes<A, LOGN, INV, 1>(v, t, sm, at, tw);
+                                         const typename A::W *__restrict__ tw, int sum) {
+    fft_passes<A, LOGN, INV, PAIR, 1>(v, t, sm, at, tw, sum);
 }
 
 // ---------------------------------------------------------------------------
@@ -315,14 +351,18 @@ template <typename R> __device__ __forceinline__ unsigned bound_of(int mag, int 
     const int d = emax - (e ? e : 1);
     return (m >> (d < 31 ? d : 31)) + 1u;
 }
-// The unit in which points of a summed bound s (each point's larger component)
-// have magnitudes |re| + |im| that add up to at most 2^61.  At least kUnitMin, the
-// finest unit that fixed_of shifts to from the smallest exponent: a line of zeros
-// or subnormals needs none below a subnormal's last bit.
+// The units of a line of points whose summed bound is s (each point's larger
+// component; |re| + |im| add up to twice that at most).  The first is at least
+// kUnitMin, the finest that fixed_of shifts to from the smallest exponent: a line
+// of zeros or subnormals needs none below a subnormal's last bit.
 constexpr int kUnitMin = -61;
-template <typename R> __device__ __forceinline__ int line_unit(int emax, unsigned s) {
-    const int unit = emax - (80 - (32 - __clz((int)s)));
-    return emax == (sizeof(R) == 8 ? 0x7ff : 0xff) ? kUnitNan : (unit < kUnitMin ? kUnitMin : unit);
+template <class A, int LOGN, bool PAIR> __device__ __forceinline__ LineScale line_scale(int emax, unsigned s) {
+    const int sum = (32 - __clz((int)s)) + 1 - 19;
+    const int b0 = scaled_passes<A, LOGN>() ? min(sum, growth_bits<PAIR>(A::points(LOGN))) : sum;
+    const int b1 = scaled_passes<A, LOGN>() ? min(sum, growth_bits<PAIR>(1 << LOGN)) : sum;
+    if (emax == (sizeof(typename A::Real) == 8 ? 0x7ff : 0xff)) return {kUnitNan, kUnitNan, sum};
+    const int first = max(emax + b0 - 62, kUnitMin);
+    return {first, first + b1 - b0, sum};
 }
 
 }  // namespace gbib

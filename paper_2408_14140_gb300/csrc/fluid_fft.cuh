@@ -50,12 +50,12 @@ struct FftGrid {
     const typename A::Mem *trig;                // [kRoots] (cos, sin)(2 pi k / kRoots)
 };
 
-// The unit of a line from its threads' points: mag[] the larger component's
+// The scale of a line from its threads' points: mag[] the larger component's
 // magnitude of each point.  FAST_T: the line's threads are neighbours in the
 // CTA; else `lanes` lines interleave.  slot[0], slot[1]: the lines' words for
 // the maximum and the sum, zero before (unused with FAST_T up to a warp).
-template <class A, int M, int TPL, bool FAST_T>
-__device__ __forceinline__ int points_unit(const int (&mag)[M], int *max_slot, int *sum_slot, int line, int lanes) {
+template <class A, int LOGN, bool PAIR, int M, int TPL, bool FAST_T>
+__device__ __forceinline__ LineScale points_scale(const int (&mag)[M], int *max_slot, int *sum_slot, int line, int lanes) {
     using R = typename A::Real;
     int h = 0;
 #pragma unroll
@@ -87,26 +87,26 @@ __device__ __forceinline__ int points_unit(const int (&mag)[M], int *max_slot, i
         __syncthreads();
         s = (unsigned)sum_slot[line];
     }
-    return line_unit<R>(emax, s);
+    return line_scale<A, LOGN, PAIR>(emax, s);
 }
 
 // A thread's points of a line to the transform's arithmetic and back; returns
-// the line's unit.
-template <class A, int E, int TPL, bool FAST_T>
-__device__ __forceinline__ int points_in(const typename A::Mem (&z)[E], typename A::C (&v)[E], int *max_slot,
+// the line's scale.
+template <class A, int LOGN, int E, int TPL, bool FAST_T>
+__device__ __forceinline__ LineScale points_in(const typename A::Mem (&z)[E], typename A::C (&v)[E], int *max_slot,
                                          int *sum_slot, int line, int lanes) {
     if constexpr (A::kFixed) {
         int mag[E];
 #pragma unroll
         for (int m = 0; m < E; ++m) mag[m] = max(magnitude(z[m].x), magnitude(z[m].y));
-        const int unit = points_unit<A, E, TPL, FAST_T>(mag, max_slot, sum_slot, line, lanes);
+        const LineScale sc = points_scale<A, LOGN, false, E, TPL, FAST_T>(mag, max_slot, sum_slot, line, lanes);
 #pragma unroll
-        for (int m = 0; m < E; ++m) v[m] = typename A::C{to_fixed(z[m].x, unit), to_fixed(z[m].y, unit)};
-        return unit;
+        for (int m = 0; m < E; ++m) v[m] = typename A::C{to_fixed(z[m].x, sc.first), to_fixed(z[m].y, sc.first)};
+        return sc;
     } else {
 #pragma unroll
         for (int m = 0; m < E; ++m) v[m] = typename A::C{z[m].x, z[m].y};
-        return 0;
+        return {0, 0, 0};
     }
 }
 template <class A> __device__ __forceinline__ typename A::Mem point_out(typename A::C v, int unit) {
@@ -163,7 +163,8 @@ k_fft_x(const typename A::Real *__restrict__ src, Spectrum<A> sp, typename A::Re
     auto at = [l](int p) { return l * S::PITCH + p + p / E; };
     grid_dep_wait();
     C v[E];
-    int unit;
+    LineScale sc = {0, 0, 0};
+    constexpr bool kPair = MODE != kXForward;
     if constexpr (MODE == kXForward) {
         Mem z[E];
 #pragma unroll
@@ -171,7 +172,7 @@ k_fft_x(const typename A::Real *__restrict__ src, Spectrum<A> sp, typename A::Re
             const R *r = src + comp + row + t + TPL * m;
             z[m] = Mem{r[0], r[plane]};
         }
-        unit = points_in<A, E, TPL, true>(z, v, s_line[0], s_line[1], l, 0);
+        sc = points_in<A, LOGN, E, TPL, true>(z, v, s_line[0], s_line[1], l, 0);
     } else {
         // Z(k) = A(k) + i B(k), Z(n0 - k) = conj A(k) + i conj B(k); real points
         // at 0 and n0/2.  The sums are formed in the transform's arithmetic.
@@ -187,13 +188,12 @@ k_fft_x(const typename A::Real *__restrict__ src, Spectrum<A> sp, typename A::Re
             mag[2 * m] = max(magnitude(a[m].x), magnitude(a[m].y));
             mag[2 * m + 1] = max(magnitude(b[m].x), magnitude(b[m].y));
         }
-        unit = 0;
-        if constexpr (A::kFixed) unit = points_unit<A, 2 * E, TPL, true>(mag, s_line[0], s_line[1], l, 0);
+        if constexpr (A::kFixed) sc = points_scale<A, LOGN, kPair, 2 * E, TPL, true>(mag, s_line[0], s_line[1], l, 0);
 #pragma unroll
         for (int m = 0; m < E; ++m) {
             if constexpr (A::kFixed) {
-                va[m] = C{to_fixed(a[m].x, unit), to_fixed(a[m].y, unit)};
-                vb[m] = C{to_fixed(b[m].x, unit), to_fixed(b[m].y, unit)};
+                va[m] = C{to_fixed(a[m].x, sc.first), to_fixed(a[m].y, sc.first)};
+                vb[m] = C{to_fixed(b[m].x, sc.first), to_fixed(b[m].y, sc.first)};
             } else {
                 va[m] = C{a[m].x, a[m].y};
                 vb[m] = C{b[m].x, b[m].y};
@@ -201,7 +201,8 @@ k_fft_x(const typename A::Real *__restrict__ src, Spectrum<A> sp, typename A::Re
             v[m] = m >= E / 2 ? C{va[m].x + vb[m].y, vb[m].x - va[m].y} : C{va[m].x - vb[m].y, va[m].y + vb[m].x};
         }
     }
-    fft_line<A, LOGN, MODE != kXForward>(v, t, sm, at, tw);
+    fft_line<A, LOGN, MODE != kXForward, kPair>(v, t, sm, at, tw, sc.sum);
+    const int unit = sc.last;
     grid_dep_launch();
     if constexpr (MODE == kXForward) {
         // separation: the thread's lower points k < n0/2 and their mirrors from
@@ -287,13 +288,13 @@ k_fft_y(Spectrum<A> sp, int logr, int log2, const typename A::W *__restrict__ tw
 #pragma unroll
     for (int m = 0; m < E; ++m) z[m] = active ? cl[(long long)(t + TPL * m) << step] : typename A::Mem{0, 0};
     C v[E];
-    const int unit = points_in<A, E, TPL, false>(z, v, s_line[0], s_line[1], l, LANES);
+    const LineScale sc = points_in<A, LOGN, E, TPL, false>(z, v, s_line[0], s_line[1], l, LANES);
     auto at = [l](int p) { return p * LANES + l; };
-    fft_line<A, LOGN, INV>(v, t, sm, at, tw);
+    fft_line<A, LOGN, INV>(v, t, sm, at, tw, sc.sum);
     grid_dep_launch();
 #pragma unroll
     for (int m = 0; m < E; ++m) {
-        z[m] = point_out<A>(v[m], unit);
+        z[m] = point_out<A>(v[m], sc.last);
         if (active) cl[(long long)(t + TPL * m) << step] = z[m];
     }
 }
@@ -367,12 +368,12 @@ k_fft_z(Spectrum<A> sp, int logr, int log1, SymbolArgs sy, const typename A::W *
 #pragma unroll
     for (int m = 0; m < E; ++m) z[m] = active ? cl[(long long)(t + TPL * m) << shift] : Mem{0, 0};
     C v[E];
-    int unit = points_in<A, E, TPL, false>(z, v, s_line[0], s_line[1], l, LANES);
+    LineScale sc = points_in<A, LOGN, E, TPL, false>(z, v, s_line[0], s_line[1], l, LANES);
     auto at = [l](int p) { return p * LANES + l; };
-    fft_line<A, LOGN, false>(v, t, sm, at, tw);
+    fft_line<A, LOGN, false>(v, t, sm, at, tw, sc.sum);
 #pragma unroll
     for (int m = 0; m < E; ++m) {
-        z[m] = point_out<A>(v[m], unit);
+        z[m] = point_out<A>(v[m], sc.last);
     }
 #pragma unroll
     for (int m = 0; m < E; ++m) {
@@ -380,13 +381,13 @@ k_fft_z(Spectrum<A> sp, int logr, int log1, SymbolArgs sy, const typename A::W *
         const R f = fs[(k <= N / 2 ? k : N - k) * LANES + l];
         z[m] = Mem{f * z[m].x, f * z[m].y};
     }
-    unit = points_in<A, E, TPL, false>(z, v, s_line[2], s_line[3], l, LANES);
-    fft_line<A, LOGN, true>(v, t, sm, at, tw);
+    sc = points_in<A, LOGN, E, TPL, false>(z, v, s_line[2], s_line[3], l, LANES);
+    fft_line<A, LOGN, true>(v, t, sm, at, tw, sc.sum);
     grid_dep_launch();
     if (active) {
 #pragma unroll
         for (int m = 0; m < E; ++m) {
-            z[m] = point_out<A>(v[m], unit);
+            z[m] = point_out<A>(v[m], sc.last);
             cl[(long long)(t + TPL * m) << shift] = z[m];
         }
     }
