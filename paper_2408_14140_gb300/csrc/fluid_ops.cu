@@ -63,20 +63,25 @@ struct RhsArgs {
     double dg[3];        // dt g
 };
 
+// The words of the fields' largest magnitudes (high words): each velocity
+// component's, the pressure's and (projection) p_old - p's.
+enum { kMaxU = 0, kMaxP = 3, kMaxOld = 4, kMaxima = 5 };
+
 // FP32 and FP64 as they stand.  kc: a cell's dt/h u_a; up / down: its states
 // towards the faces above and below, v +- (1 -+ c) m; half_slope: half the
 // monotonized-central slope from the differences a (below) and b (above),
-// min(|a|, |b|, |a + b| / 4) with their sign, 0 at extrema.
+// min(|a|, |b|, |a + b| / 4) with their sign, 0 at extrema; normal: a face's
+// normal velocity u_a as product takes it.  Arguments a and k name the component.
 template <typename R> struct PlainNum {
     using T = R;
     using V = R;
     static constexpr bool kExact = true;  // u() loses nothing
     R k, cc, cg, cl, dg[3];
-    __device__ PlainNum(const RhsArgs &a, int, int)
+    __device__ PlainNum(const RhsArgs &a, const int *)
         : k((R)a.k), cc((R)a.cc), cg((R)a.cg), cl((R)a.cl), dg{(R)a.dg[0], (R)a.dg[1], (R)a.dg[2]} {}
-    __device__ __forceinline__ V u(T x) const { return x; }
+    __device__ __forceinline__ V u(T x, int) const { return x; }
     __device__ __forceinline__ V p(T x) const { return x; }
-    __device__ __forceinline__ V kc(V v) const { return k * v; }
+    __device__ __forceinline__ V kc(V v, int) const { return k * v; }
     __device__ __forceinline__ V up(V v, V c, V m) const { return fma((R)1 - c, m, v); }
     __device__ __forceinline__ V down(V v, V c, V m) const { return fma((R)-1 - c, m, v); }
     __device__ __forceinline__ V half_slope(V a, V b) const {
@@ -94,44 +99,67 @@ template <typename R> struct PlainNum {
     }
     __device__ __forceinline__ bool positive(V x) const { return x > (R)0; }
     __device__ __forceinline__ bool negative(V x) const { return x < (R)0; }
+    __device__ __forceinline__ V normal(V un, int) const { return un; }
     __device__ __forceinline__ V product(V un, V s) const { return un * s; }
-    __device__ __forceinline__ T result(T u0, V lap, V conv, V gp, int c) const {
-        return fma(cl, lap, fma(cc, conv, fma(cg, gp, u0 + dg[c])));
+    __device__ __forceinline__ T result(T u0, V lap, V conv, V gp, int k) const {
+        return fma(cl, lap, fma(cc, conv, fma(cg, gp, u0 + dg[k])));
     }
 };
 
-// FP64 fields in 64-bit fixed point: u in units of 2^(eu), p of 2^(ep), so that
-// the field's largest |u| and |p| have 59 bits; differences and sums are then
-// exact, and what a small value loses in its conversion is 2^-60 of the
-// field's largest one.  A product is off by half a unit and the low halves' product
-// that it leaves out: at most 0.75 units in mul<64>, 1.5 in mul<62>, 2.5 in mul<61>.
-// The FP64 pipe (a warp instruction in 16 clocks of an SM) forms only the final sum.
+// FP64 fields in 64-bit fixed point: each velocity component and p in a unit of
+// its own, in which its largest value has 59 bits (one unit for all three left a component 10^-8 times the largest one's size an error of 2e-9
+// of its values).  Differences and sums are then exact, and what a small value
+// loses in its conversion is 2^-60 of its component's largest one.  A flux is the
+// state in its component's unit times the normal velocity in the largest
+// component's, so that the three axes' fluxes add up.  A product is off by half a
+// unit and the low halves' product that it leaves out: at most 0.75 units in
+// mul<64>, 1.5 in mul<62>, 2.5 in mul<61>.  The FP64 pipe (a warp instruction in
+// 16 clocks of an SM) forms only the final sum.  The CTA keeps it in shared
+// memory: in registers it spilled more.
 struct FixedNum {
     using T = double;
     using V = long long;
     static constexpr bool kExact = false;
     static constexpr int kBits = 59;
-    int eu, ep;
-    Halves kk;           // dt/h in units: c = kk v / 2^62 in Q58
-    double cc, cg, cl;   // with the units' powers of two
-    const double *dg;
-    // the ranges in which no sum overflows: |u| and |p| within 2^(+-400) and a
-    // Courant number dt/h max|u| (of the power of two above the maximum) up to 2
-    __device__ static bool fits(const RhsArgs &a, int mu, int mp) {
-        const int e = exponent_of<double>(mu), f = exponent_of<double>(mp);
-        return abs(e - 1023) <= 400 && (f <= 1 || abs(f - 1023) <= 400) && a.k * pow2(e - 1022) <= 2.0;
+    int unit[3], punit;    // to_fixed's
+    int shift[3];          // from a component's unit to the largest one's,
+    long long half[3];     // and what rounds that
+    Halves kk[3];          // dt/h in units: c = kk v / 2^62 in Q58
+    double cc[3], cl[3], cg;  // with the units' powers of two
+    double dg[3];
+    // the largest component's and a component's exponent (a component of zeros
+    // takes the largest one's unit)
+    __device__ static int largest(const int *m) { return exponent_of<double>(max(max(m[0], m[1]), m[2])); }
+    __device__ static int exponent(const int *m, int k) { return m[k] ? exponent_of<double>(m[k]) : largest(m); }
+    // the ranges in which no sum overflows: the largest |p| and each component's
+    // largest value within 2^(+-400) (or zero), and a Courant number dt/h max|u| (of
+    // the power of two above the maximum) up to 2
+    __device__ static bool fits(const RhsArgs &a, const int *m) {
+        bool in = true;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) in = in && abs(exponent(m + kMaxU, k) - 1023) <= 400;
+        const int f = exponent_of<double>(m[kMaxP]);
+        return in && (f <= 1 || abs(f - 1023) <= 400) && a.k * pow2(largest(m + kMaxU) - 1022) <= 2.0;
     }
     __device__ static double pow2(int e) { return __hiloint2double((e + 1023) << 20, 0); }
-    __device__ FixedNum(const RhsArgs &a, int mu, int mp)
-        : eu(exponent_of<double>(mu)), ep(exponent_of<double>(mp)), dg(a.dg) {
-        const int su = eu - 1022 - kBits, sp = ep > 1 ? ep - 1022 - kBits : 0;
-        kk = halves(__double2ll_rn(a.k * pow2(su) * pow2(58 + 62)));
-        cc = a.cc * pow2(2 * su + 63);
-        cg = ep > 1 ? a.cg * pow2(sp) : 0.0;  // a pressure of 0 (or below 2^-1022)
-        cl = a.cl * pow2(su);
+    __device__ FixedNum(const RhsArgs &a, const int *m) {
+        const int most = largest(m + kMaxU);
+        const int ep = exponent_of<double>(m[kMaxP]);
+        punit = ep - kBits;
+        cg = ep > 1 ? a.cg * pow2(ep - 1022 - kBits) : 0.0;  // a pressure of 0 (or below 2^-1022)
+        for (int k = 0; k < 3; ++k) {
+            const int e = exponent(m + kMaxU, k), su = e - 1022 - kBits;
+            unit[k] = e - kBits;
+            shift[k] = min(most - e, 62);
+            half[k] = (1LL << shift[k]) >> 1;
+            kk[k] = halves(__double2ll_rn(a.k * pow2(su) * pow2(58 + 62)));
+            cc[k] = a.cc * pow2(su + (most - 1022 - kBits) + 63);
+            cl[k] = a.cl * pow2(su);
+            dg[k] = a.dg[k];
+        }
     }
-    __device__ __forceinline__ V u(T x) const { return to_fixed(x, eu - kBits); }
-    __device__ __forceinline__ V p(T x) const { return to_fixed(x, ep - kBits); }
+    __device__ __forceinline__ V u(T x, int k) const { return to_fixed(x, unit[k]); }
+    __device__ __forceinline__ V p(T x) const { return to_fixed(x, punit); }
     // a b / 2^SH, rounded
     template <int SH> __device__ __forceinline__ static V mul(Halves x, Halves y) {
         const long long s = (long long)x.hi * y.hi;
@@ -139,7 +167,7 @@ struct FixedNum {
         return SH == 64 ? s + (t >> 32) : (long long)((unsigned long long)s << (64 - SH)) + (t >> (SH - 32));
     }
     // Q61: the Q58 product shifted (its rounding counts against a slope only)
-    __device__ __forceinline__ V kc(V v) const { return mul<62>(halves(v), kk) << 3; }
+    __device__ __forceinline__ V kc(V v, int a) const { return mul<62>(halves(v), kk[a]) << 3; }
     __device__ __forceinline__ V up(V v, V c, V m) const { return v + mul<61>(halves((1LL << 61) - c), halves(m)); }
     __device__ __forceinline__ V down(V v, V c, V m) const { return v - mul<61>(halves((1LL << 61) + c), halves(m)); }
     __device__ __forceinline__ V half_slope(V a, V b) const {
@@ -151,9 +179,10 @@ struct FixedNum {
     }
     __device__ __forceinline__ bool positive(V x) const { return x > 0; }
     __device__ __forceinline__ bool negative(V x) const { return x < 0; }
+    __device__ __forceinline__ V normal(V un, int a) const { return (un + half[a]) >> shift[a]; }
     __device__ __forceinline__ V product(V un, V s) const { return mul<64>(halves(un << 1), halves(s)); }
-    __device__ __forceinline__ T result(T u0, V lap, V conv, V gp, int c) const {
-        return fma(cl, (double)lap, fma(cc, (double)conv, fma(cg, (double)gp, u0 + dg[c])));
+    __device__ __forceinline__ T result(T u0, V lap, V conv, V gp, int k) const {
+        return fma(cl[k], (double)lap, fma(cc[k], (double)conv, fma(cg, (double)gp, u0 + dg[k])));
     }
 };
 
@@ -164,7 +193,7 @@ __device__ __forceinline__ void upwind_flux(const Q &q, const typename Q::V l[3]
                                             typename Q::V flux[3]) {
     const typename Q::V s = l[a] + r[a];
     const bool up = q.positive(s) && q.positive(l[a]), down = q.negative(s) && q.negative(r[a]);
-    const typename Q::V un = up ? l[a] : (down ? r[a] : 0);
+    const typename Q::V un = q.normal(up ? l[a] : (down ? r[a] : 0), a);
 #pragma unroll
     for (int c = 0; c < 3; ++c) flux[c] = q.product(un, up ? l[c] : r[c]);
 }
@@ -204,7 +233,7 @@ __device__ __forceinline__ typename Q::V states(const Q &q, typename Q::V vm, ty
 }
 
 template <class Q, int TX>
-__device__ __forceinline__ void rhs_tile(const Q q, const LevelDims &d, const typename Q::T *__restrict__ u,
+__device__ __forceinline__ void rhs_tile(const Q &q, const LevelDims &d, const typename Q::T *__restrict__ u,
                                          const typename Q::T *__restrict__ p, const RhsArgs &a,
                                          typename Q::T *__restrict__ out, RhsShared<typename Q::V, TX> &s) {
     using S = RhsTile<TX>;
@@ -252,7 +281,7 @@ __device__ __forceinline__ void rhs_tile(const Q q, const LevelDims &d, const ty
         for (int kk = k0; kk < k1; ++kk) {
 #pragma unroll
             for (int r = 0; r < S::PER; ++r)
-                if (at[r] >= 0) flat[at[r]] = q.u(raw[r]);
+                if (at[r] >= 0) flat[at[r]] = q.u(raw[r], (h + r * S::HALO) / S::ITEMS);
             if (edge) s.p[ey][ex] = q.p(praw);
             __syncthreads();  // A
             if (kk + 1 < k1) {
@@ -265,7 +294,7 @@ __device__ __forceinline__ void rhs_tile(const Q q, const LevelDims &d, const ty
             if (face) {
                 const V vn = b[(ax ? 0 : 1) * CS];
                 V up[3], down[3];
-                const V c = q.kc(vn);
+                const V c = q.kc(vn, ax ? 0 : 1);
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
                     const V *e = b + k * CS;
@@ -273,7 +302,7 @@ __device__ __forceinline__ void rhs_tile(const Q q, const LevelDims &d, const ty
                 }
                 if (low) {
                     V u1[3], d1[3], fl[3];
-                    const V c1 = q.kc(b[(ax ? 0 : 1) * CS + st]);
+                    const V c1 = q.kc(b[(ax ? 0 : 1) * CS + st], ax ? 0 : 1);
 #pragma unroll
                     for (int k = 0; k < 3; ++k) {
                         const V *e = b + k * CS + st;
@@ -300,11 +329,11 @@ __device__ __forceinline__ void rhs_tile(const Q q, const LevelDims &d, const ty
 #pragma unroll
     for (int o = 0; o < 4; ++o)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) z[o][c] = q.u(u[c * N + (size_t)((k0 + o - 2) & m2) * plane + i0]);
+        for (int c = 0; c < 3; ++c) z[o][c] = q.u(u[c * N + (size_t)((k0 + o - 2) & m2) * plane + i0], c);
     s.p[ty][tx] = q.p(p[(size_t)k0 * plane + i0]);
     {
         V l[3], r[3], x;
-        const V cl = q.kc(z[1][2]), cn = q.kc(z[2][2]);
+        const V cl = q.kc(z[1][2], 2), cn = q.kc(z[2][2], 2);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             states(q, z[0][c], z[1][c], z[2][c], cl, l[c], x);
@@ -329,7 +358,7 @@ __device__ __forceinline__ void rhs_tile(const Q q, const LevelDims &d, const ty
         if (kk + 1 < k1) praw = p[(size_t)((kk + 2) & m2) * plane + i0];
         V lap[3], conv[3], ly[3];
         {
-            const V c = q.kc(z[2][1]);
+            const V c = q.kc(z[2][1], 1);
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 V r;
@@ -339,7 +368,7 @@ __device__ __forceinline__ void rhs_tile(const Q q, const LevelDims &d, const ty
         }
         V lx[3], rx[3];
         {
-            const V c = q.kc(z[2][0]);
+            const V c = q.kc(z[2][0], 0);
 #pragma unroll
             for (int k = 0; k < 3; ++k)
                 lap[k] += states(q, s.u[k][ty + 2][tx + 1], z[2][k], s.u[k][ty + 2][tx + 3], c, lx[k], rx[k]);
@@ -381,10 +410,10 @@ __device__ __forceinline__ void rhs_tile(const Q q, const LevelDims &d, const ty
         }
         {
             V r[3], f[3], next[3];
-            const V c = q.kc(z[3][2]);
+            const V c = q.kc(z[3][2], 2);
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                z[4][k] = q.u(far[k]);
+                z[4][k] = q.u(far[k], k);
                 states(q, z[2][k], z[3][k], z[4][k], c, next[k], r[k]);
                 lap[k] += (z[3][k] - z[2][k]) - (z[2][k] - z[1][k]);
             }
@@ -416,13 +445,19 @@ __global__ void __launch_bounds__(RhsTile<TX>::T, MINB)
 k_predictor_rhs(LevelDims d, const typename Q::T *__restrict__ u, const typename Q::T *__restrict__ p, RhsArgs a,
                 const int *__restrict__ maxima, typename Q::T *__restrict__ out) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    auto &sh = *(RhsShared<typename Q::V, TX> *)smem_raw;
     grid_dep_wait();
-    int mu = 0, mp = 0;
     if constexpr (sizeof(typename Q::T) == 8) {
-        mu = maxima[0], mp = maxima[1];
-        if (FixedNum::fits(a, mu, mp) == Q::kExact) return;
+        if (FixedNum::fits(a, maxima) == Q::kExact) return;
     }
-    rhs_tile<Q, TX>(Q(a, mu, mp), d, u, p, a, out, *(RhsShared<typename Q::V, TX> *)smem_raw);
+    if constexpr (Q::kExact) {
+        rhs_tile<Q, TX>(Q(a, maxima), d, u, p, a, out, sh);
+    } else {
+        __shared__ __align__(8) unsigned char s_num[sizeof(Q)];
+        if (threadIdx.x == 0) *(Q *)s_num = Q(a, maxima);
+        __syncthreads();
+        rhs_tile<Q, TX>(*(const Q *)s_num, d, u, p, a, out, sh);
+    }
 }
 
 // The largest magnitudes (high words) of an FP64 velocity field and a nodal
@@ -434,29 +469,27 @@ __device__ __forceinline__ int largest(double2 v) { return max(magnitude(v.x), m
 template <typename V>
 __global__ void __launch_bounds__(kMaxThreads) k_field_maxima(long long N, const V *__restrict__ u, const V *__restrict__ p,
                                                               int *__restrict__ maxima) {
-    __shared__ int s_max[2];
-    if (threadIdx.x < 2) s_max[threadIdx.x] = 0;
+    __shared__ int s_max;
+    if (threadIdx.x == 0) s_max = 0;
     __syncthreads();
-    const long long step = (long long)gridDim.x * kMaxThreads;
-    int m[2] = {0, 0};
-    const long long first = (long long)blockIdx.x * kMaxThreads + threadIdx.x;
-#pragma unroll
-    for (int f = 0; f < 2; ++f) {
-        const V *v = f ? p : u;
-        const long long n = N * (long long)sizeof(double) / (long long)sizeof(V) * (f ? 1 : 3);
-        int x = 0;
+    // blockIdx.y: a velocity component or the pressure
+    const long long step = (long long)gridDim.x * kMaxThreads, n = N * (long long)sizeof(double) / (long long)sizeof(V);
+    const V *const v = blockIdx.y < 3 ? u + blockIdx.y * n : p;
+    int x = 0;
 #pragma unroll 8
-        for (long long i = first; i < n; i += step) x = max(x, largest(v[i]));
-        m[f] = __reduce_max_sync(0xffffffffu, x);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        atomicMax(&s_max[0], m[0]);
-        atomicMax(&s_max[1], m[1]);
-    }
+    for (long long i = (long long)blockIdx.x * kMaxThreads + threadIdx.x; i < n; i += step) x = max(x, largest(v[i]));
+    x = __reduce_max_sync(0xffffffffu, x);
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_max, x);
     __syncthreads();
-    if (threadIdx.x < 2) atomicMax(maxima + threadIdx.x, s_max[threadIdx.x]);
+    static_assert(kMaxU == 0 && kMaxP == 3, "the maxima's order");
+    if (threadIdx.x == 0) atomicMax(maxima + blockIdx.y, s_max);
 }
 
+// The largest |u|'s high word (the linear stencils have one unit for u: their
+// sums mix the components).
+__device__ __forceinline__ int largest_u(const int *maxima) {
+    return max(max(maxima[kMaxU], maxima[kMaxU + 1]), maxima[kMaxU + 2]);
+}
 // Maxima (high words) that the linear stencils' fixed point takes: their unit
 // is a normal double, the values finite; or 0.
 __device__ __forceinline__ bool fixed_range(int a, int b) {
@@ -548,7 +581,7 @@ __global__ void __launch_bounds__(kStencilThreads) k_projection_div(LevelDims d,
         w[0] = wk[y0 + x0], w[1] = wk[y0 + xm], w[2] = wk[ym + x0], w[3] = wk[ym + xm];
     };
     grid_dep_wait();
-    if (sizeof(T) == 8 && fixed_range(maxima[0], maxima[1])) return;  // k_projection_div_fixed
+    if (sizeof(T) == 8 && fixed_range(largest_u(maxima), maxima[kMaxP])) return;  // k_projection_div_fixed
     T am, bm, cm, a0, b0, c0, wm[4];
     DiffSum<T> xym;
     pressure((q.k0 - 1) & m2, am, bm, cm);
@@ -591,7 +624,7 @@ __global__ void __launch_bounds__(kStencilThreads) k_projection_update(LevelDims
         plane_corners(pk[i0], pk[px], pk[py], pk[pxy], gx, gy, s);
     };
     grid_dep_wait();
-    if (sizeof(T) == 8 && fixed_range(maxima[2], 0)) return;  // k_projection_update_fixed
+    if (sizeof(T) == 8 && fixed_range(maxima[kMaxOld], 0)) return;  // k_projection_update_fixed
     T gx0, gy0, s0[4], hx0 = 0, hy0 = 0, r0[4];
     corners(q, o.k0, gx0, gy0, s0);
     if (kTwo) corners(p, o.k0, hx0, hy0, r0);
@@ -651,7 +684,7 @@ k_projection_div_fixed(LevelDims d, const double *__restrict__ u, const double *
     const int ho = ((y0 + hy) & m1) * d.n0 + ((x0 + hx) & m0);
     const double *hsrc = (hc < 3 ? u + hc * N : p) + ho;
     grid_dep_wait();
-    const int mu = maxima[0], mp = maxima[1];
+    const int mu = largest_u(maxima), mp = maxima[kMaxP];
     if (!fixed_range(mu, mp)) return;  // k_projection_div
     const int eu = exponent_of<double>(mu), ep = exponent_of<double>(mp);
     // with the units (a field of zeros has none); the conversions of the two
@@ -710,7 +743,7 @@ k_projection_update_fixed(LevelDims d, double *__restrict__ u, const double *__r
     const int hx = tid <= TY ? TX : tid - TY - 1, hy = tid <= TY ? tid : TY;
     const int ho = ((y0 + hy) & m1) * d.n0 + ((x0 + hx) & m0);
     grid_dep_wait();
-    const int mq = maxima[2];
+    const int mq = maxima[kMaxOld];
     if (!fixed_range(mq, 0)) return;  // k_projection_update
     const int eq = exponent_of<double>(mq);
     double rq, rh = 0, v[3];
@@ -802,12 +835,11 @@ static cudaError_t solve(ib_ctx *ctx, const int n[3], int ncomp, const typename 
     return e;
 }
 
-// Maxima of u and p into the first of `words` zeroed words.
-static cudaError_t field_maxima(ib_ctx *ctx, size_t N, const double *u, const double *p, int *maxima, int words,
-                                cudaStream_t s) {
-    const cudaError_t e = cudaMemsetAsync(maxima, 0, words * sizeof(int), s);
+// Maxima of u and p into their words, the others zero.
+static cudaError_t field_maxima(ib_ctx *ctx, size_t N, const double *u, const double *p, int *maxima, cudaStream_t s) {
+    const cudaError_t e = cudaMemsetAsync(maxima, 0, kMaxima * sizeof(int), s);
     if (e != cudaSuccess) return e;
-    const dim3 grid(2 * ctx->sm_count);
+    const dim3 grid((ctx->sm_count + 1) / 2, 4);
     if ((((uintptr_t)u | (uintptr_t)p) & 15) == 0)
         k_field_maxima<<<grid, kMaxThreads, 0, s>>>((long long)N, (const double2 *)u, (const double2 *)p, maxima);
     else
@@ -840,7 +872,7 @@ static cudaError_t predictor_rhs(ib_ctx *ctx, const LevelDims &d, const float *u
 template <int TX>
 static cudaError_t predictor_rhs(ib_ctx *ctx, const LevelDims &d, const double *u, const double *p, const RhsArgs &a,
                                  int *maxima, double *out, cudaStream_t s) {
-    cudaError_t e = field_maxima(ctx, (size_t)d.n0 * d.n1 * d.n2, u, p, maxima, 2, s);
+    cudaError_t e = field_maxima(ctx, (size_t)d.n0 * d.n1 * d.n2, u, p, maxima, s);
     if (e == cudaSuccess) e = launch_rhs<FixedNum, TX, 2>(ctx, d, u, p, a, maxima, out, s);
     if (e == cudaSuccess) e = launch_rhs<PlainNum<double>, TX, 1>(ctx, d, u, p, a, maxima, out, s);
     return e;
@@ -857,7 +889,7 @@ static int run_predictor(ib_ctx *ctx, const ib_grid *grid, const void *u, const 
     Spectrum<A> c;
     c.c = ar.take<typename A::Mem>(3 * (N / 2));
     c.ny = ar.take<typename A::Mem>(3 * ny);
-    int *maxima = ar.take<int>(2);
+    int *maxima = ar.take<int>(kMaxima);
     if (!ar.ok()) return oom_error(ar.used, ar.cap);
     const StencilGrid sg(ctx, grid->n);
     const RhsArgs a = {dt / h, -dt / h, -dt / (4.0 * h * rho_f), 0.5 * nu * dt / (h * h), {dt * g[0], dt * g[1], dt * g[2]}};
@@ -883,7 +915,7 @@ static int run_projection(ib_ctx *ctx, const ib_grid *grid, void *u, void *p, do
     c.c = ar.take<typename A::Mem>(N / 2);
     c.ny = ar.take<typename A::Mem>((size_t)grid->n[1] * grid->n[2]);
     T *q = ar.take<T>(N);
-    int *maxima = ar.take<int>(3);
+    int *maxima = ar.take<int>(kMaxima);
     if (!ar.ok()) return oom_error(ar.used, ar.cap);
     const StencilGrid sg(ctx, grid->n);
     // p_new = rho_f (D G)^-1 D V   (Eq. ns_lp2 with L p = div((1/rho_f) grad p))
@@ -893,7 +925,7 @@ static int run_projection(ib_ctx *ctx, const ib_grid *grid, void *u, void *p, do
     const double cu = 0.25 / (h * dt), cp = 0.0625 / (h * h * rho_f), cg = dt / (4.0 * h * rho_f);
     const dim3 block1(kStencilThreads);
     if constexpr (sizeof(T) == 8) {
-        e = field_maxima(ctx, N, (const double *)u, (const double *)p, maxima, 3, s);
+        e = field_maxima(ctx, N, (const double *)u, (const double *)p, maxima, s);
         auto k = sg.d.n0 >= 32 ? k_projection_div_fixed<32> : k_projection_div_fixed<16>;
         if (e == cudaSuccess)
             e = launch_pdl(k, sg.grid, block1, 0, s, sg.d, (const double *)u, (const double *)p, cu, cp, maxima, (double *)q);
@@ -901,7 +933,7 @@ static int run_projection(ib_ctx *ctx, const ib_grid *grid, void *u, void *p, do
     if (e == cudaSuccess)
         e = launch_pdl(k_projection_div<T>, sg.grid, sg.block, 0, s, sg.d, (const T *)u, (const T *)p, cu, cp, maxima, q);
     if (e == cudaSuccess)
-        e = solve<typename A::Pressure, A>(ctx, grid->n, 1, q, c, sy, kXPressure, (T *)p, q, maxima + 2, s);
+        e = solve<typename A::Pressure, A>(ctx, grid->n, 1, q, c, sy, kXPressure, (T *)p, q, maxima + kMaxOld, s);
     if constexpr (sizeof(T) == 8) {
         auto k = sg.d.n0 >= 32 ? k_projection_update_fixed<32> : k_projection_update_fixed<16>;
         if (e == cudaSuccess) e = launch_pdl(k, sg.grid, block1, 0, s, sg.d, (double *)u, (const double *)q, cg, maxima);
