@@ -457,11 +457,12 @@ GBIB_API int particle_volume_integrals_static(const ib_grid *grid, const void *u
  * its negative adjoint.  u, p and u_star may start on any element (16-byte
  * aligned ones are read faster).  The implicit solves are exact in Fourier
  * space, so every n[a] must be a power of two in [16, 1024] (else IB_ERR_UNSUPPORTED).
- * Workspace: three half spectra (predictor: n0/2 complex numbers a line in x)
- * or one and a scalar field (projection), and for each spectrum a column of
- * n1 n2 complex numbers beside it.  FP64 fields are transformed in 64-bit fixed
- * point scaled line by line, with errors no larger than an FP64 transform's;
- * fields whose values do not fit it (not finite, or too far apart in magnitude)
+ * Workspace: at most two complex grid fields (predictor), one (projection).  FP64
+ * fields are transformed in 64-bit fixed point scaled line by line, with errors no
+ * larger than FP64 transforms'; the stencils around them hold every velocity
+ * component (predictor; the projection u as a whole) and the pressure in fixed
+ * point of 56 to 59 bits of its largest magnitude.  Fields that do not fit it (not
+ * finite, magnitudes beyond 2^+-400 or a Courant number above 2 in the predictor)
  * take FP64 stencils.
  *
  * fluid_predictor -- Step 1, Eq. (31): writes u_star = u~*,n+1 from

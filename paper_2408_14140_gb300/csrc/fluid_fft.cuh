@@ -37,10 +37,24 @@ struct SymbolArgs {
 };
 
 // The half spectrum of one field: `c` the points kx < n0/2, `ny` those of
-// kx = n0/2; fields follow one another in both.
+// kx = n0/2, one a row; fields follow one another in both.  The points of
+// 2^logg adjacent rows (or of any number, if nylog is 0) lie side by side, a
+// group every 2^(logg + nylog).  The projection keeps them at the start of the
+// right-hand side's rows that the same CTA of the x pass reads, so that it needs
+// no memory beyond two scalar fields (a point in each row instead cost the z pass
+// of 64x64x128 in FP32 2 us of 35 a call).
 template <class A> struct Spectrum {
     typename A::Mem *c, *ny;
+    int logg, nylog;
 };
+// The place of point i of 2^logg side by side, 2^(logg + step) a group.
+__device__ __forceinline__ long long grouped(long long i, int logg, int step) {
+    return ((i >> logg) << (logg + step)) + (i & ((1LL << logg) - 1));
+}
+// Lines (row pairs) of one CTA of the x passes.
+template <class A> __host__ __device__ constexpr int x_lines(int logN) {
+    return (1 << logN) / A::points(logN) >= 128 ? 1 : 128 / ((1 << logN) / A::points(logN));
+}
 
 // The launches (one field, or ncomp fields one after another in memory).
 template <class A>
@@ -126,7 +140,7 @@ enum { kXForward = 0, kXField = 1, kXPressure = 2 };
 
 template <class A, int LOGN> struct XShape {
     static constexpr int N = 1 << LOGN, E = A::points(LOGN), TPL = N / E;
-    static constexpr int LPC = TPL >= 128 ? 1 : 128 / TPL;  // lines (row pairs) of one CTA
+    static constexpr int LPC = x_lines<A>(LOGN);
     static constexpr int T = TPL * LPC;
     static constexpr int PITCH = N + N / E;                 // one point of padding per E: conflict-free writes
     static constexpr size_t smem = (size_t)LPC * PITCH * sizeof(typename A::C);
@@ -139,8 +153,7 @@ template <class A, int LOGN> struct XShape {
 // show in u.
 template <class A, int LOGN, int MODE>
 __global__ void __launch_bounds__(XShape<A, LOGN>::T)
-k_fft_x(const typename A::Real *__restrict__ src, Spectrum<A> sp, typename A::Real *__restrict__ dst,
-        typename A::Real *__restrict__ old, int *__restrict__ maxold, int log1, int log2, const typename A::W *__restrict__ tw) {
+k_fft_x(const typename A::Real *src, Spectrum<A> sp, typename A::Real *__restrict__ dst, typename A::Real *old, int *__restrict__ maxold, int log1, int log2, const typename A::W *__restrict__ tw) {
     using S = XShape<A, LOGN>;
     using C = typename A::C;
     using R = typename A::Real;
@@ -155,7 +168,7 @@ k_fft_x(const typename A::Real *__restrict__ src, Spectrum<A> sp, typename A::Re
     const long long row = ((line >> log1) * 2 * n1 + (line & (n1 - 1))) << LOGN;  // of plane 2z'
     const long long comp = (long long)blockIdx.y << (LOGN + log1 + log2);
     Mem *ca = sp.c + ((comp + row) >> 1), *cb = ca + (plane >> 1);  // the two rows' half spectra
-    Mem *na = sp.ny + ((comp + row) >> LOGN), *nb = na + n1;         // and their points n0/2
+    Mem *na = sp.ny + grouped((comp + row) >> LOGN, sp.logg, sp.nylog), *nb = na + (n1 << sp.nylog);  // and their points n0/2
     if (A::kFixed && TPL > 32) {
         if (threadIdx.x < 2 * S::LPC) (&s_line[0][0])[threadIdx.x] = 0;
         __syncthreads();
@@ -275,8 +288,8 @@ k_fft_y(Spectrum<A> sp, int logr, int log2, const typename A::W *__restrict__ tw
     const bool last = (int)blockIdx.x >= regular;
     const int q = (last ? (int)blockIdx.x - regular : (int)blockIdx.x) * LANES + l;
     const bool active = !last || q < 1 << log2;
-    const int step = last ? 0 : logr;  // log2 of the points' stride
-    typename A::Mem *cl = last ? sp.ny + ((long long)blockIdx.y << (LOGN + log2)) + ((long long)q << LOGN)
+    const int step = last ? sp.nylog : logr;  // log2 of the points' stride (grouped in the last lines)
+    typename A::Mem *cl = last ? sp.ny + ((((long long)blockIdx.y << log2) + q) << (LOGN + sp.nylog))
                                : sp.c + ((long long)blockIdx.y << (LOGN + logr + log2)) +
                                      ((long long)(q >> logr) << (LOGN + logr)) + (q & ((1 << logr) - 1));
     if (A::kFixed) {
@@ -286,7 +299,10 @@ k_fft_y(Spectrum<A> sp, int logr, int log2, const typename A::W *__restrict__ tw
     grid_dep_wait();
     typename A::Mem z[E];
 #pragma unroll
-    for (int m = 0; m < E; ++m) z[m] = active ? cl[(long long)(t + TPL * m) << step] : typename A::Mem{0, 0};
+    for (int m = 0; m < E; ++m) z[m] = last ? typename A::Mem{0, 0} : cl[(long long)(t + TPL * m) << step];
+    if (last && active)
+#pragma unroll
+        for (int m = 0; m < E; ++m) z[m] = cl[grouped(t + TPL * m, sp.logg, step)];
     C v[E];
     const LineScale sc = points_in<A, LOGN, E, TPL, false>(z, v, s_line[0], s_line[1], l, LANES);
     auto at = [l](int p) { return p * LANES + l; };
@@ -295,8 +311,11 @@ k_fft_y(Spectrum<A> sp, int logr, int log2, const typename A::W *__restrict__ tw
 #pragma unroll
     for (int m = 0; m < E; ++m) {
         z[m] = point_out<A>(v[m], sc.last);
-        if (active) cl[(long long)(t + TPL * m) << step] = z[m];
+        if (!last) cl[(long long)(t + TPL * m) << step] = z[m];
     }
+    if (last && active)
+#pragma unroll
+        for (int m = 0; m < E; ++m) cl[grouped(t + TPL * m, sp.logg, step)] = z[m];
 }
 
 // ---- z: forward, symbol, inverse --------------------------------------------
@@ -349,8 +368,8 @@ k_fft_z(Spectrum<A> sp, int logr, int log1, SymbolArgs sy, const typename A::W *
     const int q = (last ? (int)blockIdx.x - regular : (int)blockIdx.x) * LANES + l;
     const bool active = !last || q < 1 << log1;
     const int kx = last ? 1 << logr : q & ((1 << logr) - 1), ky = last ? q & ((1 << log1) - 1) : q >> logr;
-    const int shift = last ? log1 : logr + log1;  // log2 of the points' stride
-    Mem *cl = (last ? sp.ny : sp.c) + ((long long)blockIdx.y << (LOGN + shift)) + q;
+    const int shift = last ? log1 + sp.nylog : logr + log1;  // log2 of the points' stride
+    Mem *cl = (last ? sp.ny + grouped(q, sp.logg, sp.nylog) : sp.c + q) + ((long long)blockIdx.y << (LOGN + shift));
     if (A::kFixed)
         for (int i = threadIdx.x; i < 4 * LANES; i += S::T) (&s_line[0][0])[i] = 0;
     {

@@ -66,6 +66,7 @@ struct RhsArgs {
 // The words of the fields' largest magnitudes (high words): each velocity
 // component's, the pressure's and (projection) p_old - p's.
 enum { kMaxU = 0, kMaxP = 3, kMaxOld = 4, kMaxima = 5 };
+static_assert(kMaxima <= FftTables::kWords, "a fluid call's words");
 
 // FP32 and FP64 as they stand.  kc: a cell's dt/h u_a; up / down: its states
 // towards the faces above and below, v +- (1 -+ c) m; half_slope: half the
@@ -826,7 +827,7 @@ static cudaError_t solve(ib_ctx *ctx, const int n[3], int ncomp, const typename 
                          cudaStream_t s) {
     const FftGrid<X> gx = fft_grid<X>(ctx, n);
     const FftGrid<A> g = fft_grid<A>(ctx, n);
-    const Spectrum<X> cx = {c.c, c.ny};
+    const Spectrum<X> cx = {c.c, c.ny, c.logg, c.nylog};
     cudaError_t e = fft_x<X>(kXForward, gx, ncomp, src, cx, nullptr, nullptr, nullptr, s);
     if (e == cudaSuccess) e = fft_y<A>(false, g, ncomp, c, s);
     if (e == cudaSuccess) e = fft_z<A>(g, ncomp, c, sy, s);
@@ -889,7 +890,8 @@ static int run_predictor(ib_ctx *ctx, const ib_grid *grid, const void *u, const 
     Spectrum<A> c;
     c.c = ar.take<typename A::Mem>(3 * (N / 2));
     c.ny = ar.take<typename A::Mem>(3 * ny);
-    int *maxima = ar.take<int>(kMaxima);
+    c.logg = c.nylog = 0;
+    int *const maxima = ctx->fft_tab->words;
     if (!ar.ok()) return oom_error(ar.used, ar.cap);
     const StencilGrid sg(ctx, grid->n);
     const RhsArgs a = {dt / h, -dt / h, -dt / (4.0 * h * rho_f), 0.5 * nu * dt / (h * h), {dt * g[0], dt * g[1], dt * g[2]}};
@@ -913,9 +915,12 @@ static int run_projection(ib_ctx *ctx, const ib_grid *grid, void *u, void *p, do
     Arena ar(ctx);
     Spectrum<A> c;
     c.c = ar.take<typename A::Mem>(N / 2);
-    c.ny = ar.take<typename A::Mem>((size_t)grid->n[1] * grid->n[2]);
     T *q = ar.take<T>(N);
-    int *maxima = ar.take<int>(kMaxima);
+    c.ny = (typename A::Mem *)q;  // (see Spectrum)
+    c.nylog = ilog2_exact(grid->n[0]) - 1;
+    const int lines = x_lines<typename A::Pressure>(c.nylog + 1);
+    c.logg = ilog2_exact(lines < grid->n[1] ? lines : grid->n[1]);
+    int *const maxima = ctx->fft_tab->words;
     if (!ar.ok()) return oom_error(ar.used, ar.cap);
     const StencilGrid sg(ctx, grid->n);
     // p_new = rho_f (D G)^-1 D V   (Eq. ns_lp2 with L p = div((1/rho_f) grad p))

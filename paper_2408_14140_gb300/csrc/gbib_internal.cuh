@@ -236,11 +236,14 @@ constexpr int kTwiddles = twiddle_offset(0, 1);  // the table's length
 
 // Tables of the fluid step's transforms: twiddle factors (cos, -sin) in FP32
 // and as balanced Q62 halves (re hi, re lo, im hi, im lo), and (cos, sin)(2 pi
-// k / 2048) in both field types for the operators' symbols.
+// k / 2048) in both field types for the operators' symbols; and the words of a
+// fluid call (a context's calls do not overlap).
 struct FftTables {
+    static constexpr int kWords = 8;
     float2 tw32[kTwiddles], trig32[2048];
     int4 tw_fx[kTwiddles];
     double2 trig64[2048];
+    int words[kWords];
 };
 // Device copy of the tables (nullptr and a CUDA error on failure); `s` is a
 // stream of the context's, waited for.
