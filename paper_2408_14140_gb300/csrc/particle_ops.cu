@@ -188,6 +188,20 @@ __device__ __forceinline__ void volume_tables(VolTables &tb, const DevGrid &g, c
             tb.plane_off[k] = (long long)wrap_int(lo[2] + k, g.n[2]) * g.n[1] * g.n[0];
     }
 }
+// The square of the distance R + off h from a particle's centre, or below = -1
+// (lower bounds) or 0 (upper ones) where that is not positive; and the FP32 bound
+// of squares from it, with a relative margin far above their rounding (lower
+// bounds below, upper ones above).  k_volume and k_volume_plan both tell the cells
+// of alpha 1 apart by the first: the roundings are explicit, so that a cell is
+// inside for both or for neither.
+constexpr double kInside = -0.8661, kOutside = 0.8661;  // in h: past a cell's half diagonal
+__device__ __forceinline__ double bound_sq(double R, double off, double h, double below) {
+    const double b = __fma_rn(off, h, R);
+    return b > 0.0 ? __dmul_rn(b, b) : below;
+}
+__device__ __forceinline__ float lower_bound32(double sq) { return sq < 0.0 ? -1.0f : __fmul_rn((float)sq, 1.0f - 1e-5f); }
+__device__ __forceinline__ float upper_bound32(double sq) { return __fmul_rn((float)sq, 1.0f + 1e-5f); }
+
 // squared distance of a cell's centre from X_r in FP32 (one order everywhere)
 __device__ __forceinline__ float centre_sq(float xy, float z) { return __fadd_rn(xy, z); }
 
@@ -482,16 +496,14 @@ __global__ void __launch_bounds__(kVolThreads, 3) k_volume(CaseTab ct, int P, in
             }
             // squares of the bounds: cells surely inside, cells of alpha 0, the
             // node shell (a lane a bound)
-            const double off = lane == 0 ? -0.8661 : lane == 1 ? 0.8661 : lane == 2 ? -1.75 : 1.75;
-            const double b = R0 + off * g.h;
+            const double off = lane == 0 ? kInside : lane == 1 ? kOutside : lane == 2 ? -1.75 : 1.75;
             if (lane < 4) {
-                // in FP32 with a relative margin far above the rounding of the
-                // squares (the nodes and cells that matter lie 0.01 h inside the
-                // node shell and 8e-5 h inside the cell bounds); cells in the
-                // margin take the corner formula, exact for them too
-                const double sq = b > 0.0 ? b * b : (lane == 0 ? -1.0 : 0.0);
+                // (the nodes and cells that matter lie 0.01 h inside the node shell and
+                // 8e-5 h inside the cell bounds; cells in the FP32 margin take the corner
+                // formula, exact for them too)
+                const double sq = bound_sq(R0, off, g.h, lane == 0 ? -1.0 : 0.0);
                 s_sq[lane] = sq;
-                s_fsq[lane] = sq < 0.0 ? -1.0f : (float)sq * (lane & 1 ? 1.0f + 1e-5f : 1.0f - 1e-5f);
+                s_fsq[lane] = lane & 1 ? upper_bound32(sq) : lower_bound32(sq);
             }
             const double ir = 1.0 / R0;
             if (lane == 0) s_iR = ir, s_iRf = df_split_rn(ir);
@@ -765,8 +777,7 @@ __global__ void __launch_bounds__(kVolThreads, 2) k_volume_plan(CaseTab ct, int 
             okk = __all_sync(0xffffffffu, !(d > g.n[a] || d > kVolMaxBox || l < INT_MIN / 2 || l > INT_MAX / 2));
             __syncwarp();
             if (okk && (long long)s_box[3] * s_box[4] * s_box[5] > pl.cap) okk = false;  // not kept (reported then)
-            const double b = R0 - 0.8661 * g.h;
-            if (lane == 0) s_rin2 = b > 0.0 ? (float)(b * b) * (1.0f - 1e-5f) : -1.0f;
+            if (lane == 0) s_rin2 = lower_bound32(bound_sq(R0, kInside, g.h, -1.0));
         }
         if (lane == 0) s_box[6] = okk;
     }
