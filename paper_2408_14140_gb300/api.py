@@ -200,6 +200,9 @@ def make_grid(n, h, origin=(0.0, 0.0, 0.0), prec=IB_F64) -> Grid:
 class Context:
     """Owns one ``ib_ctx`` (device workspace + error latch)."""
 
+    # launch choices accepted without effect (see autotune.py)
+    INERT_CHOICES = ("gather_stage",)
+
     def __init__(self, workspace_bytes: int = 0):
         self.lib = load()
         h = ctypes.c_void_p()

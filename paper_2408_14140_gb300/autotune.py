@@ -10,8 +10,10 @@ laid out on the GPU, never the results:
 * ``volume_split``: the CTAs per particle of the volume integrals (slabs of
   cell planes; 0: one resident wave) -- the same sums, grouped differently;
 * ``gather_ctas``: resident wavefront-gather CTAs per SM (0: as many as fit);
-* ``gather_stage``: a knob the gather accepts without effect (it stages
-  nothing in shared memory).  Both gather choices leave every sum unchanged.
+* ``gather_stage``: accepted (stored choices name it) and without effect, as
+  the gather stages nothing in shared memory: a context names such choices in
+  ``INERT_CHOICES``, and they keep their default untimed.  Both gather choices
+  leave every sum unchanged.
 
 :func:`tune` times a caller-supplied step (the call sequence of the
 workload) on the device -- CUDA events on the current stream, warm-up steps
@@ -70,11 +72,14 @@ def tune(ctxs, step, space: dict | None = None, sweeps: int = 2, **timing) -> di
     """Coordinate descent over `space` (default :data:`SPACE`) on the
     contexts `ctxs` with `step`; set and return the fastest choice.
 
+    A choice that every context names inert is not varied.
+
     Returns {"choice": {...}, "ms": best, "table": [(choice, ms), ...]} with
     one table row per distinct combination timed.
     """
     space = SPACE if space is None else space
     best = {k: (DEFAULT[k] if DEFAULT.get(k) in v else v[0]) for k, v in space.items()}
+    inert = set.intersection(*(set(getattr(c, "INERT_CHOICES", ())) for c in ctxs)) if ctxs else set()
     seen: dict[tuple, float] = {}
 
     def measure(choice):
@@ -88,7 +93,7 @@ def tune(ctxs, step, space: dict | None = None, sweeps: int = 2, **timing) -> di
     for _ in range(sweeps):
         changed = False
         for k, values in space.items():
-            for v in values:
+            for v in values if k not in inert else ():
                 cand = dict(best, **{k: v})
                 ms = measure(cand)
                 if ms < best_ms:
