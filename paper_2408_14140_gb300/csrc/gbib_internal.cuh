@@ -19,8 +19,6 @@ constexpr int kRow = kTile + 3;
 constexpr int kRows = kRow * kRow;
 // Largest candidate list one tile may gather from.
 constexpr int kMaxCand = 4096;
-// Bounded spin of device-side waits (iterations of ~100 ns sleeps).
-constexpr long long kSpinLimit = 20LL * 1000 * 1000;
 
 struct DevGrid {
     int n[3];

@@ -347,11 +347,6 @@ namespace gbib {
 template <typename T> struct TileStage;
 template <> struct TileStage<float> { static constexpr int N = 256; };
 
-template <typename T>
-constexpr size_t tile_stage_bytes() {
-    return (size_t)TileStage<T>::N * 16 * sizeof(T);
-}
-
 // One tile (compact slot cs) of a gather phase over its per-cell lists: the
 // tile's candidate weights and sources are staged in shared memory (sw
 // [N][12], sA [N][4]) when they fit, then each thread takes band cells and
