@@ -12,8 +12,8 @@ laid out on the GPU, never the results:
 * ``gather_ctas``: resident wavefront-gather CTAs per SM (0: as many as fit);
 * ``gather_stage``: accepted (stored choices name it) and without effect, as
   the gather stages nothing in shared memory: a context names such choices in
-  ``INERT_CHOICES``, and they keep their default untimed.  Both gather choices
-  leave every sum unchanged.
+  ``INERT_CHOICES``, and combinations that differ in them alone share one
+  timing.  Both gather choices leave every sum unchanged.
 
 :func:`tune` times a caller-supplied step (the call sequence of the
 workload) on the device -- CUDA events on the current stream, warm-up steps
@@ -72,28 +72,31 @@ def tune(ctxs, step, space: dict | None = None, sweeps: int = 2, **timing) -> di
     """Coordinate descent over `space` (default :data:`SPACE`) on the
     contexts `ctxs` with `step`; set and return the fastest choice.
 
-    A choice that every context names inert is not varied.
-
     Returns {"choice": {...}, "ms": best, "table": [(choice, ms), ...]} with
-    one table row per distinct combination timed.
+    one table row per distinct combination; those that differ only in choices
+    that every context names inert are timed once.
     """
     space = SPACE if space is None else space
     best = {k: (DEFAULT[k] if DEFAULT.get(k) in v else v[0]) for k, v in space.items()}
     inert = set.intersection(*(set(getattr(c, "INERT_CHOICES", ())) for c in ctxs)) if ctxs else set()
     seen: dict[tuple, float] = {}
+    timed: dict[tuple, float] = {}
 
     def measure(choice):
         key = tuple(sorted(choice.items()))
         if key not in seen:
-            apply(ctxs, choice)
-            seen[key] = time_step(step, **timing)
+            effect = tuple(kv for kv in key if kv[0] not in inert)
+            if effect not in timed:
+                apply(ctxs, choice)
+                timed[effect] = time_step(step, **timing)
+            seen[key] = timed[effect]
         return seen[key]
 
     best_ms = measure(best)
     for _ in range(sweeps):
         changed = False
         for k, values in space.items():
-            for v in values if k not in inert else ():
+            for v in values:
                 cand = dict(best, **{k: v})
                 ms = measure(cand)
                 if ms < best_ms:
