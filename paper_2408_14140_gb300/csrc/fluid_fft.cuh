@@ -323,6 +323,7 @@ template <class A, int LOGN> struct ZShape {
     static constexpr int N = 1 << LOGN, E = A::points(LOGN), TPL = N / E;
     static constexpr int L0 = A::lanes(LOGN), LANES = L0 * TPL >= 128 ? L0 : 128 / TPL;
     static constexpr int T = TPL * LANES;
+    static constexpr int MINB = (A::kFixed ? 896 : 768) / T;  // 28 warps (24) an SM: 72 registers (80)
     static constexpr size_t points = (size_t)LANES * N * sizeof(typename A::C);
     static constexpr size_t smem = points + (size_t)(N / 2 + 1) * LANES * sizeof(typename A::Real);
 };
@@ -349,7 +350,7 @@ template <typename R> struct LineSymbol {
 };
 
 template <class A, int LOGN>
-__global__ void __launch_bounds__(ZShape<A, LOGN>::T)
+__global__ void __launch_bounds__(ZShape<A, LOGN>::T, ZShape<A, LOGN>::MINB)
 k_fft_z(Spectrum<A> sp, int logr, int log1, SymbolArgs sy, const typename A::W *__restrict__ tw,
         const typename A::Mem *__restrict__ trig) {
     using S = ZShape<A, LOGN>;
