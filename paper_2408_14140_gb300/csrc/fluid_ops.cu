@@ -72,7 +72,10 @@ static_assert(kMaxima <= FftTables::kWords, "a fluid call's words");
 // towards the faces above and below, v +- (1 -+ c) m; half_slope: half the
 // monotonized-central slope from the differences a (below) and b (above),
 // min(|a|, |b|, |a + b| / 4) with their sign, 0 at extrema; normal: a face's
-// normal velocity u_a as product takes it.  Arguments a and k name the component.
+// normal velocity u_a as product takes it; result: the increment is formed first
+// and u0 takes one rounding, by the varying sum (dt g alone added to u0 rounds the
+// same way in every cell of a binade: the mean velocity then drifts by up to half
+// its last bit a step).  Arguments a and k name the component.
 template <typename R> struct PlainNum {
     using T = R;
     using V = R;
@@ -103,7 +106,7 @@ template <typename R> struct PlainNum {
     __device__ __forceinline__ V normal(V un, int) const { return un; }
     __device__ __forceinline__ V product(V un, V s) const { return un * s; }
     __device__ __forceinline__ T result(T u0, V lap, V conv, V gp, int k) const {
-        return fma(cl, lap, fma(cc, conv, fma(cg, gp, u0 + dg[k])));
+        return u0 + fma(cl, lap, fma(cc, conv, fma(cg, gp, dg[k])));
     }
 };
 
@@ -183,7 +186,7 @@ struct FixedNum {
     __device__ __forceinline__ V normal(V un, int a) const { return (un + half[a]) >> shift[a]; }
     __device__ __forceinline__ V product(V un, V s) const { return mul<64>(halves(un << 1), halves(s)); }
     __device__ __forceinline__ T result(T u0, V lap, V conv, V gp, int k) const {
-        return fma(cl[k], (double)lap, fma(cc[k], (double)conv, fma(cg, (double)gp, u0 + dg[k])));
+        return u0 + fma(cl[k], (double)lap, fma(cc[k], (double)conv, fma(cg, (double)gp, dg[k])));
     }
 };
 
